@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "ds_internal.h"
+#include "step64.h"
 #include "tc.h"
 
 namespace ds {
@@ -163,8 +164,32 @@ ds_status check_grid(const ds_grid *g)
 }
 
 
+// Sums whose intermediates share 2 GiB: above that a phase fills the GPU
+// several times over and gains nothing from more products.
+int ops_in_budget(int tensors_per_op, int64_t N, int ops)
+{
+    if (tensors_per_op == 0) return 0;
+    const int64_t fit = ((int64_t)2 << 30) / ((int64_t)sizeof(double) * tensors_per_op * N);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(fit, ops));
+}
+
 // the precisions with FX operands (scales calibrated per state)
 bool is_fx(int prec) { return prec == DS_PREC_F16X10 || prec == DS_PREC_F16X13; }
+
+// the bands of component c's (tridiagonal) matrices
+Stencil stencil_of(const ds_phi_set *s, int c)
+{
+    Stencil t;
+    t.d = s->d;
+    for (int mu = 0; mu < kMaxD; ++mu) {
+        t.n[mu] = mu < s->d ? s->n[mu] : 1;
+        const double *base = s->tri_dev + (mu < s->d ? s->tri_off[c][mu] : 0);
+        t.lo[mu] = base;
+        t.di[mu] = base + t.n[mu];
+        t.up[mu] = base + 2 * t.n[mu];
+    }
+    return t;
+}
 
 bool is_tridiagonal(const double *A, int64_t n)
 {
@@ -196,7 +221,11 @@ struct ds_plan {
     std::map<double *, cudaGraphExec_t> graphs;
     int64_t launches = 0;
     tc::MixedPlan *mixed = nullptr;       // tensor-core path state
-    double *bws = nullptr;                // adjoint workspace (24 N doubles), lazily allocated
+    Sums64 sums;                          // FP64 plans: the step's Tucker sums
+    bool lean = false;                    // the workspace holds one sum on F at a time
+    double *bws = nullptr;                // adjoint workspace, lazily allocated
+    Sums64 bsums, tsums;                  // its sums; those of the diffusion-scaling gradient
+    double *tws = nullptr;                // their intermediates
     Prof prof;                            // optional per-launch event timing
     bool profiling = false;               // ds_step records events when set
     const double *fx_state = nullptr;     // FX plans: the state the scales were last set for
@@ -205,82 +234,55 @@ struct ds_plan {
 
 namespace {
 
-// acc (+)= w sum_i eta_i T(X_c, {P[c][slot][i][mu]}) (FP64 path); with
-// transpose the matrices are P^T (the adjoint operator S^T).
-int tucker_sum_f64x(ds_plan *p, int c, int slot, const double *X, double *acc, double w, bool accumulate,
-                    int transpose, double *t1, double *t2, cudaStream_t st)
+// F = K U + g(U): the stencil where every A is tridiagonal, else dense products
+int rhs_f64(ds_plan *p, const Sums64 &e, const double *U, double *F, cudaStream_t st)
 {
-    const ds_phi_set *s = p->set;
-    const int d = s->d;
-    const SplitCoeffs &co = s->co[s->scheme == DS_ETD2RKDS ? slot : kSlotEll[slot] - 1];
-    int launches = 0;
-    for (int i = 0; i < co.k; ++i) {
-        const double *in = X;
-        for (int mu = 0; mu < d; ++mu) {
-            const double *L = s->P_dev + s->P_off[c][slot][i][mu];
-            const bool last = (mu == d - 1);
-            double *out = last ? acc : ((mu % 2 == 0) ? t1 : t2);
-            p->prof.begin(st, 1, 2.0 * (double)p->N * (double)s->n[mu]);
-            launch_mode_product_f64(d, s->n, in, mu, L, transpose, out, last ? w * co.eta[i] : 1.0,
-                                    (last && (i > 0 || accumulate)) ? 1.0 : 0.0, st);
-            p->prof.end(st);
-            ++launches;
-            in = out;
-        }
-    }
-    return launches;
-}
-
-// Enqueue sum_i eta_i T(X_c, {P[c][slot][i][mu]}) into acc (FP64 path).
-int tucker_sum_f64(ds_plan *p, int c, int slot, const double *X, double *acc, double *t1,
-                   double *t2, cudaStream_t st)
-{
-    return tucker_sum_f64x(p, c, slot, X, acc, 1.0, false, 0, t1, t2, st);
-}
-
-// F = K U + g(U) with dense mode products (A not tridiagonal)
-int rhs_dense_f64(const ds_plan *p, const double *U, double *F, cudaStream_t st)
-{
-    const ds_phi_set *s = p->set;
-    int launches = 0;
-    for (int c = 0; c < 2; ++c)
-        for (int mu = 0; mu < s->d; ++mu) {
-            launch_mode_product_f64(s->d, s->n, U + c * p->N, mu, s->A_dev + s->A_off[c][mu], 0,
-                                    F + c * p->N, 1.0, mu > 0 ? 1.0 : 0.0, st);
-            ++launches;
-        }
+    if (p->set->tridiag[0] && p->set->tridiag[1]) return launch_rhs_f64(p->sten, p->model, p->N, U, F, st);
+    const int L = run_kronsum(e, U, F, 0, &p->prof, st);
     launch_add_g_f64(p->model, p->N, U, F, st);
-    return launches + 1;
+    return L + 1;
 }
 
+// out_q = S_q(X_c) of both components for the listed slots: out[q] + c N
+int sums_f64(ds_plan *p, const Sums64 &e, SumKind kind, int nslots, const int *slots, const double *X,
+             double *const *out, bool accumulate, cudaStream_t st)
+{
+    SumOp ops[2 * kSlots];
+    int n = 0;
+    for (int c = 0; c < 2; ++c)
+        for (int q = 0; q < nslots; ++q) ops[n++] = {c, slots[q], X + c * p->N, out[q] + c * p->N, accumulate};
+    return run_sums(e, kind, ops, n, &p->prof, st);
+}
+int sum_f64(ds_plan *p, const Sums64 &e, SumKind kind, int slot, const double *X, double *out, bool accumulate,
+            cudaStream_t st)
+{
+    return sums_f64(p, e, kind, 1, &slot, X, &out, accumulate, st);
+}
+
+// The three-stage schemes (real and complex splits, dense EXPRK3).  The sums
+// on F of all stages run together, unless the workspace holds only one.
 int enqueue_step_f64(ds_plan *p, double *U, cudaStream_t st)
 {
     const int64_t N = p->N;
     const double tau = p->set->tau;
-    double *F = p->ws, *a = p->ws + 2 * N, *b = p->ws + 4 * N, *D = p->ws + 6 * N;
-    double *t1 = p->ws + 8 * N, *t2 = p->ws + 9 * N;
-    int L = 0;
-    if (p->set->tridiag[0] && p->set->tridiag[1])
-        L += launch_rhs_f64(p->sten, p->model, N, U, F, st);
-    else
-        L += rhs_dense_f64(p, U, F, st);
+    double *F = p->ws, *b = p->ws + 2 * N, *D = p->ws + 4 * N, *a = p->ws + 6 * N;
+    double *as[3] = {a, a + (p->lean ? 0 : 2 * N), a + (p->lean ? 0 : 4 * N)};
+    const int slots[3] = {0, 1, 3};
+    const Sums64 &e = p->sums;
+    int L = rhs_f64(p, e, U, F, st);
     // stage U_{n2}
-    for (int c = 0; c < 2; ++c) L += tucker_sum_f64(p, c, 0, F + c * N, a + c * N, t1, t2, st);
-    launch_stage_diff_f64(p->model, N, U, a, kSlotW[0] * tau, nullptr, 0.0, D, st);
+    L += sums_f64(p, e, SumKind::plain, p->lean ? 1 : 3, slots, F, as, false, st);
+    launch_stage_diff_f64(p->model, N, U, as[0], kSlotW[0] * tau, nullptr, 0.0, D, st);
     ++L;
     // stage U_{n3}
-    for (int c = 0; c < 2; ++c) {
-        L += tucker_sum_f64(p, c, 1, F + c * N, a + c * N, t1, t2, st);
-        L += tucker_sum_f64(p, c, 2, D + c * N, b + c * N, t1, t2, st);
-    }
-    launch_stage_diff_f64(p->model, N, U, a, kSlotW[1] * tau, b, kSlotW[2] * tau, D, st);
+    if (p->lean) L += sum_f64(p, e, SumKind::plain, 1, F, a, false, st);
+    L += sum_f64(p, e, SumKind::plain, 2, D, b, false, st);
+    launch_stage_diff_f64(p->model, N, U, as[1], kSlotW[1] * tau, b, kSlotW[2] * tau, D, st);
     ++L;
     // final approximation
-    for (int c = 0; c < 2; ++c) {
-        L += tucker_sum_f64(p, c, 3, F + c * N, a + c * N, t1, t2, st);
-        L += tucker_sum_f64(p, c, 4, D + c * N, b + c * N, t1, t2, st);
-    }
-    launch_final_f64(N, U, a, kSlotW[3] * tau, b, kSlotW[4] * tau, st);
+    if (p->lean) L += sum_f64(p, e, SumKind::plain, 3, F, a, false, st);
+    L += sum_f64(p, e, SumKind::plain, 4, D, b, false, st);
+    launch_final_f64(N, U, as[2], kSlotW[3] * tau, b, kSlotW[4] * tau, st);
     ++L;
     return L;
 }
@@ -344,89 +346,31 @@ int enqueue_step_f32(ds_plan *p, double *U, cudaStream_t st)
     return L;
 }
 
-// Complex scheme (FP64): acc = Re(sum_i eta_i T(X_c, {P_i{mu}})) for real X,
-// with complex P = Pr + i Pi.  Mode 1: two real products; middle modes: four;
-// the last mode two, against the matrices with Re(eta .) folded in.
-int tucker_sum_cplx(ds_plan *p, int c, int slot, const double *X, double *acc, double *w4,
-                    cudaStream_t st)
-{
-    const ds_phi_set *s = p->set;
-    const int d = s->d;
-    const int64_t N = p->N;
-    double *Yr = w4, *Yi = w4 + N, *Zr = w4 + 2 * N, *Zi = w4 + 3 * N;
-    int L = 0;
-    auto mp = [&](const double *in, int mu, const double *M, double *out, double alpha, double beta) {
-        p->prof.begin(st, 1, 2.0 * (double)N * (double)s->n[mu]);
-        launch_mode_product_f64(d, s->n, in, mu, M, 0, out, alpha, beta, st);
-        p->prof.end(st);
-        ++L;
-    };
-    for (int i = 0; i < s->k; ++i) {
-        const int64_t o0 = s->P_off[c][slot][i][0];
-        mp(X, 0, s->P_dev + o0, Yr, 1.0, 0.0);
-        mp(X, 0, s->Pim_dev + o0, Yi, 1.0, 0.0);
-        for (int mu = 1; mu < d - 1; ++mu) {
-            const int64_t o = s->P_off[c][slot][i][mu];
-            mp(Yr, mu, s->P_dev + o, Zr, 1.0, 0.0);
-            mp(Yi, mu, s->Pim_dev + o, Zr, -1.0, 1.0);
-            mp(Yr, mu, s->Pim_dev + o, Zi, 1.0, 0.0);
-            mp(Yi, mu, s->P_dev + o, Zi, 1.0, 1.0);
-            std::swap(Yr, Zr);
-            std::swap(Yi, Zi);
-        }
-        const double *M = s->Mf_dev + s->Mf_off[c][slot][i];
-        const int64_t nn = s->n[d - 1] * s->n[d - 1];
-        mp(Yr, d - 1, M, acc, 1.0, i > 0 ? 1.0 : 0.0);
-        mp(Yi, d - 1, M + nn, acc, 1.0, 1.0);
-    }
-    return L;
-}
-
-int enqueue_step_cplx_f64(ds_plan *p, double *U, cudaStream_t st)
-{
-    const int64_t N = p->N;
-    const double tau = p->set->tau;
-    double *F = p->ws, *a = p->ws + 2 * N, *b = p->ws + 4 * N, *D = p->ws + 6 * N, *w4 = p->ws + 8 * N;
-    int L = 0;
-    if (p->set->tridiag[0] && p->set->tridiag[1])
-        L += launch_rhs_f64(p->sten, p->model, N, U, F, st);
-    else
-        L += rhs_dense_f64(p, U, F, st);
-    for (int c = 0; c < 2; ++c) L += tucker_sum_cplx(p, c, 0, F + c * N, a + c * N, w4, st);
-    launch_stage_diff_f64(p->model, N, U, a, kSlotW[0] * tau, nullptr, 0.0, D, st);
-    ++L;
-    for (int c = 0; c < 2; ++c) {
-        L += tucker_sum_cplx(p, c, 1, F + c * N, a + c * N, w4, st);
-        L += tucker_sum_cplx(p, c, 2, D + c * N, b + c * N, w4, st);
-    }
-    launch_stage_diff_f64(p->model, N, U, a, kSlotW[1] * tau, b, kSlotW[2] * tau, D, st);
-    ++L;
-    for (int c = 0; c < 2; ++c) {
-        L += tucker_sum_cplx(p, c, 3, F + c * N, a + c * N, w4, st);
-        L += tucker_sum_cplx(p, c, 4, D + c * N, b + c * N, w4, st);
-    }
-    launch_final_f64(N, U, a, kSlotW[3] * tau, b, kSlotW[4] * tau, st);
-    ++L;
-    return L;
-}
-
 // ETD2RKDS (FP64): U2 = U + tau T(F, phi_1), U <- U2 + tau 2^(d-1) T(g(U2) - G, phi_2)
 int enqueue_step_etd2_f64(ds_plan *p, double *U, cudaStream_t st)
 {
     const int64_t N = p->N;
     const double tau = p->set->tau;
-    double *F = p->ws, *a = p->ws + 2 * N, *b = p->ws + 4 * N, *D = p->ws + 6 * N;
-    double *t1 = p->ws + 8 * N, *t2 = p->ws + 9 * N;
-    int L = 0;
-    if (p->set->tridiag[0] && p->set->tridiag[1])
-        L += launch_rhs_f64(p->sten, p->model, N, U, F, st);
-    else
-        L += rhs_dense_f64(p, U, F, st);
-    for (int c = 0; c < 2; ++c) L += tucker_sum_f64(p, c, 0, F + c * N, a + c * N, t1, t2, st);
+    double *F = p->ws, *b = p->ws + 2 * N, *D = p->ws + 4 * N, *a = p->ws + 6 * N;
+    const Sums64 &e = p->sums;
+    // small products run one per launch on the FP64 pipe
+    auto sum = [&](int slot, const double *X, double *out) {
+        int L = 0;
+        bool digits = true;
+        for (int mu = 0; mu < p->set->d; ++mu) digits = digits && mm::use_digits(N / p->set->n[mu], (int)p->set->n[mu], 2);
+        if (digits) return sum_f64(p, e, SumKind::plain, slot, X, out, false, st);
+        for (int c = 0; c < 2; ++c) {
+            const SumOp op = {c, slot, X + c * N, out + c * N, false};
+            L += run_sums(e, SumKind::plain, &op, 1, &p->prof, st);
+        }
+        return L;
+    };
+    int L = rhs_f64(p, e, U, F, st);
+    L += sum(0, F, a);
     launch_stage_diff_f64(p->model, N, U, a, tau, nullptr, 0.0, D, st);
     ++L;
-    // tucker_sum applies eta = 2^(d-1) of the phi_2 term
-    for (int c = 0; c < 2; ++c) L += tucker_sum_f64(p, c, 1, D + c * N, b + c * N, t1, t2, st);
+    // the sum carries eta = 2^(d-1) of the phi_2 term
+    L += sum(1, D, b);
     launch_final_f64(N, U, a, tau, b, tau, st);
     ++L;
     return L;
@@ -438,8 +382,6 @@ int enqueue_step(ds_plan *p, double *U, cudaStream_t st, bool profile, bool cali
     int L;
     if (p->set->scheme == DS_ETD2RKDS)
         L = enqueue_step_etd2_f64(p, U, st);
-    else if (p->set->scheme == DS_EXPRK3DS_CPLX)
-        L = enqueue_step_cplx_f64(p, U, st);
     else if (p->prec == DS_PREC_F64)
         L = enqueue_step_f64(p, U, st);
     else if (p->prec == DS_PREC_F32)
@@ -760,14 +702,21 @@ ds_status ds_tucker(const ds_grid *grid, const double *X, double *Y, const doubl
         return DS_OK;
     }
     if (precision != DS_PREC_F64) return fail(DS_ERR_UNSUPPORTED, "unknown precision");
+    size_t scratch = 0;
+    for (int mu = 0; mu < d; ++mu)
+        if (mm::use_digits(N / grid->n[mu], (int)std::min<int64_t>(grid->n[mu], INT32_MAX), 1))
+            scratch = std::max(scratch, mm::scratch_bytes(N, grid->n[mu], 1, 1, true));
+    mm::Context c;
     double *tmp = nullptr;
-    DS_CUDA_TRY(cudaMallocAsync(&tmp, sizeof(double) * N * 2, st));
-    const double *in = X;
-    for (int mu = 0; mu < d; ++mu) {
-        double *out = (mu == d - 1) ? Y : tmp + (mu % 2) * N;
-        launch_mode_product_f64(d, grid->n, in, mu, L[mu], transpose, out, 1.0, 0.0, st);
-        in = out;
+    const size_t tb = mm::aligned(sizeof(double) * N * 2);
+    if (scratch && cudaMallocAsync(&tmp, tb + scratch, st) == cudaSuccess) {
+        c.ws = (uint8_t *)tmp + tb;
+        c.ws_bytes = scratch;
+    } else {
+        cudaGetLastError();
+        DS_CUDA_TRY(cudaMallocAsync(&tmp, tb, st));   // short of memory: the FP64 pipe
     }
+    tucker_f64(c, d, grid->n, X, Y, L, transpose, tmp, st);
     cudaFreeAsync(tmp, st);
     DS_CUDA_TRY(cudaGetLastError());
     return DS_OK;
@@ -777,9 +726,20 @@ ds_status ds_kronsum(const ds_phi_set *s, int c, const double *X, double *Y, voi
 {
     if (!s || !X || !Y || c < 0 || c > 1) return fail(DS_ERR_INVALID_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    for (int mu = 0; mu < s->d; ++mu)
-        launch_mode_product_f64(s->d, s->n, X, mu, s->A_dev + s->A_off[c][mu], 0, Y, 1.0,
-                                mu > 0 ? 1.0 : 0.0, st);
+    if (s->tridiag[c]) {
+        int64_t N = 1;
+        for (int mu = 0; mu < s->d; ++mu) N *= s->n[mu];
+        launch_kronsum_f64(stencil_of(s, c), N, X, Y, st);
+    } else {
+        for (int mu = 0; mu < s->d; ++mu) {
+            mm::Product p{};
+            p.A = mm::tensor_view(s->d, s->n, mu, X);
+            p.B = mm::matrix_view(s->n[mu], s->A_dev + s->A_off[c][mu], 0);
+            p.out = Y;
+            p.accumulate = mu > 0;
+            mm::launch_products_fma(&p, 1, st);
+        }
+    }
     DS_CUDA_TRY(cudaGetLastError());
     return DS_OK;
 }
@@ -811,16 +771,7 @@ ds_status ds_plan_create(const ds_grid *grid, const ds_params *params, const ds_
         p->model.model = params->model;
         for (int q = 0; q < 8; ++q) p->model.p[q] = params->p[q];
         p->set = set;
-        for (int c = 0; c < 2; ++c) {
-            p->sten[c].d = set->d;
-            for (int mu = 0; mu < kMaxD; ++mu) {
-                p->sten[c].n[mu] = mu < set->d ? set->n[mu] : 1;
-                const double *base = set->tri_dev + (mu < set->d ? set->tri_off[c][mu] : 0);
-                p->sten[c].lo[mu] = base;
-                p->sten[c].di[mu] = base + p->sten[c].n[mu];
-                p->sten[c].up[mu] = base + 2 * p->sten[c].n[mu];
-            }
-        }
+        for (int c = 0; c < 2; ++c) p->sten[c] = stencil_of(set, c);
         auto cleanup = [&](ds_status st, const char *m) { ds_plan_destroy(p); return fail(st, m); };
         if (cudaStreamCreateWithFlags(&p->st, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&p->ev_in, cudaEventDisableTiming) != cudaSuccess ||
@@ -830,11 +781,26 @@ ds_status ds_plan_create(const ds_grid *grid, const ds_params *params, const ds_
             return cleanup(DS_ERR_OOM, "status word");
         cudaMemset(p->status, 0, sizeof(DevStatus));
         if (precision == DS_PREC_F64) {
-            p->ws_count = (set->scheme == DS_EXPRK3DS_CPLX ? 12 : 10) * p->N;
+            // F, b, D, the sums on F (one pair of tensors each) and the
+            // intermediates; short of memory: one sum at a time, term by term
+            const bool etd2 = set->scheme == DS_ETD2RKDS;
+            const int per_op = sum_tensors(set, SumKind::plain), nf = etd2 ? 1 : 3;
+            int64_t zt = (int64_t)per_op * ops_in_budget(per_op, p->N, 2 * nf);
+            p->ws_count = (6 + 2 * nf + zt) * p->N;
             if (cudaMalloc(&p->ws, sizeof(double) * p->ws_count) != cudaSuccess) {
                 cudaGetLastError();
-                return cleanup(DS_ERR_OOM, "FP64 workspace");
+                p->lean = true;
+                zt = per_op / set->k;
+                p->ws_count = (8 + zt) * p->N;
+                if (cudaMalloc(&p->ws, sizeof(double) * p->ws_count) != cudaSuccess) {
+                    cudaGetLastError();
+                    return cleanup(DS_ERR_OOM, "FP64 workspace");
+                }
             }
+            std::vector<SumGroup> groups;
+            if (etd2) groups = {{SumKind::plain, {0}}, {SumKind::plain, {1}}};
+            else groups = {{SumKind::plain, {0, 1, 3}}, {SumKind::plain, {2}}, {SumKind::plain, {4}}};
+            sums_create(p->sums, set, p->N, groups, p->ws + (p->ws_count - zt * p->N), zt, p->status, p->st);
         } else if (precision == DS_PREC_F32) {
             if (!set->tridiag[0] || !set->tridiag[1])
                 return cleanup(DS_ERR_UNSUPPORTED, "reduced-precision paths need tridiagonal A_mu (use DS_PREC_F64)");
@@ -937,26 +903,6 @@ ds_status ds_integrate_ckpt(ds_plan *p, double *U, int64_t nsteps, int64_t ckpt_
     return DS_OK;
 }
 
-// dscale[c] += w sum_i eta_i sum_mu < lam_s_c, T(X_c, P with P_mu -> dP_mu) >
-static void dscale_family(ds_plan *p, int c, int slot, const double *X, const double *lam_s, double w,
-                          double *out, double *t1, double *t2, double *dscale, cudaStream_t st)
-{
-    const ds_phi_set *s = p->set;
-    const int d = s->d;
-    const SplitCoeffs &co = s->co[kSlotEll[slot] - 1];
-    for (int i = 0; i < co.k; ++i)
-        for (int md = 0; md < d; ++md) {
-            const double *in = X;
-            for (int mu = 0; mu < d; ++mu) {
-                const double *L = (mu == md ? s->dP_dev : s->P_dev) + s->P_off[c][slot][i][mu];
-                double *o = (mu == d - 1) ? out : ((mu % 2 == 0) ? t1 : t2);
-                launch_mode_product_f64(d, s->n, in, mu, L, 0, o, 1.0, 0.0, st);
-                in = o;
-            }
-            launch_dot_accum_f64(p->N, lam_s, out, w * co.eta[i], dscale + c, st);
-        }
-}
-
 ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, double *lam_n, double *dparams,
                            double *dscale, void *stream)
 {
@@ -965,71 +911,94 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
     if (p->prec != DS_PREC_F64) return fail(DS_ERR_UNSUPPORTED, "the adjoint step needs an FP64 plan");
     if (p->set->scheme != DS_EXPRK3DS_REAL) return fail(DS_ERR_UNSUPPORTED, "the adjoint covers EXPRK3DS_REAL");
     const int64_t N = p->N;
+    const ds_phi_set *s = p->set;
     if (!p->bws) {
-        cudaError_t e = cudaMalloc(&p->bws, sizeof(double) * 24 * N);
-        if (e != cudaSuccess) {
+        const int per_op = sum_tensors(s, SumKind::plain);
+        int64_t zt = (int64_t)per_op * ops_in_budget(per_op, N, 4);
+        if (cudaMalloc(&p->bws, sizeof(double) * (22 + zt) * N) != cudaSuccess) {
             cudaGetLastError();
-            p->bws = nullptr;
-            return fail(DS_ERR_OOM, "adjoint workspace");
+            zt = per_op / s->k;
+            if (cudaMalloc(&p->bws, sizeof(double) * (22 + zt) * N) != cudaSuccess) {
+                cudaGetLastError();
+                p->bws = nullptr;
+                return fail(DS_ERR_OOM, "adjoint workspace");
+            }
         }
+        sums_create(p->bsums, s, N,
+                    {{SumKind::plain, {0, 1}}, {SumKind::plain, {2}}, {SumKind::transposed, {3, 4}},
+                     {SumKind::transposed, {1, 2}}, {SumKind::transposed, {0}}},
+                    p->bws + 22 * N, zt, p->status, p->st);
+    }
+    if (dscale && !p->tws) {
+        const int per_op = sum_tensors(s, SumKind::tangent);
+        int64_t zt = (int64_t)per_op * ops_in_budget(per_op, N, 6);
+        if (cudaMalloc(&p->tws, sizeof(double) * (6 + zt) * N) != cudaSuccess) {
+            cudaGetLastError();
+            zt = per_op / s->k;
+            if (cudaMalloc(&p->tws, sizeof(double) * (6 + zt) * N) != cudaSuccess) {
+                cudaGetLastError();
+                p->tws = nullptr;
+                return fail(DS_ERR_OOM, "adjoint workspace");
+            }
+        }
+        sums_create(p->tsums, s, N,
+                    {{SumKind::tangent, {0, 1, 3}}, {SumKind::tangent, {2}}, {SumKind::tangent, {4}}},
+                    p->tws + 6 * N, zt, p->status, p->st);
     }
     cudaStream_t st = (cudaStream_t)stream;
-    const double tau = p->set->tau;
+    const double tau = s->tau;
     double *F = p->bws, *a = F + 2 * N, *b = F + 4 * N, *D2 = F + 6 * N, *U2 = F + 8 * N, *U3 = F + 10 * N;
     double *lF = F + 12 * N, *lD3 = F + 14 * N, *lD2 = F + 16 * N, *lU3 = F + 18 * N, *lU2 = F + 20 * N;
-    double *t1 = F + 22 * N, *t2 = F + 23 * N;
     const Model &m = p->model;
-    const bool tri = p->set->tridiag[0] && p->set->tridiag[1];
-    // forward recomputation of F, U2, D2, U3
-    if (tri)
-        launch_rhs_f64(p->sten, m, N, U, F, st);
-    else
-        rhs_dense_f64(p, U, F, st);
-    for (int c = 0; c < 2; ++c) tucker_sum_f64(p, c, 0, F + c * N, a + c * N, t1, t2, st);
+    const bool tri = s->tridiag[0] && s->tridiag[1];
+    const Sums64 &e = p->bsums;
+    // forward recomputation of F, U2, D2, U3 (S_3^{(1)}(F) waits in lD3's place)
+    rhs_f64(p, e, U, F, st);
+    {
+        const int q[2] = {0, 1};
+        double *out[2] = {a, lD3};
+        sums_f64(p, e, SumKind::plain, 2, q, F, out, false, st);
+    }
     launch_axpy2_f64(N, U, a, kSlotW[0] * tau, nullptr, 0.0, U2, st);
     launch_gdiff_f64(m, N, U, U2, D2, st);
-    for (int c = 0; c < 2; ++c) {
-        tucker_sum_f64(p, c, 1, F + c * N, a + c * N, t1, t2, st);
-        tucker_sum_f64(p, c, 2, D2 + c * N, b + c * N, t1, t2, st);
-    }
-    launch_axpy2_f64(N, U, a, kSlotW[1] * tau, b, kSlotW[2] * tau, U3, st);
+    sum_f64(p, e, SumKind::plain, 2, D2, b, false, st);
+    launch_axpy2_f64(N, U, lD3, kSlotW[1] * tau, b, kSlotW[2] * tau, U3, st);
     // reverse sweep
-    for (int c = 0; c < 2; ++c) {
-        tucker_sum_f64x(p, c, 3, lam + c * N, lF + c * N, kSlotW[3] * tau, false, 1, t1, t2, st);
-        tucker_sum_f64x(p, c, 4, lam + c * N, lD3 + c * N, kSlotW[4] * tau, false, 1, t1, t2, st);
+    {
+        const int q[2] = {3, 4};
+        double *out[2] = {lF, lD3};
+        sums_f64(p, e, SumKind::transposed, 2, q, lam, out, false, st);
     }
     launch_jacT_f64(m, N, U3, lD3, lU3, st);
-    for (int c = 0; c < 2; ++c) {
-        tucker_sum_f64x(p, c, 1, lU3 + c * N, lF + c * N, kSlotW[1] * tau, true, 1, t1, t2, st);
-        tucker_sum_f64x(p, c, 2, lU3 + c * N, lD2 + c * N, kSlotW[2] * tau, false, 1, t1, t2, st);
-    }
+    sum_f64(p, e, SumKind::transposed, 1, lU3, lF, true, st);
+    sum_f64(p, e, SumKind::transposed, 2, lU3, lD2, false, st);
     launch_jacT_f64(m, N, U2, lD2, lU2, st);
-    for (int c = 0; c < 2; ++c)
-        tucker_sum_f64x(p, c, 0, lU2 + c * N, lF + c * N, kSlotW[0] * tau, true, 1, t1, t2, st);
+    sum_f64(p, e, SumKind::transposed, 0, lU2, lF, true, st);
     if (dscale) {
-        // through K (F = s K U + G) and through every phi-matrix; a and b are
-        // free after U3: b <- D3 = g(U3) - g(U), a holds one Tucker output
+        // through K (F = s K U + G) and through every phi-matrix: the tangent of
+        // each sum against the adjoint of its stage; b <- D3 = g(U3) - g(U)
         launch_dot_kterm_f64(m, N, U, F, lF, dscale, st);
         launch_gdiff_f64(m, N, U, U3, b, st);
-        for (int c = 0; c < 2; ++c) {
-            const double *Fc = F + c * N;
-            double *o = a + c * N;
-            dscale_family(p, c, 0, Fc, lU2 + c * N, kSlotW[0] * tau, o, t1, t2, dscale, st);
-            dscale_family(p, c, 1, Fc, lU3 + c * N, kSlotW[1] * tau, o, t1, t2, dscale, st);
-            dscale_family(p, c, 2, D2 + c * N, lU3 + c * N, kSlotW[2] * tau, o, t1, t2, dscale, st);
-            dscale_family(p, c, 3, Fc, lam + c * N, kSlotW[3] * tau, o, t1, t2, dscale, st);
-            dscale_family(p, c, 4, b + c * N, lam + c * N, kSlotW[4] * tau, o, t1, t2, dscale, st);
-        }
+        double *o[3] = {p->tws, p->tws + 2 * N, p->tws + 4 * N};
+        auto dot = [&](int slot, const double *t, const double *adj) {
+            for (int c = 0; c < 2; ++c)
+                launch_dot_accum_f64(N, adj + c * N, t + c * N, kSlotW[slot] * tau, dscale + c, st);
+        };
+        const int q[3] = {0, 1, 3};
+        sums_f64(p, p->tsums, SumKind::tangent, 3, q, F, o, false, st);
+        dot(0, o[0], lU2);
+        dot(1, o[1], lU3);
+        dot(3, o[2], lam);
+        sum_f64(p, p->tsums, SumKind::tangent, 2, D2, o[0], false, st);
+        sum_f64(p, p->tsums, SumKind::tangent, 4, b, o[1], false, st);
+        dot(2, o[0], lU3);
+        dot(4, o[1], lam);
     }
     // K^T lam_F into F's storage
     if (tri) {
         launch_kronsumT_f64(p->sten, N, lF, F, st);
     } else {
-        for (int c = 0; c < 2; ++c)
-            for (int mu = 0; mu < p->set->d; ++mu)
-                launch_mode_product_f64(p->set->d, p->set->n, lF + c * N, mu,
-                                        p->set->A_dev + p->set->A_off[c][mu], 1, F + c * N, 1.0,
-                                        mu > 0 ? 1.0 : 0.0, st);
+        run_kronsum(e, lF, F, 1, &p->prof, st);
     }
     launch_adjoint_final_f64(m, N, U, U2, U3, lam, lU3, lU2, F, lF, lD2, lD3, lam_n, dparams, st);
     DS_CUDA_TRY(cudaGetLastError());
@@ -1495,6 +1464,10 @@ ds_status ds_plan_destroy(ds_plan *p)
     if (p->mixed) tc::mixed_plan_destroy(p->mixed);
     cudaFree(p->ws);
     cudaFree(p->bws);
+    cudaFree(p->tws);
+    sums_destroy(p->sums);
+    sums_destroy(p->bsums);
+    sums_destroy(p->tsums);
     cudaFree(p->ws32);
     cudaFree(p->P32);
     cudaFree(p->status);

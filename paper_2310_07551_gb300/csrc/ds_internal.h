@@ -48,15 +48,7 @@ ds_status check_device();
                               std::string(#expr) + ": " + cudaGetErrorString(_e));   \
     } while (0)
 
-// Strided batched FP64 GEMM: C[b] = alpha * A[b] B[b] + beta * C[b] ------
-struct DGemm {
-    int M, N, K, batch;
-    const double *A; int64_t sAm, sAk, sAb;
-    const double *B; int64_t sBk, sBn, sBb;
-    double *C; int64_t sCm, sCn, sCb;
-    double alpha, beta;
-};
-void launch_dgemm(const DGemm &g, cudaStream_t st);
+// Strided batched FP32 GEMM: C[b] = alpha * A[b] B[b] + beta * C[b] ------
 struct SGemm {
     int M, N, K, batch;
     const float *A; int64_t sAm, sAk, sAb;
@@ -67,11 +59,6 @@ struct SGemm {
 void launch_sgemm(const SGemm &g, cudaStream_t st);
 void launch_mode_product_f32(int d, const int64_t *n, const float *X, int mu, const float *L,
                              int transpose, float *Y, double alpha, double beta, cudaStream_t st);
-
-// One FP64 mu-mode product Y = X x_mu L (+ beta Y), any mode, as a GEMM.
-// L column-major n_mu x n_mu; transpose uses L^T.
-void launch_mode_product_f64(int d, const int64_t *n, const double *X, int mu, const double *L,
-                             int transpose, double *Y, double alpha, double beta, cudaStream_t st);
 
 // Reaction model ---------------------------------------------------------
 struct Model {
@@ -89,6 +76,8 @@ struct Stencil {
 // F = K U + g(U) for both components (FP64, stencil).  Returns #launches.
 int launch_rhs_f64(const Stencil *st2, const Model &m, int64_t N, const double *U, double *F,
                    cudaStream_t st);
+// Y = K X for one component (tridiagonal A)
+void launch_kronsum_f64(const Stencil &s, int64_t N, const double *X, double *Y, cudaStream_t st);
 // D = g(U + w1 a (+ w2 b)) - g(U); b may be null.
 void launch_stage_diff_f64(const Model &m, int64_t N, const double *U, const double *a, double w1,
                            const double *b, double w2, double *D, cudaStream_t st);

@@ -6,7 +6,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "ds_internal.h"
+#include "mm64.h"
 
 namespace ds {
 
@@ -87,13 +87,6 @@ __global__ void __launch_bounds__(256) k_gemm(G g)
 }
 }  // namespace
 
-void launch_dgemm(const DGemm &g, cudaStream_t st)
-{
-    if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
-    dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
-    k_gemm<double, DGemm><<<grid, 256, 0, st>>>(g);
-}
-
 void launch_sgemm(const SGemm &g, cudaStream_t st)
 {
     if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
@@ -160,12 +153,6 @@ void launch_mode_product_f32(int d, const int64_t *n, const float *X, int mu, co
     mode_product<SGemm, float>(d, n, X, mu, L, transpose, Y, alpha, beta, launch_sgemm, st);
 }
 
-void launch_mode_product_f64(int d, const int64_t *n, const double *X, int mu, const double *L,
-                             int transpose, double *Y, double alpha, double beta, cudaStream_t st)
-{
-    mode_product<DGemm, double>(d, n, X, mu, L, transpose, Y, alpha, beta, launch_dgemm, st);
-}
-
 // ---------------------------------------------------------------------------
 // Reaction terms (Section 3 models).
 // ---------------------------------------------------------------------------
@@ -205,6 +192,12 @@ __device__ __forceinline__ double stencil_point(const Stencil &s, const double *
         }
     }
     return acc;
+}
+
+__global__ void k_kronsum_f64(Stencil s, int64_t N, const double *__restrict__ X, double *__restrict__ Y)
+{
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
+        Y[p] = stencil_point(s, X, p);
 }
 
 __global__ void k_rhs_f64(Stencil s0, Stencil s1, Model m, int64_t N, const double *__restrict__ U,
@@ -482,6 +475,11 @@ int launch_rhs_f64(const Stencil *s2, const Model &m, int64_t N, const double *U
     return 1;
 }
 
+void launch_kronsum_f64(const Stencil &s, int64_t N, const double *X, double *Y, cudaStream_t st)
+{
+    k_kronsum_f64<<<grid_for(N), 256, 0, st>>>(s, N, X, Y);
+}
+
 void launch_stage_diff_f64(const Model &m, int64_t N, const double *U, const double *a, double w1,
                            const double *b, double w2, double *D, cudaStream_t st)
 {
@@ -601,35 +599,36 @@ __global__ void k_identity(int n, int nb, double *X)
     }
 }
 
+// The three phi-matrices of matrix b lie one after the other: phi_k at
+// P + (3 b + k) nn.
 // phi_k += Pw / (j + k)!  for k = 0, 1, 2
-__global__ void k_taylor_acc(int64_t tot, const double *Pw, double c0, double c1, double c2,
-                             double *p0, double *p1, double *p2)
+__global__ void k_taylor_acc(int64_t nn, const double *Pw, double c0, double c1, double c2, double *P)
 {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot;
+    const int b = blockIdx.y;
+    double *p = P + 3 * b * nn;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn;
          e += (int64_t)gridDim.x * blockDim.x) {
-        double w = Pw[e];
-        p0[e] = __dadd_rn(p0[e], __dmul_rn(c0, w));
-        p1[e] = __dadd_rn(p1[e], __dmul_rn(c1, w));
-        p2[e] = __dadd_rn(p2[e], __dmul_rn(c2, w));
+        double w = Pw[b * nn + e];
+        p[e] = __dadd_rn(p[e], __dmul_rn(c0, w));
+        p[nn + e] = __dadd_rn(p[nn + e], __dmul_rn(c1, w));
+        p[2 * nn + e] = __dadd_rn(p[2 * nn + e], __dmul_rn(c2, w));
     }
 }
 
-// squaring update; matrix b takes the new values only while it <= s_b
-__global__ void k_square_update(int64_t nn, int it, const int *s, const double *T0,
-                                const double *T1, const double *T2, double *p0, double *p1,
-                                double *p2)
+// squaring update (T: phi_0 times the three); matrix b takes the new values
+// only while it <= s_b
+__global__ void k_square_update(int64_t nn, int it, const int *s, const double *T, double *P)
 {
     const int b = blockIdx.y;
     if (it > s[b]) return;
+    const double *t = T + 3 * b * nn;
+    double *p = P + 3 * b * nn;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn;
          e += (int64_t)gridDim.x * blockDim.x) {
-        int64_t q = b * nn + e;
-        double o1 = p1[q], o2 = p2[q];
-        double n1 = __dmul_rn(__dadd_rn(T1[q], o1), 0.5);
-        double n2 = __dmul_rn(__dadd_rn(__dadd_rn(T2[q], o1), o2), 0.25);
-        p0[q] = T0[q];
-        p1[q] = n1;
-        p2[q] = n2;
+        const double o1 = p[nn + e], o2 = p[2 * nn + e];
+        p[e] = t[e];
+        p[nn + e] = __dmul_rn(__dadd_rn(t[nn + e], o1), 0.5);
+        p[2 * nn + e] = __dmul_rn(__dadd_rn(__dadd_rn(t[2 * nn + e], o1), o2), 0.25);
     }
 }
 
@@ -652,17 +651,22 @@ __global__ void k_extract_deriv(int64_t nn, const double *const *lo, const doubl
         dst[b][e] = lo[b][e] - (double)ell[b] * hi[b][e];
 }
 
-void batched_square_gemm(int n, int nb, const double *A, const double *B, double *C,
-                         cudaStream_t st)
+// C_b = A_b [B_b0 ... B_b(m-1)] for column-major n x n blocks: entry b of the
+// batch has its A at A + b sA and its m right-hand blocks, one after the
+// other, at B + b sB (products to C + b m n^2)
+void batched_products(const mm::Context &ctx, int n, int m, int nb, const double *A, int64_t sA, const double *B,
+                      int64_t sB, double *C, cudaStream_t st)
 {
-    DGemm g{};
-    int64_t nn = (int64_t)n * n;
-    g.M = n; g.N = n; g.K = n; g.batch = nb;
-    g.A = A; g.sAm = 1; g.sAk = n; g.sAb = nn;
-    g.B = B; g.sBk = 1; g.sBn = n; g.sBb = nn;
-    g.C = C; g.sCm = 1; g.sCn = n; g.sCb = nn;
-    g.alpha = 1.0; g.beta = 0.0;
-    launch_dgemm(g, st);
+    mm::Product p{};
+    p.A = mm::matrix_view(n, A, 0);
+    p.B = mm::matrix_view(n, B, 1);
+    p.B.rows = (int64_t)m * n;
+    p.A.batch = p.B.batch = nb;
+    p.A.stride = sA;
+    p.B.stride = sB;
+    p.out = C;
+    p.stride = (int64_t)m * n * n;
+    mm::run_products(ctx, &p, 1, st);
 }
 }  // namespace
 
@@ -671,12 +675,29 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     const int nb = (int)jobs.size();
     if (nb == 0) return DS_OK;
     const int64_t nn = (int64_t)n * n, tot = nn * nb;
-    // workspace: Y, Pw, T, phi0..2, T0..T2 (9 blocks) + tables
+    // workspace: Y, Pw, T, phi0..2, their products (9 blocks), tables, digit images
     double *ws = nullptr;
     DS_CUDA_TRY(cudaMallocAsync(&ws, sizeof(double) * tot * 9, st));
-    double *Y = ws, *Pw = ws + tot, *T = ws + 2 * tot;
-    double *p0 = ws + 3 * tot, *p1 = ws + 4 * tot, *p2 = ws + 5 * tot;
-    double *T0 = ws + 6 * tot, *T1 = ws + 7 * tot, *T2 = ws + 8 * tot;
+    double *Y = ws, *Pw = ws + tot, *T = ws + 2 * tot, *P = ws + 3 * tot, *T3 = ws + 6 * tot;
+    mm::Context ctx;
+    if (mm::use_digits(n, n, nb)) {
+        mm::View v = mm::matrix_view(n, nullptr, 0);
+        v.batch = nb;
+        size_t bytes = mm::image_total(v, mm::kRowBlock);
+        v.rows = 3 * (int64_t)n + 64;   // padded to whole column tiles
+        bytes += mm::image_total(v, 1);
+        if (cudaMallocAsync((void **)&ctx.ws, bytes, st) == cudaSuccess) {
+            ctx.ws_bytes = bytes;
+        } else {
+            cudaGetLastError();   // short of memory: the FP64 pipe
+            ctx.ws = nullptr;
+        }
+    }
+    auto release = [&](void *tab) {
+        cudaFreeAsync(ws, st);
+        if (ctx.ws) cudaFreeAsync(ctx.ws, st);
+        if (tab) cudaFreeAsync(tab, st);
+    };
 
     std::vector<const double *> hA(nb);
     std::vector<double> hz(nb);
@@ -684,7 +705,7 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     void *tab = nullptr;
     const size_t tab_bytes = sizeof(void *) * nb * 3 + sizeof(double) * nb * 2 + sizeof(int) * nb;
     cudaError_t e = cudaMallocAsync(&tab, tab_bytes, st);
-    if (e != cudaSuccess) { cudaFreeAsync(ws, st); return fail(DS_ERR_OOM, "phi table"); }
+    if (e != cudaSuccess) { release(nullptr); return fail(DS_ERR_OOM, "phi table"); }
     const double **dA = (const double **)tab;
     double **dSrc = (double **)((char *)tab + sizeof(void *) * nb);
     double **dDst = (double **)((char *)tab + sizeof(void *) * nb * 2);
@@ -704,7 +725,7 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     int smax = 0;
     for (int b = 0; b < nb; ++b) {
         if (!isfinite(hnorm[b])) {
-            cudaFreeAsync(ws, st); cudaFreeAsync(tab, st);
+            release(tab);
             return fail(DS_ERR_NONFINITE, "phi setup: non-finite matrix entry");
         }
         int s = 0;
@@ -720,26 +741,23 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     fact[0] = 1.0;
     for (int j = 1; j < kTaylorDeg + 4; ++j) fact[j] = fact[j - 1] * j;
     const int gl = (int)std::min<int64_t>((tot + 255) / 256, 152 * 16);
-    cudaMemsetAsync(p0, 0, sizeof(double) * tot * 3, st);
+    cudaMemsetAsync(P, 0, sizeof(double) * tot * 3, st);
     k_identity<<<gl, 256, 0, st>>>(n, nb, Pw);
     for (int j = 0; j <= kTaylorDeg; ++j) {
-        k_taylor_acc<<<gl, 256, 0, st>>>(tot, Pw, 1.0 / fact[j], 1.0 / fact[j + 1],
-                                         1.0 / fact[j + 2], p0, p1, p2);
+        k_taylor_acc<<<g2, 256, 0, st>>>(nn, Pw, 1.0 / fact[j], 1.0 / fact[j + 1], 1.0 / fact[j + 2], P);
         if (j < kTaylorDeg) {
-            batched_square_gemm(n, nb, Pw, Y, T, st);
+            batched_products(ctx, n, 1, nb, Pw, nn, Y, nn, T, st);
             std::swap(Pw, T);
         }
     }
     for (int it = 1; it <= smax; ++it) {
-        batched_square_gemm(n, nb, p0, p0, T0, st);
-        batched_square_gemm(n, nb, p0, p1, T1, st);
-        batched_square_gemm(n, nb, p0, p2, T2, st);
-        k_square_update<<<g2, 256, 0, st>>>(nn, it, ds_, T0, T1, T2, p0, p1, p2);
+        batched_products(ctx, n, 3, nb, P, 3 * nn, P, 3 * nn, T3, st);
+        k_square_update<<<g2, 256, 0, st>>>(nn, it, ds_, T3, P);
     }
     std::vector<double *> hsrc(nb), hdst(nb);
     for (int b = 0; b < nb; ++b) {
         int l = jobs[b].ell;
-        hsrc[b] = (l == 0 ? p0 : l == 1 ? p1 : p2) + b * nn;
+        hsrc[b] = P + (3 * b + l) * nn;
         hdst[b] = jobs[b].out;
     }
     cudaMemcpyAsync(dSrc, hsrc.data(), sizeof(void *) * nb, cudaMemcpyHostToDevice, st);
@@ -752,8 +770,8 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
         std::vector<int> hell(nb);
         for (int b = 0; b < nb; ++b) {
             const int l = jobs[b].ell;
-            hlo[b] = (l == 1 ? p0 : p1) + b * nn;
-            hsrc[b] = (l == 1 ? p1 : p2) + b * nn;
+            hlo[b] = P + (3 * b + l - 1) * nn;
+            hsrc[b] = P + (3 * b + l) * nn;
             hdd[b] = jobs[b].dout;
             hell[b] = l;
         }
@@ -765,10 +783,10 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
         k_extract_deriv<<<g2, 256, 0, st>>>(nn, (const double *const *)dA, (const double *const *)dSrc, ds_,
                                             (double *const *)dDst);
     }
-    cudaFreeAsync(ws, st);
-    cudaFreeAsync(tab, st);
+    release(tab);
     DS_CUDA_TRY(cudaStreamSynchronize(st));
     DS_CUDA_TRY(cudaGetLastError());
+    if (ctx.ws) return mm::take_status();
     return DS_OK;
 }
 

@@ -1,0 +1,829 @@
+// FP64 mode products on the 5th-generation tensor cores.
+//
+// GB300's FP64 pipe does 2 FMA per clock and SM (1.25 TFLOP/s in all), three
+// orders of magnitude below its FP16 tensor rate, so an FP64 contraction is
+// formed here from exact digit products.  Every fibre of an operand (the
+// entries that one output sums over) is scaled by a power of two to a 62-bit
+// fixed-point number and cut into eight balanced 8-bit digits, held as FP16
+// integers: x = 2^(e - 6) (d0 + d1 2^-8 + ... + d7 2^-56), |d0| <= 65,
+// |d1..7| <= 128.  The digit products of weight class t = p + q <= 7 (36 of
+// 64) run as FP16 MMAs into one FP32 tensor-memory accumulator per class.  An
+// accumulator holds integers below 2^24 (at most 256 contracted entries
+// between drains), so its sums are exact; the epilogue recombines the classes
+// in integers and rounds once to FP64.  What is lost is the fixed-point
+// rounding of the operands (2^-63 of a fibre's largest entry) and the classes
+// below 2^-56: about 2^-61 of the largest product, where a chain of n FP64
+// FMAs loses 2^-53 per addition.
+//
+// A fibre holding Inf or NaN carries a flag instead of an exponent: outputs
+// of a NaN fibre are NaN, those of an Inf fibre are recomputed by the FP64
+// FMA chain in the epilogue.
+#include <cuda_fp16.h>
+#include <limits.h>
+#include <stdlib.h>
+
+#include <algorithm>
+#include <atomic>
+#include <string>
+
+#include "mm64.h"
+#include "ptx.cuh"
+
+namespace ds {
+namespace mm {
+
+using namespace ptx;
+
+namespace {
+constexpr int kNanRow = INT_MAX, kInfRow = INT_MAX - 1;   // exponents of non-finite fibres
+constexpr int kChunkSlabs = 8;                            // slabs between drains: 256 entries
+constexpr int kSms = 152;
+
+// where waits that gave up are recorded for entry points without a plan
+__device__ DevStatus g_status;
+
+// ---------------------------------------------------------------------------
+// Digit images.  One warp takes 8 rows of one slab: lane = (row, 8
+// consecutive contracted entries), so that every digit plane is written as
+// 512 contiguous bytes.  WS warps (a power of two, at most 8) share the slabs
+// of a row group; each keeps the first slab it reads in registers, so a fibre
+// of up to 256 entries is read once.
+// ---------------------------------------------------------------------------
+struct SplitArgs {
+    int count;
+    int first[kMaxProd + 1];   // block prefix
+    View v[kMaxProd];
+    Image im[kMaxProd];
+};
+
+__host__ __device__ inline int split_warps(int slabs) { return slabs >= 5 ? 8 : slabs >= 3 ? 4 : slabs; }
+
+__device__ __forceinline__ void load_entries(const View &v, int64_t base, bool row_ok, int slab, int chunk, int spc,
+                                             unsigned long long (&x)[8])
+{
+    const int t = slab / spc, k0 = (slab - t * spc) * kSlab + chunk * 8;
+    const double *src = v.src[t] + base + v.I * k0;
+    const double sc = v.scale[t];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const bool ok = row_ok && k0 + j < v.n;
+        double d = ok ? src[v.I * j] : 0.0;
+        if (sc != 1.0) d = __dmul_rn(d, sc);
+        x[j] = (unsigned long long)__double_as_longlong(d);
+    }
+}
+
+// exponent e with max < 2^e of a fibre's largest magnitude (its bits)
+__device__ __forceinline__ int fibre_exp(unsigned long long mx)
+{
+    const int ef = (int)(mx >> 52);
+    if (ef == 0x7FF) return (mx & 0xFFFFFFFFFFFFFULL) ? kNanRow : kInfRow;
+    if (ef > 0) return ef - 1022;
+    return mx ? (64 - __clzll((long long)mx)) - 1074 : 0;
+}
+
+// the eight digits of 8 consecutive entries: bytes of x 2^(62 - e) + 128 in
+// every byte, one 16-byte chunk per digit plane
+__device__ __forceinline__ void store_digits(const unsigned long long (&x)[8], int e, uint8_t *dst, int64_t plane)
+{
+    uint32_t lo[8], hi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const unsigned long long b = x[j];
+        int ef = (int)(b >> 52) & 0x7FF;
+        unsigned long long m = b & 0xFFFFFFFFFFFFFULL;
+        if (ef) m |= 1ULL << 52; else ef = 1;
+        const int sh = ef - 1013 - e;   // <= 9 (<= 61 for subnormal fibres)
+        unsigned long long f;
+        if (sh >= 0) f = m << (sh & 63);
+        else f = sh < -60 ? 0ULL : (m + (1ULL << (-sh - 1))) >> -sh;
+        if (e >= kInfRow) f = 0ULL;
+        if ((long long)b < 0) f = 0ULL - f;
+        f += 0x8080808080808080ULL;
+        lo[j] = (uint32_t)f;
+        hi[j] = (uint32_t)(f >> 32);
+    }
+    const __half2 off = __half2half2(__ushort_as_half((unsigned short)0xE480));   // -1152 = -(1024 + 128)
+#pragma unroll
+    for (int p = 0; p < kDigits; ++p) {
+        uint32_t q[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t w0 = p < 4 ? hi[2 * j] : lo[2 * j], w1 = p < 4 ? hi[2 * j + 1] : lo[2 * j + 1];
+            const int b = 3 - (p & 3);
+            // FP16 1024 + byte, two entries per word
+            const uint32_t w = (__byte_perm(w0, w1, b | (b << 4) | ((4 + b) << 8) | ((4 + b) << 12)) & 0x00FF00FFu) |
+                               0x64006400u;
+            const __half2 h = __hadd2(*reinterpret_cast<const __half2 *>(&w), off);
+            q[j] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        *reinterpret_cast<uint4 *>(dst + p * plane) = make_uint4(q[0], q[1], q[2], q[3]);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_digits(const __grid_constant__ SplitArgs a)
+{
+    __shared__ unsigned long long smax[8][8];
+    int q = 0;
+    while (q + 1 < a.count && (int)blockIdx.x >= a.first[q + 1]) ++q;
+    const View &v = a.v[q];
+    const Image &im = a.im[q];
+    const int S = im.slabs, WS = split_warps(S), G = 8 / WS, spc = S / v.ncat;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int gi = warp / WS, sub = warp % WS;
+    const int64_t groups = (im.rows + 7) / 8, g = (int64_t)(blockIdx.x - a.first[q]) * G + gi;
+    const int64_t entry = g / groups, group = g - entry * groups;   // batch entry, row group in it
+    const int row = lane >> 2, chunk = lane & 3;
+    const int64_t r = group * 8 + row;
+    const bool in = gi < G && entry < v.batch, row_ok = in && r < im.rows;
+    const int64_t rg = v.r0 + r, blocks = (im.rows + im.rb - 1) / im.rb;
+    const int64_t base = row_ok ? entry * v.stride + (rg / v.I) * (v.I * v.n) + rg % v.I : 0;
+    unsigned long long x[8], y[8], mx = 0;
+    load_entries(v, base, row_ok, min(sub, S - 1), chunk, spc, x);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mx = max(mx, x[j] & 0x7FFFFFFFFFFFFFFFULL);
+    for (int s = sub + WS; s < S; s += WS) {
+        load_entries(v, base, row_ok, s, chunk, spc, y);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) mx = max(mx, y[j] & 0x7FFFFFFFFFFFFFFFULL);
+    }
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    if (chunk == 0) smax[warp][row] = mx;
+    __syncthreads();
+    if (!in) return;
+    for (int w = 0; w < WS; ++w) mx = max(mx, smax[gi * WS + w][row]);
+    const int e = fibre_exp(mx);
+    if (sub == 0 && chunk == 0 && row_ok) im.exps[entry * blocks * im.rb + r] = e;
+    const int64_t blk = r / im.rb;
+    const int rr = (int)(r - blk * im.rb);
+    const int64_t plane = (int64_t)im.rb * 64;
+    uint8_t *dst = im.data + (entry * blocks + blk) * S * kDigits * plane + rr * 64 + ((chunk ^ ((rr >> 1) & 3)) << 4);
+    if (sub < S) store_digits(x, e, dst + (int64_t)sub * kDigits * plane, plane);
+    for (int s = sub + WS; s < S; s += WS) {
+        load_entries(v, base, row_ok, s, chunk, spc, y);
+        store_digits(y, e, dst + (int64_t)s * kDigits * plane, plane);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The digit products.  One persistent CTA per SM; warp 0 copies digit blocks
+// (one contiguous block per operand and slab) into a two-stage ring, one
+// thread of warp 1 issues the MMAs, warps 2-9 drain.  A tile is 128 rows by
+// `nt` <= 64 columns: eight classes of 64 FP32 columns are all 512 columns of
+// tensor memory.  The digit planes of B lie one after the other in shared
+// memory, so digit p of A meets up to 256 / nt digits of B in one MMA, whose
+// output columns are the adjacent classes.
+// ---------------------------------------------------------------------------
+struct GProd {
+    const uint8_t *A, *B;
+    const int *eA, *eB;
+    double *out;
+    int slabs, nt, ntiles, mtiles, cols, accumulate, ncat, n;
+    int64_t rows, r0, I, IB, sA, sB, sOut;   // strides of a batch
+    const double *X[kMaxCat], *L[kMaxCat];
+    double sc[kMaxCat];
+};
+struct GArgs {
+    int count;
+    int first[kMaxProd + 1];   // tile prefix
+    DevStatus *status;
+    long long wait_limit;
+    GProd p[kMaxProd];
+};
+
+// Three warpgroups: copies and MMAs (warps 0, 1; 2 and 3 idle), then two that
+// drain.  The first gives its registers up: 128 x 40 + 256 x 232 = 384 x 168,
+// the launch's total; a drain thread holds 32 outputs as two 64-bit integers.
+constexpr int kThreads = 384, kEpiThreads = 256, kStages = 2;
+constexpr uint32_t kPlaneA = kRowBlock * 64, kStageA = kDigits * kPlaneA, kStageB = kDigits * 64 * 64;
+constexpr uint32_t kStageBytes = kStageA + kStageB;
+constexpr uint32_t kSmem = kStages * kStageBytes + 128 + 1024;
+
+// tile u: its product, batch entry, row tile and column tile
+__device__ __forceinline__ const GProd &find_unit(const GArgs &a, int u, int &entry, int &mi, int &ni)
+{
+    int q = 0;
+    while (q + 1 < a.count && u >= a.first[q + 1]) ++q;
+    const GProd &p = a.p[q];
+    const int t = u - a.first[q], row = t / p.ntiles;
+    ni = t - row * p.ntiles;
+    entry = row / p.mtiles;
+    mi = row - entry * p.mtiles;
+    return p;
+}
+
+// all eight classes of four columns, complete on return
+__device__ __forceinline__ void load_classes(uint32_t taddr, uint32_t cs, uint32_t (&v)[32])
+{
+    asm volatile(
+        "{\n\t.reg .b32 t;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%32];\n\t"
+        "add.u32 t, %32, %33;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4, %5, %6, %7}, [t];\n\t"
+        "add.u32 t, t, %33;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8, %9, %10, %11}, [t];\n\t"
+        "add.u32 t, t, %33;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12, %13, %14, %15}, [t];\n\t"
+        "add.u32 t, t, %33;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16, %17, %18, %19}, [t];\n\t"
+        "add.u32 t, t, %33;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%20, %21, %22, %23}, [t];\n\t"
+        "add.u32 t, t, %33;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%24, %25, %26, %27}, [t];\n\t"
+        "add.u32 t, t, %33;\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%28, %29, %30, %31}, [t];\n\t"
+        "tcgen05.wait::ld.sync.aligned;\n\t}\n"
+        : "=&r"(v[0]), "=&r"(v[1]), "=&r"(v[2]), "=&r"(v[3]), "=&r"(v[4]), "=&r"(v[5]), "=&r"(v[6]), "=&r"(v[7]),
+          "=&r"(v[8]), "=&r"(v[9]), "=&r"(v[10]), "=&r"(v[11]), "=&r"(v[12]), "=&r"(v[13]), "=&r"(v[14]),
+          "=&r"(v[15]), "=&r"(v[16]), "=&r"(v[17]), "=&r"(v[18]), "=&r"(v[19]), "=&r"(v[20]), "=&r"(v[21]),
+          "=&r"(v[22]), "=&r"(v[23]), "=&r"(v[24]), "=&r"(v[25]), "=&r"(v[26]), "=&r"(v[27]), "=&r"(v[28]),
+          "=&r"(v[29]), "=&r"(v[30]), "=&r"(v[31])
+        : "r"(taddr), "r"(cs)
+        : "memory");
+}
+
+// (P 2^30 + Q) 2^e rounded to nearest even, in integers: the FP64 pipe would
+// take longer than the digit products
+__device__ __forceinline__ double combine(long long P, long long Q, int e)
+{
+    long long H = P + (Q >> 30);
+    uint32_t L = (uint32_t)Q & 0x3FFFFFFFu;
+    const bool neg = H < 0;
+    if (neg) {
+        H = -H - (L ? 1 : 0);
+        L = (0u - L) & 0x3FFFFFFFu;
+    }
+    const int top = 64 - __clzll(H);
+    const int sh = max(0, top - 33);
+    const unsigned long long V = ((unsigned long long)H << (30 - sh)) | (L >> sh);
+    if (V == 0) return 0.0;
+    const int lz = __clzll((long long)V);
+    const unsigned long long M = V << lz;
+    unsigned long long m = M >> 11;
+    const uint32_t rem = (uint32_t)M & 0x7FFu;
+    m += rem > 0x400u || (rem == 0x400u && (m & 1));
+    const int E = e + sh - lz + 63;   // value in [2^E, 2^(E + 1)]
+    double r;
+    if (E >= -1022 && E <= 1022) {
+        r = __longlong_as_double((long long)(((unsigned long long)(E + 1022) << 52) + m));
+    } else {
+        r = scalbn(__longlong_as_double((long long)((1022ULL << 52) + m)), max(-3000, min(3000, E)));
+    }
+    return neg ? -r : r;
+}
+
+// the FP64 FMA chain of one output
+__device__ __forceinline__ double fma_chain(const GProd &p, int64_t entry, int64_t r, int i)
+{
+    double total = 0.0;
+    const int64_t xa = entry * p.sA + (r / p.I) * (p.I * p.n) + r % p.I;
+    const int64_t lb = entry * p.sB + (i / p.IB) * (p.IB * p.n) + i % p.IB;
+    for (int t = 0; t < p.ncat; ++t) {
+        const double *x = p.X[t] + xa, *l = p.L[t] + lb;
+        double s = 0.0;
+        for (int k = 0; k < p.n; ++k) s = fma(x[p.I * k], l[p.IB * k], s);
+        total = t ? total + p.sc[t] * s : p.sc[t] * s;
+    }
+    return total;
+}
+
+__global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_constant__ GArgs a)
+{
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_addr(smem_raw), base = (raw + 1023u) & ~1023u;
+    const uint32_t bars = base + kStages * kStageBytes;
+    uint32_t *tmem_slot = (uint32_t *)(smem_raw + (bars - raw) + 64);
+    volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+    const uint32_t FULL = bars, EMPTY = bars + 16, TFULL = bars + 32, TEMPTY = bars + 40, DRAIN = bars + 48;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int units = a.first[a.count];
+    DevStatus *const status = a.status ? a.status : &g_status;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            bar_init(FULL + 8 * s, 1);
+            bar_init(EMPTY + 8 * s, 1);
+        }
+        bar_init(TFULL, 1);
+        bar_init(TEMPTY, kEpiThreads);
+        bar_init(DRAIN, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        if (warp == 0 && lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            int issued[kStages] = {-1, -1};
+            bool ok = true;
+            for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+                int be, mi, ni;
+                const GProd &p = find_unit(a, u, be, mi, ni);
+                const uint32_t nb = (uint32_t)p.nt * 64 * kDigits;
+                const uint8_t *A = p.A + ((int64_t)be * p.mtiles + mi) * p.slabs * kStageA;
+                const uint8_t *B = p.B + ((int64_t)be * p.ntiles + ni) * p.slabs * nb;
+                for (int s = 0; s < p.slabs; ++s) {
+                    if (!bar_wait(EMPTY + 8 * stage, phase ^ 1u, abort_flag, status, 11, a.wait_limit)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t sA = base + stage * kStageBytes;
+                    bar_expect(FULL + 8 * stage, kStageA + nb);
+                    bulk_load(sA + kStageA, B + (int64_t)s * nb, nb, FULL + 8 * stage);
+                    bulk_load(sA, A + (int64_t)s * kStageA, kStageA, FULL + 8 * stage);
+                    issued[stage] = (int)phase;
+                    if (++stage == kStages) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
+                }
+            }
+            // every issued copy lands before the CTA exits
+            for (int s = 0; s < kStages; ++s)
+                if (issued[s] >= 0) {
+                    volatile int never = 0;
+                    bar_wait(FULL + 8 * s, (uint32_t)issued[s], &never, nullptr, 0, kWaitCycles);
+                }
+        }
+        if (warp == 1 && lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0, tphase = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+                int be, mi, ni;
+                const GProd &p = find_unit(a, u, be, mi, ni);
+                const uint32_t nt = (uint32_t)p.nt;
+                const int per = min((int)(256u / nt), kDigits);   // digits of B per MMA
+                for (int s = 0; ok && s < p.slabs; ++s) {
+                    const bool fresh = s % kChunkSlabs == 0;
+                    if (fresh) {
+                        if (!bar_wait(TEMPTY, tphase ^ 1u, abort_flag, status, 12, a.wait_limit)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_after();
+                        tphase ^= 1u;
+                    }
+                    if (!bar_wait(FULL + 8 * stage, phase, abort_flag, status, 13, a.wait_limit)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_after();
+                    const uint32_t sA = base + stage * kStageBytes, sB = sA + kStageA;
+#pragma unroll 1
+                    for (int ks = 0; ks < kSlab / 16; ++ks) {
+#pragma unroll 1
+                        for (int pd = 0; pd < kDigits; ++pd) {
+                            const uint64_t ad = desc_sw64(sA + pd * kPlaneA + ks * 32);
+                            const uint32_t acc = fresh && ks == 0 && pd == 0 ? 0u : 1u;
+                            const int nq = kDigits - pd;
+                            for (int q = 0; q < nq; q += per) {
+                                const int w = min(per, nq - q);
+                                const uint64_t bd = desc_sw64(sB + q * nt * 64 + ks * 32);
+                                const uint32_t d = tmem + (pd + q) * nt, id = idesc_f16(kRowBlock, w * nt);
+                                if (nq <= per) mma_f16<0>(d, ad, bd, id, acc);
+                                else if (q == 0) mma_f16<1>(d, ad, bd, id, acc);
+                                else if (q + per < nq) mma_f16<2>(d, ad, bd, id, acc);
+                                else mma_f16<3>(d, ad, bd, id, acc);
+                            }
+                        }
+                    }
+                    mma_commit_to(EMPTY + 8 * stage);
+                    if (++stage == kStages) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
+                    if (s + 1 == p.slabs || s % kChunkSlabs == kChunkSlabs - 1) mma_commit_to(TFULL);
+                }
+            }
+            mma_commit_to(DRAIN);
+            volatile int never = 0;
+            bar_wait(DRAIN, 0, &never, nullptr, 0, kWaitCycles);
+        }
+    } else {
+        // warp w reads the tensor-memory lanes 32 (w % 4) ..; the two warps of a
+        // lane quarter take half of the columns each
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+        const int quarter = warp % 4, half = (warp - 4) / 4;
+        const int m = quarter * 32 + lane;
+        uint32_t tphase = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < units; u += gridDim.x) {
+            int be, mi, ni;
+            const GProd &p = find_unit(a, u, be, mi, ni);
+            const int nt = p.nt, hc = nt / 2;
+            const int64_t r = (int64_t)mi * kRowBlock + m;
+            const bool row_ok = r < p.rows;
+            long long P[32], Q[32];
+            for (int s0 = 0; s0 < p.slabs; s0 += kChunkSlabs) {
+                ok = ok && __all_sync(0xffffffffu, bar_wait(TFULL, tphase, abort_flag, status, 14, a.wait_limit));
+                if (!ok) break;
+                tphase ^= 1u;
+                tc_after();
+                const uint32_t tq = tmem + (uint32_t)(half * hc) + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    if (g * 4 < hc) {
+                        uint32_t v[32];
+                        load_classes(tq + g * 4, (uint32_t)nt, v);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            // classes 0..2 in units of class 2, the rest in 2^-30 of that
+                            const int c0 = __float2int_rn(__uint_as_float(v[j]));
+                            const int c1 = __float2int_rn(__uint_as_float(v[4 + j]));
+                            const int c2 = __float2int_rn(__uint_as_float(v[8 + j]));
+                            const int c3 = __float2int_rn(__uint_as_float(v[12 + j]));
+                            const int c4 = __float2int_rn(__uint_as_float(v[16 + j]));
+                            const float f = fmaf(__uint_as_float(v[28 + j]), 0x1p-10f,
+                                                 fmaf(__uint_as_float(v[24 + j]), 0.25f, 64.0f * __uint_as_float(v[20 + j])));
+                            const int c5 = __float2int_rn(f);
+                            const long long hp = (long long)c0 * 65536 + ((long long)c1 * 256 + c2);
+                            const long long lp = (long long)c3 * 4194304 + ((long long)c4 * 16384 + c5);
+                            P[g * 4 + j] = s0 ? P[g * 4 + j] + hp : hp;
+                            Q[g * 4 + j] = s0 ? Q[g * 4 + j] + lp : lp;
+                        }
+                    }
+                }
+                tc_before();
+                bar_arrive(TEMPTY);
+            }
+            if (!row_ok) continue;
+            const int er = p.eA[(int64_t)be * p.mtiles * kRowBlock + r];
+            const int *eb = p.eB + (int64_t)be * p.ntiles * nt + ni * nt + half * hc;
+            const int64_t rg = p.r0 + r;
+            const int64_t o0 = (rg / p.I) * (p.I * p.cols) + rg % p.I;
+            const int c0 = ni * nt + half * hc;
+            double *out = p.out + be * p.sOut + o0 + p.I * c0;
+            bool odd = !ok || er >= kInfRow;   // some output needs more than the digits
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                if (j < hc && c0 + j < p.cols) {
+                    const int ec = __ldg(eb + j);
+                    odd = odd || ec >= kInfRow;
+                    if (!odd) {
+                        const double z = combine(P[j], Q[j], er + ec - 58);
+                        double *o = out + p.I * j;
+                        *o = p.accumulate ? __dadd_rn(*o, z) : z;
+                    }
+                }
+            }
+            if (odd) {
+                // a non-finite row or column (or an abandoned wait: NaN); the outputs
+                // before its first flagged column are already stored
+                bool seen = !ok || er >= kInfRow;
+#pragma unroll 1
+                for (int j = 0; j < hc && c0 + j < p.cols; ++j) {
+                    const int ec = __ldg(eb + j);
+                    seen = seen || ec >= kInfRow;
+                    if (!seen) continue;
+                    const double z = !ok || er == kNanRow || ec == kNanRow ? __longlong_as_double(0x7FF8000000000000LL)
+                                                                          : fma_chain(p, be, rg, c0 + j);
+                    double *o = out + p.I * j;
+                    *o = p.accumulate ? __dadd_rn(*o, z) : z;
+                }
+            }
+        }
+    }
+    tc_before();
+    __syncthreads();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 pipe's own kernel for small products: one thread per output, so
+// that even a 64 x 64 product spreads over every SM (a 64 x 64 tile would keep
+// one SM's FP64 pipe busy for 63 us).
+// ---------------------------------------------------------------------------
+struct FArgs {
+    int count;
+    int64_t first[kMaxProd + 1];   // output prefix
+    GProd p[kMaxProd];
+};
+__global__ void __launch_bounds__(128) k_fma_products(const __grid_constant__ FArgs a)
+{
+    const int64_t total = a.first[a.count];
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        int q = 0;
+        while (q + 1 < a.count && e >= a.first[q + 1]) ++q;
+        const GProd &p = a.p[q];
+        const int64_t size = p.rows * p.cols, entry = (e - a.first[q]) / size, t = e - a.first[q] - entry * size;
+        // neighbouring threads: neighbouring outputs in memory
+        int64_t r;
+        int i;
+        if (p.I == 1) {
+            r = t / p.cols;
+            i = (int)(t - r * p.cols);
+        } else {
+            const int64_t o = t / (p.I * p.cols), w = t - o * (p.I * p.cols);
+            i = (int)(w / p.I);
+            r = o * p.I + (w - i * p.I);
+        }
+        const double s = fma_chain(p, entry, r, i);
+        double *o = p.out + entry * p.sOut + t;
+        *o = p.accumulate ? __dadd_rn(*o, s) : s;
+    }
+}
+
+GProd to_gprod(const Product &s)
+{
+    GProd p{};
+    p.A = s.ia.data;
+    p.B = s.ib.data;
+    p.eA = s.ia.exps;
+    p.eB = s.ib.exps;
+    p.out = s.out;
+    p.slabs = s.ia.slabs;
+    p.nt = s.ib.rb;
+    p.cols = (int)s.B.rows;
+    p.ntiles = p.nt ? (p.cols + p.nt - 1) / p.nt : 0;
+    p.mtiles = (int)((s.A.rows + kRowBlock - 1) / kRowBlock);
+    p.sA = s.A.stride;
+    p.sB = s.B.stride;
+    p.sOut = s.stride;
+    p.accumulate = s.accumulate;
+    p.ncat = s.A.ncat;
+    p.n = s.A.n;
+    p.rows = s.A.rows;
+    p.r0 = s.A.r0;
+    p.I = s.A.I;
+    p.IB = s.B.I;
+    for (int t = 0; t < s.A.ncat; ++t) {
+        p.X[t] = s.A.src[t];
+        p.L[t] = s.B.src[t];
+        p.sc[t] = s.A.scale[t] * s.B.scale[t];
+    }
+    return p;
+}
+}  // namespace
+
+int tile_cols(int64_t rows, int cols, int products)
+{
+    const int64_t mt = (rows + kRowBlock - 1) / kRowBlock * products;
+    for (int w = 64; w > 16; w -= 16)
+        if (mt * ((cols + w - 1) / w) >= kSms) {
+            const int nb = (cols + w - 1) / w;
+            return ((cols + nb - 1) / nb + 15) / 16 * 16;
+        }
+    return 16;
+}
+
+bool use_digits(int64_t rows, int n, int count)
+{
+    const int most = rows * n > ((int64_t)1 << 20) ? 4096 : 1024;
+    return n >= 12 && n <= most && rows >= 16 && (double)rows * n * n * count > 1.5e6;
+}
+
+void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
+{
+    SplitArgs a{};
+    a.count = count;
+    for (int q = 0; q < count; ++q) {
+        a.v[q] = v[q];
+        a.im[q] = im[q];
+        const int G = 8 / split_warps(im[q].slabs);
+        const int64_t groups = (im[q].rows + 7) / 8 * v[q].batch;
+        a.first[q + 1] = a.first[q] + (int)((groups + G - 1) / G);
+    }
+    k_digits<<<a.first[count], 256, 0, st>>>(a);
+}
+
+void launch_products(const Product *s, int count, DevStatus *status, long long wait_limit, cudaStream_t st)
+{
+    static std::atomic<uint64_t> ready{0};   // devices whose shared-memory limit is raised
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 64 || !(ready.load() >> dev & 1)) {
+        cudaFuncSetAttribute(k_digit_products, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        if (dev < 64) ready.fetch_or((uint64_t)1 << dev);
+    }
+    GArgs a{};
+    a.count = count;
+    a.status = status;
+    a.wait_limit = wait_limit;
+    for (int q = 0; q < count; ++q) {
+        a.p[q] = to_gprod(s[q]);
+        a.first[q + 1] = a.first[q] + a.p[q].mtiles * a.p[q].ntiles * s[q].A.batch;
+    }
+    const int units = a.first[count];
+    if (units == 0) return;
+    k_digit_products<<<std::min(units, kSms), kThreads, kSmem, st>>>(a);
+}
+
+void launch_products_fma(const Product *s, int count, cudaStream_t st)
+{
+    FArgs a{};
+    a.count = count;
+    for (int q = 0; q < count; ++q) {
+        a.p[q] = to_gprod(s[q]);
+        a.first[q + 1] = a.first[q] + a.p[q].rows * a.p[q].cols * s[q].A.batch;
+    }
+    const int64_t total = a.first[count];
+    if (total == 0) return;
+    k_fma_products<<<(int)std::min<int64_t>((total + 127) / 128, kSms * 16), 128, 0, st>>>(a);
+}
+
+View tensor_view(int d, const int64_t *n, int mu, const double *X)
+{
+    View v{};
+    v.src[0] = X;
+    v.scale[0] = 1.0;
+    v.ncat = v.batch = 1;
+    v.n = (int)n[mu];
+    v.I = v.rows = 1;
+    for (int q = 0; q < d; ++q) {
+        if (q < mu) v.I *= n[q];
+        if (q != mu) v.rows *= n[q];
+    }
+    return v;
+}
+
+View matrix_view(int64_t n, const double *L, int transpose, double scale)
+{
+    View v{};
+    v.src[0] = L;
+    v.scale[0] = scale;
+    v.ncat = v.batch = 1;
+    v.n = (int)n;
+    v.I = transpose ? 1 : n;
+    v.rows = n;
+    return v;
+}
+
+size_t scratch_bytes(int64_t N, int64_t n, int count, int cat, bool matrices)
+{
+    const int slabs = slabs_of((int)n, cat);
+    const size_t a = aligned(image_bytes(N / n, kRowBlock, slabs) + sizeof(int) * pad_rows(N / n, kRowBlock));
+    // (the padding to whole tiles is below 64 columns)
+    const size_t b = matrices ? aligned(image_bytes(n + 64, 1, slabs) + sizeof(int) * (n + 64)) : 0;
+    // beyond 1 GiB a launch fills the GPU many times over: row blocks cost nothing
+    const size_t most = (size_t)1 << 30;
+    return std::min(count * a, std::max(most, 2 * a / (pad_rows(N / n, kRowBlock) / kRowBlock) + kAlign)) + count * b;
+}
+
+namespace {
+bool same_view(const View &a, const View &b)
+{
+    if (a.ncat != b.ncat || a.n != b.n || a.I != b.I || a.rows != b.rows || a.r0 != b.r0 || a.batch != b.batch || a.stride != b.stride) return false;
+    for (int t = 0; t < a.ncat; ++t)
+        if (a.src[t] != b.src[t] || a.scale[t] != b.scale[t]) return false;
+    return true;
+}
+double product_flops(const Product &p) { return 2.0 * p.A.batch * p.A.rows * p.B.rows * p.A.n * p.A.ncat; }
+}  // namespace
+
+int run_products(const Context &c, const Product *ps, int count, cudaStream_t st)
+{
+    int launches = 0;
+    for (int i = 0; i < count;) {
+        const bool digits = use_digits(ps[i].A.rows, ps[i].A.n, count);
+        Product p[kMaxProd];
+        View sv[kMaxProd];
+        Image si[kMaxProd];
+        int np = 0, ns = 0;
+        size_t used = 0;
+        double flops = 0.0;
+        auto place = [&](const View &v, int rb, Image &im) {   // scratch for v's image; false: no room
+            for (int q = 0; q < ns; ++q)
+                if (si[q].rb == rb && same_view(sv[q], v)) {
+                    im = si[q];
+                    return true;
+                }
+            im.rb = rb;
+            im.slabs = slabs_of(v.n, v.ncat);
+            im.rows = v.rows;
+            const size_t all = image_total(v, rb);
+            if (used + all > c.ws_bytes || ns == kMaxProd) return false;
+            im.data = c.ws + used;
+            im.exps = (int *)(im.data + image_bytes(v.rows, rb, im.slabs) * v.batch);
+            used += all;
+            sv[ns] = v;
+            si[ns++] = im;
+            return true;
+        };
+        auto add = [&](const Product &q, bool with_b) {
+            Product t = q;
+            const size_t u0 = used;
+            const int n0 = ns;
+            if ((with_b && !place(t.B, tile_cols(t.A.rows, (int)t.B.rows, count), t.ib)) ||
+                !place(t.A, kRowBlock, t.ia)) {
+                used = u0;
+                ns = n0;
+                return false;
+            }
+            p[np++] = t;
+            flops += product_flops(t);
+            return true;
+        };
+        auto flush = [&] {
+            if (ns) {
+                if (c.prof) c.prof->begin(st, 1, 0.0);
+                launch_split(sv, si, ns, st);
+                if (c.prof) c.prof->end(st);
+                ++launches;
+            }
+            if (c.prof) c.prof->begin(st, 1, flops);
+            launch_products(p, np, c.status, c.wait_limit, st);
+            if (c.prof) c.prof->end(st);
+            ++launches;
+        };
+        int j = i;
+        if (digits)
+            while (j < count && np < kMaxProd && add(ps[j], ps[j].ib.data == nullptr)) ++j;
+        if (j > i) {
+            flush();
+            i = j;
+            continue;
+        }
+        // one product whose images do not fit together: B's once (where it is cut
+        // per call), A's in row blocks
+        bool done = false;
+        if (digits && ps[i].A.batch == 1) {
+            Product t = ps[i];
+            const size_t per = image_bytes(kRowBlock, kRowBlock, slabs_of(t.A.n, t.A.ncat)) + sizeof(int) * kRowBlock;
+            const bool ok = t.ib.data || place(t.B, tile_cols(t.A.rows, (int)t.B.rows, 1), t.ib);
+            if (ok && used + per + kAlign <= c.ws_bytes) {
+                const int64_t fit = (int64_t)((c.ws_bytes - used - kAlign) / per) * kRowBlock;
+                const size_t u0 = used;
+                for (int64_t r = 0; r < ps[i].A.rows; r += fit) {
+                    Product part = t;
+                    part.A.r0 = t.A.r0 + r;
+                    part.A.rows = std::min(fit, t.A.rows - r);
+                    if (r) ns = 0;   // B's image stays
+                    used = u0;
+                    np = 0;
+                    flops = 0.0;
+                    add(part, false);
+                    flush();
+                }
+                done = true;
+            }
+        }
+        if (!done) {
+            // the FP64 pipe: every remaining product of a small phase in one launch
+            np = 0;
+            flops = 0.0;
+            const int most = digits ? 1 : kMaxProd;
+            for (j = i; j < count && np < most; ++j) {
+                p[np++] = ps[j];
+                flops += product_flops(ps[j]);
+            }
+            if (c.prof) c.prof->begin(st, 1, flops);
+            launch_products_fma(p, np, st);
+            if (c.prof) c.prof->end(st);
+            ++launches;
+        } else
+            j = i + 1;
+        i = j;
+    }
+    return launches;
+}
+
+void tucker_f64(const Context &c, int d, const int64_t *n, const double *X, double *Y, const double *const *L,
+                int transpose, double *tmp, cudaStream_t st)
+{
+    int64_t N = 1;
+    for (int q = 0; q < d; ++q) N *= n[q];
+    const double *in = X;
+    for (int mu = 0; mu < d; ++mu) {
+        Product p{};
+        p.A = tensor_view(d, n, mu, in);
+        p.B = matrix_view(n[mu], L[mu], transpose);
+        p.out = mu == d - 1 ? Y : tmp + (mu % 2) * N;
+        run_products(c, &p, 1, st);
+        in = p.out;
+    }
+}
+
+ds_status take_status()
+{
+    DevStatus h{};
+    DS_CUDA_TRY(cudaMemcpyFromSymbol(&h, g_status, sizeof h));
+    if (!h.timeout) return DS_OK;
+    const DevStatus zero{};
+    cudaMemcpyToSymbol(g_status, &zero, sizeof zero);
+    return fail(DS_ERR_TIMEOUT, "digit-product pipeline wait gave up (site " + std::to_string(h.where) + ")");
+}
+
+long long wait_limit_default()
+{
+    const char *e = getenv("DS_WAIT_LIMIT_CYCLES");
+    const long long v = e ? atoll(e) : 0;
+    return v > 0 ? v : kWaitCycles;
+}
+
+}  // namespace mm
+}  // namespace ds

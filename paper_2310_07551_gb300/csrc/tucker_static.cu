@@ -5,14 +5,15 @@
 // callback (where a nested cudaMalloc would re-enter the allocator),
 // real-time or embedded hosts that forbid allocation after start-up, and
 // plugins of frameworks that own the whole device heap.  For them the two
-// intermediate tensors of the mode-product chain live in one fixed
+// intermediate tensors of the mode-product chain, and the digit images of its
+// tensor-core products, live in one fixed
 // file-scope device array instead of temporaries.  That array is part of the
 // loaded module: every GPU on which the library is loaded holds it until the
 // process exits.
 #include <mutex>
 #include <string>
 
-#include "ds_internal.h"
+#include "mm64.h"
 
 namespace {
 
@@ -21,7 +22,11 @@ constexpr int64_t kStaticMaxPoints = (int64_t)1 << 20;
 
 // Two FP64 intermediates of kStaticMaxPoints entries each (16 MiB).  Shared
 // by every call on a device; it keeps whatever the last call left in it.
-__device__ __align__(256) double g_static_scratch[2 * kStaticMaxPoints];
+// Digit images for the tensor-core products (20 MiB): a 1024 x 1024 matrix's
+// (16 MiB) and two 128-row blocks of a tensor, which larger tensors pass
+// through block by block.
+constexpr int64_t kStaticDigits = (int64_t)20 << 20;
+__device__ __align__(256) double g_static_scratch[2 * kStaticMaxPoints + kStaticDigits / 8];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -74,15 +79,13 @@ extern "C" ds_status ds_tucker_static(const ds_grid *grid, const double *X, doub
     double *scratch = nullptr;
     r = scratch_address(&scratch);
     if (r != DS_OK) return r;
-    cudaStream_t st = (cudaStream_t)stream;
-    // every mode product writes all of its output (beta = 0), so nothing in
-    // the scratch needs clearing between calls
-    const double *in = X;
-    for (int mu = 0; mu < grid->d; ++mu) {
-        double *out = (mu == grid->d - 1) ? Y : scratch + (mu % 2) * kStaticMaxPoints;
-        ds::launch_mode_product_f64(grid->d, grid->n, in, mu, L[mu], transpose, out, 1.0, 0.0, st);
-        in = out;
-    }
+    ds::mm::Context c;
+    // every mode product writes all of its output and every digit image is
+    // written before it is read, so nothing in the scratch needs clearing
+    // between calls
+    c.ws = (uint8_t *)(scratch + 2 * kStaticMaxPoints);
+    c.ws_bytes = kStaticDigits;
+    ds::mm::tucker_f64(c, grid->d, grid->n, X, Y, L, transpose, scratch, (cudaStream_t)stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return ds::fail(DS_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     return DS_OK;
