@@ -16,6 +16,39 @@ constexpr int64_t kDenseMaxPoints = 4096;   // DS_EXPRK3_DENSE: N x N phi-matric
 constexpr int kSlots = 5;     // (s2,l1) (s3,l1) (s3,l2) (sf,l1) (sf,l2)
 constexpr int kMaxTerms = 3;
 
+// Programmatic dependent launch: a kernel launched this way may start while its
+// predecessor on the stream still runs, and orders itself behind it with
+// pdl_wait() before it touches memory that another kernel writes or reads.
+// pdl_trigger() lets the next kernel start.  Inside a stream capture the launch
+// is an ordinary one: a replayed graph's own kernel-to-kernel edges are shorter
+// (Schnakenberg 64^2, ten steps: 622 us against 735 with programmatic edges),
+// where a sequence of stream launches gains (FHN 96^3 with adjoint: 11.2 against
+// 11.8 ms).  cluster: CTAs per cluster.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &cap);
+    cudaLaunchAttribute at[2]{};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = cap == cudaStreamCaptureStatusNone;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // Split coefficients of one target function phi_l (Section 2 tables).
 struct SplitCoeffs {
     int k;                    // number of terms

@@ -196,6 +196,8 @@ __device__ __forceinline__ double stencil_point(const Stencil &s, const double *
 
 __global__ void k_kronsum_f64(Stencil s, int64_t N, const double *__restrict__ X, double *__restrict__ Y)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
         Y[p] = stencil_point(s, X, p);
 }
@@ -203,6 +205,8 @@ __global__ void k_kronsum_f64(Stencil s, int64_t N, const double *__restrict__ X
 __global__ void k_rhs_f64(Stencil s0, Stencil s1, Model m, int64_t N, const double *__restrict__ U,
                           double *__restrict__ F)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         double gu, gv;
@@ -216,6 +220,8 @@ __global__ void k_stage_diff_f64(Model m, int64_t N, const double *__restrict__ 
                                  const double *__restrict__ a, double w1,
                                  const double *__restrict__ b, double w2, double *__restrict__ D)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         double u = U[p], v = U[N + p];
@@ -236,6 +242,8 @@ __global__ void k_stage_diff_f64(Model m, int64_t N, const double *__restrict__ 
 __global__ void k_final_f64(int64_t n2, double *__restrict__ U, const double *__restrict__ a,
                             double w1, const double *__restrict__ b, double w2)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n2;
          p += (int64_t)gridDim.x * blockDim.x)
         U[p] = __dadd_rn(__dadd_rn(U[p], __dmul_rn(w1, a[p])), __dmul_rn(w2, b[p]));
@@ -243,6 +251,8 @@ __global__ void k_final_f64(int64_t n2, double *__restrict__ U, const double *__
 
 __global__ void k_add_g_f64(Model m, int64_t N, const double *__restrict__ U, double *__restrict__ F)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         double gu, gv;
@@ -302,6 +312,8 @@ __device__ __forceinline__ void dparam_point(const Model &m, double u, double v,
 __global__ void k_axpy2(int64_t n2, const double *__restrict__ U, const double *__restrict__ a, double w1,
                         const double *__restrict__ b, double w2, double *__restrict__ Y)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n2;
          p += (int64_t)gridDim.x * blockDim.x) {
         double y = __dadd_rn(U[p], __dmul_rn(w1, a[p]));
@@ -314,6 +326,8 @@ __global__ void k_axpy2(int64_t n2, const double *__restrict__ U, const double *
 __global__ void k_gdiff(Model m, int64_t N, const double *__restrict__ U, const double *__restrict__ Us,
                         double *__restrict__ D)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         double g0u, g0v, gu, gv;
@@ -328,6 +342,8 @@ __global__ void k_gdiff(Model m, int64_t N, const double *__restrict__ U, const 
 __global__ void k_jacT(Model m, int64_t N, const double *__restrict__ Us, const double *__restrict__ lam,
                        double *__restrict__ out)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         double ou, ov;
@@ -361,6 +377,8 @@ __device__ __forceinline__ double stencil_point_T(const Stencil &s, const double
 __global__ void k_kronsumT(Stencil s0, Stencil s1, int64_t N, const double *__restrict__ X,
                            double *__restrict__ Y)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         Y[p] = stencil_point_T(s0, X, p);
@@ -382,6 +400,8 @@ __global__ void __launch_bounds__(256) k_adjoint_final(Model m, int64_t N, const
                                                        const double *__restrict__ lD3,
                                                        double *__restrict__ lam_n, double *dp)
 {
+    pdl_trigger();
+    pdl_wait();
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
@@ -418,6 +438,8 @@ __global__ void __launch_bounds__(256) k_adjoint_final(Model m, int64_t N, const
 __global__ void __launch_bounds__(256) k_dot_accum(int64_t n, const double *__restrict__ a,
                                                    const double *__restrict__ b, double w, double *out)
 {
+    pdl_trigger();
+    pdl_wait();
     double s = 0.0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
          p += (int64_t)gridDim.x * blockDim.x)
@@ -436,6 +458,8 @@ __global__ void __launch_bounds__(256) k_dot_kterm(Model m, int64_t N, const dou
                                                    const double *__restrict__ F,
                                                    const double *__restrict__ lF, double *out)
 {
+    pdl_trigger();
+    pdl_wait();
     double s0 = 0.0, s1 = 0.0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
@@ -461,77 +485,85 @@ __global__ void __launch_bounds__(256) k_dot_kterm(Model m, int64_t N, const dou
     }
 }
 
-int grid_for(int64_t n)
+// Threads of a block for n points: small grids take small blocks, so that every
+// SM's FP64 pipe (16 clocks per warp instruction) has a share.
+int block_for(int64_t n)
 {
-    int64_t b = (n + 255) / 256;
-    return (int)std::min<int64_t>(b, 152 * 16);
+    int b = 256;
+    while (b > 32 && n < 2 * 152 * (int64_t)b) b /= 2;
+    return b;
+}
+int grid_for(int64_t n, int block = 256)
+{
+    int64_t b = (n + block - 1) / block;
+    return (int)std::min<int64_t>(b, 152 * 16 * (256 / block));
 }
 }  // namespace
 
 int launch_rhs_f64(const Stencil *s2, const Model &m, int64_t N, const double *U, double *F,
                    cudaStream_t st)
 {
-    k_rhs_f64<<<grid_for(N), 256, 0, st>>>(s2[0], s2[1], m, N, U, F);
+    pdl_launch(k_rhs_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s2[0], s2[1], m, N, U, F);
     return 1;
 }
 
 void launch_kronsum_f64(const Stencil &s, int64_t N, const double *X, double *Y, cudaStream_t st)
 {
-    k_kronsum_f64<<<grid_for(N), 256, 0, st>>>(s, N, X, Y);
+    pdl_launch(k_kronsum_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s, N, X, Y);
 }
 
 void launch_stage_diff_f64(const Model &m, int64_t N, const double *U, const double *a, double w1,
                            const double *b, double w2, double *D, cudaStream_t st)
 {
-    k_stage_diff_f64<<<grid_for(N), 256, 0, st>>>(m, N, U, a, w1, b, w2, D);
+    pdl_launch(k_stage_diff_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, U, a, w1, b, w2, D);
 }
 
 void launch_final_f64(int64_t N, double *U, const double *a, double w1, const double *b,
                       double w2, cudaStream_t st)
 {
-    k_final_f64<<<grid_for(2 * N), 256, 0, st>>>(2 * N, U, a, w1, b, w2);
+    pdl_launch(k_final_f64, dim3(grid_for(2 * N, block_for(2 * N))), dim3(block_for(2 * N)), 0, st, 1, 2 * N, U, a, w1, b, w2);
 }
 
 void launch_add_g_f64(const Model &m, int64_t N, const double *U, double *F, cudaStream_t st)
 {
-    k_add_g_f64<<<grid_for(N), 256, 0, st>>>(m, N, U, F);
+    pdl_launch(k_add_g_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, U, F);
 }
 
 void launch_axpy2_f64(int64_t N, const double *U, const double *a, double w1, const double *b, double w2,
                       double *Y, cudaStream_t st)
 {
-    k_axpy2<<<grid_for(2 * N), 256, 0, st>>>(2 * N, U, a, w1, b, w2, Y);
+    pdl_launch(k_axpy2, dim3(grid_for(2 * N, block_for(2 * N))), dim3(block_for(2 * N)), 0, st, 1, 2 * N, U, a, w1, b, w2, Y);
 }
 void launch_gdiff_f64(const Model &m, int64_t N, const double *U, const double *Us, double *D, cudaStream_t st)
 {
-    k_gdiff<<<grid_for(N), 256, 0, st>>>(m, N, U, Us, D);
+    pdl_launch(k_gdiff, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, U, Us, D);
 }
 void launch_jacT_f64(const Model &m, int64_t N, const double *Us, const double *lam, double *out,
                      cudaStream_t st)
 {
-    k_jacT<<<grid_for(N), 256, 0, st>>>(m, N, Us, lam, out);
+    pdl_launch(k_jacT, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, Us, lam, out);
 }
 void launch_kronsumT_f64(const Stencil *s2, int64_t N, const double *X, double *Y, cudaStream_t st)
 {
-    k_kronsumT<<<grid_for(N), 256, 0, st>>>(s2[0], s2[1], N, X, Y);
+    pdl_launch(k_kronsumT, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s2[0], s2[1], N, X, Y);
 }
 void launch_adjoint_final_f64(const Model &m, int64_t N, const double *U, const double *U2,
                               const double *U3, const double *lam, const double *lU3, const double *lU2,
                               const double *KT, const double *lF, const double *lD2, const double *lD3,
                               double *lam_n, double *dp, cudaStream_t st)
 {
-    k_adjoint_final<<<grid_for(N), 256, 0, st>>>(m, N, U, U2, U3, lam, lU3, lU2, KT, lF, lD2, lD3, lam_n, dp);
+    pdl_launch(k_adjoint_final, dim3(grid_for(N)), dim3(256), 0, st, 1, m, N, U, U2, U3, lam, lU3, lU2, KT, lF, lD2, lD3, lam_n, dp);
 }
 
 void launch_dot_accum_f64(int64_t n, const double *a, const double *b, double w, double *out,
                           cudaStream_t st)
 {
-    k_dot_accum<<<grid_for(n), 256, 0, st>>>(n, a, b, w, out);
+    pdl_launch(k_dot_accum, dim3(grid_for(n)), dim3(256), 0, st, 1, n, a, b, w, out);
 }
 void launch_dot_kterm_f64(const Model &m, int64_t N, const double *U, const double *F, const double *lF,
                           double *out, cudaStream_t st)
 {
-    k_dot_kterm<<<grid_for(N), 256, 0, st>>>(m, N, U, F, lF, out);
+    pdl_launch(k_dot_kterm, dim3(grid_for(N)), dim3(256), 0, st, 1, m, N, U, F, lF, out);
 }
 
 void launch_nonfinite_scan(const double *x, int64_t count, int *flag, cudaStream_t st)

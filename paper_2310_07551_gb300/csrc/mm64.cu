@@ -36,18 +36,19 @@ using namespace ptx;
 
 namespace {
 constexpr int kNanRow = INT_MAX, kInfRow = INT_MAX - 1;   // exponents of non-finite fibres
-constexpr int kChunkSlabs = 8;                            // slabs between drains: 256 entries
+constexpr int kChunkSlabs = 16;                           // slabs between drains: 256 entries
 constexpr int kSms = 152;
 
 // where waits that gave up are recorded for entry points without a plan
 __device__ DevStatus g_status;
 
 // ---------------------------------------------------------------------------
-// Digit images.  One warp takes 8 rows of one slab: lane = (row, 8
+// Digit images.  One warp takes 16 rows of one slab: lane = (row, 8
 // consecutive contracted entries), so that every digit plane is written as
-// 512 contiguous bytes.  WS warps (a power of two, at most 8) share the slabs
-// of a row group; each keeps the first slab it reads in registers, so a fibre
-// of up to 256 entries is read once.
+// 512 contiguous bytes.  WS warps (a power of two, at most 16) share the slabs
+// of a row group, each keeping the first slab it reads in registers, so a fibre
+// of up to 256 entries is read once.  24 bytes per entry pass through memory,
+// which bounds large tensors.
 // ---------------------------------------------------------------------------
 struct SplitArgs {
     int count;
@@ -55,21 +56,37 @@ struct SplitArgs {
     View v[kMaxProd];
     Image im[kMaxProd];
 };
+constexpr int kRowGroup = 16, kSplitWarps = 16;
 
-__host__ __device__ inline int split_warps(int slabs) { return slabs >= 5 ? 8 : slabs >= 3 ? 4 : slabs; }
+__host__ __device__ inline int split_warps(int slabs)
+{
+    int w = 1;
+    while (w < slabs && w < kSplitWarps) w *= 2;
+    return w;
+}
 
 __device__ __forceinline__ void load_entries(const View &v, int64_t base, bool row_ok, int slab, int chunk, int spc,
                                              unsigned long long (&x)[8])
 {
-    const int t = slab / spc, k0 = (slab - t * spc) * kSlab + chunk * 8;
+    const int t = slab / spc, k0 = (slab - t * spc) * kSlab + chunk * 8, left = row_ok ? v.n - k0 : 0;
     const double *src = v.src[t] + base + v.I * k0;
     const double sc = v.scale[t];
+    if (v.I == 1 && left >= 8 && ((uintptr_t)src & 15) == 0) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const bool ok = row_ok && k0 + j < v.n;
-        double d = ok ? src[v.I * j] : 0.0;
-        if (sc != 1.0) d = __dmul_rn(d, sc);
-        x[j] = (unsigned long long)__double_as_longlong(d);
+        for (int j = 0; j < 8; j += 2) {
+            const longlong2 d = *reinterpret_cast<const longlong2 *>(src + j);
+            x[j] = (unsigned long long)d.x;
+            x[j + 1] = (unsigned long long)d.y;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            x[j] = j < left ? (unsigned long long)__double_as_longlong(src[v.I * j]) : 0ULL;
+    }
+    if (sc != 1.0) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            x[j] = (unsigned long long)__double_as_longlong(__dmul_rn(__longlong_as_double((long long)x[j]), sc));
     }
 }
 
@@ -121,59 +138,75 @@ __device__ __forceinline__ void store_digits(const unsigned long long (&x)[8], i
     }
 }
 
-__global__ void __launch_bounds__(256) k_digits(const __grid_constant__ SplitArgs a)
+__device__ __forceinline__ unsigned long long largest(unsigned long long mx, const unsigned long long (&x)[8])
 {
-    __shared__ unsigned long long smax[8][8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mx = max(mx, x[j] & 0x7FFFFFFFFFFFFFFFULL);
+    return mx;
+}
+
+// IT: 32-bit row indices where every view allows it (their divisions are a
+// good part of a small launch)
+template <typename IT>
+__global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_constant__ SplitArgs a)
+{
+    __shared__ unsigned long long smax[kSplitWarps][kRowGroup];
     int q = 0;
     while (q + 1 < a.count && (int)blockIdx.x >= a.first[q + 1]) ++q;
     const View &v = a.v[q];
     const Image &im = a.im[q];
-    const int S = im.slabs, WS = split_warps(S), G = 8 / WS, spc = S / v.ncat;
+    const int S = im.slabs, WS = split_warps(S), G = kSplitWarps / WS, spc = S / v.ncat;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int gi = warp / WS, sub = warp % WS;
-    const int64_t groups = (im.rows + 7) / 8, g = (int64_t)(blockIdx.x - a.first[q]) * G + gi;
-    const int64_t entry = g / groups, group = g - entry * groups;   // batch entry, row group in it
-    const int row = lane >> 2, chunk = lane & 3;
-    const int64_t r = group * 8 + row;
-    const bool in = gi < G && entry < v.batch, row_ok = in && r < im.rows;
-    const int64_t rg = v.r0 + r, blocks = (im.rows + im.rb - 1) / im.rb;
-    const int64_t base = row_ok ? entry * v.stride + (rg / v.I) * (v.I * v.n) + rg % v.I : 0;
-    unsigned long long x[8], y[8], mx = 0;
+    const IT rows = (IT)im.rows, rb = (IT)im.rb, I = (IT)v.I;
+    const IT groups = (rows + kRowGroup - 1) / kRowGroup, g = (IT)(blockIdx.x - a.first[q]) * G + gi;
+    const IT entry = g / groups, group = g - entry * groups;   // batch entry, row group in it
+    const int row = lane >> 1, chunk = lane & 1;
+    const IT r = group * kRowGroup + row, rg = (IT)v.r0 + r;
+    const bool in = entry < (IT)v.batch, row_ok = in && r < rows;
+    const IT o = rg / I;
+    const int64_t base = (int64_t)entry * v.stride + (int64_t)o * (v.I * v.n) + (rg - o * I);
+    const IT first = r / rb, blocks = (rows + rb - 1) / rb;
+    const int rr = (int)(r - first * rb);
+    const int64_t plane = (int64_t)im.rb * 32;
+    uint8_t *dst = im.data + ((int64_t)entry * blocks + first) * S * kDigits * plane + rr * 32 +
+                   ((chunk ^ ((rr >> 2) & 1)) << 4);
+    pdl_wait();
+    unsigned long long x[8], mx = 0;
     load_entries(v, base, row_ok, min(sub, S - 1), chunk, spc, x);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) mx = max(mx, x[j] & 0x7FFFFFFFFFFFFFFFULL);
+    mx = largest(mx, x);
     for (int s = sub + WS; s < S; s += WS) {
-        load_entries(v, base, row_ok, s, chunk, spc, y);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) mx = max(mx, y[j] & 0x7FFFFFFFFFFFFFFFULL);
+        unsigned long long w[8];
+        load_entries(v, base, row_ok, s, chunk, spc, w);
+        mx = largest(mx, w);
     }
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
     if (chunk == 0) smax[warp][row] = mx;
     __syncthreads();
+    pdl_trigger();
     if (!in) return;
     for (int w = 0; w < WS; ++w) mx = max(mx, smax[gi * WS + w][row]);
     const int e = fibre_exp(mx);
-    if (sub == 0 && chunk == 0 && row_ok) im.exps[entry * blocks * im.rb + r] = e;
-    const int64_t blk = r / im.rb;
-    const int rr = (int)(r - blk * im.rb);
-    const int64_t plane = (int64_t)im.rb * 64;
-    uint8_t *dst = im.data + (entry * blocks + blk) * S * kDigits * plane + rr * 64 + ((chunk ^ ((rr >> 1) & 3)) << 4);
+    if (sub == 0 && chunk == 0 && row_ok) im.exps[(int64_t)entry * blocks * rb + r] = e;
     if (sub < S) store_digits(x, e, dst + (int64_t)sub * kDigits * plane, plane);
     for (int s = sub + WS; s < S; s += WS) {
-        load_entries(v, base, row_ok, s, chunk, spc, y);
-        store_digits(y, e, dst + (int64_t)s * kDigits * plane, plane);
+        unsigned long long w[8];
+        load_entries(v, base, row_ok, s, chunk, spc, w);
+        store_digits(w, e, dst + (int64_t)s * kDigits * plane, plane);
     }
 }
 
 // ---------------------------------------------------------------------------
-// The digit products.  One persistent CTA per SM; warp 0 copies digit blocks
-// (one contiguous block per operand and slab) into a two-stage ring, one
-// thread of warp 1 issues the MMAs, warps 2-9 drain.  A tile is 128 rows by
-// `nt` <= 64 columns: eight classes of 64 FP32 columns are all 512 columns of
-// tensor memory.  The digit planes of B lie one after the other in shared
-// memory, so digit p of A meets up to 256 / nt digits of B in one MMA, whose
-// output columns are the adjacent classes.
+// The digit products.  One persistent CTA per SM, in clusters of two that work
+// on adjacent column tiles of the same rows; warp 0 copies digit blocks (one
+// contiguous block per operand and slab) into a four-stage ring, one thread of
+// warp 1 issues the MMAs, two warpgroups drain.  A tile is 128 rows by `nt` <=
+// 64 columns: eight classes of 64 FP32 columns are all 512 columns of tensor
+// memory.  Such a tile reads 48 KiB of digits per 1152 clocks of MMAs, 42 bytes
+// per clock and SM where the L2 gives about 24, so each CTA of a pair loads half
+// of their common row block and writes it to both (32 KiB).  The digit planes of
+// B lie one after the other in shared memory, so digit p of A meets up to
+// 256 / nt digits of B in one MMA, whose output columns are the adjacent classes.
 // ---------------------------------------------------------------------------
 struct GProd {
     const uint8_t *A, *B;
@@ -186,31 +219,62 @@ struct GProd {
 };
 struct GArgs {
     int count;
-    int first[kMaxProd + 1];   // tile prefix
+    int first[kMaxProd + 1];   // prefix of tile pairs
     DevStatus *status;
     long long wait_limit;
     GProd p[kMaxProd];
 };
 
-// Three warpgroups: copies and MMAs (warps 0, 1; 2 and 3 idle), then two that
-// drain.  The first gives its registers up: 128 x 40 + 256 x 232 = 384 x 168,
-// the launch's total; a drain thread holds 32 outputs as two 64-bit integers.
-constexpr int kThreads = 384, kEpiThreads = 256, kStages = 2;
-constexpr uint32_t kPlaneA = kRowBlock * 64, kStageA = kDigits * kPlaneA, kStageB = kDigits * 64 * 64;
+// Five warpgroups: copies and MMAs (warps 0, 1; 2 and 3 idle), then four that
+// drain, of a quarter of the columns each.  The first gives registers up: 128 x
+// 32 + 512 x 112 = 640 x 96, the launch's total; a drain thread holds up to 16
+// outputs as two 64-bit integers.
+constexpr int kThreads = 640, kEpiThreads = 512, kStages = 4, kPair = 2, kEpiCols = 16;
+constexpr uint32_t kPlaneA = kRowBlock * 32, kStageA = kDigits * kPlaneA, kStageB = kDigits * 64 * 32;
 constexpr uint32_t kStageBytes = kStageA + kStageB;
 constexpr uint32_t kSmem = kStages * kStageBytes + 128 + 1024;
 
-// tile u: its product, batch entry, row tile and column tile
-__device__ __forceinline__ const GProd &find_unit(const GArgs &a, int u, int &entry, int &mi, int &ni)
+// pair of tiles u: its product (q: the product of an earlier one), batch entry,
+// row tile and this CTA's column tile (ntiles: none, where the tiles are odd)
+__device__ __forceinline__ const GProd &find_unit(const GArgs &a, int u, int &q, uint32_t rank, int &entry, int &mi, int &ni)
 {
-    int q = 0;
     while (q + 1 < a.count && u >= a.first[q + 1]) ++q;
     const GProd &p = a.p[q];
-    const int t = u - a.first[q], row = t / p.ntiles;
-    ni = t - row * p.ntiles;
+    const int pairs = (p.ntiles + kPair - 1) / kPair;
+    const int t = u - a.first[q], row = t / pairs;
+    ni = (t - row * pairs) * kPair + (int)rank;
     entry = row / p.mtiles;
     mi = row - entry * p.mtiles;
     return p;
+}
+
+// The MMAs of one slab: 36 digit products, in 12 (8, for at most 32 columns)
+// instructions.  Digit p of A stays in the collector buffer across the
+// instructions that share it.  fresh: the accumulators start at zero (digit 0 of
+// A meets every digit of B, that is every class, first).  Issued from compile-
+// time tables: with the descriptors formed in a loop one thread took 400 clocks
+// per instruction, three times the MMAs' own time.
+template <int NT>
+__device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t sA, uint32_t sB, bool fresh)
+{
+    constexpr int PER = 256 / NT < kDigits ? 256 / NT : kDigits;   // digits of B per MMA
+    const uint64_t a0 = desc_sw32(sA), b0 = desc_sw32(sB);
+#pragma unroll
+    for (int p = 0; p < kDigits; ++p) {
+        const uint64_t ad = a0 + (uint64_t)(p * kPlaneA >> 4);
+        const uint32_t acc = p == 0 && fresh ? 0u : 1u;
+        const int nq = kDigits - p;
+#pragma unroll
+        for (int q = 0; q < nq; q += PER) {
+            const int w = nq - q < PER ? nq - q : PER;
+            const uint64_t bd = b0 + (uint64_t)(q * NT * 32 >> 4);
+            const uint32_t d = tmem + (p + q) * NT, id = idesc_f16(kRowBlock, w * NT);
+            if (nq <= PER) mma_f16<0>(d, ad, bd, id, acc);
+            else if (q == 0) mma_f16<1>(d, ad, bd, id, acc);
+            else if (q + PER < nq) mma_f16<2>(d, ad, bd, id, acc);
+            else mma_f16<3>(d, ad, bd, id, acc);
+        }
+    }
 }
 
 // all eight classes of four columns, complete on return
@@ -243,33 +307,89 @@ __device__ __forceinline__ void load_classes(uint32_t taddr, uint32_t cs, uint32
         : "memory");
 }
 
-// (P 2^30 + Q) 2^e rounded to nearest even, in integers: the FP64 pipe would
-// take longer than the digit products
-__device__ __forceinline__ double combine(long long P, long long Q, int e)
+// The classes of a thread's `hc` columns as P 2^30 + Q in units of 2^-6 of class
+// 5: classes 0 .. 2 in P, the rest in Q.  ADD: on top of the earlier entries'.
+template <bool ADD>
+__device__ __forceinline__ void drain(uint32_t taddr, uint32_t cs, int hc, long long (&P)[kEpiCols], long long (&Q)[kEpiCols])
 {
-    long long H = P + (Q >> 30);
-    uint32_t L = (uint32_t)Q & 0x3FFFFFFFu;
-    const bool neg = H < 0;
-    if (neg) {
-        H = -H - (L ? 1 : 0);
-        L = (0u - L) & 0x3FFFFFFFu;
+#pragma unroll
+    for (int g = 0; g < kEpiCols / 4; ++g) {
+        if (g * 4 < hc) {
+            uint32_t v[32];
+            load_classes(taddr + g * 4, cs, v);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                auto cls = [&](int t) { return __uint_as_float(v[t * 4 + j]); };
+                const int c0 = __float2int_rn(cls(0)), c1 = __float2int_rn(cls(1)), c2 = __float2int_rn(cls(2));
+                const int c3 = __float2int_rn(cls(3)), c4 = __float2int_rn(cls(4));
+                const int c5 = __float2int_rn(fmaf(cls(7), 0x1p-10f, fmaf(cls(6), 0.25f, 64.0f * cls(5))));
+                const long long hp = (long long)c0 * 65536 + (c1 * 256 + c2);
+                const long long lp = (long long)c3 * 4194304 + ((long long)c4 * 16384 + c5);
+                P[g * 4 + j] = ADD ? P[g * 4 + j] + hp : hp;
+                Q[g * 4 + j] = ADD ? Q[g * 4 + j] + lp : lp;
+            }
+        }
     }
-    const int top = 64 - __clzll(H);
-    const int sh = max(0, top - 33);
-    const unsigned long long V = ((unsigned long long)H << (30 - sh)) | (L >> sh);
+}
+
+// P 2^30 + Q rounded to 53 bits, in 32-bit integers without branches (the FP64
+// pipe would take longer than the digit products).  The value is hi:lo, with the
+// leading bit at bit 52, times 2^(E - 52) and the sign.
+struct Rounded {
+    uint32_t lo, hi, sign;
+    int E;
+};
+__device__ __forceinline__ Rounded round_sum(long long P, long long Q, int e)
+{
+    // 96 bits: H = P + (Q >> 30) above the low 30 bits of Q; the magnitude as a
+    // ones' complement (2^-32 of H off: far below the last kept bit)
+    const long long H = P + (Q >> 30);
+    uint32_t w0 = (uint32_t)Q << 2, w1 = (uint32_t)H, w2 = (uint32_t)((unsigned long long)H >> 32);
+    const uint32_t neg = (uint32_t)((int)w2 >> 31);
+    w0 ^= neg;
+    w1 ^= neg;
+    w2 ^= neg;
+    // leading word up, then the leading bit
+    const bool z = w2 == 0;
+    w2 = z ? w1 : w2;
+    w1 = z ? w0 : w1;
+    w0 = z ? 0u : w0;
+    const int lz = __clz((int)w2);
+    const uint32_t m1 = __funnelshift_l(w1, w2, lz), m0 = __funnelshift_l(w0, w1, lz);
+    Rounded r;
+    // 53 of the 64 leading bits, to nearest; a carry moves up into the exponent
+    asm("{\n\t.reg .u32 a, b, c;\n\tadd.cc.u32 a, %2, 0x400;\n\taddc.cc.u32 b, %3, 0;\n\taddc.u32 c, 0, 0;\n\t"
+        "shf.r.clamp.b32 %0, a, b, 11;\n\tshf.r.clamp.b32 %1, b, c, 11;\n\t}"
+        : "=r"(r.lo), "=r"(r.hi)
+        : "r"(m0), "r"(m1));
+    r.sign = neg & 0x80000000u;
+    r.E = e + 93 - lz - (z ? 32 : 0);
+    if (w2 == 0) r.E = INT_MIN / 2;   // |H| = 0: left to round_rare
+    return r;
+}
+// what round_sum leaves: zero, sums below 2^-30 of class 2's unit, results
+// outside the normal range
+__device__ __noinline__ double round_rare(long long P, long long Q, int e)
+{
+    const long long H = P + (Q >> 30), L = Q & 0x3FFFFFFF;
+    const bool neg = H < 0;
+    // |H| 2^30 + |L|; below 2^64 wherever |H| < 2^34, else the low bits go
+    unsigned long long V = 0;
+    long long h = H, l = L;
+    if (neg) {
+        h = -H - (L ? 1 : 0);
+        l = L ? 0x40000000 - L : 0;
+    }
+    int sh = 0;
+    while (h >> (33 + sh)) ++sh;
+    V = ((unsigned long long)h << (30 - sh)) | ((unsigned long long)l >> sh);
     if (V == 0) return 0.0;
     const int lz = __clzll((long long)V);
-    const unsigned long long M = V << lz;
-    unsigned long long m = M >> 11;
-    const uint32_t rem = (uint32_t)M & 0x7FFu;
-    m += rem > 0x400u || (rem == 0x400u && (m & 1));
-    const int E = e + sh - lz + 63;   // value in [2^E, 2^(E + 1)]
-    double r;
-    if (E >= -1022 && E <= 1022) {
-        r = __longlong_as_double((long long)(((unsigned long long)(E + 1022) << 52) + m));
-    } else {
-        r = scalbn(__longlong_as_double((long long)((1022ULL << 52) + m)), max(-3000, min(3000, E)));
-    }
+    V <<= lz;
+    unsigned long long m = (V >> 11) + (V >> 10 & 1);
+    const int E = e + sh - lz + 63;   // m 2^(E - 52)
+    if (E < -1200) return neg ? -0.0 : 0.0;
+    const double r = scalbn((double)m, max(-2000, min(2000, E)) - 52);
     return neg ? -r : r;
 }
 
@@ -293,16 +413,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_addr(smem_raw), base = (raw + 1023u) & ~1023u;
     const uint32_t bars = base + kStages * kStageBytes;
-    uint32_t *tmem_slot = (uint32_t *)(smem_raw + (bars - raw) + 64);
+    uint32_t *tmem_slot = (uint32_t *)(smem_raw + (bars - raw) + 8 * (2 * kStages + 3));
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
-    const uint32_t FULL = bars, EMPTY = bars + 16, TFULL = bars + 32, TEMPTY = bars + 40, DRAIN = bars + 48;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t FULL = bars, EMPTY = bars + 8 * kStages, TFULL = EMPTY + 8 * kStages, TEMPTY = TFULL + 8, DRAIN = TFULL + 16;
+    const uint32_t rank = cluster_rank();
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
     const int units = a.first[a.count];
     DevStatus *const status = a.status ? a.status : &g_status;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             bar_init(FULL + 8 * s, 1);
-            bar_init(EMPTY + 8 * s, 1);
+            bar_init(EMPTY + 8 * s, kPair);   // both CTAs' MMAs are done with it
         }
         bar_init(TFULL, 1);
         bar_init(TEMPTY, kEpiThreads);
@@ -318,179 +439,187 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_before();
-    __syncthreads();
+    cluster_sync();
     tc_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_trigger();
+    pdl_wait();
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-        if (warp == 0 && lane == 0) {
-            int stage = 0;
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+        if (warp == 0) {
+            int stage = 0, q = 0, issued = 0;
             uint32_t phase = 0;
-            int issued[kStages] = {-1, -1};
             bool ok = true;
-            for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+            for (int u = blockIdx.x / kPair; ok && u < units; u += gridDim.x / kPair) {
                 int be, mi, ni;
-                const GProd &p = find_unit(a, u, be, mi, ni);
-                const uint32_t nb = (uint32_t)p.nt * 64 * kDigits;
-                const uint8_t *A = p.A + ((int64_t)be * p.mtiles + mi) * p.slabs * kStageA;
-                const uint8_t *B = p.B + ((int64_t)be * p.ntiles + ni) * p.slabs * nb;
-                for (int s = 0; s < p.slabs; ++s) {
-                    if (!bar_wait(EMPTY + 8 * stage, phase ^ 1u, abort_flag, status, 11, a.wait_limit)) {
-                        ok = false;
-                        break;
+                const GProd &p = find_unit(a, u, q, rank, be, mi, ni);
+                const uint32_t nb = (uint32_t)p.nt * 32 * kDigits;
+                const int slabs = p.slabs;
+                const uint8_t *A = p.A + ((int64_t)be * p.mtiles + mi) * slabs * kStageA + rank * (kStageA / 2);
+                const uint8_t *B = p.B + ((int64_t)be * p.ntiles + min(ni, p.ntiles - 1)) * slabs * nb;
+                for (int s = 0; s < slabs; ++s) {
+                    ok = __all_sync(0xffffffffu, bar_wait(EMPTY + 8 * stage, phase ^ 1u, abort_flag, status, 11, a.wait_limit));
+                    if (!ok) break;
+                    if (elect_one()) {
+                        const uint32_t sA = base + stage * kStageBytes;
+                        bar_expect(FULL + 8 * stage, kStageA + nb);
+                        bulk_load(sA + kStageA, B, nb, FULL + 8 * stage);
+                        bulk_load_pair(sA + rank * (kStageA / 2), A, kStageA / 2, FULL + 8 * stage);
                     }
-                    const uint32_t sA = base + stage * kStageBytes;
-                    bar_expect(FULL + 8 * stage, kStageA + nb);
-                    bulk_load(sA + kStageA, B + (int64_t)s * nb, nb, FULL + 8 * stage);
-                    bulk_load(sA, A + (int64_t)s * kStageA, kStageA, FULL + 8 * stage);
-                    issued[stage] = (int)phase;
+                    __syncwarp();
+                    A += kStageA;
+                    B += nb;
+                    ++issued;
                     if (++stage == kStages) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
             }
-            // every issued copy lands before the CTA exits
-            for (int s = 0; s < kStages; ++s)
-                if (issued[s] >= 0) {
-                    volatile int never = 0;
-                    bar_wait(FULL + 8 * s, (uint32_t)issued[s], &never, nullptr, 0, kWaitCycles);
-                }
+            // every issued copy lands, and the other CTA's last releases arrive,
+            // before the CTA exits
+            for (int s = max(0, issued - kStages); s < issued; ++s) {
+                const uint32_t st = s % kStages, ph = s / kStages & 1;
+                volatile int never = 0;
+                bar_wait(FULL + 8 * st, ph, &never, nullptr, 0, kWaitCycles);
+                if (ok) bar_wait(EMPTY + 8 * st, ph, abort_flag, nullptr, 0, kWaitCycles);
+            }
         }
-        if (warp == 1 && lane == 0) {
-            int stage = 0;
+        if (warp == 1) {
+            int stage = 0, q = 0;
             uint32_t phase = 0, tphase = 0;
             bool ok = true;
-            for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+            for (int u = blockIdx.x / kPair; ok && u < units; u += gridDim.x / kPair) {
                 int be, mi, ni;
-                const GProd &p = find_unit(a, u, be, mi, ni);
-                const uint32_t nt = (uint32_t)p.nt;
-                const int per = min((int)(256u / nt), kDigits);   // digits of B per MMA
-                for (int s = 0; ok && s < p.slabs; ++s) {
+                const GProd &p = find_unit(a, u, q, rank, be, mi, ni);
+                const int nt = p.nt, slabs = p.slabs;
+                for (int s = 0; s < slabs; ++s) {
                     const bool fresh = s % kChunkSlabs == 0;
                     if (fresh) {
-                        if (!bar_wait(TEMPTY, tphase ^ 1u, abort_flag, status, 12, a.wait_limit)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_after();
+                        ok = __all_sync(0xffffffffu, bar_wait(TEMPTY, tphase ^ 1u, abort_flag, status, 12, a.wait_limit));
+                        if (!ok) break;
                         tphase ^= 1u;
                     }
-                    if (!bar_wait(FULL + 8 * stage, phase, abort_flag, status, 13, a.wait_limit)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, bar_wait(FULL + 8 * stage, phase, abort_flag, status, 13, a.wait_limit));
+                    if (!ok) break;
                     tc_after();
                     const uint32_t sA = base + stage * kStageBytes, sB = sA + kStageA;
-#pragma unroll 1
-                    for (int ks = 0; ks < kSlab / 16; ++ks) {
-#pragma unroll 1
-                        for (int pd = 0; pd < kDigits; ++pd) {
-                            const uint64_t ad = desc_sw64(sA + pd * kPlaneA + ks * 32);
-                            const uint32_t acc = fresh && ks == 0 && pd == 0 ? 0u : 1u;
-                            const int nq = kDigits - pd;
-                            for (int q = 0; q < nq; q += per) {
-                                const int w = min(per, nq - q);
-                                const uint64_t bd = desc_sw64(sB + q * nt * 64 + ks * 32);
-                                const uint32_t d = tmem + (pd + q) * nt, id = idesc_f16(kRowBlock, w * nt);
-                                if (nq <= per) mma_f16<0>(d, ad, bd, id, acc);
-                                else if (q == 0) mma_f16<1>(d, ad, bd, id, acc);
-                                else if (q + per < nq) mma_f16<2>(d, ad, bd, id, acc);
-                                else mma_f16<3>(d, ad, bd, id, acc);
-                            }
+                    if (elect_one()) {
+                        switch (nt) {
+                        case 64: issue_slab<64>(tmem, sA, sB, fresh); break;
+                        case 48: issue_slab<48>(tmem, sA, sB, fresh); break;
+                        case 32: issue_slab<32>(tmem, sA, sB, fresh); break;
+                        default: issue_slab<16>(tmem, sA, sB, fresh); break;
                         }
+                        mma_commit_pair(EMPTY + 8 * stage);
+                        if (s + 1 == slabs || s % kChunkSlabs == kChunkSlabs - 1) mma_commit_to(TFULL);
                     }
-                    mma_commit_to(EMPTY + 8 * stage);
+                    __syncwarp();
                     if (++stage == kStages) {
                         stage = 0;
                         phase ^= 1u;
                     }
-                    if (s + 1 == p.slabs || s % kChunkSlabs == kChunkSlabs - 1) mma_commit_to(TFULL);
                 }
             }
-            mma_commit_to(DRAIN);
+            if (elect_one()) mma_commit_to(DRAIN);
+            __syncwarp();
             volatile int never = 0;
             bar_wait(DRAIN, 0, &never, nullptr, 0, kWaitCycles);
         }
     } else {
-        // warp w reads the tensor-memory lanes 32 (w % 4) ..; the two warps of a
-        // lane quarter take half of the columns each
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
-        const int quarter = warp % 4, half = (warp - 4) / 4;
+        // warp w reads the tensor-memory lanes 32 (w % 4) ..; the four warps of a
+        // lane quarter take a quarter of the columns each
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        const int quarter = warp % 4, part = (warp - 4) / 4;
         const int m = quarter * 32 + lane;
         uint32_t tphase = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < units; u += gridDim.x) {
+        int q = 0;
+        for (int u = blockIdx.x / kPair; u < units; u += gridDim.x / kPair) {
             int be, mi, ni;
-            const GProd &p = find_unit(a, u, be, mi, ni);
-            const int nt = p.nt, hc = nt / 2;
+            const GProd &p = find_unit(a, u, q, rank, be, mi, ni);
+            const int nt = p.nt, hc = nt / 4;
             const int64_t r = (int64_t)mi * kRowBlock + m;
             const bool row_ok = r < p.rows;
-            long long P[32], Q[32];
+            // exponents and addresses while the MMAs run
+            const int c0 = ni * nt + part * hc;
+            const int er = row_ok ? __ldg(p.eA + (int64_t)be * p.mtiles * kRowBlock + r) : 0;
+            const int ec = lane < hc && c0 + lane < p.cols ? __ldg(p.eB + (int64_t)be * p.ntiles * nt + c0 + lane) : 0;
+            // a column of the warp's that is not finite: every row takes the slow form
+            const bool odd_col = __any_sync(0xffffffffu, ec >= kInfRow);
+            const int64_t rg = p.r0 + r, ro = (rg | p.I) >> 32 ? rg / p.I : (int64_t)((uint32_t)rg / (uint32_t)p.I);
+            double *const out = p.out + be * p.sOut + ro * (p.I * p.cols) + (rg - ro * p.I) + p.I * c0;
+            long long P[kEpiCols], Q[kEpiCols];
             for (int s0 = 0; s0 < p.slabs; s0 += kChunkSlabs) {
                 ok = ok && __all_sync(0xffffffffu, bar_wait(TFULL, tphase, abort_flag, status, 14, a.wait_limit));
                 if (!ok) break;
                 tphase ^= 1u;
                 tc_after();
-                const uint32_t tq = tmem + (uint32_t)(half * hc) + ((uint32_t)(quarter * 32) << 16);
-#pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                    if (g * 4 < hc) {
-                        uint32_t v[32];
-                        load_classes(tq + g * 4, (uint32_t)nt, v);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            // classes 0..2 in units of class 2, the rest in 2^-30 of that
-                            const int c0 = __float2int_rn(__uint_as_float(v[j]));
-                            const int c1 = __float2int_rn(__uint_as_float(v[4 + j]));
-                            const int c2 = __float2int_rn(__uint_as_float(v[8 + j]));
-                            const int c3 = __float2int_rn(__uint_as_float(v[12 + j]));
-                            const int c4 = __float2int_rn(__uint_as_float(v[16 + j]));
-                            const float f = fmaf(__uint_as_float(v[28 + j]), 0x1p-10f,
-                                                 fmaf(__uint_as_float(v[24 + j]), 0.25f, 64.0f * __uint_as_float(v[20 + j])));
-                            const int c5 = __float2int_rn(f);
-                            const long long hp = (long long)c0 * 65536 + ((long long)c1 * 256 + c2);
-                            const long long lp = (long long)c3 * 4194304 + ((long long)c4 * 16384 + c5);
-                            P[g * 4 + j] = s0 ? P[g * 4 + j] + hp : hp;
-                            Q[g * 4 + j] = s0 ? Q[g * 4 + j] + lp : lp;
-                        }
-                    }
-                }
+                const uint32_t tq = tmem + (uint32_t)(part * hc) + ((uint32_t)(quarter * 32) << 16);
+                if (s0 == 0) drain<false>(tq, (uint32_t)nt, hc, P, Q);
+                else drain<true>(tq, (uint32_t)nt, hc, P, Q);
                 tc_before();
                 bar_arrive(TEMPTY);
             }
-            if (!row_ok) continue;
-            const int er = p.eA[(int64_t)be * p.mtiles * kRowBlock + r];
-            const int *eb = p.eB + (int64_t)be * p.ntiles * nt + ni * nt + half * hc;
-            const int64_t rg = p.r0 + r;
-            const int64_t o0 = (rg / p.I) * (p.I * p.cols) + rg % p.I;
-            const int c0 = ni * nt + half * hc;
-            double *out = p.out + be * p.sOut + o0 + p.I * c0;
-            bool odd = !ok || er >= kInfRow;   // some output needs more than the digits
+            const bool odd = !ok || odd_col || er >= kInfRow;
+            // (every lane takes part in the shuffles of the column exponents)
+            if (!__all_sync(0xffffffffu, odd)) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                if (j < hc && c0 + j < p.cols) {
-                    const int ec = __ldg(eb + j);
-                    odd = odd || ec >= kInfRow;
-                    if (!odd) {
-                        const double z = combine(P[j], Q[j], er + ec - 58);
-                        double *o = out + p.I * j;
-                        *o = p.accumulate ? __dadd_rn(*o, z) : z;
+                for (int g = 0; g < kEpiCols / 4; ++g) {
+                    if (g * 4 < hc && c0 + g * 4 < p.cols) {
+                        double z[4];
+                        bool rare = false;
+                        int e[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            e[j] = er + __shfl_sync(0xffffffffu, ec, g * 4 + j) - 58;
+                            const Rounded y = round_sum(P[g * 4 + j], Q[g * 4 + j], e[j]);
+                            const uint32_t x = (uint32_t)(y.E + 1022);   // biased exponent - 1
+                            rare |= x >= 2045u;
+                            z[j] = __hiloint2double((int)((y.hi + (x << 20)) | y.sign), (int)y.lo);
+                        }
+                        if (rare) {
+#pragma unroll 1
+                            for (int j = 0; j < 4; ++j) {
+                                const long long pj = j == 0 ? P[g * 4] : j == 1 ? P[g * 4 + 1] : j == 2 ? P[g * 4 + 2] : P[g * 4 + 3];
+                                const long long qj = j == 0 ? Q[g * 4] : j == 1 ? Q[g * 4 + 1] : j == 2 ? Q[g * 4 + 2] : Q[g * 4 + 3];
+                                const int ej = j == 0 ? e[0] : j == 1 ? e[1] : j == 2 ? e[2] : e[3];
+                                const double r = round_rare(pj, qj, ej);
+                                if (j == 0) z[0] = r;
+                                else if (j == 1) z[1] = r;
+                                else if (j == 2) z[2] = r;
+                                else z[3] = r;
+                            }
+                        }
+                        double *o = out + p.I * (g * 4);
+                        if (!row_ok || odd) continue;
+                        if (c0 + g * 4 + 3 < p.cols && !p.accumulate) {
+                            if (p.I == 1 && ((uintptr_t)o & 31) == 0) {
+                                asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(o), "d"(z[0]), "d"(z[1]),
+                                             "d"(z[2]), "d"(z[3])
+                                             : "memory");
+                            } else {
+                                o[0] = z[0];
+                                o[p.I] = z[1];
+                                o[2 * p.I] = z[2];
+                                o[3 * p.I] = z[3];
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if (c0 + g * 4 + j < p.cols) o[p.I * j] = p.accumulate ? __dadd_rn(o[p.I * j], z[j]) : z[j];
+                        }
                     }
                 }
             }
-            if (odd) {
-                // a non-finite row or column (or an abandoned wait: NaN); the outputs
-                // before its first flagged column are already stored
-                bool seen = !ok || er >= kInfRow;
+            if (odd && row_ok) {
+                // non-finite entries, or an abandoned wait (NaN)
 #pragma unroll 1
                 for (int j = 0; j < hc && c0 + j < p.cols; ++j) {
-                    const int ec = __ldg(eb + j);
-                    seen = seen || ec >= kInfRow;
-                    if (!seen) continue;
-                    const double z = !ok || er == kNanRow || ec == kNanRow ? __longlong_as_double(0x7FF8000000000000LL)
-                                                                          : fma_chain(p, be, rg, c0 + j);
+                    const int e = __ldg(p.eB + (int64_t)be * p.ntiles * nt + c0 + j);
+                    const double z = !ok || er == kNanRow || e == kNanRow ? __longlong_as_double(0x7FF8000000000000LL)
+                                                                         : fma_chain(p, be, rg, c0 + j);
                     double *o = out + p.I * j;
                     *o = p.accumulate ? __dadd_rn(*o, z) : z;
                 }
@@ -498,30 +627,40 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
         }
     }
     tc_before();
-    __syncthreads();
+    // the other CTA may still write into this one's shared memory until here
+    cluster_sync();
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
 // ---------------------------------------------------------------------------
-// The FP64 pipe's own kernel for small products: one thread per output, so
-// that even a 64 x 64 product spreads over every SM (a 64 x 64 tile would keep
-// one SM's FP64 pipe busy for 63 us).
+// The FP64 pipe's own kernel for small products: four lanes per output, each
+// with every fourth entry of the contraction, so that even a 64 x 64 product
+// spreads over every SM (a 64 x 64 tile would keep one SM's FP64 pipe busy for
+// 63 us) and the chain of dependent FMAs is a quarter of the contraction.
 // ---------------------------------------------------------------------------
 struct FArgs {
     int count;
     int64_t first[kMaxProd + 1];   // output prefix
     GProd p[kMaxProd];
 };
+constexpr int kLanes = 4;
+
 __global__ void __launch_bounds__(128) k_fma_products(const __grid_constant__ FArgs a)
 {
     const int64_t total = a.first[a.count];
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int sub = threadIdx.x % kLanes;
+    pdl_trigger();
+    pdl_wait();
+    // whole warps stay in the loop for the shuffles
+    for (int64_t e0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32 * (32 / kLanes); e0 < total;
+         e0 += (int64_t)gridDim.x * blockDim.x / kLanes) {
+        const int64_t e = min(e0 + threadIdx.x % 32 / kLanes, total - 1);
         int q = 0;
         while (q + 1 < a.count && e >= a.first[q + 1]) ++q;
         const GProd &p = a.p[q];
         const int64_t size = p.rows * p.cols, entry = (e - a.first[q]) / size, t = e - a.first[q] - entry * size;
-        // neighbouring threads: neighbouring outputs in memory
+        // neighbouring lanes: neighbouring outputs in memory
         int64_t r;
         int i;
         if (p.I == 1) {
@@ -532,9 +671,32 @@ __global__ void __launch_bounds__(128) k_fma_products(const __grid_constant__ FA
             i = (int)(w / p.I);
             r = o * p.I + (w - i * p.I);
         }
-        const double s = fma_chain(p, entry, r, i);
-        double *o = p.out + entry * p.sOut + t;
-        *o = p.accumulate ? __dadd_rn(*o, s) : s;
+        const int64_t xa = entry * p.sA + (r / p.I) * (p.I * p.n) + r % p.I;
+        const int64_t lb = entry * p.sB + (i / p.IB) * (p.IB * p.n) + i % p.IB;
+        double y = 0.0;
+        for (int c = 0; c < p.ncat; ++c) {
+            const double *x = p.X[c] + xa, *l = p.L[c] + lb;
+            double s = 0.0;
+            int k = sub;
+            for (; k + 3 * kLanes < p.n; k += 4 * kLanes) {
+                double xv[4], lv[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    xv[j] = x[p.I * (k + j * kLanes)];
+                    lv[j] = l[p.IB * (k + j * kLanes)];
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) s = fma(xv[j], lv[j], s);
+            }
+            for (; k < p.n; k += kLanes) s = fma(x[p.I * k], l[p.IB * k], s);
+            y = p.sc[c] == 1.0 && c == 0 ? s : fma(p.sc[c], s, y);
+        }
+#pragma unroll
+        for (int w = 1; w < kLanes; w *= 2) y += __shfl_xor_sync(0xffffffffu, y, w);
+        if (sub == 0 && e0 + threadIdx.x % 32 / kLanes < total) {
+            double *o = p.out + entry * p.sOut + t;
+            *o = p.accumulate ? __dadd_rn(*o, y) : y;
+        }
     }
 }
 
@@ -572,13 +734,16 @@ GProd to_gprod(const Product &s)
 
 int tile_cols(int64_t rows, int cols, int products)
 {
+    // an even number of tiles, so that no CTA of a pair idles; narrower tiles
+    // while the launch would leave SMs without one
     const int64_t mt = (rows + kRowBlock - 1) / kRowBlock * products;
-    for (int w = 64; w > 16; w -= 16)
-        if (mt * ((cols + w - 1) / w) >= kSms) {
-            const int nb = (cols + w - 1) / w;
-            return ((cols + nb - 1) / nb + 15) / 16 * 16;
-        }
-    return 16;
+    int nt = 16;
+    for (int w = 64; w >= 16; w -= 16) {
+        const int nb = (cols + w * kPair - 1) / (w * kPair) * kPair;
+        nt = std::min(w, ((cols + nb - 1) / nb + 15) / 16 * 16);
+        if (mt * ((cols + nt - 1) / nt) >= kSms) break;
+    }
+    return nt;
 }
 
 bool use_digits(int64_t rows, int n, int count)
@@ -591,14 +756,17 @@ void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
 {
     SplitArgs a{};
     a.count = count;
+    bool wide = false;
     for (int q = 0; q < count; ++q) {
         a.v[q] = v[q];
         a.im[q] = im[q];
-        const int G = 8 / split_warps(im[q].slabs);
-        const int64_t groups = (im[q].rows + 7) / 8 * v[q].batch;
+        const int G = kSplitWarps / split_warps(im[q].slabs);
+        const int64_t groups = (im[q].rows + kRowGroup - 1) / kRowGroup * v[q].batch;
         a.first[q + 1] = a.first[q] + (int)((groups + G - 1) / G);
+        wide = wide || (v[q].r0 + im[q].rows + kRowGroup * 32) * std::max(1, v[q].batch) > INT32_MAX || v[q].I > INT32_MAX;
     }
-    k_digits<<<a.first[count], 256, 0, st>>>(a);
+    if (wide) pdl_launch(k_digits<int64_t>, dim3(a.first[count]), dim3(kSplitWarps * 32), 0, st, 1, a);
+    else pdl_launch(k_digits<int>, dim3(a.first[count]), dim3(kSplitWarps * 32), 0, st, 1, a);
 }
 
 void launch_products(const Product *s, int count, DevStatus *status, long long wait_limit, cudaStream_t st)
@@ -616,11 +784,11 @@ void launch_products(const Product *s, int count, DevStatus *status, long long w
     a.wait_limit = wait_limit;
     for (int q = 0; q < count; ++q) {
         a.p[q] = to_gprod(s[q]);
-        a.first[q + 1] = a.first[q] + a.p[q].mtiles * a.p[q].ntiles * s[q].A.batch;
+        a.first[q + 1] = a.first[q] + a.p[q].mtiles * ((a.p[q].ntiles + kPair - 1) / kPair) * s[q].A.batch;
     }
     const int units = a.first[count];
     if (units == 0) return;
-    k_digit_products<<<std::min(units, kSms), kThreads, kSmem, st>>>(a);
+    pdl_launch(k_digit_products, dim3(kPair * std::min(units, kSms / kPair)), dim3(kThreads), kSmem, st, kPair, a);
 }
 
 void launch_products_fma(const Product *s, int count, cudaStream_t st)
@@ -633,7 +801,7 @@ void launch_products_fma(const Product *s, int count, cudaStream_t st)
     }
     const int64_t total = a.first[count];
     if (total == 0) return;
-    k_fma_products<<<(int)std::min<int64_t>((total + 127) / 128, kSms * 16), 128, 0, st>>>(a);
+    pdl_launch(k_fma_products, dim3((int)std::min<int64_t>((total * kLanes + 127) / 128, kSms * 16)), dim3(128), 0, st, 1, a);
 }
 
 View tensor_view(int d, const int64_t *n, int mu, const double *X)

@@ -10,7 +10,7 @@ namespace mm {
 
 constexpr int kMaxCat = 6;      // operand pairs concatenated along the contraction
 constexpr int kMaxProd = 24;    // products of one launch
-constexpr int kSlab = 32;       // contraction indices per slab (one 64-byte row of FP16 digits)
+constexpr int kSlab = 16;       // contraction indices per slab (one 32-byte row of FP16 digits)
 constexpr int kDigits = 8;
 constexpr int kRowBlock = 128;  // rows of a tensor image's block
 

@@ -55,6 +55,16 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile
     }
     return true;
 }
+// One lane of a converged warp, the same each time.  A role's loop runs on the
+// whole warp with only its asynchronous instructions under this predicate: the
+// operands then stay in uniform registers, where a lone thread moves each of
+// them there per instruction.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+    return p != 0;
+}
 // bytes, dst and src multiples of 16
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
 {
@@ -62,15 +72,34 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
+// the same into both CTAs of a cluster of two, at the same offsets in each
+__device__ __forceinline__ void bulk_load_pair(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
+                 " [%0], [%1], %2, [%3], %4;" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar), "h"((unsigned short)3)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// shared-memory matrix descriptor, K-major rows of 64 bytes in the 64-byte
-// swizzle: 8-row groups 512 bytes apart
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t addr)
+// shared-memory matrix descriptor, K-major rows of 32 bytes in the 32-byte
+// swizzle: 8-row groups 256 bytes apart
+__device__ __forceinline__ uint64_t desc_sw32(uint32_t addr)
 {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | (uint64_t)(16 >> 4) << 16 | (uint64_t)(512 >> 4) << 32 |
-           (uint64_t)1 << 46 | (uint64_t)4 << 61;
+    return (uint64_t)((addr >> 4) & 0x3FFF) | (uint64_t)(16 >> 4) << 16 | (uint64_t)(256 >> 4) << 32 |
+           (uint64_t)1 << 46 | (uint64_t)6 << 61;
 }
 // kind::f16 instruction descriptor, FP16 x FP16 -> FP32, both operands K-major
 __device__ __forceinline__ uint32_t idesc_f16(int M, int N)
@@ -97,13 +126,12 @@ __device__ __forceinline__ void mma_commit_to(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tmem_load4(uint32_t taddr, uint32_t (&v)[4])
+// the same on the barriers at that offset of both CTAs of a cluster of two
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar)
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                 : "r"(taddr));
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+                 "h"((unsigned short)3)
+                 : "memory");
 }
-__device__ __forceinline__ void tmem_load_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
 }  // namespace ptx
 }  // namespace ds
