@@ -38,6 +38,7 @@
 #include <tuple>
 #include <vector>
 
+#include "ptx.cuh"
 #include "tc.h"
 
 namespace ds {
@@ -1080,7 +1081,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #define EPI_BAR (bar0 + 8u * (2 * STAGES + 5))
 #define EPI_DEC (bar0 + 8u * (2 * STAGES + 6))
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(FULL(s), 1);
@@ -1110,8 +1111,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    // The producer's and the issuer's loops run on their whole warp, with the
+    // asynchronous instructions under elect_one(): a lone thread would move every
+    // operand of every MMA into uniform registers first, ~130 clocks each, as long
+    // as a 128 x 256 x 16 MMA itself (FX launches at (256, 256, 128): 600, 609 and
+    // 320 us with one thread, 548, 526 and 275 so).
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // ---------------- TMA producer ----------------
             int stage = 0;
             uint32_t phase = 0;
@@ -1134,28 +1140,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int it0 = sk ? itr.k0 : part * a.kpi, it1 = sk ? itr.k1 : min(it0 + a.kpi, kiters);
                 for (int it = it0; it < it1; ++it) {
                     const int tt = it / a.kchunks, kc = it % a.kchunks;
-                    if (!wait_bar(EMPTY(stage), phase ^ 1u, abort_flag, a.status, 1, a.wait_limit)) { ok = false; break; }
-                    mbar_expect_tx(FULL(stage), STAGE_BYTES);
-                    const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + STAGE_A;
-                    const int xc = (tc.s / a.xs_div) * a.xs_stride + tt, pc = tc.s * a.T + tt;
-                    if (MODE1) {
+                    ok = __all_sync(0xffffffffu, wait_bar(EMPTY(stage), phase ^ 1u, abort_flag, a.status, 1, a.wait_limit));
+                    if (!ok) break;
+                    if (ptx::elect_one()) {
+                        mbar_expect_tx(FULL(stage), STAGE_BYTES);
+                        const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + STAGE_A;
+                        const int xc = (tc.s / a.xs_div) * a.xs_stride + tt, pc = tc.s * a.T + tt;
+                        if (MODE1) {
 #pragma unroll
-                        for (int p = 0; p < NP; ++p)
-                            tma_load_4d(sA + p * A_PLANE, &a.tmA, FULL(stage), kc * BK, tc.mt * BM, p, pc);
+                            for (int p = 0; p < NP; ++p)
+                                tma_load_4d(sA + p * A_PLANE, &a.tmA, FULL(stage), kc * BK, tc.mt * BM, p, pc);
 #pragma unroll
-                        for (int p = 0; p < NP; ++p)
-                            tma_load_4d(sB + p * B_PLANE, &a.tmB, FULL(stage), kc * BK, tc.nt * BN, p, xc);
-                    } else {
+                            for (int p = 0; p < NP; ++p)
+                                tma_load_4d(sB + p * B_PLANE, &a.tmB, FULL(stage), kc * BK, tc.nt * BN, p, xc);
+                        } else {
 #pragma unroll
-                        for (int p = 0; p < NP; ++p)
+                            for (int p = 0; p < NP; ++p)
 #pragma unroll
-                            for (int h = 0; h < 2; ++h)
-                                tma_load_5d(sA + p * A_PLANE + h * (A_PLANE / 2), &a.tmA, FULL(stage),
-                                            tc.mt * BM + h * 64, kc * BK, (int)tc.o, p, xc);
+                                for (int h = 0; h < 2; ++h)
+                                    tma_load_5d(sA + p * A_PLANE + h * (A_PLANE / 2), &a.tmA, FULL(stage),
+                                                tc.mt * BM + h * 64, kc * BK, (int)tc.o, p, xc);
 #pragma unroll
-                        for (int p = 0; p < NP; ++p)
-                            tma_load_4d(sB + p * B_PLANE, &a.tmB, FULL(stage), kc * BK, tc.nt * BN, p, pc);
+                            for (int p = 0; p < NP; ++p)
+                                tma_load_4d(sB + p * B_PLANE, &a.tmB, FULL(stage), kc * BK, tc.nt * BN, p, pc);
+                        }
                     }
+                    __syncwarp();
                     issued_phase[stage] = (int)phase;
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
@@ -1168,7 +1178,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             // ---------------- MMA issuer ----------------
             const uint32_t idesc = FX ? (MODE1 ? make_idesc_f16(BM, BN, 0, 0) : make_idesc_f16(BM, BN, 1, 0))
                                       : (MODE1 ? make_idesc(BM, BN, 0, 0) : make_idesc(BM, BN, 1, 0));
@@ -1180,7 +1190,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             ItemIter<GROUPED, SK> itr(a0, gtab, gprefix, ginst, gunits);
             while (ok && itr.next()) {
                 const TcArgs &a = GROUPED ? *itr.a : a0;   // ungrouped: the kernel parameter itself
-                if (!wait_bar(TEMPTY(acc), acc_phase ^ 1u, abort_flag, a.status, 2, a.wait_limit)) break;
+                ok = __all_sync(0xffffffffu, wait_bar(TEMPTY(acc), acc_phase ^ 1u, abort_flag, a.status, 2, a.wait_limit));
+                if (!ok) break;
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)acc * ACC_COLS;
                 const int part = (int)(itr.lu % a.ksplit);
@@ -1188,74 +1199,79 @@ __global__ void __launch_bounds__(kThreads, 1)
                 constexpr bool sk = SK && !GROUPED;
                 const int it0 = sk ? itr.k0 : part * a.kpi, it1 = sk ? itr.k1 : min(it0 + a.kpi, kiters);
                 for (int it = it0; it < it1; ++it) {
-                    if (!wait_bar(FULL(stage), phase, abort_flag, a.status, 3, a.wait_limit)) { ok = false; break; }
+                    ok = __all_sync(0xffffffffu, wait_bar(FULL(stage), phase, abort_flag, a.status, 3, a.wait_limit));
+                    if (!ok) break;
                     tc_fence_after();
                     const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + STAGE_A;
-                    if constexpr (FX) {
-                        auto ad = [&](int p, int ks) {
-                            return MODE1 ? sdesc(sA + p * A_PLANE + ks * 32, 16, 512, kSw64)
-                                         : sdesc(sA + p * A_PLANE + ks * 2048, A_PLANE / 2, 1024, kSw128);
-                        };
-                        auto bd = [&](int p, int ks) { return sdesc(sB + p * B_PLANE + ks * 32, 16, 512, kSw64); };
-                        // A (= d) | B1 | B2 | B3, one tile at a time.  The products are
-                        // grouped by their A part, which the collector buffer holds
-                        // across its group (A read from shared memory 4 times per K
-                        // step instead of 10); each accumulator's first product is
-                        // in the h group.
-                        const uint32_t dB1 = tmem + BN, dB2 = tmem + 2 * BN, dB3 = tmem + 3 * BN;
+                    if (ptx::elect_one()) {
+                        if constexpr (FX) {
+                            auto ad = [&](int p, int ks) {
+                                return MODE1 ? sdesc(sA + p * A_PLANE + ks * 32, 16, 512, kSw64)
+                                             : sdesc(sA + p * A_PLANE + ks * 2048, A_PLANE / 2, 1024, kSw128);
+                            };
+                            auto bd = [&](int p, int ks) { return sdesc(sB + p * B_PLANE + ks * 32, 16, 512, kSw64); };
+                            // A (= d) | B1 | B2 | B3, one tile at a time.  The products are
+                            // grouped by their A part, which the collector buffer holds
+                            // across its group (A read from shared memory 4 times per K
+                            // step instead of 10); each accumulator's first product is
+                            // in the h group.
+                            const uint32_t dB1 = tmem + BN, dB2 = tmem + 2 * BN, dB3 = tmem + 3 * BN;
+#pragma unroll
+                            for (int ks = 0; ks < BK / 16; ++ks) {
+                                const uint32_t first = (it > it0 || ks > 0) ? 1u : 0u;
+                                const uint64_t a0 = ad(0, ks), a1 = ad(1, ks), a2 = ad(2, ks), a3 = ad(3, ks);
+                                mma_f16_coll<1>(d, a0, bd(0, ks), idesc, first);     // h h'
+                                mma_f16_coll<2>(dB1, a0, bd(1, ks), idesc, first);   // h s1'
+                                mma_f16_coll<2>(dB2, a0, bd(2, ks), idesc, first);   // h s2'
+                                mma_f16_coll<3>(dB3, a0, bd(3, ks), idesc, first);   // h s3'
+                                mma_f16_coll<1>(dB1, a1, bd(0, ks), idesc, 1u);      // s1 h'
+                                mma_f16_coll<2>(dB2, a1, bd(1, ks), idesc, 1u);      // s1 s1'
+                                if (a.fx_extra) {
+                                    mma_f16_coll<2>(dB3, a1, bd(2, ks), idesc, 1u);  // s1 s2'
+                                    mma_f16_coll<3>(dB3, a1, bd(3, ks), idesc, 1u);  // s1 s3'
+                                    mma_f16_coll<1>(dB2, a2, bd(0, ks), idesc, 1u);  // s2 h'
+                                    mma_f16_coll<2>(dB3, a2, bd(1, ks), idesc, 1u);  // s2 s1'
+                                    mma_f16_coll<3>(dB3, a2, bd(2, ks), idesc, 1u);  // s2 s2'
+                                    mma_f16_coll<1>(dB3, a3, bd(0, ks), idesc, 1u);  // s3 h'
+                                    mma_f16_coll<3>(dB3, a3, bd(1, ks), idesc, 1u);  // s3 s1'
+                                } else {
+                                    mma_f16_coll<3>(dB3, a1, bd(2, ks), idesc, 1u);  // s1 s2'
+                                    mma_f16_coll<1>(dB2, a2, bd(0, ks), idesc, 1u);  // s2 h'
+                                    mma_f16_coll<3>(dB3, a2, bd(1, ks), idesc, 1u);  // s2 s1'
+                                    mma_bf16(dB3, a3, bd(0, ks), idesc, 1u);         // s3 h'
+                                }
+                            }
+                        } else {
 #pragma unroll
                         for (int ks = 0; ks < BK / 16; ++ks) {
-                            const uint32_t first = (it > it0 || ks > 0) ? 1u : 0u;
-                            const uint64_t a0 = ad(0, ks), a1 = ad(1, ks), a2 = ad(2, ks), a3 = ad(3, ks);
-                            mma_f16_coll<1>(d, a0, bd(0, ks), idesc, first);     // h h'
-                            mma_f16_coll<2>(dB1, a0, bd(1, ks), idesc, first);   // h s1'
-                            mma_f16_coll<2>(dB2, a0, bd(2, ks), idesc, first);   // h s2'
-                            mma_f16_coll<3>(dB3, a0, bd(3, ks), idesc, first);   // h s3'
-                            mma_f16_coll<1>(dB1, a1, bd(0, ks), idesc, 1u);      // s1 h'
-                            mma_f16_coll<2>(dB2, a1, bd(1, ks), idesc, 1u);      // s1 s1'
-                            if (a.fx_extra) {
-                                mma_f16_coll<2>(dB3, a1, bd(2, ks), idesc, 1u);  // s1 s2'
-                                mma_f16_coll<3>(dB3, a1, bd(3, ks), idesc, 1u);  // s1 s3'
-                                mma_f16_coll<1>(dB2, a2, bd(0, ks), idesc, 1u);  // s2 h'
-                                mma_f16_coll<2>(dB3, a2, bd(1, ks), idesc, 1u);  // s2 s1'
-                                mma_f16_coll<3>(dB3, a2, bd(2, ks), idesc, 1u);  // s2 s2'
-                                mma_f16_coll<1>(dB3, a3, bd(0, ks), idesc, 1u);  // s3 h'
-                                mma_f16_coll<3>(dB3, a3, bd(1, ks), idesc, 1u);  // s3 s1'
-                            } else {
-                                mma_f16_coll<3>(dB3, a1, bd(2, ks), idesc, 1u);  // s1 s2'
-                                mma_f16_coll<1>(dB2, a2, bd(0, ks), idesc, 1u);  // s2 h'
-                                mma_f16_coll<3>(dB3, a2, bd(1, ks), idesc, 1u);  // s2 s1'
-                                mma_bf16(dB3, a3, bd(0, ks), idesc, 1u);         // s3 h'
+#pragma unroll
+                            for (int q = 0; q < 6; ++q) {
+                                const int pa = (q == 0 || q == 1 || q == 3) ? 0 : (q == 5 ? 2 : 1);
+                                const int pb = (q == 0 || q == 2 || q == 5) ? 0 : (q == 1 || q == 4 ? 1 : 2);
+                                uint64_t ad, bd;
+                                if (MODE1) {
+                                    ad = sdesc(sA + pa * A_PLANE + ks * 32, 16, 512, kSw64);
+                                } else {
+                                    ad = sdesc(sA + pa * A_PLANE + ks * 2048, A_PLANE / 2, 1024, kSw128);
+                                }
+                                bd = sdesc(sB + pb * B_PLANE + ks * 32, 16, 512, kSw64);
+                                if (DUAL) {
+                                    const bool first = it == it0 && ks == 0 && (q == 0 || q == 1);
+                                    mma_bf16(q == 0 ? d : d + BN, ad, bd, idesc, first ? 0u : 1u);
+                                } else {
+                                    mma_bf16(d, ad, bd, idesc, (it > it0 || ks > 0 || q > 0) ? 1u : 0u);
+                                }
                             }
                         }
-                    } else {
-#pragma unroll
-                    for (int ks = 0; ks < BK / 16; ++ks) {
-#pragma unroll
-                        for (int q = 0; q < 6; ++q) {
-                            const int pa = (q == 0 || q == 1 || q == 3) ? 0 : (q == 5 ? 2 : 1);
-                            const int pb = (q == 0 || q == 2 || q == 5) ? 0 : (q == 1 || q == 4 ? 1 : 2);
-                            uint64_t ad, bd;
-                            if (MODE1) {
-                                ad = sdesc(sA + pa * A_PLANE + ks * 32, 16, 512, kSw64);
-                            } else {
-                                ad = sdesc(sA + pa * A_PLANE + ks * 2048, A_PLANE / 2, 1024, kSw128);
-                            }
-                            bd = sdesc(sB + pb * B_PLANE + ks * 32, 16, 512, kSw64);
-                            if (DUAL) {
-                                const bool first = it == it0 && ks == 0 && (q == 0 || q == 1);
-                                mma_bf16(q == 0 ? d : d + BN, ad, bd, idesc, first ? 0u : 1u);
-                            } else {
-                                mma_bf16(d, ad, bd, idesc, (it > it0 || ks > 0 || q > 0) ? 1u : 0u);
-                            }
                         }
+                        mma_commit(EMPTY(stage));
                     }
-                    }
-                    mma_commit(EMPTY(stage));
+                    __syncwarp();
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                mma_commit(TFULL(acc));
+                if (ptx::elect_one()) mma_commit(TFULL(acc));
+                __syncwarp();
                 if constexpr (FX) {
                     acc_phase ^= 1u;   // one accumulator set: buffer 0 only
                 } else {
@@ -1263,7 +1279,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (acc == 0) acc_phase ^= 1u;
                 }
             }
-            mma_commit(DRAIN);
+            if (ptx::elect_one()) mma_commit(DRAIN);
+            __syncwarp();
             volatile int never = 0;
             wait_bar(DRAIN, 0, &never, nullptr, 0);
         }
