@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <map>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -21,6 +22,60 @@ ds_status fail(ds_status st, const std::string &msg)
 {
     set_error(msg);
     return st;
+}
+
+namespace {
+constexpr size_t kPoolKeep = (size_t)1 << 30;
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+// the current device's pool; null: none could be made (the default pool serves)
+cudaMemPool_t device_pool()
+{
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        if (cudaMemPoolCreate(&g_pool[dev], &props) != cudaSuccess) {
+            cudaGetLastError();
+            g_pool[dev] = nullptr;
+            return nullptr;
+        }
+        uint64_t keep = kPoolKeep;
+        cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    return g_pool[dev];
+}
+}  // namespace
+
+cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t st)
+{
+    cudaMemPool_t pool = device_pool();
+    if (!pool) return cudaMallocAsync(p, bytes, st);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    }
+    return e;
+}
+
+cudaError_t device_alloc(void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    cudaMemPool_t pool = e == cudaErrorMemoryAllocation ? device_pool() : nullptr;
+    if (pool) {
+        cudaGetLastError();
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -539,14 +594,14 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
                         poff += grid->n[mu] * grid->n[mu];
                     }
         s->P_count = poff;
-        cudaError_t e1 = cudaMalloc(&s->A_dev, sizeof(double) * Acount);
-        cudaError_t e2 = cudaMalloc(&s->tri_dev, sizeof(double) * toff);
-        cudaError_t e3 = cudaMalloc(&s->P_dev, sizeof(double) * poff);
+        cudaError_t e1 = pool_alloc(&s->A_dev, sizeof(double) * Acount, st);
+        cudaError_t e2 = pool_alloc(&s->tri_dev, sizeof(double) * toff, st);
+        cudaError_t e3 = pool_alloc(&s->P_dev, sizeof(double) * poff, st);
         // derivatives feed the adjoint's diffusion-scaling gradient (EXPRK3DS_REAL only)
-        cudaError_t e4 = scheme == DS_EXPRK3DS_REAL ? cudaMalloc(&s->dP_dev, sizeof(double) * poff) : cudaSuccess;
+        cudaError_t e4 = scheme == DS_EXPRK3DS_REAL ? pool_alloc(&s->dP_dev, sizeof(double) * poff, st) : cudaSuccess;
         cudaError_t e5 = cudaSuccess, e6 = cudaSuccess;
         if (scheme == DS_EXPRK3DS_CPLX) {
-            e5 = cudaMalloc(&s->Pim_dev, sizeof(double) * poff);
+            e5 = pool_alloc(&s->Pim_dev, sizeof(double) * poff, st);
             int64_t moff = 0;
             for (int c = 0; c < 2; ++c)
                 for (int q = 0; q < kSlots; ++q)
@@ -554,7 +609,7 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
                         s->Mf_off[c][q][i] = moff;
                         moff += 2 * grid->n[d - 1] * grid->n[d - 1];
                     }
-            e6 = cudaMalloc(&s->Mf_dev, sizeof(double) * moff);
+            e6 = pool_alloc(&s->Mf_dev, sizeof(double) * moff, st);
         }
         if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess ||
             e5 != cudaSuccess || e6 != cudaSuccess) {
@@ -631,12 +686,10 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
 ds_status ds_phi_set_destroy(ds_phi_set *s)
 {
     if (!s) return DS_OK;
-    cudaFree(s->A_dev);
-    cudaFree(s->tri_dev);
-    cudaFree(s->P_dev);
-    cudaFree(s->dP_dev);
-    cudaFree(s->Pim_dev);
-    cudaFree(s->Mf_dev);
+    // any stream may still read the matrices
+    cudaDeviceSynchronize();
+    for (double *p : {s->A_dev, s->tri_dev, s->P_dev, s->dP_dev, s->Pim_dev, s->Mf_dev})
+        if (p) cudaFreeAsync(p, nullptr);
     delete s;
     return DS_OK;
 }
@@ -684,7 +737,7 @@ ds_status ds_tucker(const ds_grid *grid, const double *X, double *Y, const doubl
         int64_t pm = 0;
         for (int mu = 0; mu < d; ++mu) pm += grid->n[mu] * grid->n[mu];
         float *w = nullptr;
-        DS_CUDA_TRY(cudaMallocAsync(&w, sizeof(float) * (3 * N + pm), st));
+        DS_CUDA_TRY(pool_alloc(&w, sizeof(float) * (3 * N + pm), st));
         float *x32 = w, *b0 = w + N, *b1 = w + 2 * N, *l32 = w + 3 * N;
         tc::launch_convert_f64_f32(N, X, x32, st);
         const float *in = x32;
@@ -709,12 +762,12 @@ ds_status ds_tucker(const ds_grid *grid, const double *X, double *Y, const doubl
     mm::Context c;
     double *tmp = nullptr;
     const size_t tb = mm::aligned(sizeof(double) * N * 2);
-    if (scratch && cudaMallocAsync(&tmp, tb + scratch, st) == cudaSuccess) {
+    if (scratch && pool_alloc(&tmp, tb + scratch, st) == cudaSuccess) {
         c.ws = (uint8_t *)tmp + tb;
         c.ws_bytes = scratch;
     } else {
         cudaGetLastError();
-        DS_CUDA_TRY(cudaMallocAsync(&tmp, tb, st));   // short of memory: the FP64 pipe
+        DS_CUDA_TRY(pool_alloc(&tmp, tb, st));   // short of memory: the FP64 pipe
     }
     tucker_f64(c, d, grid->n, X, Y, L, transpose, tmp, st);
     cudaFreeAsync(tmp, st);
@@ -787,12 +840,12 @@ ds_status ds_plan_create(const ds_grid *grid, const ds_params *params, const ds_
             const int per_op = sum_tensors(set, SumKind::plain), nf = etd2 ? 1 : 3;
             int64_t zt = (int64_t)per_op * ops_in_budget(per_op, p->N, 2 * nf);
             p->ws_count = (6 + 2 * nf + zt) * p->N;
-            if (cudaMalloc(&p->ws, sizeof(double) * p->ws_count) != cudaSuccess) {
+            if (device_alloc(&p->ws, sizeof(double) * p->ws_count) != cudaSuccess) {
                 cudaGetLastError();
                 p->lean = true;
                 zt = per_op / set->k;
                 p->ws_count = (8 + zt) * p->N;
-                if (cudaMalloc(&p->ws, sizeof(double) * p->ws_count) != cudaSuccess) {
+                if (device_alloc(&p->ws, sizeof(double) * p->ws_count) != cudaSuccess) {
                     cudaGetLastError();
                     return cleanup(DS_ERR_OOM, "FP64 workspace");
                 }
@@ -804,8 +857,8 @@ ds_status ds_plan_create(const ds_grid *grid, const ds_params *params, const ds_
         } else if (precision == DS_PREC_F32) {
             if (!set->tridiag[0] || !set->tridiag[1])
                 return cleanup(DS_ERR_UNSUPPORTED, "reduced-precision paths need tridiagonal A_mu (use DS_PREC_F64)");
-            if (cudaMalloc(&p->ws32, sizeof(float) * 10 * p->N) != cudaSuccess ||
-                cudaMalloc(&p->P32, sizeof(float) * set->P_count) != cudaSuccess) {
+            if (device_alloc(&p->ws32, sizeof(float) * 10 * p->N) != cudaSuccess ||
+                device_alloc(&p->P32, sizeof(float) * set->P_count) != cudaSuccess) {
                 cudaGetLastError();
                 return cleanup(DS_ERR_OOM, "FP32 workspace");
             }
@@ -915,10 +968,10 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
     if (!p->bws) {
         const int per_op = sum_tensors(s, SumKind::plain);
         int64_t zt = (int64_t)per_op * ops_in_budget(per_op, N, 4);
-        if (cudaMalloc(&p->bws, sizeof(double) * (22 + zt) * N) != cudaSuccess) {
+        if (device_alloc(&p->bws, sizeof(double) * (22 + zt) * N) != cudaSuccess) {
             cudaGetLastError();
             zt = per_op / s->k;
-            if (cudaMalloc(&p->bws, sizeof(double) * (22 + zt) * N) != cudaSuccess) {
+            if (device_alloc(&p->bws, sizeof(double) * (22 + zt) * N) != cudaSuccess) {
                 cudaGetLastError();
                 p->bws = nullptr;
                 return fail(DS_ERR_OOM, "adjoint workspace");
@@ -932,10 +985,10 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
     if (dscale && !p->tws) {
         const int per_op = sum_tensors(s, SumKind::tangent);
         int64_t zt = (int64_t)per_op * ops_in_budget(per_op, N, 6);
-        if (cudaMalloc(&p->tws, sizeof(double) * (6 + zt) * N) != cudaSuccess) {
+        if (device_alloc(&p->tws, sizeof(double) * (6 + zt) * N) != cudaSuccess) {
             cudaGetLastError();
             zt = per_op / s->k;
-            if (cudaMalloc(&p->tws, sizeof(double) * (6 + zt) * N) != cudaSuccess) {
+            if (device_alloc(&p->tws, sizeof(double) * (6 + zt) * N) != cudaSuccess) {
                 cudaGetLastError();
                 p->tws = nullptr;
                 return fail(DS_ERR_OOM, "adjoint workspace");

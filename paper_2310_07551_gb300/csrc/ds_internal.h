@@ -81,6 +81,19 @@ ds_status check_device();
                               std::string(#expr) + ": " + cudaGetErrorString(_e));   \
     } while (0)
 
+// Stream-ordered device memory for workspaces of one call and for phi-sets, from
+// a pool of the library's own per device.  The pool keeps up to 1 GiB between
+// calls (the default pool gives everything back at each synchronisation, and
+// mapping it again took 0.9 of the 1.3 ms of a 256^3 split-BF16 Tucker operator);
+// it is emptied when an allocation fails.
+cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t st);
+template <typename T>
+cudaError_t pool_alloc(T **p, size_t bytes, cudaStream_t st) { return pool_alloc((void **)p, bytes, st); }
+// cudaMalloc that empties the pool and tries again where memory is short
+cudaError_t device_alloc(void **p, size_t bytes);
+template <typename T>
+cudaError_t device_alloc(T **p, size_t bytes) { return device_alloc((void **)p, bytes); }
+
 // Strided batched FP32 GEMM: C[b] = alpha * A[b] B[b] + beta * C[b] ------
 struct SGemm {
     int M, N, K, batch;

@@ -709,7 +709,7 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     const int64_t nn = (int64_t)n * n, tot = nn * nb;
     // workspace: Y, Pw, T, phi0..2, their products (9 blocks), tables, digit images
     double *ws = nullptr;
-    DS_CUDA_TRY(cudaMallocAsync(&ws, sizeof(double) * tot * 9, st));
+    DS_CUDA_TRY(pool_alloc(&ws, sizeof(double) * tot * 9, st));
     double *Y = ws, *Pw = ws + tot, *T = ws + 2 * tot, *P = ws + 3 * tot, *T3 = ws + 6 * tot;
     mm::Context ctx;
     if (mm::use_digits(n, n, nb)) {
@@ -718,7 +718,7 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
         size_t bytes = mm::image_total(v, mm::kRowBlock);
         v.rows = 3 * (int64_t)n + 64;   // padded to whole column tiles
         bytes += mm::image_total(v, 1);
-        if (cudaMallocAsync((void **)&ctx.ws, bytes, st) == cudaSuccess) {
+        if (pool_alloc((void **)&ctx.ws, bytes, st) == cudaSuccess) {
             ctx.ws_bytes = bytes;
         } else {
             cudaGetLastError();   // short of memory: the FP64 pipe
@@ -736,7 +736,7 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     for (int b = 0; b < nb; ++b) { hA[b] = jobs[b].A; hz[b] = jobs[b].z; }
     void *tab = nullptr;
     const size_t tab_bytes = sizeof(void *) * nb * 3 + sizeof(double) * nb * 2 + sizeof(int) * nb;
-    cudaError_t e = cudaMallocAsync(&tab, tab_bytes, st);
+    cudaError_t e = pool_alloc(&tab, tab_bytes, st);
     if (e != cudaSuccess) { release(nullptr); return fail(DS_ERR_OOM, "phi table"); }
     const double **dA = (const double **)tab;
     double **dSrc = (double **)((char *)tab + sizeof(void *) * nb);
@@ -874,7 +874,7 @@ ds_status phi_batch_cplx(int n, const std::vector<PhiJobC> &jobs, cudaStream_t s
     if (nb == 0) return DS_OK;
     const int64_t m = 2 * (int64_t)n, mm = m * m;
     double *buf = nullptr;
-    DS_CUDA_TRY(cudaMallocAsync(&buf, sizeof(double) * mm * nb * 2, st));
+    DS_CUDA_TRY(pool_alloc(&buf, sizeof(double) * mm * nb * 2, st));
     double *emb = buf, *res = buf + mm * nb;
     std::vector<PhiJob> rj(nb);
     for (int b = 0; b < nb; ++b) {

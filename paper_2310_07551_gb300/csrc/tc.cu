@@ -2941,11 +2941,65 @@ __global__ void k_absmax(int64_t N, const double *__restrict__ X, FxScales *f, i
     if ((threadIdx.x & 31) == 0 && mb) atomicMax(&f->maxbits[k], mb);
 }
 
+// |a| (a > 0) rounded to BF16 to nearest even: the bits of a 2^e with the leading
+// bit of a at 2^(e + bits - 1); a becomes the signed remainder
+__device__ __forceinline__ uint32_t take_bf16(long long &a, int e)
+{
+    const int lz = __clzll(a);
+    const unsigned long long A = (unsigned long long)a << lz;
+    uint32_t q = (uint32_t)(A >> 56);
+    const uint32_t rest = (uint32_t)(A >> 24);   // 32 bits below q; the ones below those only break ties
+    q += rest > 0x80000000u || (rest == 0x80000000u && ((A & 0xFFFFFFu) || (q & 1)));
+    const int sh = 56 - lz;
+    a = sh >= 0 ? a - (long long)((unsigned long long)q << sh) : 0;
+    return (uint32_t)((e + 63 - lz + 127) << 7) + q - 128;
+}
+// split3 in integers (the FP64 pipe's conversions took 216 us for 256^3 entries,
+// memory 35): the same three parts
+__device__ __forceinline__ void split3_int(double x, uint32_t (&o)[3])
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)(b >> 52) & 0x7FF;
+    o[0] = o[1] = o[2] = 0;
+    if (ex < 1023 - 60 || ex > 1023 + 126) {
+        // zero, parts that may leave BF16's normal range, infinities, NaN
+        bf16 p[3];
+        split3(x, p[0], p[1], p[2]);
+        for (int k = 0; k < 3; ++k) o[k] = __bfloat16_as_ushort(p[k]);
+        return;
+    }
+    uint32_t sign = (uint32_t)(b >> 48) & 0x8000u;
+    long long a = (long long)((b & 0xFFFFFFFFFFFFFULL) | 1ULL << 52);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (a == 0) break;
+        o[k] = sign | take_bf16(a, ex - 1075);
+        if (a < 0) {
+            a = -a;
+            sign ^= 0x8000u;
+        }
+    }
+}
+// N a multiple of 8
 __global__ void k_split_tensor(int64_t N, const double *__restrict__ X, bf16 *__restrict__ out)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-         p += (int64_t)gridDim.x * blockDim.x)
-        store_planes(out, N, p, X[p]);
+    const bool wide = ((uintptr_t)X & 15) == 0;
+    for (int64_t p = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); p < N;
+         p += 4 * (int64_t)gridDim.x * blockDim.x) {
+        double x[4];
+        if (wide) {
+            const double2 a = *reinterpret_cast<const double2 *>(X + p), b = *reinterpret_cast<const double2 *>(X + p + 2);
+            x[0] = a.x, x[1] = a.y, x[2] = b.x, x[3] = b.y;
+        } else {
+            for (int j = 0; j < 4; ++j) x[j] = X[p + j];
+        }
+        uint32_t o[4][3];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) split3_int(x[j], o[j]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            *reinterpret_cast<uint2 *>(out + k * N + p) = make_uint2(o[0][k] | o[1][k] << 16, o[2][k] | o[3][k] << 16);
+    }
 }
 
 __global__ void k_f32_to_f64(int64_t N, const float *__restrict__ a, double *__restrict__ y)
@@ -4947,7 +5001,7 @@ ds_status tucker_mixed(const ds_grid *grid, const double *X, double *Y, const do
     }
     char *ws = nullptr;
     const size_t bytes = sizeof(bf16) * (6 * N + pmax) + sizeof(float) * N + 256;
-    DS_CUDA_TRY(cudaMallocAsync((void **)&ws, bytes, st));
+    DS_CUDA_TRY(pool_alloc((void **)&ws, bytes, st));
     bf16 *A0 = (bf16 *)ws, *A1 = A0 + 3 * N, *Pp = A1 + 3 * N;
     float *outf = (float *)(((uintptr_t)(Pp + pmax) + 255) & ~(uintptr_t)255);
     k_split_tensor<<<pw_grid(N), 256, 0, st>>>(N, X, A0);
@@ -5002,7 +5056,7 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
     char *ws = nullptr;
     const size_t bytes = sizeof(__half) * (8 * N + pmax) + sizeof(float) * psmax + sizeof(FxScales) +
                          sizeof(FxMatJob) * kMaxD + 1024;
-    DS_CUDA_TRY(cudaMallocAsync((void **)&ws, bytes, st));
+    DS_CUDA_TRY(pool_alloc((void **)&ws, bytes, st));
     __half *A0 = (__half *)ws, *A1 = A0 + 4 * N, *Pp = A1 + 4 * N;
     char *tail = (char *)(((uintptr_t)(Pp + pmax) + 255) & ~(uintptr_t)255);
     FxScales *fxs = (FxScales *)tail;
