@@ -271,13 +271,15 @@ struct ds_plan {
     int64_t ws_count = 0;
     float *ws32 = nullptr;                // FP32 path workspace
     float *P32 = nullptr;                 // FP32 copies of the phi-matrices
+    float *z32 = nullptr;                 // its intermediates (in ws32)
+    int64_t z32_tensors = 0;
     DevStatus *status = nullptr;          // device error word
     Stencil sten[2];
     std::map<double *, cudaGraphExec_t> graphs;
     int64_t launches = 0;
     tc::MixedPlan *mixed = nullptr;       // tensor-core path state
     Sums64 sums;                          // FP64 plans: the step's Tucker sums
-    bool lean = false;                    // the workspace holds one sum on F at a time
+    bool lean = false;                    // (FP64, FP32) the workspace holds one sum on F at a time
     double *bws = nullptr;                // adjoint workspace, lazily allocated
     Sums64 bsums, tsums;                  // its sums; those of the diffusion-scaling gradient
     double *tws = nullptr;                // their intermediates
@@ -342,28 +344,56 @@ int enqueue_step_f64(ds_plan *p, double *U, cudaStream_t st)
     return L;
 }
 
-// FP32 CUDA-core path: same sequence as the FP64 path with FP32 operands
-int tucker_sum_f32(ds_plan *p, int c, int slot, const float *X, float *acc, float *t1, float *t2,
-                   cudaStream_t st)
+// FP32 CUDA-core path: the FP64 path's sequence with FP32 operands.  Each mode of
+// all listed sums (both components) is one phase; a sum's terms are added in
+// order in its last mode.
+int sums_f32(ds_plan *p, int nslots, const int *slots, const float *X, float *const *out, cudaStream_t st)
 {
     const ds_phi_set *s = p->set;
-    const int d = s->d;
-    const SplitCoeffs &co = s->co[kSlotEll[slot] - 1];
+    const int d = s->d, per_op = sum_tensors(s, SumKind::plain), nops = 2 * nslots;
+    const int64_t N = p->N;
+    const int fit = (int)(p->z32_tensors / per_op), at_once = std::max(1, std::min(fit, nops));
+    const int terms = fit > 0 ? s->k : 1;
     int launches = 0;
-    for (int i = 0; i < co.k; ++i) {
-        const float *in = X;
-        for (int mu = 0; mu < d; ++mu) {
-            const float *L = p->P32 + s->P_off[c][slot][i][mu];
-            const bool last = (mu == d - 1);
-            float *out = last ? acc : ((mu % 2 == 0) ? t1 : t2);
-            p->prof.begin(st, 1, 2.0 * (double)p->N * (double)s->n[mu]);
-            launch_mode_product_f32(d, s->n, in, mu, L, 0, out, last ? co.eta[i] : 1.0,
-                                    (last && i > 0) ? 1.0 : 0.0, st);
-            p->prof.end(st);
-            ++launches;
-            in = out;
-        }
-    }
+    for (int b = 0; b < nops; b += at_once)
+        for (int i0 = 0; i0 < s->k; i0 += terms)
+            for (int mu = 0; mu < d; ++mu) {
+                std::vector<F32Product> ps;
+                for (int q = b; q < std::min(nops, b + at_once); ++q) {
+                    const int c = q / nslots, slot = slots[q % nslots];
+                    const SplitCoeffs &co = s->co[kSlotEll[slot] - 1];
+                    float *z = p->z32 + N * per_op * (q - b);
+                    F32Product sum{};
+                    for (int t = 0; t < terms; ++t) {
+                        const float *L = p->P32 + s->P_off[c][slot][i0 + t][mu];
+                        const float *in = mu == 0 ? X + c * N : z + N * (((mu - 1) % 2) * terms + t);
+                        if (mu < d - 1) {
+                            F32Product one{};
+                            one.X[0] = in;
+                            one.L[0] = L;
+                            one.alpha[0] = 1.0f;
+                            one.nterm = 1;
+                            one.Y = z + N * ((mu % 2) * terms + t);
+                            ps.push_back(one);
+                        } else {
+                            sum.X[t] = in;
+                            sum.L[t] = L;
+                            sum.alpha[t] = (float)co.eta[i0 + t];
+                            sum.nterm = t + 1;
+                        }
+                    }
+                    if (mu == d - 1) {
+                        sum.accumulate = i0 > 0;
+                        sum.Y = out[q % nslots] + c * N;
+                        ps.push_back(sum);
+                    }
+                }
+                double flops = 0.0;
+                for (const F32Product &f : ps) flops += 2.0 * (double)N * (double)s->n[mu] * f.nterm;
+                p->prof.begin(st, 1, flops);
+                launches += launch_products_f32(d, s->n, mu, 0, ps.data(), (int)ps.size(), st);
+                p->prof.end(st);
+            }
     return launches;
 }
 
@@ -371,33 +401,26 @@ int enqueue_step_f32(ds_plan *p, double *U, cudaStream_t st)
 {
     const int64_t N = p->N;
     const double tau = p->set->tau;
-    float *F = p->ws32, *a = F + 2 * N, *b = F + 4 * N, *D = F + 6 * N, *t1 = F + 8 * N, *t2 = F + 9 * N;
+    float *F = p->ws32, *b = F + 2 * N, *D = F + 4 * N, *a = F + 6 * N;
+    float *as[3] = {a, a + (p->lean ? 0 : 2 * N), a + (p->lean ? 0 : 4 * N)};
+    const int slots[3] = {0, 1, 3};
     int L = 0;
-    p->prof.begin(st, 2, 0.0);
-    tc::launch_rhs_f32(p->sten, p->model, N, U, F, st);
-    p->prof.end(st);
-    ++L;
-    for (int c = 0; c < 2; ++c) L += tucker_sum_f32(p, c, 0, F + c * N, a + c * N, t1, t2, st);
-    p->prof.begin(st, 2, 0.0);
-    tc::launch_stage_f32(p->model, N, U, a, kSlotW[0] * tau, nullptr, 0.0, D, st);
-    p->prof.end(st);
-    ++L;
-    for (int c = 0; c < 2; ++c) {
-        L += tucker_sum_f32(p, c, 1, F + c * N, a + c * N, t1, t2, st);
-        L += tucker_sum_f32(p, c, 2, D + c * N, b + c * N, t1, t2, st);
-    }
-    p->prof.begin(st, 2, 0.0);
-    tc::launch_stage_f32(p->model, N, U, a, kSlotW[1] * tau, b, kSlotW[2] * tau, D, st);
-    p->prof.end(st);
-    ++L;
-    for (int c = 0; c < 2; ++c) {
-        L += tucker_sum_f32(p, c, 3, F + c * N, a + c * N, t1, t2, st);
-        L += tucker_sum_f32(p, c, 4, D + c * N, b + c * N, t1, t2, st);
-    }
-    p->prof.begin(st, 2, 0.0);
-    tc::launch_final_f32(N, U, a, kSlotW[3] * tau, b, kSlotW[4] * tau, st);
-    p->prof.end(st);
-    ++L;
+    auto sum = [&](int slot, const float *X, float *out) { L += sums_f32(p, 1, &slot, X, &out, st); };
+    auto pointwise = [&](auto launch) {
+        p->prof.begin(st, 2, 0.0);
+        launch();
+        p->prof.end(st);
+        ++L;
+    };
+    pointwise([&] { tc::launch_rhs_f32(p->sten, p->model, N, U, F, st); });
+    L += sums_f32(p, p->lean ? 1 : 3, slots, F, as, st);
+    pointwise([&] { tc::launch_stage_f32(p->model, N, U, as[0], kSlotW[0] * tau, nullptr, 0.0, D, st); });
+    if (p->lean) sum(1, F, a);
+    sum(2, D, b);
+    pointwise([&] { tc::launch_stage_f32(p->model, N, U, as[1], kSlotW[1] * tau, b, kSlotW[2] * tau, D, st); });
+    if (p->lean) sum(3, F, a);
+    sum(4, D, b);
+    pointwise([&] { tc::launch_final_f32(N, U, as[2], kSlotW[3] * tau, b, kSlotW[4] * tau, st); });
     return L;
 }
 
@@ -745,7 +768,13 @@ ds_status ds_tucker(const ds_grid *grid, const double *X, double *Y, const doubl
         for (int mu = 0; mu < d; ++mu) {
             tc::launch_convert_f64_f32(grid->n[mu] * grid->n[mu], L[mu], pl, st);
             float *out = (mu % 2 == 0) ? b0 : b1;
-            launch_mode_product_f32(d, grid->n, in, mu, pl, transpose, out, 1.0, 0.0, st);
+            F32Product one{};
+            one.X[0] = in;
+            one.L[0] = pl;
+            one.alpha[0] = 1.0f;
+            one.nterm = 1;
+            one.Y = out;
+            launch_products_f32(d, grid->n, mu, transpose, &one, 1, st);
             in = out;
             pl += grid->n[mu] * grid->n[mu];
         }
@@ -857,11 +886,21 @@ ds_status ds_plan_create(const ds_grid *grid, const ds_params *params, const ds_
         } else if (precision == DS_PREC_F32) {
             if (!set->tridiag[0] || !set->tridiag[1])
                 return cleanup(DS_ERR_UNSUPPORTED, "reduced-precision paths need tridiagonal A_mu (use DS_PREC_F64)");
-            if (device_alloc(&p->ws32, sizeof(float) * 10 * p->N) != cudaSuccess ||
-                device_alloc(&p->P32, sizeof(float) * set->P_count) != cudaSuccess) {
+            // as the FP64 plans' workspace
+            const int per_op = sum_tensors(set, SumKind::plain);
+            p->z32_tensors = (int64_t)per_op * ops_in_budget(per_op, p->N, 6);
+            bool ok = device_alloc(&p->ws32, sizeof(float) * (12 + p->z32_tensors) * p->N) == cudaSuccess;
+            if (!ok) {
+                cudaGetLastError();
+                p->lean = true;
+                p->z32_tensors = per_op / set->k;
+                ok = device_alloc(&p->ws32, sizeof(float) * (8 + p->z32_tensors) * p->N) == cudaSuccess;
+            }
+            if (!ok || device_alloc(&p->P32, sizeof(float) * set->P_count) != cudaSuccess) {
                 cudaGetLastError();
                 return cleanup(DS_ERR_OOM, "FP32 workspace");
             }
+            p->z32 = p->ws32 + (p->lean ? 8 : 12) * p->N;
             tc::launch_convert_f64_f32(set->P_count, set->P_dev, p->P32, 0);
         } else {
             r = tc::mixed_plan_create(grid, set, p->status, &p->mixed, precision == DS_PREC_BF16X6C,

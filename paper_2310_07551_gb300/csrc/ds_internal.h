@@ -94,17 +94,17 @@ cudaError_t device_alloc(void **p, size_t bytes);
 template <typename T>
 cudaError_t device_alloc(T **p, size_t bytes) { return device_alloc((void **)p, bytes); }
 
-// Strided batched FP32 GEMM: C[b] = alpha * A[b] B[b] + beta * C[b] ------
-struct SGemm {
-    int M, N, K, batch;
-    const float *A; int64_t sAm, sAk, sAb;
-    const float *B; int64_t sBk, sBn, sBb;
-    float *C; int64_t sCm, sCn, sCb;
-    double alpha, beta;
+// FP32 mode products on the CUDA cores, one launch per kMaxProducts32 of them:
+// Y = sum_t alpha_t X_t x_mu L_t (+ Y), term after term (one FMA each).  L column-major n_mu x n_mu; transpose uses L^T.  Returns the
+// number of launches.
+constexpr int kMaxProducts32 = 24;
+struct F32Product {
+    const float *X[kMaxTerms], *L[kMaxTerms];
+    float alpha[kMaxTerms];
+    int nterm, accumulate;
+    float *Y;
 };
-void launch_sgemm(const SGemm &g, cudaStream_t st);
-void launch_mode_product_f32(int d, const int64_t *n, const float *X, int mu, const float *L,
-                             int transpose, float *Y, double alpha, double beta, cudaStream_t st);
+int launch_products_f32(int d, const int64_t *n, int mu, int transpose, const F32Product *p, int count, cudaStream_t st);
 
 // Reaction model ---------------------------------------------------------
 struct Model {

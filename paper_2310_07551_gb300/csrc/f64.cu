@@ -1,6 +1,5 @@
-// FP64 kernels: strided batched DGEMM (mu-mode products, phi setup),
-// the stencil form of the Kronecker-sum action with the reaction term, the
-// pointwise stage kernels of EXPRK3DS_REAL and the phi-function evaluation.
+// FP32 mode products on the CUDA cores; FP64 kernels: the stencil form of the
+// Kronecker-sum action with the reaction term, the pointwise stage kernels of EXPRK3DS_REAL and the phi-function evaluation.
 #include <math.h>
 
 #include <algorithm>
@@ -11,146 +10,190 @@
 namespace ds {
 
 // ---------------------------------------------------------------------------
-// Strided batched GEMM (FP64, and FP32 for the CUDA-core FP32 path).
-// 64x64 output tile, K chunks of 16, 256 threads,
-// 4x4 outputs per thread.  GB300's FP64 pipe is narrow, so the kernel is
-// built to keep it fed rather than to save bandwidth: each operand tile is
-// staged once in shared memory with whichever index has unit stride mapped
-// to consecutive threads.
+// FP32 mode products on the CUDA cores: Y(i, f) = sum over terms of alpha sum_j
+// L(i, j) X(j, f) (+ Y) over the fibres f of a mode, entry (j, f) of a tensor at
+// (f / I) (I n) + f % I + I j.  A block takes up to 128 rows i (a multiple of
+// eight, n cut evenly, so that n = 100 pads to 104) by 64 fibres, counted through
+// all slices; a thread 8 x 8 outputs, 64 FMAs per four 16-byte shared-memory
+// loads, each output one FMA chain in ascending j.  The next 16 entries of the
+// contraction are fetched while the current ones are used.  One product of 10^6
+// points is 16k threads, a third of what the SMs hold at 8 x 8 outputs each, so
+// the products of a phase share a launch (FitzHugh-Nagumo 100^3, two steps: 3.25 ms
+// with 64 x 64 tiles of 4 x 4 outputs per thread and a launch per product, 5.8 with
+// this tile and a launch per product, 2.14 so; 4 x 8 outputs for the launches of two
+// products: 2.24).  18 products of 100 entries each run at 21 TFLOP/s, the FMA pipe
+// 43 % busy: the padding (104 of 100 rows, 112 of 100 entries) and the copies'
+// addresses take the rest.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16;
+constexpr int kSgRows = 128, kSgCols = 64, kSgK = 16, TR = 8;   // TR: rows per thread
 
-template <typename T, typename G>
-__global__ void __launch_bounds__(256) k_gemm(G g)
+struct SProd {
+    int n, rows;          // contracted size; rows per block
+    int64_t I, fibres;
+    int64_t sLi, sLj;
+    bool wide_l, wide_x;  // rows of L, fibres of X in aligned groups of four
+    F32Product p[kMaxProducts32];
+};
+
+__global__ void __launch_bounds__(kSgRows, 4) k_mode_f32(const __grid_constant__ SProd g)
 {
-    __shared__ T As[BK][BM + 1];
-    __shared__ T Bs[BK][BN + 1];
-    const int t = threadIdx.x;
-    const int tx = t % 16, ty = t / 16;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int b = blockIdx.z;
-    const T *A = g.A + (int64_t)b * g.sAb;
-    const T *B = g.B + (int64_t)b * g.sBb;
-    T *C = g.C + (int64_t)b * g.sCb;
-    const bool a_m_fast = (g.sAm == 1);
-    const bool b_n_fast = (g.sBn == 1);
-
-    T acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-
-    for (int k0 = 0; k0 < g.K; k0 += BK) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            int e = t + 256 * r;
-            int mm, kk;
-            if (a_m_fast) { mm = e % BM; kk = e / BM; } else { kk = e % BK; mm = e / BK; }
-            int gm = m0 + mm, gk = k0 + kk;
-            As[kk][mm] = (gm < g.M && gk < g.K) ? A[gm * g.sAm + gk * g.sAk] : T(0);
-            int nn, kb;
-            if (b_n_fast) { nn = e % BN; kb = e / BN; } else { kb = e % BK; nn = e / BK; }
-            int gn = n0 + nn, gkb = k0 + kb;
-            Bs[kb][nn] = (gn < g.N && gkb < g.K) ? B[gkb * g.sBk + gn * g.sBn] : T(0);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            T a[4], bb[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
-        }
-        __syncthreads();
+    __shared__ __align__(16) float Ls[2][kSgK][kSgRows + 4];
+    __shared__ __align__(16) float Xs[2][kSgK][kSgCols + 4];
+    __shared__ int64_t off[kSgCols];
+    const F32Product &p = g.p[blockIdx.z];
+    const int t = threadIdx.x, nt = blockDim.x, rows = g.rows;
+    const int64_t f0 = (int64_t)blockIdx.x * kSgCols;
+    const int i0 = blockIdx.y * rows;
+    for (int c = t; c < kSgCols; c += nt) {
+        const int64_t f = f0 + c, o = f / g.I;
+        off[c] = f < g.fibres ? o * (g.I * g.n) + (f - o * g.I) : -1;
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int gm = m0 + ty + 16 * i;
-        if (gm >= g.M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int gn = n0 + tx + 16 * j;
-            if (gn >= g.N) continue;
-            T *c = C + gm * g.sCm + gn * g.sCn;
-            T v = (T)g.alpha * acc[i][j];
-            if (g.beta != 0.0) v = v + (T)g.beta * *c;
-            *c = v;
-        }
-    }
-}
-}  // namespace
-
-void launch_sgemm(const SGemm &g, cudaStream_t st)
-{
-    if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
-    dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
-    k_gemm<float, SGemm><<<grid, 256, 0, st>>>(g);
-}
-
-namespace {
-// A mode product's GEMM with 64-bit sizes, launched as chunks that each fit
-// the launch limits: at most 65535 batch entries (gridDim.z), 65535 row
-// tiles of 64 (gridDim.y) and 2^30 columns (int indexing inside k_gemm).
-// Each chunk is an independent GEMM on offset pointers, so the result is the
-// same as one launch would give.
-constexpr int64_t kMaxBatch = 65535, kMaxRows = 65535 * (int64_t)BM, kMaxCols = (int64_t)1 << 30;
-
-template <typename G, typename T>
-void launch_chunked(int64_t M, int64_t N, int64_t K, int64_t batch, const T *A, int64_t sAm, int64_t sAk,
-                    int64_t sAb, const T *B, int64_t sBk, int64_t sBn, int64_t sBb, T *C, int64_t sCm,
-                    int64_t sCn, int64_t sCb, double alpha, double beta, void (*launch)(const G &, cudaStream_t),
-                    cudaStream_t st)
-{
-    for (int64_t b0 = 0; b0 < batch; b0 += kMaxBatch)
-        for (int64_t m0 = 0; m0 < M; m0 += kMaxRows)
-            for (int64_t n0 = 0; n0 < N; n0 += kMaxCols) {
-                G g{};
-                g.M = (int)std::min(kMaxRows, M - m0);
-                g.N = (int)std::min(kMaxCols, N - n0);
-                g.K = (int)K;
-                g.batch = (int)std::min(kMaxBatch, batch - b0);
-                g.A = A + b0 * sAb + m0 * sAm;
-                g.sAm = sAm; g.sAk = sAk; g.sAb = sAb;
-                g.B = B + b0 * sBb + n0 * sBn;
-                g.sBk = sBk; g.sBn = sBn; g.sBb = sBb;
-                g.C = C + b0 * sCb + m0 * sCm + n0 * sCn;
-                g.sCm = sCm; g.sCn = sCn; g.sCb = sCb;
-                g.alpha = alpha;
-                g.beta = beta;
-                launch(g, st);
+    __syncthreads();
+    const int tx = t % 8, ti = t / 8;   // fibres 4 tx .. and 32 + 4 tx .., rows TR ti ..
+    const bool li_fast = g.sLi == 1, x_fast = g.I > 1;
+    // The next chunk's copies run behind the FMAs; out-of-range entries arrive as
+    // zero.  Four entries per copy where rows (fibres) of four are aligned; else
+    // single ones, eight lanes along the fast index.
+    auto copy4 = [](float *dst, const float *src, bool ok) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                     "l"(src), "r"(ok ? 4 : 0)
+                     : "memory");
+    };
+    auto copy16 = [](float *dst, const float *src, bool ok) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                     "l"(src), "r"(ok ? 16 : 0)
+                     : "memory");
+    };
+    const int step = nt / 8, quads = rows / 4;
+    auto fill = [&](int buf, const float *X, const float *L, int k0) {
+        if (g.wide_l) {
+            for (int k = t / quads, i = t % quads * 4; k < kSgK;) {
+                const bool in = k0 + k < g.n && i0 + i < g.n;
+                copy16(&Ls[buf][k][i], in ? L + i0 + i + (int64_t)(k0 + k) * g.n : L, in);
+                i += 4 * nt;   // the next of this thread's quads
+                while (i >= rows) i -= rows, ++k;
             }
-}
-
-// Y = X x_mu L (+ beta Y) as a GEMM; L(i, j) = L[i + m j], transposed L[j + m i]
-template <typename G, typename T>
-void mode_product(int d, const int64_t *n, const T *X, int mu, const T *L, int transpose, T *Y, double alpha,
-                  double beta, void (*launch)(const G &, cudaStream_t), cudaStream_t st)
-{
-    int64_t I = 1, O = 1, m = n[mu];
-    for (int q = 0; q < mu; ++q) I *= n[q];
-    for (int q = mu + 1; q < d; ++q) O *= n[q];
-    const int64_t sLi = transpose ? m : 1, sLj = transpose ? 1 : m;
-    if (mu == 0)
-        // Y[r][i] = sum_j X[r][j] L(i, j): M = fibres r, N = i, K = j
-        launch_chunked<G, T>(O, m, m, 1, X, m, 1, 0, L, sLj, sLi, 0, Y, m, 1, 0, alpha, beta, launch, st);
-    else
-        // per outer index o: Y[o][i][x] = sum_j L(i, j) X[o][j][x]
-        launch_chunked<G, T>(m, I, m, O, L, sLi, sLj, 0, X, I, 1, I * m, Y, I, 1, I * m, alpha, beta, launch,
-                             st);
+        } else if (li_fast) {
+            for (int i = t; i < rows; i += nt)
+#pragma unroll
+                for (int k = 0; k < kSgK; ++k) {
+                    const bool in = i0 + i < g.n && k0 + k < g.n;
+                    copy4(&Ls[buf][k][i], in ? L + i0 + i + (k0 + k) * g.sLj : L, in);
+                }
+        } else {
+            for (int i = ti; i < rows; i += step)
+#pragma unroll
+                for (int k = tx; k < kSgK; k += 8) {
+                    const bool in = k0 + k < g.n && i0 + i < g.n;
+                    copy4(&Ls[buf][k][i], in ? L + (i0 + i) * g.sLi + (k0 + k) * g.sLj : L, in);
+                }
+        }
+        if (g.wide_x) {
+            for (int e = t; e < kSgK * kSgCols / 4; e += nt) {
+                const int k = e / (kSgCols / 4), c = e % (kSgCols / 4) * 4;
+                const int64_t o = off[c];
+                const bool in = k0 + k < g.n && o >= 0;
+                copy16(&Xs[buf][k][c], in ? X + o + g.I * (k0 + k) : X, in);
+            }
+        } else if (x_fast) {
+            for (int k = ti; k < kSgK; k += step)
+#pragma unroll
+                for (int c = tx; c < kSgCols; c += 8) {
+                    const int64_t o = off[c];
+                    const bool in = k0 + k < g.n && o >= 0;
+                    copy4(&Xs[buf][k][c], in ? X + o + g.I * (k0 + k) : X, in);
+                }
+        } else {
+            for (int c = ti; c < kSgCols; c += step) {
+                const int64_t o = off[c];
+#pragma unroll
+                for (int k = tx; k < kSgK; k += 8) {
+                    const bool in = k0 + k < g.n && o >= 0;
+                    copy4(&Xs[buf][k][c], in ? X + o + k0 + k : X, in);
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto landed = [] {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+    };
+    for (int term = 0; term < p.nterm; ++term) {
+        const float *X = p.X[term], *L = p.L[term], alpha = p.alpha[term];
+        float acc[TR][8];
+#pragma unroll
+        for (int r = 0; r < TR; ++r)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[r][c] = 0.0f;
+        fill(0, X, L, 0);
+        landed();
+        int buf = 0;
+        for (int k0 = 0; k0 < g.n; k0 += kSgK) {
+            if (k0 + kSgK < g.n) fill(buf ^ 1, X, L, k0 + kSgK);
+#pragma unroll 4
+            for (int k = 0; k < kSgK; ++k) {
+                float a[TR];
+#pragma unroll
+                for (int r = 0; r < TR; r += 4)
+                    *reinterpret_cast<float4 *>(&a[r]) = *reinterpret_cast<const float4 *>(&Ls[buf][k][ti * TR + r]);
+                const float4 b0 = *reinterpret_cast<const float4 *>(&Xs[buf][k][tx * 4]);
+                const float4 b1 = *reinterpret_cast<const float4 *>(&Xs[buf][k][32 + tx * 4]);
+                const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+                for (int r = 0; r < TR; ++r)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
+            }
+            landed();
+            buf ^= 1;
+        }
+        // a thread adds its own outputs' terms, in order
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int64_t o = off[(c < 4 ? 0 : 28) + tx * 4 + c];
+            if (o < 0) continue;
+#pragma unroll
+            for (int r = 0; r < TR; ++r) {
+                const int i = i0 + ti * TR + r;
+                if (ti * TR + r >= rows || i >= g.n) continue;
+                float *y = p.Y + o + g.I * i;
+                *y = term > 0 || p.accumulate ? __fmaf_rn(alpha, acc[r][c], *y) : __fmul_rn(alpha, acc[r][c]);
+            }
+        }
+    }
 }
 }  // namespace
 
-void launch_mode_product_f32(int d, const int64_t *n, const float *X, int mu, const float *L,
-                             int transpose, float *Y, double alpha, double beta, cudaStream_t st)
+int launch_products_f32(int d, const int64_t *n, int mu, int transpose, const F32Product *p, int count, cudaStream_t st)
 {
-    mode_product<SGemm, float>(d, n, X, mu, L, transpose, Y, alpha, beta, launch_sgemm, st);
+    SProd g{};
+    g.n = (int)n[mu];
+    g.I = g.fibres = 1;
+    for (int q = 0; q < d; ++q) {
+        if (q < mu) g.I *= n[q];
+        if (q != mu) g.fibres *= n[q];
+    }
+    g.sLi = transpose ? n[mu] : 1;
+    g.sLj = transpose ? 1 : n[mu];
+    g.wide_l = !transpose && g.n % 4 == 0;
+    g.wide_x = g.I % 4 == 0;
+    for (int q = 0; q < count; ++q)
+        for (int t = 0; t < p[q].nterm; ++t) {
+            g.wide_l = g.wide_l && ((uintptr_t)p[q].L[t] & 15) == 0;
+            g.wide_x = g.wide_x && ((uintptr_t)p[q].X[t] & 15) == 0;
+        }
+    const int blocks = (g.n + kSgRows - 1) / kSgRows;
+    g.rows = ((g.n + blocks - 1) / blocks + 7) / 8 * 8;
+    int launches = 0;
+    for (int q = 0; q < count; q += kMaxProducts32, ++launches) {
+        const int m = std::min(kMaxProducts32, count - q);
+        std::copy(p + q, p + q + m, g.p);
+        const dim3 grid((unsigned)((g.fibres + kSgCols - 1) / kSgCols), (unsigned)((g.n + g.rows - 1) / g.rows), m);
+        k_mode_f32<<<grid, std::max(32, g.rows), 0, st>>>(g);
+    }
+    return launches;
 }
 
 // ---------------------------------------------------------------------------
