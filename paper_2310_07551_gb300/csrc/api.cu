@@ -242,6 +242,7 @@ Stencil stencil_of(const ds_phi_set *s, int c)
         t.lo[mu] = base;
         t.di[mu] = base + t.n[mu];
         t.up[mu] = base + 2 * t.n[mu];
+        t.sum[mu] = base + 3 * t.n[mu];
     }
     return t;
 }
@@ -592,7 +593,7 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
                 s->tri_off[c][mu] = toff;
                 if (!is_tridiagonal(hA.data() + off, grid->n[mu])) s->tridiag[c] = false;
                 off += grid->n[mu] * grid->n[mu];
-                toff += 3 * grid->n[mu];
+                toff += 4 * grid->n[mu];
             }
         }
         std::vector<double> htri(toff, 0.0);
@@ -600,11 +601,12 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
             for (int mu = 0; mu < d; ++mu) {
                 const int64_t n = grid->n[mu];
                 const double *Am = hA.data() + s->A_off[c][mu];
-                double *lo = htri.data() + s->tri_off[c][mu], *di = lo + n, *up = lo + 2 * n;
+                double *lo = htri.data() + s->tri_off[c][mu], *di = lo + n, *up = lo + 2 * n, *sum = lo + 3 * n;
                 for (int64_t i = 0; i < n; ++i) {
                     lo[i] = i > 0 ? Am[i + n * (i - 1)] : 0.0;
                     di[i] = Am[i + n * i];
                     up[i] = i + 1 < n ? Am[i + n * (i + 1)] : 0.0;
+                    sum[i] = (lo[i] + di[i]) + up[i];
                 }
             }
         // phi-matrix layout [c][slot][i][mu]

@@ -117,6 +117,7 @@ struct Stencil {
     int d;
     int64_t n[kMaxD];
     const double *lo[kMaxD], *di[kMaxD], *up[kMaxD];   // device arrays of length n_mu
+    const double *sum[kMaxD];                          // row sums (lo + di) + up
 };
 
 // F = K U + g(U) for both components (FP64, stencil).  Returns #launches.
@@ -242,7 +243,7 @@ struct ds_phi_set {
     double *A_dev = nullptr;                // copy of A, column-major blocks
     int64_t A_off[2][ds::kMaxD];
     bool tridiag[2];                        // every A_{c,mu} tridiagonal
-    double *tri_dev = nullptr;              // [c][mu][3][n_mu]
+    double *tri_dev = nullptr;              // [c][mu][4][n_mu]: bands, row sums
     int64_t tri_off[2][ds::kMaxD];
     double *P_dev = nullptr;                // FP64 phi-matrices, column-major blocks
     double *dP_dev = nullptr;               // their derivatives w.r.t. a scaling of A (same offsets)

@@ -202,60 +202,85 @@ int launch_products_f32(int d, const int64_t *n, int mu, int transpose, const F3
 __device__ __forceinline__ void react(const Model &m, double u, double v, double &gu, double &gv)
 {
     if (m.model == DS_SCHNAKENBERG) {
-        double u2v = __dmul_rn(__dmul_rn(u, u), v);
-        gu = __dmul_rn(m.p[0], __dadd_rn(__dsub_rn(m.p[1], u), u2v));
-        gv = __dmul_rn(m.p[0], __dsub_rn(m.p[2], u2v));
+        const double u2v = u * u * v;
+        gu = m.p[0] * ((m.p[1] - u) + u2v);
+        gv = m.p[0] * (m.p[2] - u2v);
     } else if (m.model == DS_FHN) {
-        gu = __dsub_rn(__dsub_rn(u, __dmul_rn(__dmul_rn(u, u), u)), v);
-        gv = __dmul_rn(m.p[0], __dsub_rn(__dsub_rn(u, __dmul_rn(m.p[1], v)), m.p[2]));
+        gu = fma(-u * u, u, u - v);
+        gv = m.p[0] * fma(-m.p[1], v, u - m.p[2]);
     } else {
         gu = 0.0;
         gv = 0.0;
     }
 }
 
-namespace {
-// K U for one point of one component: sum over modes of the tridiagonal row,
-// each row summed left to right (lower, diagonal, upper), modes in order.
-__device__ __forceinline__ double stencil_point(const Stencil &s, const double *U, int64_t p)
+// g(u + du, v + dv) - g(u, v) as the polynomial in the increments: no
+// cancellation, and fewer operations than g twice (the pointwise kernels are
+// bound by the FP64 pipe, 16 clocks per warp instruction and SM)
+__device__ __forceinline__ void react_difference(const Model &m, double u, double v, double du, double dv, double &Du,
+                                                 double &Dv)
 {
+    if (m.model == DS_SCHNAKENBERG) {
+        const double q = du * fma(2.0, u, du);                  // (u + du)^2 - u^2
+        const double w = fma(q, v + dv, u * u * dv);            // (u + du)^2 (v + dv) - u^2 v
+        Du = m.p[0] * (w - du);
+        Dv = -m.p[0] * w;
+    } else if (m.model == DS_FHN) {
+        const double c = fma(3.0 * u, u + du, du * du);         // ((u + du)^3 - u^3) / du
+        Du = fma(-du, c, du - dv);
+        Dv = m.p[0] * fma(-m.p[1], dv, du);
+    } else {
+        Du = 0.0;
+        Dv = 0.0;
+    }
+}
+
+namespace {
+// K U for one point of one component: each tridiagonal row as lo (u- - u) + up (u+ -
+// u) + (row sum) u, so that a constant state gives exactly zero where the rows sum
+// to zero, and neighbouring values lose nothing in their difference; all in one
+// chain of FMAs.  IT: 32-bit indices where the grid allows them.
+template <typename IT>
+__device__ __forceinline__ double stencil_point(const Stencil &s, const double *U, IT p)
+{
+    const double u = U[p];
     double acc = 0.0;
-    int64_t stride = 1, rest = p;
+    IT stride = 1, rest = p;
 #pragma unroll
     for (int mu = 0; mu < kMaxD; ++mu) {
         if (mu < s.d) {
-            int64_t nm = s.n[mu];
-            int64_t i = rest % nm;
-            rest /= nm;
-            double r = __dmul_rn(s.di[mu][i], U[p]);
-            if (i > 0) r = __dadd_rn(__dmul_rn(s.lo[mu][i], U[p - stride]), r);
-            if (i + 1 < nm) r = __dadd_rn(r, __dmul_rn(s.up[mu][i], U[p + stride]));
-            acc = __dadd_rn(acc, r);
+            const IT nm = (IT)s.n[mu], q = rest / nm, i = rest - q * nm;
+            rest = q;
+            if (i > 0) acc = fma(s.lo[mu][i], U[p - stride] - u, acc);
+            if (i + 1 < nm) acc = fma(s.up[mu][i], U[p + stride] - u, acc);
+            const double rs = s.sum[mu][i];
+            if (__double_as_longlong(rs)) acc = fma(rs, u, acc);
             stride *= nm;
         }
     }
     return acc;
 }
 
-__global__ void k_kronsum_f64(Stencil s, int64_t N, const double *__restrict__ X, double *__restrict__ Y)
+template <typename IT>
+__global__ void k_kronsum_f64(Stencil s, IT N, const double *__restrict__ X, double *__restrict__ Y)
 {
     pdl_trigger();
     pdl_wait();
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
-        Y[p] = stencil_point(s, X, p);
+    for (IT p = (IT)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (IT)gridDim.x * blockDim.x)
+        Y[p] = stencil_point<IT>(s, X, p);
 }
 
-__global__ void k_rhs_f64(Stencil s0, Stencil s1, Model m, int64_t N, const double *__restrict__ U,
+template <typename IT>
+__global__ void k_rhs_f64(Stencil s0, Stencil s1, Model m, IT N, const double *__restrict__ U,
                           double *__restrict__ F)
 {
     pdl_trigger();
     pdl_wait();
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-         p += (int64_t)gridDim.x * blockDim.x) {
+    for (IT p = (IT)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (IT)gridDim.x * blockDim.x) {
         double gu, gv;
         react(m, U[p], U[N + p], gu, gv);
-        F[p] = __dadd_rn(stencil_point(s0, U, p), gu);
-        F[N + p] = __dadd_rn(stencil_point(s1, U + N, p), gv);
+        F[p] = stencil_point<IT>(s0, U, p) + gu;
+        F[N + p] = stencil_point<IT>(s1, U + N, p) + gv;
     }
 }
 
@@ -267,18 +292,12 @@ __global__ void k_stage_diff_f64(Model m, int64_t N, const double *__restrict__ 
     pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
-        double u = U[p], v = U[N + p];
-        double us = __dadd_rn(u, __dmul_rn(w1, a[p]));
-        double vs = __dadd_rn(v, __dmul_rn(w1, a[N + p]));
+        double du = w1 * a[p], dv = w1 * a[N + p];
         if (b) {
-            us = __dadd_rn(us, __dmul_rn(w2, b[p]));
-            vs = __dadd_rn(vs, __dmul_rn(w2, b[N + p]));
+            du = fma(w2, b[p], du);
+            dv = fma(w2, b[N + p], dv);
         }
-        double g0u, g0v, gu, gv;
-        react(m, u, v, g0u, g0v);
-        react(m, us, vs, gu, gv);
-        D[p] = __dsub_rn(gu, g0u);
-        D[N + p] = __dsub_rn(gv, g0v);
+        react_difference(m, U[p], U[N + p], du, dv, D[p], D[N + p]);
     }
 }
 
@@ -289,7 +308,7 @@ __global__ void k_final_f64(int64_t n2, double *__restrict__ U, const double *__
     pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n2;
          p += (int64_t)gridDim.x * blockDim.x)
-        U[p] = __dadd_rn(__dadd_rn(U[p], __dmul_rn(w1, a[p])), __dmul_rn(w2, b[p]));
+        U[p] = fma(w2, b[p], fma(w1, a[p], U[p]));
 }
 
 __global__ void k_add_g_f64(Model m, int64_t N, const double *__restrict__ U, double *__restrict__ F)
@@ -359,8 +378,8 @@ __global__ void k_axpy2(int64_t n2, const double *__restrict__ U, const double *
     pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n2;
          p += (int64_t)gridDim.x * blockDim.x) {
-        double y = __dadd_rn(U[p], __dmul_rn(w1, a[p]));
-        if (b) y = __dadd_rn(y, __dmul_rn(w2, b[p]));
+        double y = fma(w1, a[p], U[p]);
+        if (b) y = fma(w2, b[p], y);
         Y[p] = y;
     }
 }
@@ -373,11 +392,8 @@ __global__ void k_gdiff(Model m, int64_t N, const double *__restrict__ U, const 
     pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
-        double g0u, g0v, gu, gv;
-        react(m, U[p], U[N + p], g0u, g0v);
-        react(m, Us[p], Us[N + p], gu, gv);
-        D[p] = __dsub_rn(gu, g0u);
-        D[N + p] = __dsub_rn(gv, g0v);
+        const double u = U[p], v = U[N + p];
+        react_difference(m, u, v, Us[p] - u, Us[N + p] - v, D[p], D[N + p]);
     }
 }
 
@@ -397,35 +413,33 @@ __global__ void k_jacT(Model m, int64_t N, const double *__restrict__ Us, const 
 }
 
 // K^T x for one point of one component (transposed tridiagonal rows)
-__device__ __forceinline__ double stencil_point_T(const Stencil &s, const double *X, int64_t p)
+template <typename IT>
+__device__ __forceinline__ double stencil_point_T(const Stencil &s, const double *X, IT p)
 {
     double acc = 0.0;
-    int64_t stride = 1, rest = p;
+    IT stride = 1, rest = p;
 #pragma unroll
     for (int mu = 0; mu < kMaxD; ++mu) {
         if (mu < s.d) {
-            const int64_t nm = s.n[mu];
-            const int64_t i = rest % nm;
-            rest /= nm;
-            double r = s.di[mu][i] * X[p];
-            if (i > 0) r += s.up[mu][i - 1] * X[p - stride];
-            if (i + 1 < nm) r += s.lo[mu][i + 1] * X[p + stride];
-            acc += r;
+            const IT nm = (IT)s.n[mu], q = rest / nm, i = rest - q * nm;
+            rest = q;
+            acc = fma(s.di[mu][i], X[p], acc);
+            if (i > 0) acc = fma(s.up[mu][i - 1], X[p - stride], acc);
+            if (i + 1 < nm) acc = fma(s.lo[mu][i + 1], X[p + stride], acc);
             stride *= nm;
         }
     }
     return acc;
 }
 
-__global__ void k_kronsumT(Stencil s0, Stencil s1, int64_t N, const double *__restrict__ X,
-                           double *__restrict__ Y)
+template <typename IT>
+__global__ void k_kronsumT(Stencil s0, Stencil s1, IT N, const double *__restrict__ X, double *__restrict__ Y)
 {
     pdl_trigger();
     pdl_wait();
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        Y[p] = stencil_point_T(s0, X, p);
-        Y[N + p] = stencil_point_T(s1, X + N, p);
+    for (IT p = (IT)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (IT)gridDim.x * blockDim.x) {
+        Y[p] = stencil_point_T<IT>(s0, X, p);
+        Y[N + p] = stencil_point_T<IT>(s1, X + N, p);
     }
 }
 
@@ -546,13 +560,16 @@ int grid_for(int64_t n, int block = 256)
 int launch_rhs_f64(const Stencil *s2, const Model &m, int64_t N, const double *U, double *F,
                    cudaStream_t st)
 {
-    pdl_launch(k_rhs_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s2[0], s2[1], m, N, U, F);
+    const dim3 grid(grid_for(N, block_for(N))), block(block_for(N));
+    // (headroom for the stride past the end)
+    if (N < (int64_t)1 << 30) pdl_launch(k_rhs_f64<int>, grid, block, 0, st, 1, s2[0], s2[1], m, (int)N, U, F);
+    else pdl_launch(k_rhs_f64<int64_t>, grid, block, 0, st, 1, s2[0], s2[1], m, N, U, F);
     return 1;
 }
 
 void launch_kronsum_f64(const Stencil &s, int64_t N, const double *X, double *Y, cudaStream_t st)
 {
-    pdl_launch(k_kronsum_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s, N, X, Y);
+    pdl_launch(k_kronsum_f64<int64_t>, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s, N, X, Y);
 }
 
 void launch_stage_diff_f64(const Model &m, int64_t N, const double *U, const double *a, double w1,
@@ -588,7 +605,9 @@ void launch_jacT_f64(const Model &m, int64_t N, const double *Us, const double *
 }
 void launch_kronsumT_f64(const Stencil *s2, int64_t N, const double *X, double *Y, cudaStream_t st)
 {
-    pdl_launch(k_kronsumT, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s2[0], s2[1], N, X, Y);
+    const dim3 grid(grid_for(N, block_for(N))), block(block_for(N));
+    if (N < (int64_t)1 << 30) pdl_launch(k_kronsumT<int>, grid, block, 0, st, 1, s2[0], s2[1], (int)N, X, Y);
+    else pdl_launch(k_kronsumT<int64_t>, grid, block, 0, st, 1, s2[0], s2[1], N, X, Y);
 }
 void launch_adjoint_final_f64(const Model &m, int64_t N, const double *U, const double *U2,
                               const double *U3, const double *lam, const double *lU3, const double *lU2,

@@ -5,7 +5,7 @@
 // formed here from exact digit products.  Every fibre of an operand (the
 // entries that one output sums over) is scaled by a power of two to a 62-bit
 // fixed-point number and cut into eight balanced 8-bit digits, held as FP16
-// integers: x = 2^(e - 6) (d0 + d1 2^-8 + ... + d7 2^-56), |d0| <= 65,
+// integers: x = 2^(e - 6) (d0 + d1 2^-8 + ... + d7 2^-56), |d0| <= 64,
 // |d1..7| <= 128.  The digit products of weight class t = p + q <= 7 (36 of
 // 64) run as FP16 MMAs into one FP32 tensor-memory accumulator per class.  An
 // accumulator holds integers below 2^24 (at most 256 contracted entries
@@ -45,10 +45,11 @@ __device__ DevStatus g_status;
 // ---------------------------------------------------------------------------
 // Digit images.  One warp takes 16 rows of one slab: lane = (row, 8
 // consecutive contracted entries), so that every digit plane is written as
-// 512 contiguous bytes.  WS warps (a power of two, at most 16) share the slabs
-// of a row group, each keeping the first slab it reads in registers, so a fibre
-// of up to 256 entries is read once.  24 bytes per entry pass through memory,
-// which bounds large tensors.
+// 512 contiguous bytes.  Up to 16 warps share the slabs of a row group, each
+// keeping the first slab it reads in registers, so a fibre of up to 256 entries
+// is read once.  24 bytes per entry pass through memory, which bounds large
+// tensors; blocks are as small as the slabs allow, so that one block's loads run
+// behind another's stores.
 // ---------------------------------------------------------------------------
 struct SplitArgs {
     int count;
@@ -58,12 +59,7 @@ struct SplitArgs {
 };
 constexpr int kRowGroup = 16, kSplitWarps = 16;
 
-__host__ __device__ inline int split_warps(int slabs)
-{
-    int w = 1;
-    while (w < slabs && w < kSplitWarps) w *= 2;
-    return w;
-}
+__host__ __device__ inline int split_warps(int slabs) { return slabs < kSplitWarps ? slabs : kSplitWarps; }
 
 __device__ __forceinline__ void load_entries(const View &v, int64_t base, bool row_ok, int slab, int chunk, int spc,
                                              unsigned long long (&x)[8])
@@ -155,7 +151,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
     while (q + 1 < a.count && (int)blockIdx.x >= a.first[q + 1]) ++q;
     const View &v = a.v[q];
     const Image &im = a.im[q];
-    const int S = im.slabs, WS = split_warps(S), G = kSplitWarps / WS, spc = S / v.ncat;
+    const int S = im.slabs, WS = split_warps(S), G = blockDim.x / 32 / WS, spc = S / v.ncat;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int gi = warp / WS, sub = warp % WS;
     const IT rows = (IT)im.rows, rb = (IT)im.rb, I = (IT)v.I;
@@ -163,7 +159,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
     const IT entry = g / groups, group = g - entry * groups;   // batch entry, row group in it
     const int row = lane >> 1, chunk = lane & 1;
     const IT r = group * kRowGroup + row, rg = (IT)v.r0 + r;
-    const bool in = entry < (IT)v.batch, row_ok = in && r < rows;
+    const bool in = gi < G && entry < (IT)v.batch, row_ok = in && r < rows;
     const IT o = rg / I;
     const int64_t base = (int64_t)entry * v.stride + (int64_t)o * (v.I * v.n) + (rg - o * I);
     const IT first = r / rb, blocks = (rows + rb - 1) / rb;
@@ -320,8 +316,12 @@ __device__ __forceinline__ void drain(uint32_t taddr, uint32_t cs, int hc, long 
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 auto cls = [&](int t) { return __uint_as_float(v[t * 4 + j]); };
-                const int c0 = __float2int_rn(cls(0)), c1 = __float2int_rn(cls(1)), c2 = __float2int_rn(cls(2));
-                const int c3 = __float2int_rn(cls(3)), c4 = __float2int_rn(cls(4));
+                // |class 0| <= 2^20, |class 1| <= 2^22: integers by adding 1.5 2^23
+                // (the conversion unit takes 16 values per clock and SM, as long for
+                // six classes as the MMAs of 96 entries)
+                const int c0 = __float_as_int(cls(0) + 12582912.0f) - 0x4B400000;
+                const int c1 = __float_as_int(cls(1) + 12582912.0f) - 0x4B400000;
+                const int c2 = __float2int_rn(cls(2)), c3 = __float2int_rn(cls(3)), c4 = __float2int_rn(cls(4));
                 const int c5 = __float2int_rn(fmaf(cls(7), 0x1p-10f, fmaf(cls(6), 0.25f, 64.0f * cls(5))));
                 const long long hp = (long long)c0 * 65536 + (c1 * 256 + c2);
                 const long long lp = (long long)c3 * 4194304 + ((long long)c4 * 16384 + c5);
@@ -757,16 +757,20 @@ void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
     SplitArgs a{};
     a.count = count;
     bool wide = false;
+    int warps = 1;
+    for (int q = 0; q < count; ++q) warps = std::max(warps, split_warps(im[q].slabs));
+    warps *= std::max(1, 8 / warps);
     for (int q = 0; q < count; ++q) {
         a.v[q] = v[q];
         a.im[q] = im[q];
-        const int G = kSplitWarps / split_warps(im[q].slabs);
+        const int G = warps / split_warps(im[q].slabs);
         const int64_t groups = (im[q].rows + kRowGroup - 1) / kRowGroup * v[q].batch;
         a.first[q + 1] = a.first[q] + (int)((groups + G - 1) / G);
         wide = wide || (v[q].r0 + im[q].rows + kRowGroup * 32) * std::max(1, v[q].batch) > INT32_MAX || v[q].I > INT32_MAX;
     }
-    if (wide) pdl_launch(k_digits<int64_t>, dim3(a.first[count]), dim3(kSplitWarps * 32), 0, st, 1, a);
-    else pdl_launch(k_digits<int>, dim3(a.first[count]), dim3(kSplitWarps * 32), 0, st, 1, a);
+    const dim3 grid(a.first[count]), block(warps * 32);
+    if (wide) pdl_launch(k_digits<int64_t>, grid, block, 0, st, 1, a);
+    else pdl_launch(k_digits<int>, grid, block, 0, st, 1, a);
 }
 
 void launch_products(const Product *s, int count, DevStatus *status, long long wait_limit, cudaStream_t st)
