@@ -640,25 +640,28 @@ void launch_nonfinite_scan(const double *x, int64_t count, int *flag, cudaStream
 //   phi_1(2Y) = (phi_0(Y) phi_1(Y) + phi_1(Y)) / 2,
 //   phi_2(2Y) = (phi_0(Y) phi_2(Y) + phi_1(Y) + phi_2(Y)) / 4.
 // Matrix b is squared exactly s_b times, s_b the least s >= 0 with
-// ||2^-s z_b A_b||_1 <= 1/2.
+// ||2^-s z_b A_b||_1 <= 1/2; the batch is sorted by s_b, so that each squaring
+// runs on the matrices that still need it.  The Taylor polynomials in Y = 2^-s z A
+// are evaluated in blocks of four powers (Paterson & Stockmeyer 1973): Y^2, then
+// Y^3 and Y^4, then three Horner steps in Y^4 on the three polynomials together,
+// 12 matrix products instead of one per degree.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int kTaylorDeg = 16;
 
-__global__ void k_build_X(int64_t nn, const double *const *Asrc, const double *z, double *X)
+__global__ void k_build_X(int64_t nn, const double *const *Asrc, const double *z, double *X, int64_t stride)
 {
     const int b = blockIdx.y;
     const double *A = Asrc[b];
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn;
          e += (int64_t)gridDim.x * blockDim.x)
-        X[b * nn + e] = z[b] * A[e];
+        X[b * stride + e] = z[b] * A[e];
 }
 
 // one block per matrix: column abs-sum maximum
-__global__ void k_norm1(int n, const double *X, double *out)
+__global__ void k_norm1(int n, const double *X, int64_t stride, double *out)
 {
     const int b = blockIdx.x;
-    const double *M = X + (int64_t)b * n * n;
+    const double *M = X + b * stride;
     __shared__ double red[256];
     double best = 0.0;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
@@ -675,46 +678,34 @@ __global__ void k_norm1(int n, const double *X, double *out)
     if (threadIdx.x == 0) out[b] = red[0];
 }
 
-__global__ void k_scale_pow2(int64_t nn, const int *s, double *X)
+// The powers of matrix b lie one after the other (Y^k at Q + (4 b + k - 1) nn), and
+// so do its three phi-matrices (phi_k at P + (3 b + k) nn).
+// T_k = sum_{j < 4} c_jk Y^j + (top: c_4k Y^4, else R_k), c_jk = 1 / (4 i + j + k)!
+struct TaylorBlock {
+    double c[5][3];
+};
+__global__ void k_taylor_block(int n, int64_t nn, bool top, TaylorBlock t, const double *Q, const double *R, double *T)
 {
     const int b = blockIdx.y;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn;
-         e += (int64_t)gridDim.x * blockDim.x)
-        X[b * nn + e] = ldexp(X[b * nn + e], -s[b]);
-}
-
-__global__ void k_identity(int n, int nb, double *X)
-{
-    int64_t nn = (int64_t)n * n, tot = nn * nb;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r = e % nn;
-        X[e] = ((r % n) == (r / n)) ? 1.0 : 0.0;
+    const double *y = Q + 4 * b * nn;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn; e += (int64_t)gridDim.x * blockDim.x) {
+        const bool diag = e % n == e / n;
+        const double y1 = y[e], y2 = y[nn + e], y3 = y[2 * nn + e], y4 = top ? y[3 * nn + e] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            double v = top ? t.c[4][k] * y4 : R[(3 * b + k) * nn + e];
+            v = fma(t.c[3][k], y3, v);
+            v = fma(t.c[2][k], y2, v);
+            v = fma(t.c[1][k], y1, v);
+            T[(3 * b + k) * nn + e] = diag ? v + t.c[0][k] : v;
+        }
     }
 }
 
-// The three phi-matrices of matrix b lie one after the other: phi_k at
-// P + (3 b + k) nn.
-// phi_k += Pw / (j + k)!  for k = 0, 1, 2
-__global__ void k_taylor_acc(int64_t nn, const double *Pw, double c0, double c1, double c2, double *P)
+// squaring update (T: phi_0 times the three)
+__global__ void k_square_update(int64_t nn, const double *T, double *P)
 {
     const int b = blockIdx.y;
-    double *p = P + 3 * b * nn;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        double w = Pw[b * nn + e];
-        p[e] = __dadd_rn(p[e], __dmul_rn(c0, w));
-        p[nn + e] = __dadd_rn(p[nn + e], __dmul_rn(c1, w));
-        p[2 * nn + e] = __dadd_rn(p[2 * nn + e], __dmul_rn(c2, w));
-    }
-}
-
-// squaring update (T: phi_0 times the three); matrix b takes the new values
-// only while it <= s_b
-__global__ void k_square_update(int64_t nn, int it, const int *s, const double *T, double *P)
-{
-    const int b = blockIdx.y;
-    if (it > s[b]) return;
     const double *t = T + 3 * b * nn;
     double *p = P + 3 * b * nn;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn;
@@ -745,11 +736,11 @@ __global__ void k_extract_deriv(int64_t nn, const double *const *lo, const doubl
         dst[b][e] = lo[b][e] - (double)ell[b] * hi[b][e];
 }
 
-// C_b = A_b [B_b0 ... B_b(m-1)] for column-major n x n blocks: entry b of the
-// batch has its A at A + b sA and its m right-hand blocks, one after the
-// other, at B + b sB (products to C + b m n^2)
+// C_b = A_b [B_b0 ... B_b(m-1)] for column-major n x n blocks, entries b of the
+// batch sA, sB, sC apart, a right-hand entry's m blocks one after the other (and
+// the products')
 void batched_products(const mm::Context &ctx, int n, int m, int nb, const double *A, int64_t sA, const double *B,
-                      int64_t sB, double *C, cudaStream_t st)
+                      int64_t sB, double *C, int64_t sC, cudaStream_t st)
 {
     mm::Product p{};
     p.A = mm::matrix_view(n, A, 0);
@@ -759,7 +750,7 @@ void batched_products(const mm::Context &ctx, int n, int m, int nb, const double
     p.A.stride = sA;
     p.B.stride = sB;
     p.out = C;
-    p.stride = (int64_t)m * n * n;
+    p.stride = sC;
     mm::run_products(ctx, &p, 1, st);
 }
 }  // namespace
@@ -769,10 +760,10 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     const int nb = (int)jobs.size();
     if (nb == 0) return DS_OK;
     const int64_t nn = (int64_t)n * n, tot = nn * nb;
-    // workspace: Y, Pw, T, phi0..2, their products (9 blocks), tables, digit images
+    // workspace: Y .. Y^4, phi0..2, their products (10 blocks), tables, digit images
     double *ws = nullptr;
-    DS_CUDA_TRY(pool_alloc(&ws, sizeof(double) * tot * 9, st));
-    double *Y = ws, *Pw = ws + tot, *T = ws + 2 * tot, *P = ws + 3 * tot, *T3 = ws + 6 * tot;
+    DS_CUDA_TRY(pool_alloc(&ws, sizeof(double) * tot * 10, st));
+    double *Q = ws, *P = ws + 4 * tot, *T = ws + 7 * tot;
     mm::Context ctx;
     if (mm::use_digits(n, n, nb)) {
         mm::View v = mm::matrix_view(n, nullptr, 0);
@@ -810,8 +801,8 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     cudaMemcpyAsync(dz, hz.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st);
 
     dim3 g2((unsigned)std::min<int64_t>((nn + 255) / 256, 1024), nb);
-    k_build_X<<<g2, 256, 0, st>>>(nn, dA, dz, Y);
-    k_norm1<<<nb, 256, 0, st>>>(n, Y, dnorm);
+    k_build_X<<<g2, 256, 0, st>>>(nn, dA, dz, Q, 4 * nn);
+    k_norm1<<<nb, 256, 0, st>>>(n, Q, 4 * nn, dnorm);
     std::vector<double> hnorm(nb);
     cudaMemcpyAsync(hnorm.data(), dnorm, sizeof(double) * nb, cudaMemcpyDeviceToHost, st);
     DS_CUDA_TRY(cudaStreamSynchronize(st));
@@ -827,32 +818,47 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
         hs[b] = s;
         smax = std::max(smax, s);
     }
-    cudaMemcpyAsync(ds_, hs.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st);
-    k_scale_pow2<<<g2, 256, 0, st>>>(nn, ds_, Y);
+    // the batch in order of falling s; Y = (2^-s z) A
+    std::vector<int> perm(nb), sp(nb);
+    for (int b = 0; b < nb; ++b) perm[b] = b;
+    std::stable_sort(perm.begin(), perm.end(), [&](int x, int y) { return hs[x] > hs[y]; });
+    for (int b = 0; b < nb; ++b) {
+        sp[b] = hs[perm[b]];
+        hA[b] = jobs[perm[b]].A;
+        hz[b] = ldexp(jobs[perm[b]].z, -sp[b]);
+    }
+    cudaMemcpyAsync(dA, hA.data(), sizeof(void *) * nb, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(dz, hz.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st);
+    k_build_X<<<g2, 256, 0, st>>>(nn, dA, dz, Q, 4 * nn);
 
     // Taylor: phi_k(Y) = sum_j Y^j / (j + k)!
-    double fact[kTaylorDeg + 4];
-    fact[0] = 1.0;
-    for (int j = 1; j < kTaylorDeg + 4; ++j) fact[j] = fact[j - 1] * j;
-    const int gl = (int)std::min<int64_t>((tot + 255) / 256, 152 * 16);
-    cudaMemsetAsync(P, 0, sizeof(double) * tot * 3, st);
-    k_identity<<<gl, 256, 0, st>>>(n, nb, Pw);
-    for (int j = 0; j <= kTaylorDeg; ++j) {
-        k_taylor_acc<<<g2, 256, 0, st>>>(nn, Pw, 1.0 / fact[j], 1.0 / fact[j + 1], 1.0 / fact[j + 2], P);
-        if (j < kTaylorDeg) {
-            batched_products(ctx, n, 1, nb, Pw, nn, Y, nn, T, st);
-            std::swap(Pw, T);
-        }
+    batched_products(ctx, n, 1, nb, Q, 4 * nn, Q, 4 * nn, Q + nn, 4 * nn, st);              // Y^2
+    batched_products(ctx, n, 2, nb, Q + nn, 4 * nn, Q, 4 * nn, Q + 2 * nn, 4 * nn, st);     // Y^3, Y^4
+    auto block = [](int i) {
+        double fact[20] = {1.0};
+        for (int j = 1; j < 20; ++j) fact[j] = fact[j - 1] * j;
+        TaylorBlock t;
+        for (int j = 0; j < 5; ++j)
+            for (int k = 0; k < 3; ++k) t.c[j][k] = 1.0 / fact[4 * i + j + k];
+        return t;
+    };
+    k_taylor_block<<<g2, 256, 0, st>>>(n, nn, true, block(3), Q, nullptr, P);
+    for (int i = 2; i >= 0; --i) {
+        batched_products(ctx, n, 3, nb, Q + 3 * nn, 4 * nn, P, 3 * nn, T, 3 * nn, st);
+        k_taylor_block<<<g2, 256, 0, st>>>(n, nn, false, block(i), Q, T, P);
     }
     for (int it = 1; it <= smax; ++it) {
-        batched_products(ctx, n, 3, nb, P, 3 * nn, P, 3 * nn, T3, st);
-        k_square_update<<<g2, 256, 0, st>>>(nn, it, ds_, T3, P);
+        int active = 0;
+        while (active < nb && sp[active] >= it) ++active;
+        batched_products(ctx, n, 3, active, P, 3 * nn, P, 3 * nn, T, 3 * nn, st);
+        k_square_update<<<dim3(g2.x, active), 256, 0, st>>>(nn, T, P);
     }
     std::vector<double *> hsrc(nb), hdst(nb);
     for (int b = 0; b < nb; ++b) {
-        int l = jobs[b].ell;
+        const PhiJob &job = jobs[perm[b]];
+        const int l = job.ell;
         hsrc[b] = P + (3 * b + l) * nn;
-        hdst[b] = jobs[b].out;
+        hdst[b] = job.out;
     }
     cudaMemcpyAsync(dSrc, hsrc.data(), sizeof(void *) * nb, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(dDst, hdst.data(), sizeof(void *) * nb, cudaMemcpyHostToDevice, st);
@@ -863,10 +869,11 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
         std::vector<double *> hlo(nb), hdd(nb);
         std::vector<int> hell(nb);
         for (int b = 0; b < nb; ++b) {
-            const int l = jobs[b].ell;
+            const PhiJob &job = jobs[perm[b]];
+            const int l = job.ell;
             hlo[b] = P + (3 * b + l - 1) * nn;
             hsrc[b] = P + (3 * b + l) * nn;
-            hdd[b] = jobs[b].dout;
+            hdd[b] = job.dout;
             hell[b] = l;
         }
         // the tables are reused: dA <- lo, dSrc <- hi, dDst <- dout, ds_ <- ell

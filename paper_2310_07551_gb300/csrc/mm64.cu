@@ -861,7 +861,8 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
 {
     int launches = 0;
     for (int i = 0; i < count;) {
-        const bool digits = use_digits(ps[i].A.rows, ps[i].A.n, count);
+        const int many = count * ps[i].A.batch;   // products in a launch
+        const bool digits = use_digits(ps[i].A.rows, ps[i].A.n, many);
         Product p[kMaxProd];
         View sv[kMaxProd];
         Image si[kMaxProd];
@@ -890,7 +891,7 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
             Product t = q;
             const size_t u0 = used;
             const int n0 = ns;
-            if ((with_b && !place(t.B, tile_cols(t.A.rows, (int)t.B.rows, count), t.ib)) ||
+            if ((with_b && !place(t.B, tile_cols(t.A.rows, (int)t.B.rows, many), t.ib)) ||
                 !place(t.A, kRowBlock, t.ia)) {
                 used = u0;
                 ns = n0;
