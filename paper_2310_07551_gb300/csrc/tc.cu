@@ -4558,8 +4558,23 @@ ds_status mixed_group_create(const std::vector<MixedPlan *> &mps, const std::vec
             std::vector<TcArgs> tab(ninst), tab_sep, tab_s(ninst);
             std::vector<StageArgs> stab, stab_s;
             std::vector<int64_t> prefix(ninst), sprefix, prefix_sep;
-            int64_t units = 0, units_sep = 0, points = 0, off = 0;
+            int64_t units = 0, units_sep = 0, points = 0;
+            // longest contractions first: the units of a wave then take about as
+            // long, and the last wave holds the short ones
+            std::vector<int> by_k(ninst);
+            std::vector<int64_t> offs(ninst);
             for (int i = 0; i < ninst; ++i) {
+                by_k[i] = i;
+                offs[i] = i ? offs[i - 1] + mps[i - 1]->N : 0;
+            }
+            auto length = [&](int i) {
+                const TcArgs &a = mps[i]->C[g][mu][mps[i]->compensated ? 0 : 1].args;
+                return a.T * a.kchunks;
+            };
+            std::stable_sort(by_k.begin(), by_k.end(), [&](int x, int y) { return length(x) > length(y); });
+            for (int q = 0; q < ninst; ++q) {
+                const int i = by_k[q];
+                const int64_t off = offs[i];
                 // 128-column tiles (with dual accumulators for compensated plans): a
                 // batch's problems are small, and the narrower tiles fill the SMs
                 // better (measured on the 64-instance Schnakenberg batch)
@@ -4572,9 +4587,9 @@ ds_status mixed_group_create(const std::vector<MixedPlan *> &mps, const std::vec
                     a.U = U[i];
                     a.model = mf;
                 }
-                tab[i] = a;
-                tab_s[i] = a;
-                if (a.epi) tab_s[i].U = Us + 2 * off;
+                tab[q] = a;
+                tab_s[q] = a;
+                if (a.epi) tab_s[q].U = Us + 2 * off;
                 if (last) {
                     ModeLaunch S = mps[i]->Csep[g][w];
                     set_split(S, 1, nullptr);
@@ -4588,11 +4603,10 @@ ds_status mixed_group_create(const std::vector<MixedPlan *> &mps, const std::vec
                     sprefix.push_back(points);
                     points += mps[i]->N;
                 }
-                prefix[i] = units;
+                prefix[q] = units;
                 units += a.num_units;
-                off += mps[i]->N;
                 sl.flops += launch_flops(L, L.N);
-                if (i == 0) {
+                if (q == 0) {
                     sl.mode1 = L.mode1;
                     sl.bn = L.bn;
                     sl.dual = L.dual;
