@@ -1110,6 +1110,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // (the prologue above runs behind the previous launch)
+    pdl_trigger();
+    pdl_wait();
 
     // The producer's and the issuer's loops run on their whole warp, with the
     // asynchronous instructions under elect_one(): a lone thread would move every
@@ -1255,12 +1258,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                                     ad = sdesc(sA + pa * A_PLANE + ks * 2048, A_PLANE / 2, 1024, kSw128);
                                 }
                                 bd = sdesc(sB + pb * B_PLANE + ks * 32, 16, 512, kSw64);
-                                if (DUAL) {
-                                    const bool first = it == it0 && ks == 0 && (q == 0 || q == 1);
-                                    mma_bf16(q == 0 ? d : d + BN, ad, bd, idesc, first ? 0u : 1u);
-                                } else {
-                                    mma_bf16(d, ad, bd, idesc, (it > it0 || ks > 0 || q > 0) ? 1u : 0u);
-                                }
+                                // (the first two products share their A part, which the
+                                // collector buffer keeps)
+                                const uint32_t dq = DUAL && q > 0 ? d + BN : d;
+                                const bool first = it == it0 && ks == 0 && (q == 0 || (DUAL && q == 1));
+                                if (q == 0) mma_f16_coll<1>(dq, ad, bd, idesc, first ? 0u : 1u);
+                                else if (q == 1) mma_f16_coll<3>(dq, ad, bd, idesc, first ? 0u : 1u);
+                                else mma_bf16(dq, ad, bd, idesc, 1u);
                             }
                         }
                         }
@@ -2215,6 +2219,8 @@ __global__ void __launch_bounds__(TX * TY, 1) k_rhs_tiled(const __grid_constant_
                                                           const RhsArgs *__restrict__ gtab,
                                                           const int *__restrict__ gprefix, int ginst)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ float sh[2][2][TY + 2][TX + 2];   // [component][hi, lo][y][x], one-point halo
     int gi = 0, lb = 0;
     if (GROUPED) {
@@ -2358,6 +2364,8 @@ __global__ void __launch_bounds__(TX * TY, 3) k_rhs_fx(const __grid_constant__ R
                                                        const RhsArgs *__restrict__ gtab,
                                                        const int *__restrict__ gprefix, int ginst)
 {
+    pdl_trigger();
+    pdl_wait();
     constexpr int HX = TX + 2, HY = TY + 2;
     constexpr int NHALO = TY > 1 ? 2 * (TX + TY) : 2;
     static_assert(NHALO <= TX * TY, "one halo point per thread");
@@ -2552,14 +2560,14 @@ static void launch_rhs_tiled(const StencilF &s0, const StencilF &s1, const Model
     const bool small = N < ((int64_t)1 << 31);
     if (s0.d == 3) {
         if (small)
-            k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, false><<<g, RT3_X * RT3_Y, 0, st>>>(a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, false>, dim3(g), dim3(RT3_X * RT3_Y), 0, st, 1, a, nullptr, nullptr, 0);
         else
-            k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int64_t, false><<<g, RT3_X * RT3_Y, 0, st>>>(a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int64_t, false>, dim3(g), dim3(RT3_X * RT3_Y), 0, st, 1, a, nullptr, nullptr, 0);
     } else {
         if (small)
-            k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, false><<<g, RT2_X, 0, st>>>(a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, false>, dim3(g), dim3(RT2_X), 0, st, 1, a, nullptr, nullptr, 0);
         else
-            k_rhs_tiled<RT2_X, 1, RT2_Z, int64_t, false><<<g, RT2_X, 0, st>>>(a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int64_t, false>, dim3(g), dim3(RT2_X), 0, st, 1, a, nullptr, nullptr, 0);
     }
 }
 
@@ -2570,16 +2578,16 @@ static void launch_rhs_group(int d, const RhsArgs *tab, const int *prefix, int n
 {
     if (fx) {
         if (d == 3)
-            k_rhs_fx<RT3_X, RT3_Y, RT3_Z, true><<<blocks, RT3_X * RT3_Y, 0, st>>>(RhsArgs{}, tab, prefix, ninst);
+            pdl_launch(k_rhs_fx<RT3_X, RT3_Y, RT3_Z, true>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, 1, RhsArgs{}, tab, prefix, ninst);
         else
-            k_rhs_fx<RT2_X, 1, RT2_Z, true><<<blocks, RT2_X, 0, st>>>(RhsArgs{}, tab, prefix, ninst);
+            pdl_launch(k_rhs_fx<RT2_X, 1, RT2_Z, true>, dim3(blocks), dim3(RT2_X), 0, st, 1, RhsArgs{}, tab, prefix, ninst);
         return;
     }
     if (d == 3)
-        k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, true><<<blocks, RT3_X * RT3_Y, 0, st>>>(RhsArgs{}, tab, prefix,
+        pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, true>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, 1, RhsArgs{}, tab, prefix,
                                                                                          ninst);
     else
-        k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, true><<<blocks, RT2_X, 0, st>>>(RhsArgs{}, tab, prefix, ninst);
+        pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, true>, dim3(blocks), dim3(RT2_X), 0, st, 1, RhsArgs{}, tab, prefix, ninst);
 }
 
 // Separate (unfused) stage kernels, used when timing at plan creation finds them
@@ -2591,6 +2599,8 @@ __global__ void k_stage_planes(ModelF m, int64_t N, const double *__restrict__ U
                                int64_t cs_a, const float *__restrict__ b, int64_t cs_b,
                                bf16 *__restrict__ Dp)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         float hu, lu, hv, lv;
@@ -2614,6 +2624,8 @@ __global__ void k_stage_planes(ModelF m, int64_t N, const double *__restrict__ U
 __global__ void k_final_mixed(int64_t N, double *__restrict__ U, const float *__restrict__ a, int64_t cs_a,
                               const float *__restrict__ b, int64_t cs_b)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
          p += (int64_t)gridDim.x * blockDim.x) {
         U[p] += widen_f(a[p] + b[p]);
@@ -2696,6 +2708,8 @@ __device__ __forceinline__ void stage_fx_record(FxScales *fxs, int slot, const f
 }
 __global__ void k_stage_fx(const __grid_constant__ StageFx a)
 {
+    pdl_trigger();
+    pdl_wait();
     float mx[2] = {0.0f, 0.0f};
     bool over = false;
     // every lane of a warp runs the same number of iterations (the shuffle
@@ -2723,6 +2737,8 @@ __global__ void k_final_fx(int64_t N, double *__restrict__ U, const float *__res
                            const float *__restrict__ al, int64_t cs_a, const float *__restrict__ bh,
                            const float *__restrict__ bl, int64_t cs_b)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
         final_fx_point(N, U, ah, al, cs_a, bh, bl, cs_b, p);
 }
@@ -2854,6 +2870,8 @@ __device__ __forceinline__ void fx_rescale_slot(FxScales *f, int k, bool reset)
 }
 __global__ void k_fx_rescale(FxScales *f, int first, int count, int reset)
 {
+    pdl_trigger();
+    pdl_wait();
     const int k = first + (int)threadIdx.x;
     if ((int)threadIdx.x >= count || k >= kFxSlots) return;
     fx_rescale_slot(f, k, reset != 0);
@@ -3343,6 +3361,8 @@ __device__ __forceinline__ void store_planes4(bf16 *dst, int64_t plane, int64_t 
 __global__ void k_split_reduce(int64_t total, int64_t N, int ksplit, const float *__restrict__ ws, int out_kind,
                                void *out)
 {
+    pdl_trigger();
+    pdl_wait();
     for (int64_t e = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); e < total;
          e += 4 * (int64_t)gridDim.x * blockDim.x) {
         const float4 v = part_sum4(ws, total, ksplit, e);
@@ -3359,6 +3379,8 @@ __global__ void k_split_reduce(int64_t total, int64_t N, int ksplit, const float
 // kernel's, applied to the part sums (summed in part order).
 __global__ void k_split_reduce_epi(const __grid_constant__ TcArgs a)
 {
+    pdl_trigger();
+    pdl_wait();
     const int64_t N = a.out_ps, ps = a.part_stride;
     const int S2 = a.S / 2;
     const int64_t total = a.epi == 2 ? (int64_t)a.S * N : (int64_t)S2 * N;
@@ -3430,43 +3452,43 @@ static void launch_tc_k(bool mode1, int bn, bool dual, int grid, cudaStream_t st
             constexpr uint32_t sm = TileCfg<128, 4>::SMEM_BYTES;
             if (a.out_kind == 0) {
                 if (mode1)
-                    k_mode_tc<true, 128, false, GROUPED, false, 1><<<grid, kThreads, sm, st>>>(a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<true, 128, false, GROUPED, false, 1>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
                 else
-                    k_mode_tc<false, 128, false, GROUPED, false, 1><<<grid, kThreads, sm, st>>>(a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<false, 128, false, GROUPED, false, 1>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
             } else if (a.out_kind == 1) {
                 if (mode1)
-                    k_mode_tc<true, 128, false, GROUPED, false, 2><<<grid, kThreads, sm, st>>>(a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<true, 128, false, GROUPED, false, 2>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
                 else
-                    k_mode_tc<false, 128, false, GROUPED, false, 2><<<grid, kThreads, sm, st>>>(a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<false, 128, false, GROUPED, false, 2>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
             } else if constexpr (!GROUPED) {
                 if (mode1)
-                    k_mode_tc<true, 128, false, false, false, 3><<<grid, kThreads, sm, st>>>(a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<true, 128, false, false, false, 3>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
                 else
-                    k_mode_tc<false, 128, false, false, false, 3><<<grid, kThreads, sm, st>>>(a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<false, 128, false, false, false, 3>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
             }
         }
         return;
     }
     if (bn == 256) {
         if (mode1)
-            k_mode_tc<true, 256, false, GROUPED, SK><<<grid, kThreads, TileCfg<256>::SMEM_BYTES, st>>>(a, gtab, gprefix,
+            pdl_launch(k_mode_tc<true, 256, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<256>::SMEM_BYTES, st, 1, a, gtab, gprefix,
                                                                                                   ginst, gunits);
         else
-            k_mode_tc<false, 256, false, GROUPED, SK><<<grid, kThreads, TileCfg<256>::SMEM_BYTES, st>>>(a, gtab, gprefix,
+            pdl_launch(k_mode_tc<false, 256, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<256>::SMEM_BYTES, st, 1, a, gtab, gprefix,
                                                                                                    ginst, gunits);
     } else if (!dual) {
         if (mode1)
-            k_mode_tc<true, 128, false, GROUPED, SK><<<grid, kThreads, TileCfg<128>::SMEM_BYTES, st>>>(a, gtab, gprefix,
+            pdl_launch(k_mode_tc<true, 128, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
                                                                                                   ginst, gunits);
         else
-            k_mode_tc<false, 128, false, GROUPED, SK><<<grid, kThreads, TileCfg<128>::SMEM_BYTES, st>>>(a, gtab, gprefix,
+            pdl_launch(k_mode_tc<false, 128, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
                                                                                                    ginst, gunits);
     } else {
         if (mode1)
-            k_mode_tc<true, 128, true, GROUPED, SK><<<grid, kThreads, TileCfg<128>::SMEM_BYTES, st>>>(a, gtab, gprefix,
+            pdl_launch(k_mode_tc<true, 128, true, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
                                                                                                  ginst, gunits);
         else
-            k_mode_tc<false, 128, true, GROUPED, SK><<<grid, kThreads, TileCfg<128>::SMEM_BYTES, st>>>(a, gtab, gprefix,
+            pdl_launch(k_mode_tc<false, 128, true, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
                                                                                                   ginst, gunits);
     }
 }
@@ -3534,9 +3556,9 @@ static void launch(const ModeLaunch &L, cudaStream_t st, double *U = nullptr, co
         const int64_t total = a.part_stride;
         const int g = (int)std::min<int64_t>((total / 4 + 255) / 256, 152 * 8);
         if (a.epi)
-            k_split_reduce_epi<<<g, 256, 0, st>>>(a);
+            pdl_launch(k_split_reduce_epi, dim3(g), dim3(256), 0, st, 1, a);
         else
-            k_split_reduce<<<g, 256, 0, st>>>(total, L.N, a.ksplit, a.part_ws, a.out_kind, a.out);
+            pdl_launch(k_split_reduce, dim3(g), dim3(256), 0, st, 1, total, L.N, a.ksplit, a.part_ws, a.out_kind, a.out);
     }
 }
 
@@ -3780,11 +3802,11 @@ static void launch_stage_kernel(const MixedPlan *mp, int g, const ModelF &mf, do
 {
     const int64_t N = mp->N;
     if (g == 0)
-        k_stage_planes<<<pw_grid(N), 256, 0, st>>>(mf, N, U, mp->incF, 3 * N, nullptr, 0, mp->Dp);
+        pdl_launch(k_stage_planes, dim3(pw_grid(N)), dim3(256), 0, st, 1, mf, N, U, mp->incF, 3 * N, nullptr, 0, mp->Dp);
     else if (g == 1)
-        k_stage_planes<<<pw_grid(N), 256, 0, st>>>(mf, N, U, mp->incF + N, 3 * N, mp->incD, N, mp->Dp);
+        pdl_launch(k_stage_planes, dim3(pw_grid(N)), dim3(256), 0, st, 1, mf, N, U, mp->incF + N, 3 * N, mp->incD, N, mp->Dp);
     else
-        k_final_mixed<<<pw_grid(N), 256, 0, st>>>(N, U, mp->incF + 2 * N, 3 * N, mp->incD, N);
+        pdl_launch(k_final_mixed, dim3(pw_grid(N)), dim3(256), 0, st, 1, N, U, mp->incF + 2 * N, 3 * N, mp->incD, N);
 }
 
 // For each group, time its last mode with the fused epilogue against the
@@ -4390,9 +4412,9 @@ static void launch_rhs_fx(MixedPlan *mp, const Model &model, double *U, bool mea
     const dim3 g = rhs_tiles(mp->stf[0]);
     const unsigned blocks = g.x * g.y * g.z;
     if (mp->d == 3)
-        k_rhs_fx<RT3_X, RT3_Y, RT3_Z, false><<<blocks, RT3_X * RT3_Y, 0, st>>>(a, nullptr, nullptr, 0);
+        pdl_launch(k_rhs_fx<RT3_X, RT3_Y, RT3_Z, false>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, 1, a, nullptr, nullptr, 0);
     else
-        k_rhs_fx<RT2_X, 1, RT2_Z, false><<<blocks, RT2_X, 0, st>>>(a, nullptr, nullptr, 0);
+        pdl_launch(k_rhs_fx<RT2_X, 1, RT2_Z, false>, dim3(blocks), dim3(RT2_X), 0, st, 1, a, nullptr, nullptr, 0);
 }
 
 int enqueue_rhs_mixed(MixedPlan *mp, const Model &model, double *U, cudaStream_t st)
@@ -4874,7 +4896,7 @@ int enqueue_step_mixed(MixedPlan *mp, const ds_phi_set *set, const Model &model,
         // from that and then writes it.
         // reset: the calibrating step starts each slot's exponent history
         auto rescale = [&](int first, int count, bool reset) {
-            k_fx_rescale<<<1, 32, 0, st>>>(mp->fxs, first, count, reset ? 1 : 0);
+            pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, 1, mp->fxs, first, count, reset ? 1 : 0);
             ++L;
         };
         auto rhs = [&](bool measure) {
@@ -4950,7 +4972,7 @@ int enqueue_step_mixed(MixedPlan *mp, const ds_phi_set *set, const Model &model,
             sa.measure = measure ? 1 : 0;
             sa.model = mdf;
             P.begin(st, 2, 0.0, (double)N * (g == 1 ? 48.0 : 64.0));
-            k_stage_fx<<<pw_grid(N), 256, 0, st>>>(sa);
+            pdl_launch(k_stage_fx, dim3(pw_grid(N)), dim3(256), 0, st, 1, sa);
             P.end(st);
             ++L;
         };
@@ -4969,7 +4991,7 @@ int enqueue_step_mixed(MixedPlan *mp, const ds_phi_set *set, const Model &model,
         }
         // U += tau S_f(F) + 3tau/2 S_f(D3), both as double-floats
         P.begin(st, 2, 0.0, (double)N * 64.0);
-        k_final_fx<<<pw_grid(N), 256, 0, st>>>(N, U, mp->incF + 2 * N, mp->incFlo + 2 * N, 3 * N, mp->incD,
+        pdl_launch(k_final_fx, dim3(pw_grid(N)), dim3(256), 0, st, 1, N, U, mp->incF + 2 * N, mp->incFlo + 2 * N, 3 * N, mp->incD,
                                                mp->incDlo, N);
         P.end(st);
         ++L;
@@ -5082,7 +5104,7 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
     DS_CUDA_TRY(cudaMemcpyAsync(fxs, &h, sizeof(h), cudaMemcpyHostToDevice, st));
     DS_CUDA_TRY(cudaMemcpyAsync(jobs, hj, sizeof(FxMatJob) * d, cudaMemcpyHostToDevice, st));
     k_absmax<<<pw_grid(N), 256, 0, st>>>(N, X, fxs, 0);
-    k_fx_rescale<<<1, 32, 0, st>>>(fxs, 0, 1, 1);
+    pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, 1, fxs, 0, 1, 1);
     k_split_tensor_fx<<<pw_grid(N), 256, 0, st>>>(N, X, fxs, 0, A0);
     __half *pcur = Pp;
     float *pscur = pscale;
@@ -5108,7 +5130,7 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
             ModeLaunch mm = ml;
             mm.args.fx_measure = 1;
             launch(mm, st);
-            k_fx_rescale<<<1, 32, 0, st>>>(fxs, mu + 1, 1, 1);
+            pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, 1, fxs, mu + 1, 1, 1);
         }
         launch(ml, st);
         in = bufs[mu % 2];
