@@ -43,9 +43,9 @@ constexpr int kSms = 152;
 __device__ DevStatus g_status;
 
 // ---------------------------------------------------------------------------
-// Digit images.  One warp takes 16 rows of one slab: lane = (row, 8
-// consecutive contracted entries), so that every digit plane is written as
-// 512 contiguous bytes.  Up to 16 warps share the slabs of a row group, each
+// Digit images.  One warp takes 2E rows of one slab: lane = (row, E consecutive
+// contracted entries), so that every digit plane is written as 64 E contiguous
+// bytes.  Up to 16 warps share the slabs of a row group, each
 // keeping the first slab it reads in registers, so a fibre of up to 256 entries
 // is read once.  24 bytes per entry pass through memory, which bounds large
 // tensors; blocks are as small as the slabs allow, so that one block's loads run
@@ -57,31 +57,32 @@ struct SplitArgs {
     View v[kMaxProd];
     Image im[kMaxProd];
 };
-constexpr int kRowGroup = 16, kSplitWarps = 16;
+constexpr int kSplitWarps = 16;
 
 __host__ __device__ inline int split_warps(int slabs) { return slabs < kSplitWarps ? slabs : kSplitWarps; }
 
+template <int E>
 __device__ __forceinline__ void load_entries(const View &v, int64_t base, bool row_ok, int slab, int chunk, int spc,
-                                             unsigned long long (&x)[8])
+                                             unsigned long long (&x)[E])
 {
-    const int t = slab / spc, k0 = (slab - t * spc) * kSlab + chunk * 8, left = row_ok ? v.n - k0 : 0;
+    const int t = slab / spc, k0 = (slab - t * spc) * kSlab + chunk * E, left = row_ok ? v.n - k0 : 0;
     const double *src = v.src[t] + base + v.I * k0;
     const double sc = v.scale[t];
-    if (v.I == 1 && left >= 8 && ((uintptr_t)src & 15) == 0) {
+    if (v.I == 1 && left >= E && ((uintptr_t)src & 15) == 0) {
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
+        for (int j = 0; j < E; j += 2) {
             const longlong2 d = *reinterpret_cast<const longlong2 *>(src + j);
             x[j] = (unsigned long long)d.x;
             x[j + 1] = (unsigned long long)d.y;
         }
     } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+        for (int j = 0; j < E; ++j)
             x[j] = j < left ? (unsigned long long)__double_as_longlong(src[v.I * j]) : 0ULL;
     }
     if (sc != 1.0) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+        for (int j = 0; j < E; ++j)
             x[j] = (unsigned long long)__double_as_longlong(__dmul_rn(__longlong_as_double((long long)x[j]), sc));
     }
 }
@@ -95,13 +96,14 @@ __device__ __forceinline__ int fibre_exp(unsigned long long mx)
     return mx ? (64 - __clzll((long long)mx)) - 1074 : 0;
 }
 
-// the eight digits of 8 consecutive entries: bytes of x 2^(62 - e) + 128 in
-// every byte, one 16-byte chunk per digit plane
-__device__ __forceinline__ void store_digits(const unsigned long long (&x)[8], int e, uint8_t *dst, int64_t plane)
+// the eight digits of E consecutive entries: bytes of x 2^(62 - e) + 128 in
+// every byte, one chunk of 2 E bytes per digit plane
+template <int E>
+__device__ __forceinline__ void store_digits(const unsigned long long (&x)[E], int e, uint8_t *dst, int64_t plane)
 {
-    uint32_t lo[8], hi[8];
+    uint32_t lo[E], hi[E];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < E; ++j) {
         const unsigned long long b = x[j];
         int ef = (int)(b >> 52) & 0x7FF;
         unsigned long long m = b & 0xFFFFFFFFFFFFFULL;
@@ -119,9 +121,9 @@ __device__ __forceinline__ void store_digits(const unsigned long long (&x)[8], i
     const __half2 off = __half2half2(__ushort_as_half((unsigned short)0xE480));   // -1152 = -(1024 + 128)
 #pragma unroll
     for (int p = 0; p < kDigits; ++p) {
-        uint32_t q[4];
+        uint32_t q[E / 2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < E / 2; ++j) {
             const uint32_t w0 = p < 4 ? hi[2 * j] : lo[2 * j], w1 = p < 4 ? hi[2 * j + 1] : lo[2 * j + 1];
             const int b = 3 - (p & 3);
             // FP16 1024 + byte, two entries per word
@@ -130,23 +132,27 @@ __device__ __forceinline__ void store_digits(const unsigned long long (&x)[8], i
             const __half2 h = __hadd2(*reinterpret_cast<const __half2 *>(&w), off);
             q[j] = *reinterpret_cast<const uint32_t *>(&h);
         }
-        *reinterpret_cast<uint4 *>(dst + p * plane) = make_uint4(q[0], q[1], q[2], q[3]);
+        if constexpr (E == 8) *reinterpret_cast<uint4 *>(dst + p * plane) = make_uint4(q[0], q[1], q[2], q[3]);
+        else *reinterpret_cast<uint2 *>(dst + p * plane) = make_uint2(q[0], q[1]);
     }
 }
 
-__device__ __forceinline__ unsigned long long largest(unsigned long long mx, const unsigned long long (&x)[8])
+template <int E>
+__device__ __forceinline__ unsigned long long largest(unsigned long long mx, const unsigned long long (&x)[E])
 {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) mx = max(mx, x[j] & 0x7FFFFFFFFFFFFFFFULL);
+    for (int j = 0; j < E; ++j) mx = max(mx, x[j] & 0x7FFFFFFFFFFFFFFFULL);
     return mx;
 }
 
 // IT: 32-bit row indices where every view allows it (their divisions are a
 // good part of a small launch)
-template <typename IT>
+template <typename IT, int E>
 __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_constant__ SplitArgs a)
 {
-    __shared__ unsigned long long smax[kSplitWarps][kRowGroup];
+    static_assert(E == 8 || E == 4, "16 or 8 bytes of a digit plane per thread");
+    constexpr int kRows = 2 * E, kLaneBits = E == 8 ? 1 : 2;   // rows per warp, log2 of the lanes per row
+    __shared__ unsigned long long smax[kSplitWarps][kRows];
     int q = 0;
     while (q + 1 < a.count && (int)blockIdx.x >= a.first[q + 1]) ++q;
     const View &v = a.v[q];
@@ -155,10 +161,10 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int gi = warp / WS, sub = warp % WS;
     const IT rows = (IT)im.rows, rb = (IT)im.rb, I = (IT)v.I;
-    const IT groups = (rows + kRowGroup - 1) / kRowGroup, g = (IT)(blockIdx.x - a.first[q]) * G + gi;
+    const IT groups = (rows + kRows - 1) / kRows, g = (IT)(blockIdx.x - a.first[q]) * G + gi;
     const IT entry = g / groups, group = g - entry * groups;   // batch entry, row group in it
-    const int row = lane >> 1, chunk = lane & 1;
-    const IT r = group * kRowGroup + row, rg = (IT)v.r0 + r;
+    const int row = lane >> kLaneBits, chunk = lane & ((1 << kLaneBits) - 1);
+    const IT r = group * kRows + row, rg = (IT)v.r0 + r;
     const bool in = gi < G && entry < (IT)v.batch, row_ok = in && r < rows;
     const IT o = rg / I;
     const int64_t base = (int64_t)entry * v.stride + (int64_t)o * (v.I * v.n) + (rg - o * I);
@@ -166,17 +172,18 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
     const int rr = (int)(r - first * rb);
     const int64_t plane = (int64_t)im.rb * 32;
     uint8_t *dst = im.data + ((int64_t)entry * blocks + first) * S * kDigits * plane + rr * 32 +
-                   ((chunk ^ ((rr >> 2) & 1)) << 4);
+                   (E == 8 ? (chunk ^ ((rr >> 2) & 1)) << 4 : (((chunk >> 1) ^ ((rr >> 2) & 1)) << 4) + ((chunk & 1) << 3));
     pdl_wait();
-    unsigned long long x[8], mx = 0;
+    unsigned long long x[E], mx = 0;
     load_entries(v, base, row_ok, min(sub, S - 1), chunk, spc, x);
     mx = largest(mx, x);
     for (int s = sub + WS; s < S; s += WS) {
-        unsigned long long w[8];
+        unsigned long long w[E];
         load_entries(v, base, row_ok, s, chunk, spc, w);
         mx = largest(mx, w);
     }
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    if constexpr (E == 4) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
     if (chunk == 0) smax[warp][row] = mx;
     __syncthreads();
     pdl_trigger();
@@ -186,7 +193,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
     if (sub == 0 && chunk == 0 && row_ok) im.exps[(int64_t)entry * blocks * rb + r] = e;
     if (sub < S) store_digits(x, e, dst + (int64_t)sub * kDigits * plane, plane);
     for (int s = sub + WS; s < S; s += WS) {
-        unsigned long long w[8];
+        unsigned long long w[E];
         load_entries(v, base, row_ok, s, chunk, spc, w);
         store_digits(w, e, dst + (int64_t)s * kDigits * plane, plane);
     }
@@ -195,8 +202,8 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
 // ---------------------------------------------------------------------------
 // The digit products.  One persistent CTA per SM, in clusters of two that work
 // on adjacent column tiles of the same rows; warp 0 copies digit blocks (one
-// contiguous block per operand and slab) into a four-stage ring, one thread of
-// warp 1 issues the MMAs, two warpgroups drain.  A tile is 128 rows by `nt` <=
+// contiguous block per operand and slab) into a four-stage ring, warp 1 issues
+// the MMAs, four warpgroups drain.  A tile is 128 rows by `nt` <=
 // 64 columns: eight classes of 64 FP32 columns are all 512 columns of tensor
 // memory.  Such a tile reads 48 KiB of digits per 1152 clocks of MMAs, 42 bytes
 // per clock and SM where the L2 gives about 24, so each CTA of a pair loads half
@@ -646,33 +653,39 @@ struct FArgs {
 };
 constexpr int kLanes = 4;
 
+// IT: 32-bit indices where the launch allows them (its divisions cost as much as
+// a short contraction)
+template <typename IT>
 __global__ void __launch_bounds__(128) k_fma_products(const __grid_constant__ FArgs a)
 {
-    const int64_t total = a.first[a.count];
+    const IT total = (IT)a.first[a.count];
     const int sub = threadIdx.x % kLanes;
     pdl_trigger();
     pdl_wait();
     // whole warps stay in the loop for the shuffles
-    for (int64_t e0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32 * (32 / kLanes); e0 < total;
-         e0 += (int64_t)gridDim.x * blockDim.x / kLanes) {
-        const int64_t e = min(e0 + threadIdx.x % 32 / kLanes, total - 1);
+    for (IT e0 = ((IT)blockIdx.x * blockDim.x + threadIdx.x) / 32 * (32 / kLanes); e0 < total;
+         e0 += (IT)gridDim.x * blockDim.x / kLanes) {
+        const IT e = min(e0 + (IT)(threadIdx.x % 32 / kLanes), total - 1);
         int q = 0;
-        while (q + 1 < a.count && e >= a.first[q + 1]) ++q;
+        while (q + 1 < a.count && e >= (IT)a.first[q + 1]) ++q;
         const GProd &p = a.p[q];
-        const int64_t size = p.rows * p.cols, entry = (e - a.first[q]) / size, t = e - a.first[q] - entry * size;
+        const IT I = (IT)p.I, cols = (IT)p.cols, IB = (IT)p.IB;
+        const IT size = (IT)p.rows * cols, entry = (e - (IT)a.first[q]) / size, t = e - (IT)a.first[q] - entry * size;
         // neighbouring lanes: neighbouring outputs in memory
-        int64_t r;
-        int i;
-        if (p.I == 1) {
-            r = t / p.cols;
-            i = (int)(t - r * p.cols);
+        IT o, x0, i;
+        if (I == 1) {
+            o = t / cols;
+            i = t - o * cols;
+            x0 = 0;
         } else {
-            const int64_t o = t / (p.I * p.cols), w = t - o * (p.I * p.cols);
-            i = (int)(w / p.I);
-            r = o * p.I + (w - i * p.I);
+            o = t / (I * cols);
+            const IT w = t - o * (I * cols);
+            i = w / I;
+            x0 = w - i * I;
         }
-        const int64_t xa = entry * p.sA + (r / p.I) * (p.I * p.n) + r % p.I;
-        const int64_t lb = entry * p.sB + (i / p.IB) * (p.IB * p.n) + i % p.IB;
+        const int64_t xa = (int64_t)entry * p.sA + (int64_t)o * (p.I * p.n) + x0;
+        const IT ob = i / IB;
+        const int64_t lb = (int64_t)entry * p.sB + (int64_t)ob * (p.IB * p.n) + (i - ob * IB);
         double y = 0.0;
         for (int c = 0; c < p.ncat; ++c) {
             const double *x = p.X[c] + xa, *l = p.L[c] + lb;
@@ -693,9 +706,9 @@ __global__ void __launch_bounds__(128) k_fma_products(const __grid_constant__ FA
         }
 #pragma unroll
         for (int w = 1; w < kLanes; w *= 2) y += __shfl_xor_sync(0xffffffffu, y, w);
-        if (sub == 0 && e0 + threadIdx.x % 32 / kLanes < total) {
-            double *o = p.out + entry * p.sOut + t;
-            *o = p.accumulate ? __dadd_rn(*o, y) : y;
+        if (sub == 0 && e0 + (IT)(threadIdx.x % 32 / kLanes) < total) {
+            double *z = p.out + (int64_t)entry * p.sOut + t;
+            *z = p.accumulate ? __dadd_rn(*z, y) : y;
         }
     }
 }
@@ -732,27 +745,42 @@ GProd to_gprod(const Product &s)
 }
 }  // namespace
 
-int tile_cols(int64_t rows, int cols, int products)
+int tile_cols(int64_t rows, int cols, int products, int slabs)
 {
-    // an even number of tiles, so that no CTA of a pair idles; narrower tiles
-    // while the launch would leave SMs without one
+    // the width whose waves take the least: clocks per tile measured in the kernel,
+    // at 64 columns 1365 per slab (smem and L2 bound) and 6500 for the drain, at 48
+    // 1111 and 5100, at 32 900 and 3800, at 16 estimated; a pair of CTAs takes two
+    // tiles, the second idle where the tiles are odd
+    static const struct {
+        int nt, slab, tile;
+    } kCost[] = {{64, 1365, 6500}, {48, 1111, 5100}, {32, 900, 3800}, {16, 750, 2800}};
     const int64_t mt = (rows + kRowBlock - 1) / kRowBlock * products;
-    int nt = 16;
-    for (int w = 64; w >= 16; w -= 16) {
-        const int nb = (cols + w * kPair - 1) / (w * kPair) * kPair;
-        nt = std::min(w, ((cols + nb - 1) / nb + 15) / 16 * 16);
-        if (mt * ((cols + nt - 1) / nt) >= kSms) break;
+    int best = 16;
+    double least = 0.0;
+    for (const auto &c : kCost) {
+        const int64_t pairs = mt * (((cols + c.nt - 1) / c.nt + kPair - 1) / kPair), slots = kSms / kPair;
+        const double t = (double)((pairs + slots - 1) / slots) * ((double)slabs * c.slab + c.tile);
+        if (least == 0.0 || t < least) {
+            least = t;
+            best = c.nt;
+        }
     }
-    return nt;
+    // the same number of tiles, evenly wide
+    const int nb = (cols + best - 1) / best;
+    return std::min(best, ((cols + nb - 1) / nb + 15) / 16 * 16);
 }
 
 bool use_digits(int64_t rows, int n, int count)
 {
     const int most = rows * n > ((int64_t)1 << 20) ? 4096 : 1024;
-    return n >= 12 && n <= most && rows >= 16 && (double)rows * n * n * count > 1.5e6;
+    // 1.5e6 FMAs take the FP64 pipe about as long as the two launches of a digit
+    // product take at least (7 and 9 + 5 us); row tiles of 128 that are mostly padding
+    // move the line (twelve products of 64 x 64: 9 against 14 us)
+    return n >= 12 && n <= most && rows >= 16 && (double)rows * n * n * count > 1.5e6 * std::max(1.0, 160.0 / rows);
 }
 
-void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
+template <int E>
+static void split_as(const View *v, const Image *im, int count, cudaStream_t st)
 {
     SplitArgs a{};
     a.count = count;
@@ -764,13 +792,24 @@ void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
         a.v[q] = v[q];
         a.im[q] = im[q];
         const int G = warps / split_warps(im[q].slabs);
-        const int64_t groups = (im[q].rows + kRowGroup - 1) / kRowGroup * v[q].batch;
+        const int64_t groups = (im[q].rows + 2 * E - 1) / (2 * E) * v[q].batch;
         a.first[q + 1] = a.first[q] + (int)((groups + G - 1) / G);
-        wide = wide || (v[q].r0 + im[q].rows + kRowGroup * 32) * std::max(1, v[q].batch) > INT32_MAX || v[q].I > INT32_MAX;
+        wide = wide || (v[q].r0 + im[q].rows + 2 * E * 32) * std::max(1, v[q].batch) > INT32_MAX || v[q].I > INT32_MAX;
     }
     const dim3 grid(a.first[count]), block(warps * 32);
-    if (wide) pdl_launch(k_digits<int64_t>, grid, block, 0, st, 1, a);
-    else pdl_launch(k_digits<int>, grid, block, 0, st, 1, a);
+    if (wide) pdl_launch(k_digits<int64_t, E>, grid, block, 0, st, 1, a);
+    else pdl_launch(k_digits<int, E>, grid, block, 0, st, 1, a);
+}
+
+void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
+{
+    // Where eight entries per thread leave half of the SMs' warps empty, four: a
+    // chain of dependent work half as long (301 x 150, 150 x 301 and their matrices
+    // 8.4 -> 7.0 us; eighteen tensors of 96^3, with warps for all SMs, 45 -> 49 us).
+    int64_t threads = 0;
+    for (int q = 0; q < count; ++q) threads += im[q].rows * v[q].batch * im[q].slabs * (kSlab / 8);
+    if (threads < (int64_t)kSms * 512) split_as<4>(v, im, count, st);
+    else split_as<8>(v, im, count, st);
 }
 
 void launch_products(const Product *s, int count, DevStatus *status, long long wait_limit, cudaStream_t st)
@@ -805,7 +844,10 @@ void launch_products_fma(const Product *s, int count, cudaStream_t st)
     }
     const int64_t total = a.first[count];
     if (total == 0) return;
-    pdl_launch(k_fma_products, dim3((int)std::min<int64_t>((total * kLanes + 127) / 128, kSms * 16)), dim3(128), 0, st, 1, a);
+    const dim3 grid((int)std::min<int64_t>((total * kLanes + 127) / 128, kSms * 16));
+    // (headroom for the stride past the end and the thread index)
+    if (total < (int64_t)1 << 28) pdl_launch(k_fma_products<int>, grid, dim3(128), 0, st, 1, a);
+    else pdl_launch(k_fma_products<int64_t>, grid, dim3(128), 0, st, 1, a);
 }
 
 View tensor_view(int d, const int64_t *n, int mu, const double *X)
@@ -891,7 +933,7 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
             Product t = q;
             const size_t u0 = used;
             const int n0 = ns;
-            if ((with_b && !place(t.B, tile_cols(t.A.rows, (int)t.B.rows, many), t.ib)) ||
+            if ((with_b && !place(t.B, tile_cols(t.A.rows, (int)t.B.rows, many, slabs_of(t.A.n, t.A.ncat)), t.ib)) ||
                 !place(t.A, kRowBlock, t.ia)) {
                 used = u0;
                 ns = n0;
@@ -927,7 +969,7 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
         if (digits && ps[i].A.batch == 1) {
             Product t = ps[i];
             const size_t per = image_bytes(kRowBlock, kRowBlock, slabs_of(t.A.n, t.A.ncat)) + sizeof(int) * kRowBlock;
-            const bool ok = t.ib.data || place(t.B, tile_cols(t.A.rows, (int)t.B.rows, 1), t.ib);
+            const bool ok = t.ib.data || place(t.B, tile_cols(t.A.rows, (int)t.B.rows, 1, slabs_of(t.A.n, t.A.ncat)), t.ib);
             if (ok && used + per + kAlign <= c.ws_bytes) {
                 const int64_t fit = (int64_t)((c.ws_bytes - used - kAlign) / per) * kRowBlock;
                 const size_t u0 = used;

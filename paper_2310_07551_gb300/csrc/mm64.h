@@ -102,8 +102,8 @@ void tucker_f64(const Context &c, int d, const int64_t *n, const double *X, doub
                 int transpose, double *tmp, cudaStream_t st);
 
 // Columns per tile (a multiple of 16, at most 64) for matrices of `cols`
-// columns, chosen so that `products` products of `rows` rows fill the SMs.
-int tile_cols(int64_t rows, int cols, int products);
+// columns in a launch of `products` products of `rows` rows and `slabs` slabs.
+int tile_cols(int64_t rows, int cols, int products, int slabs);
 
 // Digit images of up to kMaxProd views (one launch).
 void launch_split(const View *v, const Image *im, int count, cudaStream_t st);

@@ -166,7 +166,7 @@ void sums_create(Sums64 &e, const ds_phi_set *s, int64_t N, const std::vector<Su
         for (const Product &p : ps) {
             Image &im = e.images[view_key(p.B)];
             if (im.rb) continue;   // already listed
-            im.rb = mm::tile_cols(p.A.rows, (int)p.B.rows, count);
+            im.rb = mm::tile_cols(p.A.rows, (int)p.B.rows, count, mm::slabs_of(p.B.n, p.B.ncat));
             im.slabs = mm::slabs_of(p.B.n, p.B.ncat);
             im.rows = p.B.rows;
             offs.push_back(bytes);

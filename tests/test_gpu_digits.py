@@ -121,3 +121,18 @@ def test_non_finite_entries(ds, special, where):
     assert np.array_equal(np.isinf(got), inf) and np.array_equal(got[inf] > 0, ref[inf] > 0)
     fin = np.isfinite(ref)
     assert np.allclose(got[fin], ref[fin], rtol=0, atol=64 * 2.0**-52)
+
+
+@pytest.mark.parametrize("n,mode", [(470, 0), (513, 0), (470, 2), (513, 2)])
+def test_long_tensors(ds, n, mode):
+    """tensors whose digit images have eight entries per thread (shorter ones have
+    four), contracted along the first mode and along a strided one; a sample of rows"""
+    rng = np.random.default_rng(n + mode)
+    X, L = (rng.standard_normal((m, n)) * 10.0 ** rng.uniform(-3, 3, (m, n)) * 10.0 ** rng.integers(-40, 40, (m, 1))
+            for m in (11**3, n))
+    T = np.moveaxis(X.reshape(11, 11, 11, n), 3, 3 - mode)
+    Ls = [torch.from_numpy(L if mu == mode else np.eye(11)).cuda() for mu in range(4)]
+    got = ds.tucker(torch.from_numpy(T.copy()).cuda(), Ls).cpu().numpy()
+    got = np.moveaxis(got, 3 - mode, 3).reshape(11**3, n)
+    r = np.r_[0:16, 120:130, 1000:1010, 1315:1331]
+    check(got[r], X[r], L)
