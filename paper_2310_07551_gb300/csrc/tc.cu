@@ -7,11 +7,12 @@
 // with FP32 accumulation in tensor memory; the dropped products have weight
 // <= 2^-24 relative to the leading one.
 //
-// Kernel structure (one persistent CTA per SM, 192 threads):
-//   warp 0      TMA producer: BF16 plane tiles of both operands into a
-//               3-stage shared-memory ring (cp.async.bulk.tensor, swizzled)
-//   warp 1      tensor-memory allocator and single-thread tcgen05.mma issuer
-//   warps 2-5   epilogue: tcgen05.ld of the FP32 accumulator, scaling and
+// Kernel structure (one persistent CTA per SM, 320 threads):
+//   warp 0      TMA producer: BF16 plane tiles of the tensor (cp.async.bulk.tensor,
+//               swizzled) and phi-matrix tile images (cp.async.bulk) into a
+//               shared-memory ring
+//   warp 1      tensor-memory allocator and tcgen05.mma issuer (elected thread)
+//   warps 2-9   epilogue: tcgen05.ld of the FP32 accumulator, scaling and
 //               the store of BF16 planes or FP32 values
 // Two 128x256 FP32 accumulators (512 TMEM columns) let the epilogue of one
 // tile overlap the MMAs of the next.  Every mbarrier wait is bounded; a wait
@@ -69,6 +70,25 @@ struct TileCfg {
     static constexpr uint32_t SPILL_BYTES = NP == 4 ? 32u * 256u * 4u : 0u;
     static constexpr uint32_t SMEM_BYTES = SPILL_OFF + SPILL_BYTES + 1024;
 };
+// A phi-matrix is stored as images of its shared-memory tiles: [K chunk of 32]
+// [row block of 128][plane], each an 8 KiB tile of 64-byte rows in the 64-byte
+// swizzle, zero padded.  The planes of a tile then arrive in one contiguous bulk
+// copy (three pairs for 256 columns).  A tensor-map copy costs by box row, not by
+// byte (32-byte rows, half as long, took the FX mode-1 launch of 256^3 from 1069 to
+// 1399 us).  As images instead of 64-byte-row boxes: that launch 1069 -> 1007 us, its
+// split-BF16 launches 231 -> 224 us; FX launches along other modes, whose tensor boxes
+// have 128-byte rows, are as fast either way.
+__host__ __device__ inline int phi_row_blocks(int64_t n) { return (int)((n + 255) / 256 * 2); }
+__host__ __device__ inline int64_t phi_elems(int64_t n, int planes)
+{
+    return (n + 31) / 32 * phi_row_blocks(n) * planes * 4096;
+}
+// entry (i, j) of plane 0; plane p lies p 4096 entries on
+__device__ __forceinline__ int64_t phi_offset(int n, int planes, int i, int j)
+{
+    return ((int64_t)(j >> 5) * phi_row_blocks(n) + (i >> 7)) * planes * 4096 + (i & 127) * 32 +
+           ((((j >> 3) & 3) ^ ((i >> 1) & 3)) << 3) + (j & 7);
+}
 constexpr long long kTimeoutCycles = 4000000000LL;   // ~2 s at 2 GHz
 
 // UMMA shared-memory descriptor layout types
@@ -138,8 +158,9 @@ struct ModelF {
 };
 
 struct alignas(128) TcArgs {
-    CUtensorMap tmA;
-    CUtensorMap tmB;
+    CUtensorMap tmX;          // the tensor planes
+    const bf16 *phi;          // phi-matrix images [S T] (phi_offset)
+    int phi_blocks;           // their row blocks
     int S, T, xs_stride, xs_div, n;
     int mtiles, ntiles, kchunks, out_kind;
     // tile order.  Mode-1 launches: 0 row tiles fastest, then stacks, then
@@ -1132,8 +1153,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             while (ok && itr.next()) {
                 const TcArgs &a = GROUPED ? *itr.a : a0;   // ungrouped: the kernel parameter itself
                 if (GROUPED && itr.a != seen) {
-                    tmap_acquire(&a.tmA);
-                    tmap_acquire(&a.tmB);
+                    tmap_acquire(&a.tmX);
                     seen = itr.a;
                 }
                 int part;
@@ -1149,23 +1169,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                         mbar_expect_tx(FULL(stage), STAGE_BYTES);
                         const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + STAGE_A;
                         const int xc = (tc.s / a.xs_div) * a.xs_stride + tt, pc = tc.s * a.T + tt;
+                        const bf16 *img = a.phi + ((int64_t)(pc * a.kchunks + kc) * a.phi_blocks +
+                                                   (MODE1 ? tc.mt : tc.nt * (BN / BM))) * (NP * 4096);
                         if (MODE1) {
+                            ptx::bulk_load(sA, img, STAGE_A, FULL(stage));
 #pragma unroll
                             for (int p = 0; p < NP; ++p)
-                                tma_load_4d(sA + p * A_PLANE, &a.tmA, FULL(stage), kc * BK, tc.mt * BM, p, pc);
-#pragma unroll
-                            for (int p = 0; p < NP; ++p)
-                                tma_load_4d(sB + p * B_PLANE, &a.tmB, FULL(stage), kc * BK, tc.nt * BN, p, xc);
+                                tma_load_4d(sB + p * B_PLANE, &a.tmX, FULL(stage), kc * BK, tc.nt * BN, p, xc);
                         } else {
+                            if (BN == BM) {
+                                ptx::bulk_load(sB, img, NP * B_PLANE, FULL(stage));
+                            } else {
+#pragma unroll
+                                for (int p = 0; p < NP; ++p)
+#pragma unroll
+                                    for (int h = 0; h < BN / BM; ++h)
+                                        ptx::bulk_load(sB + p * B_PLANE + h * A_PLANE, img + (h * NP + p) * 4096, A_PLANE,
+                                                       FULL(stage));
+                            }
 #pragma unroll
                             for (int p = 0; p < NP; ++p)
 #pragma unroll
                                 for (int h = 0; h < 2; ++h)
-                                    tma_load_5d(sA + p * A_PLANE + h * (A_PLANE / 2), &a.tmA, FULL(stage),
+                                    tma_load_5d(sA + p * A_PLANE + h * (A_PLANE / 2), &a.tmX, FULL(stage),
                                                 tc.mt * BM + h * 64, kc * BK, (int)tc.o, p, xc);
-#pragma unroll
-                            for (int p = 0; p < NP; ++p)
-                                tma_load_4d(sB + p * B_PLANE, &a.tmB, FULL(stage), kc * BK, tc.nt * BN, p, pc);
                         }
                     }
                     __syncwarp();
@@ -2833,18 +2860,17 @@ __global__ void k_stage_group(const StageArgs *__restrict__ tab, const int64_t *
     }
 }
 
-// dense column-major FP64 matrix (optionally transposed, scaled) -> BF16
-// planes [plane][i][j] with leading dimension ldp (zero padded)
-__global__ void k_split_matrix(int n, int ldp, const double *__restrict__ L, int transpose, double scale,
-                               bf16 *__restrict__ out)
+// dense column-major FP64 matrix (optionally transposed, scaled) -> BF16 image
+__global__ void k_split_matrix(int n, const double *__restrict__ L, int transpose, double scale, bf16 *__restrict__ out)
 {
-    const int64_t plane = (int64_t)n * ldp;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < plane;
+    const int cols = (n + 31) / 32 * 32;
+    const int64_t total = (int64_t)phi_row_blocks(n) * 128 * cols;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / ldp), j = (int)(e % ldp);
+        const int i = (int)(e / cols), j = (int)(e % cols);
         double x = 0.0;
-        if (j < n) x = scale * (transpose ? L[j + (int64_t)n * i] : L[i + (int64_t)n * j]);
-        store_planes(out, plane, e, x);
+        if (i < n && j < n) x = scale * (transpose ? L[j + (int64_t)n * i] : L[i + (int64_t)n * j]);
+        store_planes(out, 4096, phi_offset(n, 3, i, j), x);
     }
 }
 
@@ -2886,8 +2912,8 @@ __global__ void k_fx_rescale_group(FxScales *const *__restrict__ tab, int count)
 // FX planes of phi-matrices, one block per output row i of stack s: the row
 // of every term t < T (matrix src[s T + t], column-major n x n, times
 // scale[s T + t]) shares one exponent sigma = ceil(log2 max_{t,j} |.|) - 11;
-// pscale[s n + i] = 2^sigma and planes [pc][4][n][ldp] (zero padded) hold
-// the FX split of each entry times 2^-sigma.
+// pscale[s n + i] = 2^sigma and the images [pc] hold the FX split of each entry
+// times 2^-sigma (blocks of rows i >= n: their zeros).
 struct FxMatJob {
     const double *src;
     double scale;
@@ -2897,7 +2923,7 @@ __device__ __forceinline__ double fx_job_at(const FxMatJob &J, int n, int i, int
 {
     return J.scale * (J.transpose ? J.src[j + (int64_t)n * i] : J.src[i + (int64_t)n * j]);
 }
-__global__ void k_split_matrix_fx(int n, int ldp, int T, const FxMatJob *__restrict__ jobs, __half *__restrict__ out,
+__global__ void k_split_matrix_fx(int n, int T, const FxMatJob *__restrict__ jobs, __half *__restrict__ out,
                                   float *__restrict__ pscale)
 {
     const int i = blockIdx.x, s = blockIdx.y;
@@ -2905,7 +2931,7 @@ __global__ void k_split_matrix_fx(int n, int ldp, int T, const FxMatJob *__restr
     double mx = 0.0;
     for (int t = 0; t < T; ++t) {
         const FxMatJob J = jobs[s * T + t];
-        for (int j = threadIdx.x; j < n; j += blockDim.x) mx = fmax(mx, fabs(fx_job_at(J, n, i, j)));
+        for (int j = threadIdx.x; j < n && i < n; j += blockDim.x) mx = fmax(mx, fabs(fx_job_at(J, n, i, j)));
     }
     red[threadIdx.x] = mx;
     __syncthreads();
@@ -2920,18 +2946,18 @@ __global__ void k_split_matrix_fx(int n, int ldp, int T, const FxMatJob *__restr
         const double fr = frexp(mx, &e);   // mx = fr 2^e, fr in [0.5, 1)
         sig = (fr == 0.5 ? e - 1 : e) - 11;
     }
-    if (threadIdx.x == 0) pscale[(int64_t)s * n + i] = ldexpf(1.0f, sig);
+    if (threadIdx.x == 0 && i < n) pscale[(int64_t)s * n + i] = ldexpf(1.0f, sig);
     const double inv = ldexp(1.0, -sig);
-    const int64_t plane = (int64_t)n * ldp;
+    const int cols = (n + 31) / 32 * 32;
     for (int t = 0; t < T; ++t) {
         const FxMatJob J = jobs[s * T + t];
-        __half *o = out + (int64_t)(s * T + t) * 4 * plane + (int64_t)i * ldp;
-        for (int j = threadIdx.x; j < ldp; j += blockDim.x) {
+        for (int j = threadIdx.x; j < cols; j += blockDim.x) {
+            __half *o = out + (s * T + t) * phi_elems(n, 4) + phi_offset(n, 4, i, j);
             __half q[4];
-            if (j < n) fx_split_d(fx_job_at(J, n, i, j) * inv, q);
+            if (i < n && j < n) fx_split_d(fx_job_at(J, n, i, j) * inv, q);
             else q[0] = q[1] = q[2] = q[3] = __float2half(0.0f);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) o[j + k * plane] = q[k];
+            for (int k = 0; k < 4; ++k) o[k * 4096] = q[k];
         }
     }
 }
@@ -3165,10 +3191,10 @@ static int num_sms()
 static int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // Describe Y_s = sum_t X_{(s / xs_div) xs + t} x_mu P_{s T + t} for s < S, t < T.
-//   X: BF16 planes [xcombos][3][N];  P: BF16 planes [pcombos][3][n_mu][ldp]
+//   X: BF16 planes [xcombos][3][N];  P: images [S T]
 //   out: planes [S][3][N] (out_kind 0) or FP32 [S][N] (out_kind 1)
 static ds_status describe(ModeLaunch &L, int d, const int64_t *n, int mu, const bf16 *X, int xcombos,
-                          const bf16 *P, int pcombos, int ldp, int S, int T, int xs_stride, int xs_div,
+                          const bf16 *P, int S, int T, int xs_stride, int xs_div,
                           void *out, int out_kind, float alpha, DevStatus *status, int bn = 256,
                           bool dual = false, bool fx = false)
 {
@@ -3196,14 +3222,10 @@ static ds_status describe(ModeLaunch &L, int d, const int64_t *n, int mu, const 
     if (mu == 0) {
         L.mode1 = true;
         const int64_t R = O;
-        uint64_t pd[4] = {(uint64_t)nm, (uint64_t)nm, NPL, (uint64_t)pcombos};
-        uint64_t ps[3] = {ldp * e2, nm * ldp * e2, NPL * nm * ldp * e2};
-        uint32_t pb[4] = {BK, BM, 1, 1};
         uint64_t xd[4] = {(uint64_t)nm, (uint64_t)R, NPL, (uint64_t)xcombos};
         uint64_t xs[3] = {nm * e2, N * e2, NPL * N * e2};
         uint32_t xb[4] = {BK, (uint32_t)BN, 1, 1};
-        ok = make_map(&a.tmA, P, 4, pd, ps, pb, CU_TENSOR_MAP_SWIZZLE_64B) &&
-             make_map(&a.tmB, X, 4, xd, xs, xb, CU_TENSOR_MAP_SWIZZLE_64B);
+        ok = make_map(&a.tmX, X, 4, xd, xs, xb, CU_TENSOR_MAP_SWIZZLE_64B);
         a.mtiles = (int)cdiv(nm, BM);
         a.ntiles = (int)cdiv(R, BN);
         a.num_tiles = (int64_t)a.mtiles * S * a.ntiles;
@@ -3214,11 +3236,7 @@ static ds_status describe(ModeLaunch &L, int d, const int64_t *n, int mu, const 
         uint64_t xd[5] = {(uint64_t)I, (uint64_t)nm, (uint64_t)O, NPL, (uint64_t)xcombos};
         uint64_t xs[4] = {I * e2, I * nm * e2, N * e2, NPL * N * e2};
         uint32_t xb[5] = {64, BK, 1, 1, 1};
-        uint64_t pd[4] = {(uint64_t)nm, (uint64_t)nm, NPL, (uint64_t)pcombos};
-        uint64_t ps[3] = {ldp * e2, nm * ldp * e2, NPL * nm * ldp * e2};
-        uint32_t pb[4] = {BK, (uint32_t)BN, 1, 1};
-        ok = make_map(&a.tmA, X, 5, xd, xs, xb, CU_TENSOR_MAP_SWIZZLE_128B) &&
-             make_map(&a.tmB, P, 4, pd, ps, pb, CU_TENSOR_MAP_SWIZZLE_64B);
+        ok = make_map(&a.tmX, X, 5, xd, xs, xb, CU_TENSOR_MAP_SWIZZLE_128B);
         a.mtiles = (int)cdiv(I, BM);
         a.ntiles = (int)cdiv(nm, BN);
         a.num_tiles = (int64_t)S * O * a.mtiles * a.ntiles;
@@ -3232,6 +3250,8 @@ static ds_status describe(ModeLaunch &L, int d, const int64_t *n, int mu, const 
     a.xs_div = xs_div;
     a.n = (int)nm;
     a.kchunks = (int)cdiv(nm, BK);
+    a.phi = P;
+    a.phi_blocks = phi_row_blocks(nm);
     a.out_kind = out_kind;
     a.out = out;
     a.out_ps = N;
@@ -3725,7 +3745,6 @@ static int autotune_launch(ModeLaunch *c, int ncand, float *ws, float *skws, int
     return best;
 }
 
-static int round8(int64_t n) { return (int)((n + 7) / 8 * 8); }
 
 static ds_status check_shape(int d, const int64_t *n)
 {
@@ -3985,7 +4004,7 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
     //            last mode: 3k combos with w_q tau eta^{(1)}_i folded in
     //   group D2 (slot 2), D3 (slot 4): k combos per mode; last mode folds w eta^{(2)}
     const int Fslots[3] = {0, 1, 3};
-    // phi planes, per (group, mode): [c][combo][plane][n_mu][ldp]
+    // phi images, per (group, mode): [c][combo]
     //   group F: 3k combos (stage q' in {slot 0, 1, 3}, term i); the last mode's
     //            matrices carry w_q tau eta^{(1)}_i
     //   group D2 (slot 2), D3 (slot 4): k combos; last mode carries w eta^{(2)}
@@ -3999,7 +4018,7 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
         for (int mu = 0; mu < d; ++mu) {
             goff[g][mu] = total;
             const int combos = g == 0 ? 3 * k : k;
-            total += (int64_t)2 * combos * (fxg(g) ? 4 : 3) * mp->n[mu] * round8(mp->n[mu]);
+            total += 2 * combos * phi_elems(mp->n[mu], fxg(g) ? 4 : 3);
         }
     auto cleanup = [&](ds_status s, const char *msg) {
         mixed_plan_destroy(mp);
@@ -4048,7 +4067,6 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
             if (fxg(g)) {
                 // FX planes of the group: per stack s one row scale over its T terms
                 const int64_t nm = mp->n[mu];
-                const int ldp = round8(nm);
                 const bool last = (mu == d - 1);
                 const int combos = g == 0 ? 3 * k : k, T = last ? k : 1;
                 std::vector<FxMatJob> jobs(2 * combos);
@@ -4060,14 +4078,13 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
                                                  last ? kSlotW[slot] * tau * co.eta[i] : 1.0, 0};
                     }
                 cudaMemcpy(mp->fx_jobs, jobs.data(), sizeof(FxMatJob) * jobs.size(), cudaMemcpyHostToDevice);
-                k_split_matrix_fx<<<dim3((unsigned)nm, (unsigned)(2 * combos / T)), 256>>>(
-                    (int)nm, ldp, T, mp->fx_jobs, (__half *)(mp->Pp + goff[g][mu]), mp->pscale + mp->pscale_off[g][mu]);
+                k_split_matrix_fx<<<dim3((unsigned)phi_row_blocks(nm) * 128, (unsigned)(2 * combos / T)), 256>>>(
+                    (int)nm, T, mp->fx_jobs, (__half *)(mp->Pp + goff[g][mu]), mp->pscale + mp->pscale_off[g][mu]);
                 cudaDeviceSynchronize();   // the job table is reused for the next mode
                 continue;
             }
             const int64_t nm = mp->n[mu];
-            const int ldp = round8(nm);
-            const int64_t psz = 3 * nm * ldp;
+            const int64_t psz = phi_elems(nm, 3);
             const bool last = (mu == d - 1);
             const int combos = g == 0 ? 3 * k : k;
             for (int c = 0; c < 2; ++c)
@@ -4079,7 +4096,7 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
                     const double scale = last ? kSlotW[slot] * tau * co.eta[i] : 1.0;
                     const double *src = set->P_dev + set->P_off[c][slot][i][mu];
                     bf16 *dst = mp->Pp + goff[g][mu] + (int64_t)(c * combos + cb) * psz;
-                    k_split_matrix<<<pw_grid(nm * ldp), 256>>>((int)nm, ldp, src, 0, scale, dst);
+                    k_split_matrix<<<pw_grid(psz / 3), 256>>>((int)nm, src, 0, scale, dst);
                 }
         }
     // launch descriptors: stack index s = c * S0 + combo
@@ -4089,7 +4106,6 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
         bf16 *Zs[2] = {mp->Z1, mp->Z2};
         for (int mu = 0; mu < d; ++mu) {
             const bf16 *P = mp->Pp + goff[g][mu];
-            const int ldp = round8(mp->n[mu]);
             const bool last = (mu == d - 1);
             const bf16 *X = mu == 0 ? Xin : Zs[(mu - 1) % 2];
             const int xcombos = mu == 0 ? 2 : 2 * S0;
@@ -4110,7 +4126,7 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
             for (int w = 0; w < 2; ++w) {
                 ModeLaunch &Cw = mp->C[g][mu][w];
                 // compensated plans have one candidate: 128-column tiles, two accumulators
-                r = describe(Cw, d, mp->n, mu, X, xcombos, P, 2 * S0, ldp, S, T, xs, xdiv, out, kind, 1.0f,
+                r = describe(Cw, d, mp->n, mu, X, xcombos, P, S, T, xs, xdiv, out, kind, 1.0f,
                              status, (w || compensated) ? 128 : 256, compensated, fxg(g));
                 if (r != DS_OK) { mixed_plan_destroy(mp); return r; }
                 if (fxg(g)) {
@@ -5033,7 +5049,7 @@ ds_status tucker_mixed(const ds_grid *grid, const double *X, double *Y, const do
     int64_t N = 1, pmax = 0;
     for (int q = 0; q < d; ++q) {
         N *= grid->n[q];
-        pmax += 3 * grid->n[q] * round8(grid->n[q]);
+        pmax += phi_elems(grid->n[q], 3);
     }
     char *ws = nullptr;
     const size_t bytes = sizeof(bf16) * (6 * N + pmax) + sizeof(float) * N + 256;
@@ -5046,17 +5062,17 @@ ds_status tucker_mixed(const ds_grid *grid, const double *X, double *Y, const do
     bf16 *bufs[2] = {A1, A0};
     for (int mu = 0; mu < d; ++mu) {
         const int64_t nm = grid->n[mu];
-        const int ldp = round8(nm);
-        k_split_matrix<<<pw_grid(nm * ldp), 256, 0, st>>>((int)nm, ldp, L[mu], transpose, 1.0, pcur);
+        const int64_t psz = phi_elems(nm, 3);
+        k_split_matrix<<<pw_grid(psz / 3), 256, 0, st>>>((int)nm, L[mu], transpose, 1.0, pcur);
         const bool last = (mu == d - 1);
         void *out = last ? (void *)outf : (void *)bufs[mu % 2];
         ModeLaunch ml;
-        r = describe(ml, d, grid->n, mu, in, 1, pcur, 1, ldp, 1, 1, 0, 1, out, last ? 1 : 0, 1.0f, status,
+        r = describe(ml, d, grid->n, mu, in, 1, pcur, 1, 1, 0, 1, out, last ? 1 : 0, 1.0f, status,
                      compensated ? 128 : 256, compensated);
         if (r != DS_OK) { cudaFreeAsync(ws, st); return r; }
         launch(ml, st);
         in = bufs[mu % 2];
-        pcur += 3 * nm * ldp;
+        pcur += psz;
     }
     k_f32_to_f64<<<pw_grid(N), 256, 0, st>>>(N, outf, Y);
     cudaFreeAsync(ws, st);
@@ -5086,7 +5102,7 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
     int64_t N = 1, pmax = 0, psmax = 0;
     for (int q = 0; q < d; ++q) {
         N *= grid->n[q];
-        pmax += 4 * grid->n[q] * round8(grid->n[q]);
+        pmax += phi_elems(grid->n[q], 4);
         psmax += grid->n[q];
     }
     char *ws = nullptr;
@@ -5112,12 +5128,11 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
     __half *bufs[2] = {A1, A0};
     for (int mu = 0; mu < d; ++mu) {
         const int64_t nm = grid->n[mu];
-        const int ldp = round8(nm);
-        k_split_matrix_fx<<<dim3((unsigned)nm, 1), 256, 0, st>>>((int)nm, ldp, 1, jobs + mu, pcur, pscur);
+        k_split_matrix_fx<<<dim3((unsigned)phi_row_blocks(nm) * 128, 1), 256, 0, st>>>((int)nm, 1, jobs + mu, pcur, pscur);
         const bool last = (mu == d - 1);
         void *out = last ? (void *)Y : (void *)bufs[mu % 2];
         ModeLaunch ml;
-        r = describe(ml, d, grid->n, mu, (const bf16 *)in, 1, (const bf16 *)pcur, 1, ldp, 1, 1, 0, 1, out,
+        r = describe(ml, d, grid->n, mu, (const bf16 *)in, 1, (const bf16 *)pcur, 1, 1, 0, 1, out,
                      last ? 2 : 0, 1.0f, status, 128, false, true);
         if (r != DS_OK) { cudaFreeAsync(ws, st); return r; }
         ml.args.fxs = fxs;
@@ -5134,7 +5149,7 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
         }
         launch(ml, st);
         in = bufs[mu % 2];
-        pcur += 4 * nm * ldp;
+        pcur += phi_elems(nm, 4);
         pscur += nm;
     }
     DS_CUDA_TRY(cudaStreamSynchronize(st));
