@@ -54,7 +54,10 @@ typedef enum {
 } ds_status;
 
 /* Arithmetic of the mu-mode contractions.
- *   DS_PREC_F64    : FP64 everywhere (FP64 FMA pipe).
+ *   DS_PREC_F64    : FP64 everywhere.  Large contractions are sums of exact
+ *                    products of 8-bit digits on the tensor cores (operands
+ *                    as 62-bit fixed point per fibre, the sum rounded to
+ *                    FP64 once), small ones FP64 FMA chains.
  *   DS_PREC_F32    : FP32 mode products on the CUDA cores (FP32 FMA, FP32
  *                    intermediates and stage sums), FP64 state -- the
  *                    design of the paper's single-precision GPU runs.
@@ -217,8 +220,10 @@ ds_status ds_phi_get_ex(const ds_phi_set *set, int c, int slot, int term, int mu
  *      F16X10 the intermediates are FX parts scaled by their exact largest
  *      magnitude and the last product is formed in double-float).  Y is
  *      written in FP64.
- *   Temporary device memory is allocated per call and released before the
- *   call returns (stream-ordered).
+ *   Temporary device memory comes from a memory pool of the library, stream-
+ *   ordered, and is returned to it before the call returns.  The pool keeps
+ *   at most 1 GiB per device across calls and gives everything back before
+ *   an allocation of the library is refused.
  *   Errors: DS_ERR_INVALID_ARG, DS_ERR_UNSUPPORTED (precision/shape),
  *   DS_ERR_OOM, DS_ERR_CUDA. */
 ds_status ds_tucker(const ds_grid *grid, const double *X, double *Y,
@@ -230,10 +235,11 @@ ds_status ds_tucker(const ds_grid *grid, const double *X, double *Y,
  * that forbid allocation after start-up, plugins whose framework owns the
  * device heap.  The paper has no counterpart; this is a property of the
  * library, not of the method.
- *   It allocates nothing.  Its two intermediate tensors live in one fixed
- *   device array inside the library (16 MiB: two FP64 tensors of up to
- *   1,048,576 points), which every GPU that loads the library holds until
- *   the process exits.  Grids with more than 1,048,576 points are rejected
+ *   It allocates nothing.  Its two intermediate tensors and the digits of
+ *   its contractions live in one fixed device array inside the library (36
+ *   MiB: two FP64 tensors of up to 1,048,576 points and 20 MiB of digits;
+ *   contractions whose digits need more run in blocks of rows), which every
+ *   GPU that loads the library holds until the process exits.  Grids with more than 1,048,576 points are rejected
  *   with DS_ERR_INVALID_ARG; use ds_tucker for them.
  *   The first call on each device looks up the array's device address
  *   (cudaGetSymbolAddress) with that device current and keeps it for the
@@ -313,10 +319,14 @@ ds_status ds_integrate_ckpt(ds_plan *plan, double *U, int64_t nsteps, int64_t ck
  *     A_{c,mu} at s_c = 1; for A = delta_c D, dL/d delta_c = dL/ds_c /
  *     delta_c).  It flows through K (<lam_F, K U>) and through every
  *     phi-matrix: d/ds phi_l(s Z) = phi_{l-1}(Z) - l phi_l(Z) (from the
- *     power series), formed once by ds_phi_setup.  Costs d extra Tucker
- *     operators per Tucker operator of the step.
+ *     power series), formed once by ds_phi_setup.  The tangent of a Tucker
+ *     operator is carried through its modes (the product rule, two products
+ *     per mode), so this costs about two more Tucker operators per Tucker
+ *     operator of the step.
  *   Errors: DS_ERR_INVALID_ARG, DS_ERR_UNSUPPORTED (non-FP64 plan), DS_ERR_OOM
- *   (first call allocates a 24 N-double workspace). */
+ *   (the first call allocates a workspace of 22 N doubles and the
+ *   intermediates, the first with dscale 6 N and theirs: intermediates of as
+ *   many Tucker operators as fit 2 GiB, of one term where memory is short). */
 ds_status ds_step_backward(ds_plan *plan, const double *U, const double *lam, double *lam_n,
                            double *dparams, double *dscale, void *stream);
 
