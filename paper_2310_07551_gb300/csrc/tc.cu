@@ -281,9 +281,9 @@ __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity)
 __device__ __noinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                       DevStatus *st, int site, long long limit = kTimeoutCycles)
 {
-    if (mbar_try(bar, parity)) return true;
-    const long long t0 = clock64();
     const bool short_limit = limit < kTimeoutCycles;
+    if (short_limit ? mbar_test(bar, parity) : mbar_try(bar, parity)) return true;
+    const long long t0 = clock64();
     uint32_t it = 0;
     while (true) {
         if (short_limit ? mbar_test(bar, parity) : mbar_try(bar, parity)) return true;
