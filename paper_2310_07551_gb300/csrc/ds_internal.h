@@ -23,12 +23,12 @@ constexpr int kMaxTerms = 3;
 // is an ordinary one: a replayed graph's own kernel-to-kernel edges are shorter
 // (Schnakenberg 64^2, ten steps: 622 us against 735 with programmatic edges),
 // where a sequence of stream launches gains (FHN 96^3 with adjoint: 11.2 against
-// 11.8 ms).  cluster: CTAs per cluster.
+// 11.8 ms).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>
-cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster, A... args)
+cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
@@ -37,14 +37,11 @@ cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
     cfg.stream = st;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(st, &cap);
-    cudaLaunchAttribute at[2]{};
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = cap == cudaStreamCaptureStatusNone;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = cluster;
-    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = cap == cudaStreamCaptureStatusNone;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 #endif

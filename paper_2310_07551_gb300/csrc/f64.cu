@@ -562,70 +562,70 @@ int launch_rhs_f64(const Stencil *s2, const Model &m, int64_t N, const double *U
 {
     const dim3 grid(grid_for(N, block_for(N))), block(block_for(N));
     // (headroom for the stride past the end)
-    if (N < (int64_t)1 << 30) pdl_launch(k_rhs_f64<int>, grid, block, 0, st, 1, s2[0], s2[1], m, (int)N, U, F);
-    else pdl_launch(k_rhs_f64<int64_t>, grid, block, 0, st, 1, s2[0], s2[1], m, N, U, F);
+    if (N < (int64_t)1 << 30) pdl_launch(k_rhs_f64<int>, grid, block, 0, st, s2[0], s2[1], m, (int)N, U, F);
+    else pdl_launch(k_rhs_f64<int64_t>, grid, block, 0, st, s2[0], s2[1], m, N, U, F);
     return 1;
 }
 
 void launch_kronsum_f64(const Stencil &s, int64_t N, const double *X, double *Y, cudaStream_t st)
 {
-    pdl_launch(k_kronsum_f64<int64_t>, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, s, N, X, Y);
+    pdl_launch(k_kronsum_f64<int64_t>, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, s, N, X, Y);
 }
 
 void launch_stage_diff_f64(const Model &m, int64_t N, const double *U, const double *a, double w1,
                            const double *b, double w2, double *D, cudaStream_t st)
 {
-    pdl_launch(k_stage_diff_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, U, a, w1, b, w2, D);
+    pdl_launch(k_stage_diff_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, m, N, U, a, w1, b, w2, D);
 }
 
 void launch_final_f64(int64_t N, double *U, const double *a, double w1, const double *b,
                       double w2, cudaStream_t st)
 {
-    pdl_launch(k_final_f64, dim3(grid_for(2 * N, block_for(2 * N))), dim3(block_for(2 * N)), 0, st, 1, 2 * N, U, a, w1, b, w2);
+    pdl_launch(k_final_f64, dim3(grid_for(2 * N, block_for(2 * N))), dim3(block_for(2 * N)), 0, st, 2 * N, U, a, w1, b, w2);
 }
 
 void launch_add_g_f64(const Model &m, int64_t N, const double *U, double *F, cudaStream_t st)
 {
-    pdl_launch(k_add_g_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, U, F);
+    pdl_launch(k_add_g_f64, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, m, N, U, F);
 }
 
 void launch_axpy2_f64(int64_t N, const double *U, const double *a, double w1, const double *b, double w2,
                       double *Y, cudaStream_t st)
 {
-    pdl_launch(k_axpy2, dim3(grid_for(2 * N, block_for(2 * N))), dim3(block_for(2 * N)), 0, st, 1, 2 * N, U, a, w1, b, w2, Y);
+    pdl_launch(k_axpy2, dim3(grid_for(2 * N, block_for(2 * N))), dim3(block_for(2 * N)), 0, st, 2 * N, U, a, w1, b, w2, Y);
 }
 void launch_gdiff_f64(const Model &m, int64_t N, const double *U, const double *Us, double *D, cudaStream_t st)
 {
-    pdl_launch(k_gdiff, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, U, Us, D);
+    pdl_launch(k_gdiff, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, m, N, U, Us, D);
 }
 void launch_jacT_f64(const Model &m, int64_t N, const double *Us, const double *lam, double *out,
                      cudaStream_t st)
 {
-    pdl_launch(k_jacT, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, 1, m, N, Us, lam, out);
+    pdl_launch(k_jacT, dim3(grid_for(N, block_for(N))), dim3(block_for(N)), 0, st, m, N, Us, lam, out);
 }
 void launch_kronsumT_f64(const Stencil *s2, int64_t N, const double *X, double *Y, cudaStream_t st)
 {
     const dim3 grid(grid_for(N, block_for(N))), block(block_for(N));
-    if (N < (int64_t)1 << 30) pdl_launch(k_kronsumT<int>, grid, block, 0, st, 1, s2[0], s2[1], (int)N, X, Y);
-    else pdl_launch(k_kronsumT<int64_t>, grid, block, 0, st, 1, s2[0], s2[1], N, X, Y);
+    if (N < (int64_t)1 << 30) pdl_launch(k_kronsumT<int>, grid, block, 0, st, s2[0], s2[1], (int)N, X, Y);
+    else pdl_launch(k_kronsumT<int64_t>, grid, block, 0, st, s2[0], s2[1], N, X, Y);
 }
 void launch_adjoint_final_f64(const Model &m, int64_t N, const double *U, const double *U2,
                               const double *U3, const double *lam, const double *lU3, const double *lU2,
                               const double *KT, const double *lF, const double *lD2, const double *lD3,
                               double *lam_n, double *dp, cudaStream_t st)
 {
-    pdl_launch(k_adjoint_final, dim3(grid_for(N)), dim3(256), 0, st, 1, m, N, U, U2, U3, lam, lU3, lU2, KT, lF, lD2, lD3, lam_n, dp);
+    pdl_launch(k_adjoint_final, dim3(grid_for(N)), dim3(256), 0, st, m, N, U, U2, U3, lam, lU3, lU2, KT, lF, lD2, lD3, lam_n, dp);
 }
 
 void launch_dot_accum_f64(int64_t n, const double *a, const double *b, double w, double *out,
                           cudaStream_t st)
 {
-    pdl_launch(k_dot_accum, dim3(grid_for(n)), dim3(256), 0, st, 1, n, a, b, w, out);
+    pdl_launch(k_dot_accum, dim3(grid_for(n)), dim3(256), 0, st, n, a, b, w, out);
 }
 void launch_dot_kterm_f64(const Model &m, int64_t N, const double *U, const double *F, const double *lF,
                           double *out, cudaStream_t st)
 {
-    pdl_launch(k_dot_kterm, dim3(grid_for(N)), dim3(256), 0, st, 1, m, N, U, F, lF, out);
+    pdl_launch(k_dot_kterm, dim3(grid_for(N)), dim3(256), 0, st, m, N, U, F, lF, out);
 }
 
 void launch_nonfinite_scan(const double *x, int64_t count, int *flag, cudaStream_t st)

@@ -200,14 +200,18 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
 }
 
 // ---------------------------------------------------------------------------
-// The digit products.  One persistent CTA per SM, in clusters of two that work
-// on adjacent column tiles of the same rows; warp 0 copies digit blocks (one
+// The digit products.  One persistent CTA per SM; warp 0 copies digit blocks (one
 // contiguous block per operand and slab) into a four-stage ring, warp 1 issues
 // the MMAs, four warpgroups drain.  A tile is 128 rows by `nt` <=
 // 64 columns: eight classes of 64 FP32 columns are all 512 columns of tensor
 // memory.  Such a tile reads 48 KiB of digits per 1152 clocks of MMAs, 42 bytes
-// per clock and SM where the L2 gives about 24, so each CTA of a pair loads half
-// of their common row block and writes it to both (32 KiB).  The digit planes of
+// per clock and SM, which the L2 does not always give; but sharing the row block
+// between two CTAs costs more than it saves.  Each CTA for itself: 301 x 150 four
+// steps 570 us, complex 150 x 150 305 us, Tucker 201 x 150 x 67 142 us, 96^3 with
+// adjoint 9.98 ms; a cluster of two that loads half of the rows each and multicasts
+// them: 616, 311, 153, 10.06; halves passed on from shared memory to shared memory:
+// 893, 513, 189, 13.1.  (Multicast loads are out of the library in any case: it also
+// runs on several GPUs.)  The digit planes of
 // B lie one after the other in shared memory, so digit p of A meets up to
 // 256 / nt digits of B in one MMA, whose output columns are the adjacent classes.
 // ---------------------------------------------------------------------------
@@ -222,7 +226,7 @@ struct GProd {
 };
 struct GArgs {
     int count;
-    int first[kMaxProd + 1];   // prefix of tile pairs
+    int first[kMaxProd + 1];   // prefix of tiles
     DevStatus *status;
     long long wait_limit;
     GProd p[kMaxProd];
@@ -232,20 +236,21 @@ struct GArgs {
 // drain, of a quarter of the columns each.  The first gives registers up: 128 x
 // 32 + 512 x 112 = 640 x 96, the launch's total; a drain thread holds up to 16
 // outputs as two 64-bit integers.
-constexpr int kThreads = 640, kEpiThreads = 512, kStages = 4, kPair = 2, kEpiCols = 16;
+constexpr int kThreads = 640, kEpiThreads = 512, kStages = 4, kEpiCols = 16;
 constexpr uint32_t kPlaneA = kRowBlock * 32, kStageA = kDigits * kPlaneA, kStageB = kDigits * 64 * 32;
 constexpr uint32_t kStageBytes = kStageA + kStageB;
+constexpr uint32_t kBars = 2 * kStages + 3;
 constexpr uint32_t kSmem = kStages * kStageBytes + 128 + 1024;
+static_assert(8 * kBars + 8 <= 128, "barriers and two words behind the ring");
 
-// pair of tiles u: its product (q: the product of an earlier one), batch entry,
-// row tile and this CTA's column tile (ntiles: none, where the tiles are odd)
-__device__ __forceinline__ const GProd &find_unit(const GArgs &a, int u, int &q, uint32_t rank, int &entry, int &mi, int &ni)
+// tile u: its product (q: the product of an earlier one), batch entry, row tile and
+// column tile
+__device__ __forceinline__ const GProd &find_tile(const GArgs &a, int u, int &q, int &entry, int &mi, int &ni)
 {
     while (q + 1 < a.count && u >= a.first[q + 1]) ++q;
     const GProd &p = a.p[q];
-    const int pairs = (p.ntiles + kPair - 1) / kPair;
-    const int t = u - a.first[q], row = t / pairs;
-    ni = (t - row * pairs) * kPair + (int)rank;
+    const int t = u - a.first[q], row = t / p.ntiles;
+    ni = t - row * p.ntiles;
     entry = row / p.mtiles;
     mi = row - entry * p.mtiles;
     return p;
@@ -420,23 +425,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_addr(smem_raw), base = (raw + 1023u) & ~1023u;
     const uint32_t bars = base + kStages * kStageBytes;
-    uint32_t *tmem_slot = (uint32_t *)(smem_raw + (bars - raw) + 8 * (2 * kStages + 3));
+    uint32_t *tmem_slot = (uint32_t *)(smem_raw + (bars - raw) + 8 * kBars);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
-    const uint32_t FULL = bars, EMPTY = bars + 8 * kStages, TFULL = EMPTY + 8 * kStages, TEMPTY = TFULL + 8, DRAIN = TFULL + 16;
-    const uint32_t rank = cluster_rank();
+    const uint32_t FULL = bars, EMPTY = FULL + 8 * kStages, TFULL = EMPTY + 8 * kStages, TEMPTY = TFULL + 8, DRAIN = TFULL + 16;
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
-    const int units = a.first[a.count];
+    const int tiles = a.first[a.count];
     DevStatus *const status = a.status ? a.status : &g_status;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
-            bar_init(FULL + 8 * s, 1);
-            bar_init(EMPTY + 8 * s, kPair);   // both CTAs' MMAs are done with it
-        }
+        for (int s = 0; s < 2 * kStages; ++s) bar_init(bars + 8 * s, 1);
         bar_init(TFULL, 1);
         bar_init(TEMPTY, kEpiThreads);
         bar_init(DRAIN, 1);
         *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_before();
-    cluster_sync();
+    __syncthreads();
     tc_after();
     const uint32_t tmem = *tmem_slot;
     pdl_trigger();
@@ -458,21 +458,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
             int stage = 0, q = 0, issued = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int u = blockIdx.x / kPair; ok && u < units; u += gridDim.x / kPair) {
+            for (int u = blockIdx.x; ok && u < tiles; u += gridDim.x) {
                 int be, mi, ni;
-                const GProd &p = find_unit(a, u, q, rank, be, mi, ni);
+                const GProd &p = find_tile(a, u, q, be, mi, ni);
                 const uint32_t nb = (uint32_t)p.nt * 32 * kDigits;
                 const int slabs = p.slabs;
-                const uint8_t *A = p.A + ((int64_t)be * p.mtiles + mi) * slabs * kStageA + rank * (kStageA / 2);
-                const uint8_t *B = p.B + ((int64_t)be * p.ntiles + min(ni, p.ntiles - 1)) * slabs * nb;
+                const uint8_t *A = p.A + ((int64_t)be * p.mtiles + mi) * slabs * kStageA;
+                const uint8_t *B = p.B + ((int64_t)be * p.ntiles + ni) * slabs * nb;
                 for (int s = 0; s < slabs; ++s) {
                     ok = __all_sync(0xffffffffu, bar_wait(EMPTY + 8 * stage, phase ^ 1u, abort_flag, status, 11, a.wait_limit));
                     if (!ok) break;
                     if (elect_one()) {
                         const uint32_t sA = base + stage * kStageBytes;
                         bar_expect(FULL + 8 * stage, kStageA + nb);
+                        bulk_load(sA, A, kStageA, FULL + 8 * stage);
                         bulk_load(sA + kStageA, B, nb, FULL + 8 * stage);
-                        bulk_load_pair(sA + rank * (kStageA / 2), A, kStageA / 2, FULL + 8 * stage);
                     }
                     __syncwarp();
                     A += kStageA;
@@ -484,22 +484,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                     }
                 }
             }
-            // every issued copy lands, and the other CTA's last releases arrive,
-            // before the CTA exits
-            for (int s = max(0, issued - kStages); s < issued; ++s) {
-                const uint32_t st = s % kStages, ph = s / kStages & 1;
-                volatile int never = 0;
-                bar_wait(FULL + 8 * st, ph, &never, nullptr, 0, kWaitCycles);
-                if (ok) bar_wait(EMPTY + 8 * st, ph, abort_flag, nullptr, 0, kWaitCycles);
-            }
+            // every issued copy lands before the CTA exits
+            volatile int never = 0;
+            for (int s = max(0, issued - kStages); s < issued; ++s)
+                bar_wait(FULL + 8 * (s % kStages), s / kStages & 1, &never, nullptr, 0, kWaitCycles);
         }
         if (warp == 1) {
             int stage = 0, q = 0;
             uint32_t phase = 0, tphase = 0;
             bool ok = true;
-            for (int u = blockIdx.x / kPair; ok && u < units; u += gridDim.x / kPair) {
+            for (int u = blockIdx.x; ok && u < tiles; u += gridDim.x) {
                 int be, mi, ni;
-                const GProd &p = find_unit(a, u, q, rank, be, mi, ni);
+                const GProd &p = find_tile(a, u, q, be, mi, ni);
                 const int nt = p.nt, slabs = p.slabs;
                 for (int s = 0; s < slabs; ++s) {
                     const bool fresh = s % kChunkSlabs == 0;
@@ -519,7 +515,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                         case 32: issue_slab<32>(tmem, sA, sB, fresh); break;
                         default: issue_slab<16>(tmem, sA, sB, fresh); break;
                         }
-                        mma_commit_pair(EMPTY + 8 * stage);
+                        mma_commit_to(EMPTY + 8 * stage);
                         if (s + 1 == slabs || s % kChunkSlabs == kChunkSlabs - 1) mma_commit_to(TFULL);
                     }
                     __syncwarp();
@@ -543,9 +539,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
         uint32_t tphase = 0;
         bool ok = true;
         int q = 0;
-        for (int u = blockIdx.x / kPair; u < units; u += gridDim.x / kPair) {
+        for (int u = blockIdx.x; u < tiles; u += gridDim.x) {
             int be, mi, ni;
-            const GProd &p = find_unit(a, u, q, rank, be, mi, ni);
+            const GProd &p = find_tile(a, u, q, be, mi, ni);
             const int nt = p.nt, hc = nt / 4;
             const int64_t r = (int64_t)mi * kRowBlock + m;
             const bool row_ok = r < p.rows;
@@ -634,8 +630,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
         }
     }
     tc_before();
-    // the other CTA may still write into this one's shared memory until here
-    cluster_sync();
+    __syncthreads();
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
@@ -749,8 +744,7 @@ int tile_cols(int64_t rows, int cols, int products, int slabs)
 {
     // the width whose waves take the least: clocks per tile measured in the kernel,
     // at 64 columns 1365 per slab (smem and L2 bound) and 6500 for the drain, at 48
-    // 1111 and 5100, at 32 900 and 3800, at 16 estimated; a pair of CTAs takes two
-    // tiles, the second idle where the tiles are odd
+    // 1111 and 5100, at 32 900 and 3800, at 16 estimated
     static const struct {
         int nt, slab, tile;
     } kCost[] = {{64, 1365, 6500}, {48, 1111, 5100}, {32, 900, 3800}, {16, 750, 2800}};
@@ -758,8 +752,8 @@ int tile_cols(int64_t rows, int cols, int products, int slabs)
     int best = 16;
     double least = 0.0;
     for (const auto &c : kCost) {
-        const int64_t pairs = mt * (((cols + c.nt - 1) / c.nt + kPair - 1) / kPair), slots = kSms / kPair;
-        const double t = (double)((pairs + slots - 1) / slots) * ((double)slabs * c.slab + c.tile);
+        const int64_t tiles = mt * ((cols + c.nt - 1) / c.nt);
+        const double t = (double)((tiles + kSms - 1) / kSms) * ((double)slabs * c.slab + c.tile);
         if (least == 0.0 || t < least) {
             least = t;
             best = c.nt;
@@ -797,8 +791,8 @@ static void split_as(const View *v, const Image *im, int count, cudaStream_t st)
         wide = wide || (v[q].r0 + im[q].rows + 2 * E * 32) * std::max(1, v[q].batch) > INT32_MAX || v[q].I > INT32_MAX;
     }
     const dim3 grid(a.first[count]), block(warps * 32);
-    if (wide) pdl_launch(k_digits<int64_t, E>, grid, block, 0, st, 1, a);
-    else pdl_launch(k_digits<int, E>, grid, block, 0, st, 1, a);
+    if (wide) pdl_launch(k_digits<int64_t, E>, grid, block, 0, st, a);
+    else pdl_launch(k_digits<int, E>, grid, block, 0, st, a);
 }
 
 void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
@@ -827,11 +821,11 @@ void launch_products(const Product *s, int count, DevStatus *status, long long w
     a.wait_limit = wait_limit;
     for (int q = 0; q < count; ++q) {
         a.p[q] = to_gprod(s[q]);
-        a.first[q + 1] = a.first[q] + a.p[q].mtiles * ((a.p[q].ntiles + kPair - 1) / kPair) * s[q].A.batch;
+        a.first[q + 1] = a.first[q] + a.p[q].mtiles * a.p[q].ntiles * s[q].A.batch;
     }
-    const int units = a.first[count];
-    if (units == 0) return;
-    pdl_launch(k_digit_products, dim3(kPair * std::min(units, kSms / kPair)), dim3(kThreads), kSmem, st, kPair, a);
+    const int tiles = a.first[count];
+    if (tiles == 0) return;
+    pdl_launch(k_digit_products, dim3(std::min(tiles, kSms)), dim3(kThreads), kSmem, st, a);
 }
 
 void launch_products_fma(const Product *s, int count, cudaStream_t st)
@@ -846,8 +840,8 @@ void launch_products_fma(const Product *s, int count, cudaStream_t st)
     if (total == 0) return;
     const dim3 grid((int)std::min<int64_t>((total * kLanes + 127) / 128, kSms * 16));
     // (headroom for the stride past the end and the thread index)
-    if (total < (int64_t)1 << 28) pdl_launch(k_fma_products<int>, grid, dim3(128), 0, st, 1, a);
-    else pdl_launch(k_fma_products<int64_t>, grid, dim3(128), 0, st, 1, a);
+    if (total < (int64_t)1 << 28) pdl_launch(k_fma_products<int>, grid, dim3(128), 0, st, a);
+    else pdl_launch(k_fma_products<int64_t>, grid, dim3(128), 0, st, a);
 }
 
 View tensor_view(int d, const int64_t *n, int mu, const double *X)

@@ -2587,14 +2587,14 @@ static void launch_rhs_tiled(const StencilF &s0, const StencilF &s1, const Model
     const bool small = N < ((int64_t)1 << 31);
     if (s0.d == 3) {
         if (small)
-            pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, false>, dim3(g), dim3(RT3_X * RT3_Y), 0, st, 1, a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, false>, dim3(g), dim3(RT3_X * RT3_Y), 0, st, a, nullptr, nullptr, 0);
         else
-            pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int64_t, false>, dim3(g), dim3(RT3_X * RT3_Y), 0, st, 1, a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int64_t, false>, dim3(g), dim3(RT3_X * RT3_Y), 0, st, a, nullptr, nullptr, 0);
     } else {
         if (small)
-            pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, false>, dim3(g), dim3(RT2_X), 0, st, 1, a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, false>, dim3(g), dim3(RT2_X), 0, st, a, nullptr, nullptr, 0);
         else
-            pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int64_t, false>, dim3(g), dim3(RT2_X), 0, st, 1, a, nullptr, nullptr, 0);
+            pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int64_t, false>, dim3(g), dim3(RT2_X), 0, st, a, nullptr, nullptr, 0);
     }
 }
 
@@ -2605,16 +2605,16 @@ static void launch_rhs_group(int d, const RhsArgs *tab, const int *prefix, int n
 {
     if (fx) {
         if (d == 3)
-            pdl_launch(k_rhs_fx<RT3_X, RT3_Y, RT3_Z, true>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, 1, RhsArgs{}, tab, prefix, ninst);
+            pdl_launch(k_rhs_fx<RT3_X, RT3_Y, RT3_Z, true>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, RhsArgs{}, tab, prefix, ninst);
         else
-            pdl_launch(k_rhs_fx<RT2_X, 1, RT2_Z, true>, dim3(blocks), dim3(RT2_X), 0, st, 1, RhsArgs{}, tab, prefix, ninst);
+            pdl_launch(k_rhs_fx<RT2_X, 1, RT2_Z, true>, dim3(blocks), dim3(RT2_X), 0, st, RhsArgs{}, tab, prefix, ninst);
         return;
     }
     if (d == 3)
-        pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, true>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, 1, RhsArgs{}, tab, prefix,
+        pdl_launch(k_rhs_tiled<RT3_X, RT3_Y, RT3_Z, int32_t, true>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, RhsArgs{}, tab, prefix,
                                                                                          ninst);
     else
-        pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, true>, dim3(blocks), dim3(RT2_X), 0, st, 1, RhsArgs{}, tab, prefix, ninst);
+        pdl_launch(k_rhs_tiled<RT2_X, 1, RT2_Z, int32_t, true>, dim3(blocks), dim3(RT2_X), 0, st, RhsArgs{}, tab, prefix, ninst);
 }
 
 // Separate (unfused) stage kernels, used when timing at plan creation finds them
@@ -3472,43 +3472,43 @@ static void launch_tc_k(bool mode1, int bn, bool dual, int grid, cudaStream_t st
             constexpr uint32_t sm = TileCfg<128, 4>::SMEM_BYTES;
             if (a.out_kind == 0) {
                 if (mode1)
-                    pdl_launch(k_mode_tc<true, 128, false, GROUPED, false, 1>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<true, 128, false, GROUPED, false, 1>, dim3(grid), dim3(kThreads), sm, st, a, gtab, gprefix, ginst, gunits);
                 else
-                    pdl_launch(k_mode_tc<false, 128, false, GROUPED, false, 1>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<false, 128, false, GROUPED, false, 1>, dim3(grid), dim3(kThreads), sm, st, a, gtab, gprefix, ginst, gunits);
             } else if (a.out_kind == 1) {
                 if (mode1)
-                    pdl_launch(k_mode_tc<true, 128, false, GROUPED, false, 2>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<true, 128, false, GROUPED, false, 2>, dim3(grid), dim3(kThreads), sm, st, a, gtab, gprefix, ginst, gunits);
                 else
-                    pdl_launch(k_mode_tc<false, 128, false, GROUPED, false, 2>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<false, 128, false, GROUPED, false, 2>, dim3(grid), dim3(kThreads), sm, st, a, gtab, gprefix, ginst, gunits);
             } else if constexpr (!GROUPED) {
                 if (mode1)
-                    pdl_launch(k_mode_tc<true, 128, false, false, false, 3>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<true, 128, false, false, false, 3>, dim3(grid), dim3(kThreads), sm, st, a, gtab, gprefix, ginst, gunits);
                 else
-                    pdl_launch(k_mode_tc<false, 128, false, false, false, 3>, dim3(grid), dim3(kThreads), sm, st, 1, a, gtab, gprefix, ginst, gunits);
+                    pdl_launch(k_mode_tc<false, 128, false, false, false, 3>, dim3(grid), dim3(kThreads), sm, st, a, gtab, gprefix, ginst, gunits);
             }
         }
         return;
     }
     if (bn == 256) {
         if (mode1)
-            pdl_launch(k_mode_tc<true, 256, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<256>::SMEM_BYTES, st, 1, a, gtab, gprefix,
+            pdl_launch(k_mode_tc<true, 256, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<256>::SMEM_BYTES, st, a, gtab, gprefix,
                                                                                                   ginst, gunits);
         else
-            pdl_launch(k_mode_tc<false, 256, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<256>::SMEM_BYTES, st, 1, a, gtab, gprefix,
+            pdl_launch(k_mode_tc<false, 256, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<256>::SMEM_BYTES, st, a, gtab, gprefix,
                                                                                                    ginst, gunits);
     } else if (!dual) {
         if (mode1)
-            pdl_launch(k_mode_tc<true, 128, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
+            pdl_launch(k_mode_tc<true, 128, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, a, gtab, gprefix,
                                                                                                   ginst, gunits);
         else
-            pdl_launch(k_mode_tc<false, 128, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
+            pdl_launch(k_mode_tc<false, 128, false, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, a, gtab, gprefix,
                                                                                                    ginst, gunits);
     } else {
         if (mode1)
-            pdl_launch(k_mode_tc<true, 128, true, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
+            pdl_launch(k_mode_tc<true, 128, true, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, a, gtab, gprefix,
                                                                                                  ginst, gunits);
         else
-            pdl_launch(k_mode_tc<false, 128, true, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, 1, a, gtab, gprefix,
+            pdl_launch(k_mode_tc<false, 128, true, GROUPED, SK>, dim3(grid), dim3(kThreads), TileCfg<128>::SMEM_BYTES, st, a, gtab, gprefix,
                                                                                                   ginst, gunits);
     }
 }
@@ -3576,9 +3576,9 @@ static void launch(const ModeLaunch &L, cudaStream_t st, double *U = nullptr, co
         const int64_t total = a.part_stride;
         const int g = (int)std::min<int64_t>((total / 4 + 255) / 256, 152 * 8);
         if (a.epi)
-            pdl_launch(k_split_reduce_epi, dim3(g), dim3(256), 0, st, 1, a);
+            pdl_launch(k_split_reduce_epi, dim3(g), dim3(256), 0, st, a);
         else
-            pdl_launch(k_split_reduce, dim3(g), dim3(256), 0, st, 1, total, L.N, a.ksplit, a.part_ws, a.out_kind, a.out);
+            pdl_launch(k_split_reduce, dim3(g), dim3(256), 0, st, total, L.N, a.ksplit, a.part_ws, a.out_kind, a.out);
     }
 }
 
@@ -3821,11 +3821,11 @@ static void launch_stage_kernel(const MixedPlan *mp, int g, const ModelF &mf, do
 {
     const int64_t N = mp->N;
     if (g == 0)
-        pdl_launch(k_stage_planes, dim3(pw_grid(N)), dim3(256), 0, st, 1, mf, N, U, mp->incF, 3 * N, nullptr, 0, mp->Dp);
+        pdl_launch(k_stage_planes, dim3(pw_grid(N)), dim3(256), 0, st, mf, N, U, mp->incF, 3 * N, nullptr, 0, mp->Dp);
     else if (g == 1)
-        pdl_launch(k_stage_planes, dim3(pw_grid(N)), dim3(256), 0, st, 1, mf, N, U, mp->incF + N, 3 * N, mp->incD, N, mp->Dp);
+        pdl_launch(k_stage_planes, dim3(pw_grid(N)), dim3(256), 0, st, mf, N, U, mp->incF + N, 3 * N, mp->incD, N, mp->Dp);
     else
-        pdl_launch(k_final_mixed, dim3(pw_grid(N)), dim3(256), 0, st, 1, N, U, mp->incF + 2 * N, 3 * N, mp->incD, N);
+        pdl_launch(k_final_mixed, dim3(pw_grid(N)), dim3(256), 0, st, N, U, mp->incF + 2 * N, 3 * N, mp->incD, N);
 }
 
 // For each group, time its last mode with the fused epilogue against the
@@ -4428,9 +4428,9 @@ static void launch_rhs_fx(MixedPlan *mp, const Model &model, double *U, bool mea
     const dim3 g = rhs_tiles(mp->stf[0]);
     const unsigned blocks = g.x * g.y * g.z;
     if (mp->d == 3)
-        pdl_launch(k_rhs_fx<RT3_X, RT3_Y, RT3_Z, false>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, 1, a, nullptr, nullptr, 0);
+        pdl_launch(k_rhs_fx<RT3_X, RT3_Y, RT3_Z, false>, dim3(blocks), dim3(RT3_X * RT3_Y), 0, st, a, nullptr, nullptr, 0);
     else
-        pdl_launch(k_rhs_fx<RT2_X, 1, RT2_Z, false>, dim3(blocks), dim3(RT2_X), 0, st, 1, a, nullptr, nullptr, 0);
+        pdl_launch(k_rhs_fx<RT2_X, 1, RT2_Z, false>, dim3(blocks), dim3(RT2_X), 0, st, a, nullptr, nullptr, 0);
 }
 
 int enqueue_rhs_mixed(MixedPlan *mp, const Model &model, double *U, cudaStream_t st)
@@ -4912,7 +4912,7 @@ int enqueue_step_mixed(MixedPlan *mp, const ds_phi_set *set, const Model &model,
         // from that and then writes it.
         // reset: the calibrating step starts each slot's exponent history
         auto rescale = [&](int first, int count, bool reset) {
-            pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, 1, mp->fxs, first, count, reset ? 1 : 0);
+            pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, mp->fxs, first, count, reset ? 1 : 0);
             ++L;
         };
         auto rhs = [&](bool measure) {
@@ -4988,7 +4988,7 @@ int enqueue_step_mixed(MixedPlan *mp, const ds_phi_set *set, const Model &model,
             sa.measure = measure ? 1 : 0;
             sa.model = mdf;
             P.begin(st, 2, 0.0, (double)N * (g == 1 ? 48.0 : 64.0));
-            pdl_launch(k_stage_fx, dim3(pw_grid(N)), dim3(256), 0, st, 1, sa);
+            pdl_launch(k_stage_fx, dim3(pw_grid(N)), dim3(256), 0, st, sa);
             P.end(st);
             ++L;
         };
@@ -5007,7 +5007,7 @@ int enqueue_step_mixed(MixedPlan *mp, const ds_phi_set *set, const Model &model,
         }
         // U += tau S_f(F) + 3tau/2 S_f(D3), both as double-floats
         P.begin(st, 2, 0.0, (double)N * 64.0);
-        pdl_launch(k_final_fx, dim3(pw_grid(N)), dim3(256), 0, st, 1, N, U, mp->incF + 2 * N, mp->incFlo + 2 * N, 3 * N, mp->incD,
+        pdl_launch(k_final_fx, dim3(pw_grid(N)), dim3(256), 0, st, N, U, mp->incF + 2 * N, mp->incFlo + 2 * N, 3 * N, mp->incD,
                                                mp->incDlo, N);
         P.end(st);
         ++L;
@@ -5120,7 +5120,7 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
     DS_CUDA_TRY(cudaMemcpyAsync(fxs, &h, sizeof(h), cudaMemcpyHostToDevice, st));
     DS_CUDA_TRY(cudaMemcpyAsync(jobs, hj, sizeof(FxMatJob) * d, cudaMemcpyHostToDevice, st));
     k_absmax<<<pw_grid(N), 256, 0, st>>>(N, X, fxs, 0);
-    pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, 1, fxs, 0, 1, 1);
+    pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, fxs, 0, 1, 1);
     k_split_tensor_fx<<<pw_grid(N), 256, 0, st>>>(N, X, fxs, 0, A0);
     __half *pcur = Pp;
     float *pscur = pscale;
@@ -5145,7 +5145,7 @@ ds_status tucker_fx(const ds_grid *grid, const double *X, double *Y, const doubl
             ModeLaunch mm = ml;
             mm.args.fx_measure = 1;
             launch(mm, st);
-            pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, 1, fxs, mu + 1, 1, 1);
+            pdl_launch(k_fx_rescale, dim3(1), dim3(32), 0, st, fxs, mu + 1, 1, 1);
         }
         launch(ml, st);
         in = bufs[mu % 2];
