@@ -884,7 +884,7 @@ ds_status ds_plan_create(const ds_grid *grid, const ds_params *params, const ds_
             std::vector<SumGroup> groups;
             if (etd2) groups = {{SumKind::plain, {0}}, {SumKind::plain, {1}}};
             else groups = {{SumKind::plain, {0, 1, 3}}, {SumKind::plain, {2}}, {SumKind::plain, {4}}};
-            sums_create(p->sums, set, p->N, groups, p->ws + (p->ws_count - zt * p->N), zt, p->status, p->st);
+            sums_create(p->sums, set, p->N, groups, p->ws + (p->ws_count - zt * p->N), zt, p->st);
         } else if (precision == DS_PREC_F32) {
             if (!set->tridiag[0] || !set->tridiag[1])
                 return cleanup(DS_ERR_UNSUPPORTED, "reduced-precision paths need tridiagonal A_mu (use DS_PREC_F64)");
@@ -1021,7 +1021,7 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
         sums_create(p->bsums, s, N,
                     {{SumKind::plain, {0, 1}}, {SumKind::plain, {2}}, {SumKind::transposed, {3, 4}},
                      {SumKind::transposed, {1, 2}}, {SumKind::transposed, {0}}},
-                    p->bws + 22 * N, zt, p->status, p->st);
+                    p->bws + 22 * N, zt, p->st);
     }
     if (dscale && !p->tws) {
         const int per_op = sum_tensors(s, SumKind::tangent);
@@ -1037,7 +1037,7 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
         }
         sums_create(p->tsums, s, N,
                     {{SumKind::tangent, {0, 1, 3}}, {SumKind::tangent, {2}}, {SumKind::tangent, {4}}},
-                    p->tws + 6 * N, zt, p->status, p->st);
+                    p->tws + 6 * N, zt, p->st);
     }
     cudaStream_t st = (cudaStream_t)stream;
     const double tau = s->tau;

@@ -887,7 +887,6 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
     release(tab);
     DS_CUDA_TRY(cudaStreamSynchronize(st));
     DS_CUDA_TRY(cudaGetLastError());
-    if (ctx.ws) return mm::take_status();
     return DS_OK;
 }
 

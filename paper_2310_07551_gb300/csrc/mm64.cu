@@ -17,14 +17,14 @@
 //
 // A fibre holding Inf or NaN carries a flag instead of an exponent: outputs
 // of a NaN fibre are NaN, those of an Inf fibre are recomputed by the FP64
-// FMA chain in the epilogue.
+// FMA chain in the epilogue.  So are the outputs behind a bounded wait that gave
+// up: a call that meets one is slow, and its results are right.
 #include <cuda_fp16.h>
 #include <limits.h>
 #include <stdlib.h>
 
 #include <algorithm>
 #include <atomic>
-#include <string>
 
 #include "mm64.h"
 #include "ptx.cuh"
@@ -38,9 +38,6 @@ namespace {
 constexpr int kNanRow = INT_MAX, kInfRow = INT_MAX - 1;   // exponents of non-finite fibres
 constexpr int kChunkSlabs = 16;                           // slabs between drains: 256 entries
 constexpr int kSms = 152;
-
-// where waits that gave up are recorded for entry points without a plan
-__device__ DevStatus g_status;
 
 // ---------------------------------------------------------------------------
 // Digit images.  One warp takes 2E rows of one slab: lane = (row, E consecutive
@@ -227,7 +224,6 @@ struct GProd {
 struct GArgs {
     int count;
     int first[kMaxProd + 1];   // prefix of tiles
-    DevStatus *status;
     long long wait_limit;
     GProd p[kMaxProd];
 };
@@ -430,7 +426,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
     const uint32_t FULL = bars, EMPTY = FULL + 8 * kStages, TFULL = EMPTY + 8 * kStages, TEMPTY = TFULL + 8, DRAIN = TFULL + 16;
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
     const int tiles = a.first[a.count];
-    DevStatus *const status = a.status ? a.status : &g_status;
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2 * kStages; ++s) bar_init(bars + 8 * s, 1);
         bar_init(TFULL, 1);
@@ -466,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                 const uint8_t *A = p.A + ((int64_t)be * p.mtiles + mi) * slabs * kStageA;
                 const uint8_t *B = p.B + ((int64_t)be * p.ntiles + ni) * slabs * nb;
                 for (int s = 0; s < slabs; ++s) {
-                    ok = __all_sync(0xffffffffu, bar_wait(EMPTY + 8 * stage, phase ^ 1u, abort_flag, status, 11, a.wait_limit));
+                    ok = __all_sync(0xffffffffu, bar_wait(EMPTY + 8 * stage, phase ^ 1u, abort_flag, a.wait_limit));
                     if (!ok) break;
                     if (elect_one()) {
                         const uint32_t sA = base + stage * kStageBytes;
@@ -487,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
             // every issued copy lands before the CTA exits
             volatile int never = 0;
             for (int s = max(0, issued - kStages); s < issued; ++s)
-                bar_wait(FULL + 8 * (s % kStages), s / kStages & 1, &never, nullptr, 0, kWaitCycles);
+                bar_wait(FULL + 8 * (s % kStages), s / kStages & 1, &never, kWaitCycles);
         }
         if (warp == 1) {
             int stage = 0, q = 0;
@@ -500,11 +495,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                 for (int s = 0; s < slabs; ++s) {
                     const bool fresh = s % kChunkSlabs == 0;
                     if (fresh) {
-                        ok = __all_sync(0xffffffffu, bar_wait(TEMPTY, tphase ^ 1u, abort_flag, status, 12, a.wait_limit));
+                        ok = __all_sync(0xffffffffu, bar_wait(TEMPTY, tphase ^ 1u, abort_flag, a.wait_limit));
                         if (!ok) break;
                         tphase ^= 1u;
                     }
-                    ok = __all_sync(0xffffffffu, bar_wait(FULL + 8 * stage, phase, abort_flag, status, 13, a.wait_limit));
+                    ok = __all_sync(0xffffffffu, bar_wait(FULL + 8 * stage, phase, abort_flag, a.wait_limit));
                     if (!ok) break;
                     tc_after();
                     const uint32_t sA = base + stage * kStageBytes, sB = sA + kStageA;
@@ -528,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
             if (elect_one()) mma_commit_to(DRAIN);
             __syncwarp();
             volatile int never = 0;
-            bar_wait(DRAIN, 0, &never, nullptr, 0, kWaitCycles);
+            bar_wait(DRAIN, 0, &never, kWaitCycles);
         }
     } else {
         // warp w reads the tensor-memory lanes 32 (w % 4) ..; the four warps of a
@@ -555,7 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
             double *const out = p.out + be * p.sOut + ro * (p.I * p.cols) + (rg - ro * p.I) + p.I * c0;
             long long P[kEpiCols], Q[kEpiCols];
             for (int s0 = 0; s0 < p.slabs; s0 += kChunkSlabs) {
-                ok = ok && __all_sync(0xffffffffu, bar_wait(TFULL, tphase, abort_flag, status, 14, a.wait_limit));
+                ok = ok && __all_sync(0xffffffffu, bar_wait(TFULL, tphase, abort_flag, a.wait_limit));
                 if (!ok) break;
                 tphase ^= 1u;
                 tc_after();
@@ -617,12 +612,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                 }
             }
             if (odd && row_ok) {
-                // non-finite entries, or an abandoned wait (NaN)
+                // non-finite entries, or a wait gave up (every later output of this warp)
 #pragma unroll 1
                 for (int j = 0; j < hc && c0 + j < p.cols; ++j) {
                     const int e = __ldg(p.eB + (int64_t)be * p.ntiles * nt + c0 + j);
-                    const double z = !ok || er == kNanRow || e == kNanRow ? __longlong_as_double(0x7FF8000000000000LL)
-                                                                         : fma_chain(p, be, rg, c0 + j);
+                    const double z = er == kNanRow || e == kNanRow ? __longlong_as_double(0x7FF8000000000000LL)
+                                                                   : fma_chain(p, be, rg, c0 + j);
                     double *o = out + p.I * j;
                     *o = p.accumulate ? __dadd_rn(*o, z) : z;
                 }
@@ -806,7 +801,7 @@ void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
     else split_as<8>(v, im, count, st);
 }
 
-void launch_products(const Product *s, int count, DevStatus *status, long long wait_limit, cudaStream_t st)
+void launch_products(const Product *s, int count, long long wait_limit, cudaStream_t st)
 {
     static std::atomic<uint64_t> ready{0};   // devices whose shared-memory limit is raised
     int dev = 0;
@@ -817,7 +812,6 @@ void launch_products(const Product *s, int count, DevStatus *status, long long w
     }
     GArgs a{};
     a.count = count;
-    a.status = status;
     a.wait_limit = wait_limit;
     for (int q = 0; q < count; ++q) {
         a.p[q] = to_gprod(s[q]);
@@ -945,7 +939,7 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
                 ++launches;
             }
             if (c.prof) c.prof->begin(st, 1, flops);
-            launch_products(p, np, c.status, c.wait_limit, st);
+            launch_products(p, np, c.wait_limit, st);
             if (c.prof) c.prof->end(st);
             ++launches;
         };
@@ -1015,16 +1009,6 @@ void tucker_f64(const Context &c, int d, const int64_t *n, const double *X, doub
         run_products(c, &p, 1, st);
         in = p.out;
     }
-}
-
-ds_status take_status()
-{
-    DevStatus h{};
-    DS_CUDA_TRY(cudaMemcpyFromSymbol(&h, g_status, sizeof h));
-    if (!h.timeout) return DS_OK;
-    const DevStatus zero{};
-    cudaMemcpyToSymbol(g_status, &zero, sizeof zero);
-    return fail(DS_ERR_TIMEOUT, "digit-product pipeline wait gave up (site " + std::to_string(h.where) + ")");
 }
 
 long long wait_limit_default()

@@ -62,12 +62,10 @@ inline size_t image_bytes(int64_t rows, int rb, int slabs)
 // cycles a pipeline wait may take (the test hook DS_WAIT_LIMIT_CYCLES, else ~2 s)
 long long wait_limit_default();
 
-// Scratch of run_products for digit images, and where waits that gave up and
-// launch times are recorded.
+// Scratch of run_products for digit images, and where launch times are recorded.
 struct Context {
     uint8_t *ws = nullptr;
     size_t ws_bytes = 0;
-    DevStatus *status = nullptr;   // null: one per device, see take_status
     long long wait_limit = wait_limit_default();
     Prof *prof = nullptr;
 };
@@ -108,17 +106,13 @@ int tile_cols(int64_t rows, int cols, int products, int slabs);
 // Digit images of up to kMaxProd views (one launch).
 void launch_split(const View *v, const Image *im, int count, cudaStream_t st);
 // Up to kMaxProd products on their images (one launch).
-void launch_products(const Product *p, int count, DevStatus *status, long long wait_limit, cudaStream_t st);
+void launch_products(const Product *p, int count, long long wait_limit, cudaStream_t st);
 // The same products on the FP64 pipe, one thread per output (one launch;
 // images unused): small products.
 void launch_products_fma(const Product *p, int count, cudaStream_t st);
 // Whether a mode product of this shape runs on the tensor cores (count
 // products in the launch).
 bool use_digits(int64_t rows, int n, int count);
-
-// DS_ERR_TIMEOUT (once) if a wait of a launch without a status word of its own
-// gave up; call it after a synchronisation.
-ds_status take_status();
 
 }  // namespace mm
 }  // namespace ds

@@ -35,21 +35,29 @@ __device__ __forceinline__ bool bar_try(uint32_t bar, uint32_t parity)
                  : "memory");
     return ok != 0;
 }
-// Waits for the phase at most `limit` cycles; false when the wait gave up or
-// another wait of the CTA did.  The first to give up records its site.
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, DevStatus *st,
-                                      int site, long long limit)
+__device__ __forceinline__ bool bar_test(uint32_t bar, uint32_t parity)
 {
-    if (bar_try(bar, parity)) return true;
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}\n"
+                 : "=r"(ok)
+                 : "r"(bar), "r"(parity)
+                 : "memory");
+    return ok != 0;
+}
+// Waits for the phase at most `limit` cycles; false when the wait gave up or
+// another wait of the CTA did.  A limit below the usual one is a test's: then every
+// probe returns at once, where try_wait may suspend the thread until the phase
+// completes.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long limit)
+{
+    const bool at_once = limit < kWaitCycles;
+    if (bar_test(bar, parity)) return true;
     const long long t0 = clock64();
-    while (!bar_try(bar, parity)) {
+    while (!(at_once ? bar_test(bar, parity) : bar_try(bar, parity))) {
         if (*abort_flag) return false;
         if (clock64() - t0 > limit) {
             *abort_flag = 1;
-            if (st) {
-                atomicExch(&st->timeout, 1);
-                atomicExch(&st->where, site);
-            }
             return false;
         }
     }

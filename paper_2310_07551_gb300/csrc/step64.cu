@@ -147,13 +147,12 @@ int sum_tensors(const ds_phi_set *s, SumKind kind)
 }
 
 void sums_create(Sums64 &e, const ds_phi_set *s, int64_t N, const std::vector<SumGroup> &groups, double *z,
-                 int64_t z_tensors, DevStatus *status, cudaStream_t st)
+                 int64_t z_tensors, cudaStream_t st)
 {
     e.set = s;
     e.N = N;
     e.z = z;
     e.z_tensors = z_tensors;
-    e.ctx.status = status;
     // the phases' matrices and the scratch of the largest phase
     std::vector<View> views;
     std::vector<Image> ims;

@@ -43,7 +43,7 @@ int sum_tensors(const ds_phi_set *s, SumKind kind);
 // it waits for).  Where memory is short the sums still run: matrices cut per
 // call, or products on the FP64 pipe.
 void sums_create(Sums64 &e, const ds_phi_set *s, int64_t N, const std::vector<SumGroup> &groups, double *z,
-                 int64_t z_tensors, DevStatus *status, cudaStream_t st);
+                 int64_t z_tensors, cudaStream_t st);
 void sums_destroy(Sums64 &e);
 // Runs independent sums of one kind; returns the number of launches.
 int run_sums(const Sums64 &e, SumKind kind, const SumOp *ops, int count, Prof *prof, cudaStream_t st);
