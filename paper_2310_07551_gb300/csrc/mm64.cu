@@ -349,14 +349,15 @@ struct Rounded {
 };
 __device__ __forceinline__ Rounded round_sum(long long P, long long Q, int e)
 {
-    // 96 bits: H = P + (Q >> 30) above the low 30 bits of Q; the magnitude as a
-    // ones' complement (2^-32 of H off: far below the last kept bit)
+    // 96 bits: H = P + (Q >> 30) above the low 30 bits of Q; their
+    // magnitude
     const long long H = P + (Q >> 30);
     uint32_t w0 = (uint32_t)Q << 2, w1 = (uint32_t)H, w2 = (uint32_t)((unsigned long long)H >> 32);
     const uint32_t neg = (uint32_t)((int)w2 >> 31);
-    w0 ^= neg;
-    w1 ^= neg;
-    w2 ^= neg;
+    asm("{\n\t.reg .u32 a, b, c;\n\txor.b32 a, %0, %3;\n\txor.b32 b, %1, %3;\n\txor.b32 c, %2, %3;\n\t"
+        "sub.cc.u32 %0, a, %3;\n\tsubc.cc.u32 %1, b, %3;\n\tsubc.u32 %2, c, %3;\n\t}"
+        : "+r"(w0), "+r"(w1), "+r"(w2)
+        : "r"(neg));
     // leading word up, then the leading bit
     const bool z = w2 == 0;
     w2 = z ? w1 : w2;
