@@ -57,9 +57,13 @@ typedef enum {
  *   DS_PREC_F64    : FP64 everywhere.  Large contractions are sums of exact
  *                    products of 8-bit digits on the tensor cores (operands
  *                    as 62-bit fixed point per fibre, the sum rounded to
- *                    FP64 once), small ones FP64 FMA chains.  The outputs
- *                    behind a wait of the digit products that gave up are
- *                    FMA chains too: no call fails for it.
+ *                    FP64 once), small ones FP64 FMA chains.  Outputs whose
+ *                    terms are small against their fibres' largest entries
+ *                    (sum of magnitudes below 2^-8 of the product of the
+ *                    largest) are FMA chains too, so that entries of any
+ *                    size keep their relative accuracy.  So are the outputs
+ *                    behind a wait of the digit products that gave up: no
+ *                    call fails for it.
  *   DS_PREC_F32    : FP32 mode products on the CUDA cores (FP32 FMA, FP32
  *                    intermediates and stage sums), FP64 state -- the
  *                    design of the paper's single-precision GPU runs.

@@ -1064,10 +1064,11 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
         sums_f64(p, e, SumKind::transposed, 2, q, lam, out, false, st);
     }
     launch_jacT_f64(m, N, U3, lD3, lU3, st);
-    sum_f64(p, e, SumKind::transposed, 1, lU3, lF, true, st);
+    sum_f64(p, e, SumKind::transposed, 1, lU3, a, false, st);
     sum_f64(p, e, SumKind::transposed, 2, lU3, lD2, false, st);
     launch_jacT_f64(m, N, U2, lD2, lU2, st);
-    sum_f64(p, e, SumKind::transposed, 0, lU2, lF, true, st);
+    sum_f64(p, e, SumKind::transposed, 0, lU2, b, false, st);
+    launch_axpy2_f64(N, lF, a, 1.0, b, 1.0, lF, st);
     if (dscale) {
         // through K (F = s K U + G) and through every phi-matrix: the tangent of
         // each sum against the adjoint of its stage; b <- D3 = g(U3) - g(U)

@@ -371,8 +371,9 @@ __device__ __forceinline__ void dparam_point(const Model &m, double u, double v,
 }
 
 // Y = U + w1 a (+ w2 b), 2 N values
-__global__ void k_axpy2(int64_t n2, const double *__restrict__ U, const double *__restrict__ a, double w1,
-                        const double *__restrict__ b, double w2, double *__restrict__ Y)
+// (Y may be U)
+__global__ void k_axpy2(int64_t n2, const double *U, const double *__restrict__ a, double w1,
+                        const double *__restrict__ b, double w2, double *Y)
 {
     pdl_trigger();
     pdl_wait();
@@ -770,7 +771,7 @@ ds_status phi_batch_f64(int n, const std::vector<PhiJob> &jobs, cudaStream_t st)
         v.batch = nb;
         size_t bytes = mm::image_total(v, mm::kRowBlock);
         v.rows = 3 * (int64_t)n + 64;   // padded to whole column tiles
-        bytes += mm::image_total(v, 1);
+        bytes += mm::image_total(v, 1) + mm::kAlign + mm::left_bytes(n, 3 * n, nb);
         if (pool_alloc((void **)&ctx.ws, bytes, st) == cudaSuccess) {
             ctx.ws_bytes = bytes;
         } else {

@@ -7,13 +7,23 @@
 // fixed-point number and cut into eight balanced 8-bit digits, held as FP16
 // integers: x = 2^(e - 6) (d0 + d1 2^-8 + ... + d7 2^-56), |d0| <= 64,
 // |d1..7| <= 128.  The digit products of weight class t = p + q <= 7 (36 of
-// 64) run as FP16 MMAs into one FP32 tensor-memory accumulator per class.  An
-// accumulator holds integers below 2^24 (at most 256 contracted entries
-// between drains), so its sums are exact; the epilogue recombines the classes
-// in integers and rounds once to FP64.  What is lost is the fixed-point
-// rounding of the operands (2^-63 of a fibre's largest entry) and the classes
-// below 2^-56: about 2^-61 of the largest product, where a chain of n FP64
-// FMAs loses 2^-53 per addition.
+// 64) run as FP16 MMAs into one FP32 tensor-memory accumulator per class, the
+// epilogue recombines the classes in integers and rounds once to FP64.  (The error-free
+// splitting of matrix products of Ozaki, Ogita, Oishi and Rump, 2012, with digits of
+// a fixed radix.)
+//
+// What it loses, per contracted entry and in units of the product 2^(ex + el) of the
+// two fibres' powers of two: the dropped classes, below 2^-59.2 (seven digit products of
+// at most 2^14 at 2^-76); the operands' rounding, 2^-62.  Accumulators: at most 256
+// entries are contracted between drains, which bounds class t by t 2^22: classes 0 to
+// 4 stay below 2^24 and are exact; 5 to 7 may pass it, where nearly all of more than 200
+// entries have extreme digits of the same sign, and then lose a unit (2^-52, 2^-60,
+// 2^-68) per MMA.  The drain keeps 2^-66 of class 7 and 2^-60 of the sum.  A chain of
+// n FMAs loses 2^-53 of a partial sum per entry, so the digits are the better where
+// the sum S of the terms' magnitudes is not small against 2^(ex + el).  Where it is
+// (identity or graded matrices, localised states), small entries have few digits of
+// their own: such outputs, S below 2^-8, become FMA chains (k_settle), so that every
+// output is within n 2^-51 S of its sum, as a chain is within n 2^-53 S.
 //
 // A fibre holding Inf or NaN carries a flag instead of an exponent: outputs
 // of a NaN fibre are NaN, those of an Inf fibre are recomputed by the FP64
@@ -25,6 +35,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "mm64.h"
 #include "ptx.cuh"
@@ -35,7 +46,15 @@ namespace mm {
 using namespace ptx;
 
 namespace {
-constexpr int kNanRow = INT_MAX, kInfRow = INT_MAX - 1;   // exponents of non-finite fibres
+constexpr int kNanRow = 32767, kInfRow = 32766, kZeroRow = -16384;   // exponents of non-finite and zero fibres
+// Digit sums below 2^-kWeak of their fibres' 2^exponents are looked into (settle).  At
+// 2^-8 the dropped classes weigh about as much as an FMA chain's roundings (a random
+// walk: 2^-54 sqrt(n) of S); one power of two more would send 4 to 8 times as many outputs of
+// a smooth state to the chains (Schnakenberg 301 x 150 at step 1200, second mode: 0.09 %
+// of them, 0.5 % at 2^-7).
+// entries of at least 2^-kBig of their fibre's are flagged as big, so that one that is
+// big in both fibres is a term of 2^-kWeak.
+constexpr int kWeak = 8, kBig = kWeak / 2;
 constexpr int kChunkSlabs = 16;                           // slabs between drains: 256 entries
 constexpr int kSms = 152;
 
@@ -50,6 +69,7 @@ constexpr int kSms = 152;
 // ---------------------------------------------------------------------------
 struct SplitArgs {
     int count;
+    int *reset;                // set to zero (the products' count of outputs left to k_settle)
     int first[kMaxProd + 1];   // block prefix
     View v[kMaxProd];
     Image im[kMaxProd];
@@ -90,15 +110,17 @@ __device__ __forceinline__ int fibre_exp(unsigned long long mx)
     const int ef = (int)(mx >> 52);
     if (ef == 0x7FF) return (mx & 0xFFFFFFFFFFFFFULL) ? kNanRow : kInfRow;
     if (ef > 0) return ef - 1022;
-    return mx ? (64 - __clzll((long long)mx)) - 1074 : 0;
+    return mx ? (64 - __clzll((long long)mx)) - 1074 : kZeroRow;
 }
+// magnitude of a slab whose largest entry has these bits: below 2^(code - 1023); 0: all zero
+__device__ __forceinline__ uint32_t slab_code(unsigned long long mx) { return mx ? (uint32_t)(mx >> 52) + 1 : 0u; }
 
 // the eight digits of E consecutive entries: bytes of x 2^(62 - e) + 128 in
-// every byte, one chunk of 2 E bytes per digit plane
+// every byte, one chunk of 2 E bytes per digit plane.  Returns a bit per big entry.
 template <int E>
-__device__ __forceinline__ void store_digits(const unsigned long long (&x)[E], int e, uint8_t *dst, int64_t plane)
+__device__ __forceinline__ uint32_t store_digits(const unsigned long long (&x)[E], int e, uint8_t *dst, int64_t plane)
 {
-    uint32_t lo[E], hi[E];
+    uint32_t lo[E], hi[E], big = 0;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
         const unsigned long long b = x[j];
@@ -110,6 +132,7 @@ __device__ __forceinline__ void store_digits(const unsigned long long (&x)[E], i
         if (sh >= 0) f = m << (sh & 63);
         else f = sh < -60 ? 0ULL : (m + (1ULL << (-sh - 1))) >> -sh;
         if (e >= kInfRow) f = 0ULL;
+        if (f >> (62 - kBig)) big |= 1u << j;
         if ((long long)b < 0) f = 0ULL - f;
         f += 0x8080808080808080ULL;
         lo[j] = (uint32_t)f;
@@ -132,6 +155,7 @@ __device__ __forceinline__ void store_digits(const unsigned long long (&x)[E], i
         if constexpr (E == 8) *reinterpret_cast<uint4 *>(dst + p * plane) = make_uint4(q[0], q[1], q[2], q[3]);
         else *reinterpret_cast<uint2 *>(dst + p * plane) = make_uint2(q[0], q[1]);
     }
+    return big;
 }
 
 template <int E>
@@ -142,6 +166,18 @@ __device__ __forceinline__ unsigned long long largest(unsigned long long mx, con
     return mx;
 }
 
+// a slab's mask and code of a row from its lanes' parts; all lanes of a warp
+template <int E>
+__device__ __forceinline__ void join_lanes(uint32_t &big, uint32_t &code, int chunk)
+{
+    big <<= chunk * E;
+#pragma unroll
+    for (int w = 1; w < kSlab / E; w *= 2) {
+        big |= __shfl_xor_sync(0xffffffffu, big, w);
+        code = max(code, __shfl_xor_sync(0xffffffffu, code, w));
+    }
+}
+
 // IT: 32-bit row indices where every view allows it (their divisions are a
 // good part of a small launch)
 template <typename IT, int E>
@@ -150,6 +186,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
     static_assert(E == 8 || E == 4, "16 or 8 bytes of a digit plane per thread");
     constexpr int kRows = 2 * E, kLaneBits = E == 8 ? 1 : 2;   // rows per warp, log2 of the lanes per row
     __shared__ unsigned long long smax[kSplitWarps][kRows];
+    __shared__ int speak[kSplitWarps][kRows];   // the slab of that entry
     int q = 0;
     while (q + 1 < a.count && (int)blockIdx.x >= a.first[q + 1]) ++q;
     const View &v = a.v[q];
@@ -171,28 +208,57 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
     uint8_t *dst = im.data + ((int64_t)entry * blocks + first) * S * kDigits * plane + rr * 32 +
                    (E == 8 ? (chunk ^ ((rr >> 2) & 1)) << 4 : (((chunk >> 1) ^ ((rr >> 2) & 1)) << 4) + ((chunk & 1) << 3));
     pdl_wait();
-    unsigned long long x[E], mx = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && a.reset) *a.reset = 0;
+    unsigned long long x[E];
     load_entries(v, base, row_ok, min(sub, S - 1), chunk, spc, x);
-    mx = largest(mx, x);
+    unsigned long long mx = largest(0ULL, x);
+    const uint32_t code = slab_code(mx);
+    int peak = min(sub, S - 1);
     for (int s = sub + WS; s < S; s += WS) {
         unsigned long long w[E];
         load_entries(v, base, row_ok, s, chunk, spc, w);
-        mx = largest(mx, w);
+        const unsigned long long m = largest(0ULL, w);
+        if (m > mx) {
+            mx = m;
+            peak = s;
+        }
     }
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    if constexpr (E == 4) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    if (chunk == 0) smax[warp][row] = mx;
+#pragma unroll
+    for (int w = 1; w < kSlab / E; w *= 2) {
+        const unsigned long long m = __shfl_xor_sync(0xffffffffu, mx, w);
+        const int o = __shfl_xor_sync(0xffffffffu, peak, w);
+        if (m > mx) {
+            mx = m;
+            peak = o;
+        }
+    }
+    if (chunk == 0) {
+        smax[warp][row] = mx;
+        speak[warp][row] = peak;
+    }
     __syncthreads();
     pdl_trigger();
     if (!in) return;
     for (int w = 0; w < WS; ++w) mx = max(mx, smax[gi * WS + w][row]);
     const int e = fibre_exp(mx);
-    if (sub == 0 && chunk == 0 && row_ok) im.exps[(int64_t)entry * blocks * rb + r] = e;
-    if (sub < S) store_digits(x, e, dst + (int64_t)sub * kDigits * plane, plane);
+    if (sub == 0 && chunk == 0 && row_ok) {
+        int w = 0;
+        while (w < WS - 1 && smax[gi * WS + w][row] != mx) ++w;
+        im.exps[(int64_t)entry * blocks * rb + r] = speak[gi * WS + w][row] << 16 | (e & 0xFFFF);
+    }
+    const int64_t at = ((int64_t)entry * blocks + first) * S * im.rb + rr;   // of the row's mask and code in slab 0
+    auto note = [&](int s, uint32_t big, uint32_t code) {
+        join_lanes<E>(big, code, chunk);
+        if (chunk == 0 && row_ok) {
+            im.masks[at + (int64_t)s * im.rb] = (uint16_t)big;
+            im.codes[at + (int64_t)s * im.rb] = (uint16_t)code;
+        }
+    };
+    if (sub < S) note(sub, store_digits(x, e, dst + (int64_t)sub * kDigits * plane, plane), code);
     for (int s = sub + WS; s < S; s += WS) {
         unsigned long long w[E];
         load_entries(v, base, row_ok, s, chunk, spc, w);
-        store_digits(w, e, dst + (int64_t)s * kDigits * plane, plane);
+        note(s, store_digits(w, e, dst + (int64_t)s * kDigits * plane, plane), slab_code(largest(0ULL, w)));
     }
 }
 
@@ -215,15 +281,25 @@ __global__ void __launch_bounds__(kSplitWarps * 32, 2) k_digits(const __grid_con
 struct GProd {
     const uint8_t *A, *B;
     const int *eA, *eB;
+    const uint16_t *mA, *mB, *cA, *cB;   // masks and codes
     double *out;
     int slabs, nt, ntiles, mtiles, cols, accumulate, ncat, n;
     int64_t rows, r0, I, IB, sA, sB, sOut;   // strides of a batch
     const double *X[kMaxCat], *L[kMaxCat];
     double sc[kMaxCat];
 };
+// Outputs of a tile that a drain leaves to k_settle: four columns (the first: c) of 32
+// rows (a lane quarter), words[j] the rows' bits in column c + j.
+struct Left {
+    uint16_t prod, c;
+    int entry, mi, ni;         // (ni: tile times four, plus the quarter)
+    uint32_t words[4];
+};
 struct GArgs {
     int count;
     int first[kMaxProd + 1];   // prefix of tiles
+    int *nleft;
+    Left *left;                // room for every tile's
     long long wait_limit;
     GProd p[kMaxProd];
 };
@@ -311,7 +387,7 @@ __device__ __forceinline__ void load_classes(uint32_t taddr, uint32_t cs, uint32
         : "memory");
 }
 
-// The classes of a thread's `hc` columns as P 2^30 + Q in units of 2^-6 of class
+// The classes of a thread's `hc` columns as P 2^38 + Q in units of 2^-14 of class
 // 5: classes 0 .. 2 in P, the rest in Q.  ADD: on top of the earlier entries'.
 template <bool ADD>
 __device__ __forceinline__ void drain(uint32_t taddr, uint32_t cs, int hc, long long (&P)[kEpiCols], long long (&Q)[kEpiCols])
@@ -330,9 +406,9 @@ __device__ __forceinline__ void drain(uint32_t taddr, uint32_t cs, int hc, long 
                 const int c0 = __float_as_int(cls(0) + 12582912.0f) - 0x4B400000;
                 const int c1 = __float_as_int(cls(1) + 12582912.0f) - 0x4B400000;
                 const int c2 = __float2int_rn(cls(2)), c3 = __float2int_rn(cls(3)), c4 = __float2int_rn(cls(4));
-                const int c5 = __float2int_rn(fmaf(cls(7), 0x1p-10f, fmaf(cls(6), 0.25f, 64.0f * cls(5))));
+                const int c5 = __float2int_rn(cls(5)), c6 = __float2int_rn(fmaf(cls(7), 0.25f, 64.0f * cls(6)));
                 const long long hp = (long long)c0 * 65536 + (c1 * 256 + c2);
-                const long long lp = (long long)c3 * 4194304 + ((long long)c4 * 16384 + c5);
+                const long long lp = (long long)c3 * 1073741824 + ((long long)c4 * 4194304 + ((long long)c5 * 16384 + c6));
                 P[g * 4 + j] = ADD ? P[g * 4 + j] + hp : hp;
                 Q[g * 4 + j] = ADD ? Q[g * 4 + j] + lp : lp;
             }
@@ -340,7 +416,7 @@ __device__ __forceinline__ void drain(uint32_t taddr, uint32_t cs, int hc, long 
     }
 }
 
-// P 2^30 + Q rounded to 53 bits, in 32-bit integers without branches (the FP64
+// P 2^38 + Q rounded to 53 bits, in 32-bit integers without branches (the FP64
 // pipe would take longer than the digit products).  The value is hi:lo, with the
 // leading bit at bit 52, times 2^(E - 52) and the sign.
 struct Rounded {
@@ -349,10 +425,10 @@ struct Rounded {
 };
 __device__ __forceinline__ Rounded round_sum(long long P, long long Q, int e)
 {
-    // 96 bits: H = P + (Q >> 30) above the low 30 bits of Q; their
+    // 96 bits: H = P + (Q >> 38) above 32 of the low 38 bits of Q; their
     // magnitude
-    const long long H = P + (Q >> 30);
-    uint32_t w0 = (uint32_t)Q << 2, w1 = (uint32_t)H, w2 = (uint32_t)((unsigned long long)H >> 32);
+    const long long H = P + (Q >> 38);
+    uint32_t w0 = (uint32_t)(Q >> 6), w1 = (uint32_t)H, w2 = (uint32_t)((unsigned long long)H >> 32);
     const uint32_t neg = (uint32_t)((int)w2 >> 31);
     asm("{\n\t.reg .u32 a, b, c;\n\txor.b32 a, %0, %3;\n\txor.b32 b, %1, %3;\n\txor.b32 c, %2, %3;\n\t"
         "sub.cc.u32 %0, a, %3;\n\tsubc.cc.u32 %1, b, %3;\n\tsubc.u32 %2, c, %3;\n\t}"
@@ -380,23 +456,18 @@ __device__ __forceinline__ Rounded round_sum(long long P, long long Q, int e)
 // outside the normal range
 __device__ __noinline__ double round_rare(long long P, long long Q, int e)
 {
-    const long long H = P + (Q >> 30), L = Q & 0x3FFFFFFF;
+    const long long H = P + (Q >> 38), L = Q & 0x3FFFFFFFFF;
     const bool neg = H < 0;
-    // |H| 2^30 + |L|; below 2^64 wherever |H| < 2^34, else the low bits go
-    unsigned long long V = 0;
-    long long h = H, l = L;
-    if (neg) {
-        h = -H - (L ? 1 : 0);
-        l = L ? 0x40000000 - L : 0;
-    }
+    // |H| 2^38 + |L|; the low bits go where it is 2^63 or more
+    const long long h = neg ? -H - (L ? 1 : 0) : H, l = neg && L ? 0x4000000000 - L : L;
     int sh = 0;
-    while (h >> (33 + sh)) ++sh;
-    V = ((unsigned long long)h << (30 - sh)) | ((unsigned long long)l >> sh);
+    while (h >> (25 + sh)) ++sh;
+    unsigned long long V = ((unsigned long long)h << (38 - sh)) | ((unsigned long long)l >> sh);
     if (V == 0) return 0.0;
     const int lz = __clzll((long long)V);
     V <<= lz;
     unsigned long long m = (V >> 11) + (V >> 10 & 1);
-    const int E = e + sh - lz + 63;   // m 2^(E - 52)
+    const int E = e - 8 + sh - lz + 63;   // m 2^(E - 52)
     if (E < -1200) return neg ? -0.0 : 0.0;
     const double r = scalbn((double)m, max(-2000, min(2000, E)) - 52);
     return neg ? -r : r;
@@ -415,6 +486,252 @@ __device__ __forceinline__ double fma_chain(const GProd &p, int64_t entry, int64
         total = t ? total + p.sc[t] * s : p.sc[t] * s;
     }
     return total;
+}
+
+// Lower bound, in units of 2^-28 of the fibres' 2^exponents, of the summed magnitudes of
+// the terms of slab s (of every concatenated operand) of row m and column c of a tile,
+// from its two leading digits v = 256 d0 + d1: |v| stands for at least |v| - 1/2.
+__device__ __forceinline__ float leading_terms(const GProd &p, const uint8_t *A, const uint8_t *B, int spc, int s, int m, int c)
+{
+    const int nt = p.nt, sa = (m >> 2) & 1, sb = (c >> 2) & 1;
+    float sum = 0.0f;
+    for (int t = 0; t < p.ncat; ++t) {
+        const uint4 *a = reinterpret_cast<const uint4 *>(A + (int64_t)(t * spc + s) * kStageA + m * 32);
+        const uint4 *b = reinterpret_cast<const uint4 *>(B + (int64_t)(t * spc + s) * (nt * 32 * kDigits) + c * 32);
+        uint4 x[2][2], y[2][2];   // digit, half of the slab
+#pragma unroll
+        for (int d = 0; d < 2; ++d)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                x[d][h] = __ldg(a + d * (kPlaneA / 16) + (h ^ sa));
+                y[d][h] = __ldg(b + d * (nt * 2) + (h ^ sb));
+            }
+        auto pair = [](uint32_t lead, uint32_t next) {   // two entries' |v| - 1/2, not negative
+            const float2 u = __half22float2(*reinterpret_cast<const __half2 *>(&lead)), w = __half22float2(*reinterpret_cast<const __half2 *>(&next));
+            return make_float2(fmaxf(fabsf(fmaf(256.0f, u.x, w.x)) - 0.5f, 0.0f), fmaxf(fabsf(fmaf(256.0f, u.y, w.y)) - 0.5f, 0.0f));
+        };
+        auto quad = [&](const uint4 &x0, const uint4 &x1, const uint4 &y0, const uint4 &y1) {
+            const uint32_t xl[4] = {x0.x, x0.y, x0.z, x0.w}, xn[4] = {x1.x, x1.y, x1.z, x1.w};
+            const uint32_t yl[4] = {y0.x, y0.y, y0.z, y0.w}, yn[4] = {y1.x, y1.y, y1.z, y1.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 u = pair(xl[q], xn[q]), v = pair(yl[q], yn[q]);
+                sum = fmaf(u.x, v.x, fmaf(u.y, v.y, sum));
+            }
+        };
+        quad(x[0][0], x[1][0], y[0][0], y[1][0]);
+        quad(x[0][1], x[1][1], y[0][1], y[1][1]);
+    }
+    return sum;
+}
+
+// Outputs that are small against the largest entries of their fibres (Left): four
+// columns of 32 rows, by W warps.  The digit sum stands where the leading digits, in the
+// slab with the column's largest entry, show terms that add up to 2^-kWeak of the
+// fibres' 2^exponents (a zero crossing of a smooth state has them, but none that is big
+// in both fibres).  The others become FMA chains.  (accumulate: all of them; their
+// digit sums were not added.)
+//   Few of them: sixteen lanes for an output, each with eight entries on their way.
+// Many (graded operands): a lane per row, the columns' chains over every fourth slab (in
+// each of four warps), first those whose bounds are within 2^-24 of the largest, then
+// those that are not beyond 2^-56 of the sums so far.  The FP64 pipe bounds that: a
+// DFMA of a warp takes its quarter of the SM 64 clocks.  W does not change a sum's
+// order.
+constexpr int kFew = 32, kSettleThreads = 128;
+struct SettleShared {
+    uint32_t keep[4];
+    int most[4][32];
+    double part[4][4][32];   // warp, column, row
+};
+template <int W>
+__device__ __forceinline__ void settle(const GProd &p, const Left &g, SettleShared &sh)
+{
+    const uint32_t all = 0xffffffffu;
+    const int tid = threadIdx.x % (32 * W), warp = tid / 32, lane = tid % 32;
+    const int S = p.slabs, ncat = p.ncat, spc = S / ncat, n = p.n, nt = p.nt;
+    const int mi = g.mi, ni = g.ni / 4, m0 = g.ni % 4 * 32, c = g.c;
+    const int64_t I = p.I, IB = p.IB, entry = g.entry;
+    auto place = [&](int row, int64_t &x, int64_t &y) {   // a row's first entry, its output in the first column
+        const int64_t rg = p.r0 + (int64_t)mi * kRowBlock + m0 + row;
+        const int64_t ro = (rg | I) >> 32 ? rg / I : (int64_t)((uint32_t)rg / (uint32_t)I);
+        x = entry * p.sA + ro * (I * n) + (rg - ro * I);
+        y = entry * p.sOut + ro * (I * p.cols) + (rg - ro * I) + I * (ni * nt + c);
+    };
+    auto column = [&](int j) {   // first entry of a column of L
+        const uint32_t col = (uint32_t)min(ni * nt + c + j, p.cols - 1), o = col / (uint32_t)IB;
+        return entry * p.sB + o * (IB * n) + (col - o * (uint32_t)IB);
+    };
+    auto put = [&](int64_t y, int j, double t) {
+        double *o = p.out + y + I * j;
+        *o = p.accumulate ? __dadd_rn(*o, t) : t;
+    };
+    uint32_t words[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        words[j] = g.words[j];
+        if (words[j] && !p.accumulate && (W == 1 || j == warp)) {
+            const uint8_t *const A = p.A + (entry * p.mtiles + mi) * S * kStageA, *const B = p.B + (entry * p.ntiles + ni) * S * (nt * 32 * kDigits);
+            const int w = __ldg(p.eB + (entry * p.ntiles + ni) * nt + c + j), s = (w >> 16) % spc;
+            if constexpr (W == 1) {
+                // (graded operands: the slab's bound says no as soon)
+                const int er = (int16_t)__ldg(p.eA + (entry * p.mtiles + mi) * kRowBlock + m0 + lane);
+                int b = 0;
+                for (int t = 0; t < ncat; ++t)
+                    b = max(b, (int)__ldg(p.cA + ((entry * p.mtiles + mi) * S + t * spc + s) * kRowBlock + m0 + lane) +
+                                   (int)__ldg(p.cB + ((entry * p.ntiles + ni) * S + t * spc + s) * nt + c + j));
+                // 16 ncat <= 96 products below 2^(b - 2046)
+                if (!__any_sync(all, (words[j] >> lane & 1) && b - 2046 + 7 > er + (int16_t)w - kWeak)) continue;
+            }
+            words[j] &= __ballot_sync(all, leading_terms(p, A, B, spc, s, m0 + lane, c + j) < 1.001f * (float)(1 << (28 - kWeak)));
+        }
+    }
+    if constexpr (W > 1) {
+        __syncthreads();   // (the outputs before are done with the shared memory)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (tid == 32 * j) sh.keep[j] = words[j];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) words[j] = sh.keep[j];
+    }
+    const int count = __popc(words[0]) + __popc(words[1]) + __popc(words[2]) + __popc(words[3]);
+    if (count == 0) return;
+    if (count <= kFew) {
+        constexpr int step = 16, share = 32 * W / step;
+        const int sub = tid % step;
+        for (int first = 0; first < count; first += share) {
+            int mine = min(first + tid / step, count - 1), j = 0;   // (the last one again where they run out)
+            while (mine >= __popc(words[j])) mine -= __popc(words[j++]);
+            int64_t xs, ys;
+            place((int)__fns(words[j], 0, mine + 1), xs, ys);
+            const int64_t ls = column(j);
+            double total = 0.0;
+            for (int t = 0; t < ncat; ++t) {
+                const double *x = p.X[t] + xs, *l = p.L[t] + ls;
+                double sum = 0.0;
+                for (int k0 = sub; k0 - sub < n; k0 += 8 * step) {
+                    double xv[8], lv[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int k = k0 + i * step;
+                        xv[i] = k < n ? x[I * k] : 0.0;
+                        lv[i] = k < n ? l[IB * k] : 0.0;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (k0 - sub + i * step < n) sum = fma(xv[i], lv[i], sum);
+                }
+                total = fma(p.sc[t], sum, total);
+            }
+#pragma unroll
+            for (int w = step / 2; w; w /= 2) total += __shfl_xor_sync(all, total, w);
+            if (sub == 0 && first + tid / step < count) put(ys, j, total);
+        }
+        return;
+    }
+    uint32_t weak = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) weak |= (words[j] >> lane & 1) << j;
+    const uint16_t *ca = p.cA + (entry * p.mtiles + mi) * S * kRowBlock + m0 + lane, *cb = p.cB + (entry * p.ntiles + ni) * S * nt + c;
+    // products of slab s in these columns are below 2^(bound - 2046); 0: all zero
+    auto bound = [&](int s) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(cb + s * nt));
+        const uint32_t r = __ldg(ca + s * kRowBlock);
+        const uint32_t b = max(max(words[0] ? v.x & 0xFFFFu : 0u, words[1] ? v.x >> 16 : 0u),
+                               max(words[2] ? v.y & 0xFFFFu : 0u, words[3] ? v.y >> 16 : 0u));
+        return weak && r && b ? (int)(r + b) : 0;
+    };
+    int most = 0;
+#pragma unroll 4
+    for (int s = warp; s < S; s += W) most = max(most, bound(s));
+    if constexpr (W > 1) {
+        sh.most[warp][lane] = most;
+        __syncthreads();
+        most = max(max(sh.most[0][lane], sh.most[1][lane]), max(sh.most[2][lane], sh.most[3][lane]));
+    }
+    int64_t xs, ys;
+    place(lane, xs, ys);
+    // lane: two entries of a slab of column lane / 8
+    const int64_t ls = column(lane / 8);
+    const int ki = lane % 8 * 2, from = max(most - 24, 1);
+    int floor = from;   // slabs of a smaller bound do not matter (yet)
+    double total[4] = {};
+    for (int pass = 0; pass < 2; ++pass) {
+        double half[4] = {}, quarter[4] = {};   // (W = 1) parts 0 (+ 1), part 2
+#pragma unroll 1
+        for (int first = W == 1 ? 0 : warp; first < (W == 1 ? 4 : warp + 1); ++first) {
+            double mine[4] = {}, sum[4] = {};
+            int t = 0;
+            for (int s = first; s < S; s += 4) {
+                const int b = bound(s), u = s / spc;
+                if (!__any_sync(all, b && b >= floor) || (pass && __any_sync(all, b >= from))) continue;
+                if (u != t) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        mine[j] = fma(p.sc[t], sum[j], mine[j]);
+                        sum[j] = 0.0;
+                    }
+                    t = u;
+                }
+                const int k0 = (s - u * spc) * kSlab;
+                const double *x = p.X[u] + xs, *l = p.L[u] + ls;
+                double xv[kSlab];
+#pragma unroll
+                for (int i = 0; i < kSlab; ++i) xv[i] = weak && k0 + i < n ? x[I * (k0 + i)] : 0.0;
+                const double l0 = k0 + ki < n ? l[IB * (k0 + ki)] : 0.0, l1 = k0 + ki + 1 < n ? l[IB * (k0 + ki + 1)] : 0.0;
+#pragma unroll
+                for (int i = 0; i < kSlab; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (words[j]) sum[j] = fma(xv[i], __shfl_sync(all, i & 1 ? l1 : l0, j * 8 + i / 2), sum[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                mine[j] = fma(p.sc[t], sum[j], mine[j]);
+                if constexpr (W > 1) {
+                    sh.part[warp][j][lane] = mine[j];
+                } else if (words[j]) {
+                    if (first == 0) half[j] = mine[j];
+                    else if (first == 1) half[j] += mine[j];
+                    else if (first == 2) quarter[j] = mine[j];
+                    else total[j] += half[j] + (quarter[j] + mine[j]);
+                }
+            }
+        }
+        if constexpr (W > 1) {
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (words[j]) total[j] += (sh.part[0][j][lane] + sh.part[1][j][lane]) + (sh.part[2][j][lane] + sh.part[3][j][lane]);
+            __syncthreads();
+        }
+        // S slabs of 16 products below 2^(b - 2046) are below 2^-56 of |total|
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (pass == 0 && (weak >> j & 1)) {
+                const int e = total[j] == 0.0 ? -100000 : ilogb(total[j]);
+                floor = min(floor, e - 56 + 2046 - 4 - (32 - __clz(S)));
+            }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if ((W == 1 || j == warp) && (weak >> j & 1)) put(ys, j, total[j]);
+}
+
+// A kernel of its own because what is left to it clusters: settled by the CTA of their
+// tile, ten groups of outputs took 240k clocks where the other CTAs took 40k.  A block
+// takes a group where they are few (latency), each of its warps one where they are many.
+__global__ void __launch_bounds__(kSettleThreads, 4) k_settle(const __grid_constant__ GArgs a)
+{
+    __shared__ SettleShared sh;
+    pdl_trigger();
+    pdl_wait();
+    const int items = *a.nleft;
+    if (items <= 2 * (int)gridDim.x) {
+        for (int i = blockIdx.x; i < items; i += gridDim.x) settle<4>(a.p[a.left[i].prod], a.left[i], sh);
+    } else {
+        for (int i = blockIdx.x * 4 + threadIdx.x / 32; i < items; i += gridDim.x * 4) settle<1>(a.p[a.left[i].prod], a.left[i], sh);
+    }
 }
 
 __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_constant__ GArgs a)
@@ -538,24 +855,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
         for (int u = blockIdx.x; u < tiles; u += gridDim.x) {
             int be, mi, ni;
             const GProd &p = find_tile(a, u, q, be, mi, ni);
-            const int nt = p.nt, hc = nt / 4;
+            const int nt = p.nt, hc = nt / 4, cw = part * hc;   // the warp's first column in the tile
             const int64_t r = (int64_t)mi * kRowBlock + m;
             const bool row_ok = r < p.rows;
-            // exponents and addresses while the MMAs run
-            const int c0 = ni * nt + part * hc;
-            const int er = row_ok ? __ldg(p.eA + (int64_t)be * p.mtiles * kRowBlock + r) : 0;
-            const int ec = lane < hc && c0 + lane < p.cols ? __ldg(p.eB + (int64_t)be * p.ntiles * nt + c0 + lane) : 0;
-            // a column of the warp's that is not finite: every row takes the slow form
-            const bool odd_col = __any_sync(0xffffffffu, ec >= kInfRow);
+            const int c0 = ni * nt + cw;
             const int64_t rg = p.r0 + r, ro = (rg | p.I) >> 32 ? rg / p.I : (int64_t)((uint32_t)rg / (uint32_t)p.I);
             double *const out = p.out + be * p.sOut + ro * (p.I * p.cols) + (rg - ro * p.I) + p.I * c0;
+            // exponents, and where the columns have their largest entries, while the MMAs run
+            const int er = row_ok ? (int16_t)__ldg(p.eA + (int64_t)be * p.mtiles * kRowBlock + r) : 0;
+            const int wc = lane < hc && c0 + lane < p.cols ? __ldg(p.eB + (int64_t)be * p.ntiles * nt + c0 + lane) : 0;
+            // a column of the warp's that is not finite: every row takes the slow form
+            const bool odd_col = __any_sync(0xffffffffu, (int16_t)wc >= kInfRow);
             long long P[kEpiCols], Q[kEpiCols];
             for (int s0 = 0; s0 < p.slabs; s0 += kChunkSlabs) {
                 ok = ok && __all_sync(0xffffffffu, bar_wait(TFULL, tphase, abort_flag, a.wait_limit));
                 if (!ok) break;
                 tphase ^= 1u;
                 tc_after();
-                const uint32_t tq = tmem + (uint32_t)(part * hc) + ((uint32_t)(quarter * 32) << 16);
+                const uint32_t tq = tmem + (uint32_t)cw + ((uint32_t)(quarter * 32) << 16);
                 if (s0 == 0) drain<false>(tq, (uint32_t)nt, hc, P, Q);
                 else drain<true>(tq, (uint32_t)nt, hc, P, Q);
                 tc_before();
@@ -564,6 +881,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
             const bool odd = !ok || odd_col || er >= kInfRow;
             // (every lane takes part in the shuffles of the column exponents)
             if (!__all_sync(0xffffffffu, odd)) {
+                uint32_t weak = 0;   // columns whose sums are small against their fibres
+                const bool mine = row_ok && !odd;
 #pragma unroll
                 for (int g = 0; g < kEpiCols / 4; ++g) {
                     if (g * 4 < hc && c0 + g * 4 < p.cols) {
@@ -572,10 +891,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                         int e[4];
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            e[j] = er + __shfl_sync(0xffffffffu, ec, g * 4 + j) - 58;
+                            e[j] = er + (int16_t)__shfl_sync(0xffffffffu, wc, g * 4 + j) - 58;
                             const Rounded y = round_sum(P[g * 4 + j], Q[g * 4 + j], e[j]);
                             const uint32_t x = (uint32_t)(y.E + 1022);   // biased exponent - 1
                             rare |= x >= 2045u;
+                            if (y.E < e[j] + 58 - kWeak) weak |= 1u << (g * 4 + j);
                             z[j] = __hiloint2double((int)((y.hi + (x << 20)) | y.sign), (int)y.lo);
                         }
                         if (rare) {
@@ -592,7 +912,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                             }
                         }
                         double *o = out + p.I * (g * 4);
-                        if (!row_ok || odd) continue;
+                        if (!mine) continue;
                         if (c0 + g * 4 + 3 < p.cols && !p.accumulate) {
                             if (p.I == 1 && ((uintptr_t)o & 31) == 0) {
                                 asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(o), "d"(z[0]), "d"(z[1]),
@@ -607,16 +927,78 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                         } else {
 #pragma unroll
                             for (int j = 0; j < 4; ++j)
-                                if (c0 + g * 4 + j < p.cols) o[p.I * j] = p.accumulate ? __dadd_rn(o[p.I * j], z[j]) : z[j];
+                                if (c0 + g * 4 + j < p.cols) {
+                                    // (weak sums are not added: settle does that)
+                                    if (!p.accumulate) o[p.I * j] = z[j];
+                                    else if (er == kZeroRow || !(weak >> (g * 4 + j) & 1)) o[p.I * j] = __dadd_rn(o[p.I * j], z[j]);
+                                }
                         }
                     }
+                }
+                if (!mine || er == kZeroRow) weak = 0;
+                // Small by cancellation, or because the terms are?  The digits stand where
+                // an entry is big in both fibres, in the slab where the column has its
+                // largest (of any concatenated operand).
+                uint32_t hold = 0;   // (lane: column) rows left to settle
+                uint32_t cols = __reduce_or_sync(0xffffffffu, weak);
+                if (cols && !p.accumulate) {
+                    const int S = p.slabs, spc = S / p.ncat, s = (wc >> 16) % spc;
+                    const uint16_t *const ma = p.mA + ((int64_t)be * p.mtiles + mi) * S * kRowBlock + m;
+                    const uint16_t *const mb = p.mB + ((int64_t)be * p.ntiles + ni) * S * nt + cw + lane;
+                    for (int t0 = 0; t0 < p.ncat; t0 += 3) {
+                        uint32_t b[3];
+#pragma unroll
+                        for (int t = 0; t < 3; ++t)
+                            b[t] = (cols >> lane & 1) && t0 + t < p.ncat ? __ldg(mb + (int64_t)((t0 + t) * spc + s) * nt) : 0u;
+                        // (columns that have it in the same slab together)
+                        for (uint32_t left = cols; left;) {
+                            const int at = __shfl_sync(0xffffffffu, s, __ffs((int)left) - 1);
+                            uint32_t same = __ballot_sync(0xffffffffu, s == at) & left, r[3];
+                            left &= ~same;
+#pragma unroll
+                            for (int t = 0; t < 3; ++t) r[t] = t0 + t < p.ncat ? __ldg(ma + (int64_t)((t0 + t) * spc + at) * kRowBlock) : 0u;
+                            for (; same; same &= same - 1) {
+                                const int j = __ffs((int)same) - 1;
+                                uint32_t found = 0;
+#pragma unroll
+                                for (int t = 0; t < 3; ++t) found |= r[t] & __shfl_sync(0xffffffffu, b[t], j);
+                                if (found) weak &= ~(1u << j);
+                            }
+                        }
+                    }
+                    cols = __reduce_or_sync(0xffffffffu, weak);
+                }
+                for (; cols; cols &= cols - 1) {
+                    const int j = __ffs((int)cols) - 1;
+                    const bool zero = (int16_t)__shfl_sync(0xffffffffu, wc, j) == kZeroRow;
+                    const uint32_t rows = __ballot_sync(0xffffffffu, !zero && c0 + j < p.cols && (weak >> j & 1));
+                    if (lane == j) hold = rows;
+                }
+                const uint32_t some = __ballot_sync(0xffffffffu, hold);
+                if (some) {
+                    // (groups of four columns, a lane each)
+                    const uint32_t groups = (some | some >> 1 | some >> 2 | some >> 3) & 0x1111u;
+                    int at = lane == 0 ? atomicAdd(a.nleft, __popc(groups)) : 0;
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(groups & ((1u << (lane & ~3)) - 1));
+                    if (lane < 16 && (groups >> (lane & ~3) & 1)) {
+                        Left &g = a.left[at];
+                        g.words[lane % 4] = hold;
+                        if (lane % 4 == 0) {
+                            g.prod = (uint16_t)q;
+                            g.c = (uint16_t)(cw + lane);
+                            g.entry = be;
+                            g.mi = mi;
+                            g.ni = ni * 4 + quarter;
+                        }
+                    }
+                    __syncwarp();
                 }
             }
             if (odd && row_ok) {
                 // non-finite entries, or a wait gave up (every later output of this warp)
 #pragma unroll 1
                 for (int j = 0; j < hc && c0 + j < p.cols; ++j) {
-                    const int e = __ldg(p.eB + (int64_t)be * p.ntiles * nt + c0 + j);
+                    const int e = (int16_t)__ldg(p.eB + (int64_t)be * p.ntiles * nt + c0 + j);
                     const double z = er == kNanRow || e == kNanRow ? __longlong_as_double(0x7FF8000000000000LL)
                                                                    : fma_chain(p, be, rg, c0 + j);
                     double *o = out + p.I * j;
@@ -711,6 +1093,10 @@ GProd to_gprod(const Product &s)
     p.B = s.ib.data;
     p.eA = s.ia.exps;
     p.eB = s.ib.exps;
+    p.mA = s.ia.masks;
+    p.mB = s.ib.masks;
+    p.cA = s.ia.codes;
+    p.cB = s.ib.codes;
     p.out = s.out;
     p.slabs = s.ia.slabs;
     p.nt = s.ib.rb;
@@ -770,10 +1156,11 @@ bool use_digits(int64_t rows, int n, int count)
 }
 
 template <int E>
-static void split_as(const View *v, const Image *im, int count, cudaStream_t st)
+static void split_as(const View *v, const Image *im, int count, int *reset, cudaStream_t st)
 {
     SplitArgs a{};
     a.count = count;
+    a.reset = reset;
     bool wide = false;
     int warps = 1;
     for (int q = 0; q < count; ++q) warps = std::max(warps, split_warps(im[q].slabs));
@@ -791,18 +1178,18 @@ static void split_as(const View *v, const Image *im, int count, cudaStream_t st)
     else pdl_launch(k_digits<int, E>, grid, block, 0, st, a);
 }
 
-void launch_split(const View *v, const Image *im, int count, cudaStream_t st)
+void launch_split(const View *v, const Image *im, int count, int *reset, cudaStream_t st)
 {
     // Where eight entries per thread leave half of the SMs' warps empty, four: a
     // chain of dependent work half as long (301 x 150, 150 x 301 and their matrices
     // 8.4 -> 7.0 us; eighteen tensors of 96^3, with warps for all SMs, 45 -> 49 us).
     int64_t threads = 0;
     for (int q = 0; q < count; ++q) threads += im[q].rows * v[q].batch * im[q].slabs * (kSlab / 8);
-    if (threads < (int64_t)kSms * 512) split_as<4>(v, im, count, st);
-    else split_as<8>(v, im, count, st);
+    if (threads < (int64_t)kSms * 512) split_as<4>(v, im, count, reset, st);
+    else split_as<8>(v, im, count, reset, st);
 }
 
-void launch_products(const Product *s, int count, long long wait_limit, cudaStream_t st)
+int launch_products(const Product *s, int count, uint8_t *left, long long wait_limit, cudaStream_t st)
 {
     static std::atomic<uint64_t> ready{0};   // devices whose shared-memory limit is raised
     int dev = 0;
@@ -819,8 +1206,12 @@ void launch_products(const Product *s, int count, long long wait_limit, cudaStre
         a.first[q + 1] = a.first[q] + a.p[q].mtiles * a.p[q].ntiles * s[q].A.batch;
     }
     const int tiles = a.first[count];
-    if (tiles == 0) return;
+    if (tiles == 0) return 0;
+    a.nleft = (int *)left;
+    a.left = (Left *)(left + kAlign);
     pdl_launch(k_digit_products, dim3(std::min(tiles, kSms)), dim3(kThreads), kSmem, st, a);
+    pdl_launch(k_settle, dim3((int)std::min<int64_t>(kSms * 4, (int64_t)tiles * 64)), dim3(kSettleThreads), 0, st, a);
+    return 2;
 }
 
 void launch_products_fma(const Product *s, int count, cudaStream_t st)
@@ -869,12 +1260,12 @@ View matrix_view(int64_t n, const double *L, int transpose, double scale)
 size_t scratch_bytes(int64_t N, int64_t n, int count, int cat, bool matrices)
 {
     const int slabs = slabs_of((int)n, cat);
-    const size_t a = aligned(image_bytes(N / n, kRowBlock, slabs) + sizeof(int) * pad_rows(N / n, kRowBlock));
+    const size_t a = aligned(image_total(N / n, kRowBlock, slabs) + left_bytes(N / n, (int)n, 1));
     // (the padding to whole tiles is below 64 columns)
-    const size_t b = matrices ? aligned(image_bytes(n + 64, 1, slabs) + sizeof(int) * (n + 64)) : 0;
+    const size_t b = matrices ? aligned(image_total(n + 64, 1, slabs)) : 0;
     // beyond 1 GiB a launch fills the GPU many times over: row blocks cost nothing
     const size_t most = (size_t)1 << 30;
-    return std::min(count * a, std::max(most, 2 * a / (pad_rows(N / n, kRowBlock) / kRowBlock) + kAlign)) + count * b;
+    return kAlign + std::min(count * a, std::max(most, 2 * a / (pad_rows(N / n, kRowBlock) / kRowBlock) + kAlign)) + count * b;
 }
 
 namespace {
@@ -898,7 +1289,7 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
         View sv[kMaxProd];
         Image si[kMaxProd];
         int np = 0, ns = 0;
-        size_t used = 0;
+        size_t used = 0, lists = kAlign;   // (from the start of the scratch) images; at its end: left outputs
         double flops = 0.0;
         auto place = [&](const View &v, int rb, Image &im) {   // scratch for v's image; false: no room
             for (int q = 0; q < ns; ++q)
@@ -910,9 +1301,8 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
             im.slabs = slabs_of(v.n, v.ncat);
             im.rows = v.rows;
             const size_t all = image_total(v, rb);
-            if (used + all > c.ws_bytes || ns == kMaxProd) return false;
-            im.data = c.ws + used;
-            im.exps = (int *)(im.data + image_bytes(v.rows, rb, im.slabs) * v.batch);
+            if (used + lists + all > c.ws_bytes || ns == kMaxProd) return false;
+            im.place(c.ws + used, v.batch);
             used += all;
             sv[ns] = v;
             si[ns++] = im;
@@ -920,11 +1310,13 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
         };
         auto add = [&](const Product &q, bool with_b) {
             Product t = q;
-            const size_t u0 = used;
+            const size_t u0 = used, l0 = lists;
             const int n0 = ns;
-            if ((with_b && !place(t.B, tile_cols(t.A.rows, (int)t.B.rows, many, slabs_of(t.A.n, t.A.ncat)), t.ib)) ||
+            lists += left_bytes(t.A.rows, (int)t.B.rows, t.A.batch);
+            if (used + lists > c.ws_bytes || (with_b && !place(t.B, tile_cols(t.A.rows, (int)t.B.rows, many, slabs_of(t.A.n, t.A.ncat)), t.ib)) ||
                 !place(t.A, kRowBlock, t.ia)) {
                 used = u0;
+                lists = l0;
                 ns = n0;
                 return false;
             }
@@ -935,14 +1327,13 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
         auto flush = [&] {
             if (ns) {
                 if (c.prof) c.prof->begin(st, 1, 0.0);
-                launch_split(sv, si, ns, st);
+                launch_split(sv, si, ns, (int *)(c.ws + (c.ws_bytes - lists) / kAlign * kAlign), st);
                 if (c.prof) c.prof->end(st);
                 ++launches;
             }
             if (c.prof) c.prof->begin(st, 1, flops);
-            launch_products(p, np, c.wait_limit, st);
+            launches += launch_products(p, np, c.ws + (c.ws_bytes - lists) / kAlign * kAlign, c.wait_limit, st);
             if (c.prof) c.prof->end(st);
-            ++launches;
         };
         int j = i;
         if (digits)
@@ -957,10 +1348,10 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
         bool done = false;
         if (digits && ps[i].A.batch == 1) {
             Product t = ps[i];
-            const size_t per = image_bytes(kRowBlock, kRowBlock, slabs_of(t.A.n, t.A.ncat)) + sizeof(int) * kRowBlock;
+            const size_t per = image_total(kRowBlock, kRowBlock, slabs_of(t.A.n, t.A.ncat)) + left_bytes(kRowBlock, (int)t.B.rows, 1);
             const bool ok = t.ib.data || place(t.B, tile_cols(t.A.rows, (int)t.B.rows, 1, slabs_of(t.A.n, t.A.ncat)), t.ib);
-            if (ok && used + per + kAlign <= c.ws_bytes) {
-                const int64_t fit = (int64_t)((c.ws_bytes - used - kAlign) / per) * kRowBlock;
+            if (ok && used + per + 2 * kAlign <= c.ws_bytes) {
+                const int64_t fit = (int64_t)((c.ws_bytes - used - 2 * kAlign) / per) * kRowBlock;
                 const size_t u0 = used;
                 for (int64_t r = 0; r < ps[i].A.rows; r += fit) {
                     Product part = t;
@@ -968,6 +1359,7 @@ int run_products(const Context &c, const Product *ps, int count, cudaStream_t st
                     part.A.rows = std::min(fit, t.A.rows - r);
                     if (r) ns = 0;   // B's image stays
                     used = u0;
+                    lists = kAlign;
                     np = 0;
                     flops = 0.0;
                     add(part, false);

@@ -30,13 +30,17 @@ struct View {
 
 // The digit image of a view: blocks of `rb` rows; per block and slab the
 // eight digit planes [rb][kSlab] in FP16, swizzled as the tensor core reads
-// them; one exponent per row.  A batch's images follow one another, each in
-// whole blocks.
+// them; per row its exponent (low half) and the slab of its largest entry.  Per block,
+// slab and row also a mask, a bit per entry that is big against the exponent, and a
+// code, the slab's own magnitude.  A batch's images follow one another, each in whole
+// blocks; so do its exponents, its masks and its codes.
 struct Image {
     uint8_t *data;
     int *exps;
+    uint16_t *masks, *codes;
     int rb, slabs;
     int64_t rows;
+    void place(uint8_t *at, int batch);
 };
 
 // out(r, i) (+)= sum over the contraction of A(r, k) B(i, k); element (r, i)
@@ -53,10 +57,31 @@ struct Product {
 
 inline int slabs_of(int n, int ncat) { return ncat * ((n + kSlab - 1) / kSlab); }
 inline int64_t pad_rows(int64_t rows, int rb) { return (rows + rb - 1) / rb * rb; }
-// data and exponents
+// data
 inline size_t image_bytes(int64_t rows, int rb, int slabs)
 {
     return (size_t)pad_rows(rows, rb) * slabs * kSlab * 2 * kDigits;
+}
+
+// data, exponents, masks and codes of one image
+inline size_t image_total(int64_t rows, int rb, int slabs)
+{
+    return image_bytes(rows, rb, slabs) + sizeof(int) * pad_rows(rows, rb) * (1 + slabs);
+}
+inline void Image::place(uint8_t *at, int batch)
+{
+    data = at;
+    exps = (int *)(data + image_bytes(rows, rb, slabs) * batch);
+    masks = (uint16_t *)(exps + pad_rows(rows, rb) * batch);
+    codes = masks + pad_rows(rows, rb) * slabs * batch;
+}
+
+// room for what the digit products of `rows` x `cols` outputs may leave to the FMA
+// chains: 32 bytes for each four columns of 32 rows of a tile (and, once for a launch,
+// kAlign for their count)
+inline size_t left_bytes(int64_t rows, int cols, int batch)
+{
+    return (size_t)pad_rows(rows, kRowBlock) * ((cols + 63) / 4 + 1) * batch;
 }
 
 // cycles a pipeline wait may take (the test hook DS_WAIT_LIMIT_CYCLES, else ~2 s)
@@ -88,11 +113,11 @@ int run_products(const Context &c, const Product *p, int count, cudaStream_t st)
 // tensors of N points and n x n matrices, `cat` concatenated terms, matrices
 // cut per call or not.
 size_t scratch_bytes(int64_t N, int64_t n, int count, int cat, bool matrices);
-// An image's bytes with its exponents, for a batch.
+// A view's images in all, for a batch.
 inline size_t image_total(const View &v, int rb)
 {
     const int slabs = v.ncat * ((v.n + kSlab - 1) / kSlab);
-    return aligned((image_bytes(v.rows, rb, slabs) + sizeof(int) * pad_rows(v.rows, rb)) * v.batch);
+    return aligned(image_total(v.rows, rb, slabs) * v.batch);
 }
 // Y = X x_1 L_1 ... x_d L_d (L^T with transpose), chained mode products; tmp:
 // two tensors of N = prod n entries.
@@ -103,11 +128,12 @@ void tucker_f64(const Context &c, int d, const int64_t *n, const double *X, doub
 // columns in a launch of `products` products of `rows` rows and `slabs` slabs.
 int tile_cols(int64_t rows, int cols, int products, int slabs);
 
-// Digit images of up to kMaxProd views (one launch).
-void launch_split(const View *v, const Image *im, int count, cudaStream_t st);
-// Up to kMaxProd products on their images (one launch).
-void launch_products(const Product *p, int count, long long wait_limit, cudaStream_t st);
-// The same products on the FP64 pipe, one thread per output (one launch;
+// Digit images of up to kMaxProd views (one launch); reset: null, or a word to zero.
+void launch_split(const View *v, const Image *im, int count, int *reset, cudaStream_t st);
+// Up to kMaxProd products on their images.  left: a word, zero before the call, and
+// from kAlign on the products' left_bytes.  Returns the number of launches.
+int launch_products(const Product *p, int count, uint8_t *left, long long wait_limit, cudaStream_t st);
+// The same products on the FP64 pipe, four threads per output (one launch;
 // images unused): small products.
 void launch_products_fma(const Product *p, int count, cudaStream_t st);
 // Whether a mode product of this shape runs on the tensor cores (count

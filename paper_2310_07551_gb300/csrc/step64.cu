@@ -208,12 +208,11 @@ void sums_create(Sums64 &e, const ds_phi_set *s, int64_t N, const std::vector<Su
     }
     for (size_t q = 0; q < views.size(); ++q) {
         Image &im = ims[q];
-        im.data = e.mats + offs[q];
-        im.exps = (int *)(im.data + mm::image_bytes(im.rows, im.rb, im.slabs));
+        im.place(e.mats + offs[q], 1);
         e.images[view_key(views[q])] = im;
     }
     for (size_t q = 0; q < views.size(); q += mm::kMaxProd)
-        mm::launch_split(&views[q], &ims[q], (int)std::min<size_t>(mm::kMaxProd, views.size() - q), st);
+        mm::launch_split(&views[q], &ims[q], (int)std::min<size_t>(mm::kMaxProd, views.size() - q), nullptr, st);
     cudaStreamSynchronize(st);
 }
 
