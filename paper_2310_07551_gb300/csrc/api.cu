@@ -619,28 +619,36 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
                         poff += grid->n[mu] * grid->n[mu];
                     }
         s->P_count = poff;
-        cudaError_t e1 = pool_alloc(&s->A_dev, sizeof(double) * Acount, st);
-        cudaError_t e2 = pool_alloc(&s->tri_dev, sizeof(double) * toff, st);
-        cudaError_t e3 = pool_alloc(&s->P_dev, sizeof(double) * poff, st);
-        // derivatives feed the adjoint's diffusion-scaling gradient (EXPRK3DS_REAL only)
-        cudaError_t e4 = scheme == DS_EXPRK3DS_REAL ? pool_alloc(&s->dP_dev, sizeof(double) * poff, st) : cudaSuccess;
-        cudaError_t e5 = cudaSuccess, e6 = cudaSuccess;
-        if (scheme == DS_EXPRK3DS_CPLX) {
-            e5 = pool_alloc(&s->Pim_dev, sizeof(double) * poff, st);
-            int64_t moff = 0;
+        // one block: the matrices, their bands, the phi-matrices, their derivatives (which
+        // feed the adjoint's diffusion-scaling gradient; EXPRK3DS_REAL only) or imaginary parts
+        int64_t moff = 0;
+        if (scheme == DS_EXPRK3DS_CPLX)
             for (int c = 0; c < 2; ++c)
                 for (int q = 0; q < kSlots; ++q)
                     for (int i = 0; i < s->k; ++i) {
                         s->Mf_off[c][q][i] = moff;
                         moff += 2 * grid->n[d - 1] * grid->n[d - 1];
                     }
-            e6 = pool_alloc(&s->Mf_dev, sizeof(double) * moff, st);
-        }
-        if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess ||
-            e5 != cudaSuccess || e6 != cudaSuccess) {
+        int64_t count = 0;
+        auto part = [&](int64_t entries) {   // on a 256-byte boundary
+            const int64_t at = count;
+            count += (entries + 31) / 32 * 32;
+            return at;
+        };
+        const int64_t oA = part(Acount), oT = part(toff), oP = part(poff), oD = part(scheme == DS_EXPRK3DS_REAL ? poff : 0),
+                      oI = part(scheme == DS_EXPRK3DS_CPLX ? poff : 0), oM = part(moff);
+        if (device_alloc(&s->block, sizeof(double) * count) != cudaSuccess) {
             cudaGetLastError();
             ds_phi_set_destroy(s);
             return fail(DS_ERR_OOM, "phi-set device allocation");
+        }
+        s->A_dev = s->block + oA;
+        s->tri_dev = s->block + oT;
+        s->P_dev = s->block + oP;
+        if (scheme == DS_EXPRK3DS_REAL) s->dP_dev = s->block + oD;
+        if (scheme == DS_EXPRK3DS_CPLX) {
+            s->Pim_dev = s->block + oI;
+            s->Mf_dev = s->block + oM;
         }
         cudaMemcpyAsync(s->A_dev, hA.data(), sizeof(double) * Acount, cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(s->tri_dev, htri.data(), sizeof(double) * toff, cudaMemcpyHostToDevice, st);
@@ -711,10 +719,8 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
 ds_status ds_phi_set_destroy(ds_phi_set *s)
 {
     if (!s) return DS_OK;
-    // any stream may still read the matrices
-    cudaDeviceSynchronize();
-    for (double *p : {s->A_dev, s->tri_dev, s->P_dev, s->dP_dev, s->Pim_dev, s->Mf_dev})
-        if (p) cudaFreeAsync(p, nullptr);
+    // waits for the work of the block's device, whichever is current
+    cudaFree(s->block);
     delete s;
     return DS_OK;
 }

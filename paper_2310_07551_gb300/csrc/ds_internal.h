@@ -78,7 +78,7 @@ ds_status check_device();
                               std::string(#expr) + ": " + cudaGetErrorString(_e));   \
     } while (0)
 
-// Stream-ordered device memory for workspaces of one call and for phi-sets, from
+// Stream-ordered device memory for workspaces of one call, from
 // a pool of the library's own per device.  The pool keeps up to 1 GiB between
 // calls (the default pool gives everything back at each synchronisation, and
 // mapping it again took 0.9 of the 1.3 ms of a 256^3 split-BF16 Tucker operator);
@@ -237,6 +237,7 @@ struct ds_phi_set {
     int k;
     double tau;
     ds::SplitCoeffs co[2];                  // [l-1]
+    double *block = nullptr;                // device memory of all that follows
     double *A_dev = nullptr;                // copy of A, column-major blocks
     int64_t A_off[2][ds::kMaxD];
     bool tridiag[2];                        // every A_{c,mu} tridiagonal
