@@ -867,7 +867,7 @@ ds_status ds_plan_create(const ds_grid *grid, const ds_params *params, const ds_
             cudaEventCreateWithFlags(&p->ev_in, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&p->ev_out, cudaEventDisableTiming) != cudaSuccess)
             return cleanup(DS_ERR_CUDA, "stream/event creation");
-        if (cudaMalloc(&p->status, sizeof(DevStatus)) != cudaSuccess)
+        if (device_alloc(&p->status, sizeof(DevStatus)) != cudaSuccess)
             return cleanup(DS_ERR_OOM, "status word");
         cudaMemset(p->status, 0, sizeof(DevStatus));
         if (precision == DS_PREC_F64) {

@@ -194,13 +194,13 @@ void sums_create(Sums64 &e, const ds_phi_set *s, int64_t N, const std::vector<Su
                 kron_products(s, nullptr, nullptr, mu, tr, N, ps);
                 phase(ps);
             }
-    if (scratch && cudaMalloc(&e.ctx.ws, scratch) == cudaSuccess) {
+    if (scratch && device_alloc(&e.ctx.ws, scratch) == cudaSuccess) {
         e.ctx.ws_bytes = scratch;
     } else {
         cudaGetLastError();
         e.ctx.ws = nullptr;
     }
-    if (views.empty() || cudaMalloc(&e.mats, bytes) != cudaSuccess) {
+    if (views.empty() || device_alloc(&e.mats, bytes) != cudaSuccess) {
         cudaGetLastError();
         e.mats = nullptr;
         e.images.clear();

@@ -3974,8 +3974,8 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
                 oq += 3 * nm;
             }
         }
-        if (cudaMalloc(&mp->bands, sizeof(float) * hb.size()) != cudaSuccess ||
-            (fx && cudaMalloc(&mp->cf4, sizeof(float4) * cq.size()) != cudaSuccess)) {
+        if (device_alloc(&mp->bands, sizeof(float) * hb.size()) != cudaSuccess ||
+            (fx && device_alloc(&mp->cf4, sizeof(float4) * cq.size()) != cudaSuccess)) {
             cudaGetLastError();
             cudaFree(mp->bands);
             delete mp;
@@ -4024,15 +4024,15 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
         mixed_plan_destroy(mp);
         return fail(s, msg);
     };
-    if (cudaMalloc(&mp->Pp, sizeof(bf16) * total) != cudaSuccess ||
-        cudaMalloc(&mp->Fp, sizeof(bf16) * 2 * npF * N) != cudaSuccess ||
-        cudaMalloc(&mp->Dp, sizeof(bf16) * (fx_all ? 8 : 6) * N) != cudaSuccess ||
-        cudaMalloc(&mp->Z1, sizeof(bf16) * 6 * npF * k * N) != cudaSuccess ||
-        (d >= 3 && cudaMalloc(&mp->Z2, sizeof(bf16) * 6 * npF * k * N) != cudaSuccess) ||
-        cudaMalloc(&mp->incF, sizeof(float) * 6 * N) != cudaSuccess ||
-        cudaMalloc(&mp->incD, sizeof(float) * 2 * N) != cudaSuccess ||
-        (fx_all && (cudaMalloc(&mp->incFlo, sizeof(float) * 6 * N) != cudaSuccess ||
-                    cudaMalloc(&mp->incDlo, sizeof(float) * 2 * N) != cudaSuccess))) {
+    if (device_alloc(&mp->Pp, sizeof(bf16) * total) != cudaSuccess ||
+        device_alloc(&mp->Fp, sizeof(bf16) * 2 * npF * N) != cudaSuccess ||
+        device_alloc(&mp->Dp, sizeof(bf16) * (fx_all ? 8 : 6) * N) != cudaSuccess ||
+        device_alloc(&mp->Z1, sizeof(bf16) * 6 * npF * k * N) != cudaSuccess ||
+        (d >= 3 && device_alloc(&mp->Z2, sizeof(bf16) * 6 * npF * k * N) != cudaSuccess) ||
+        device_alloc(&mp->incF, sizeof(float) * 6 * N) != cudaSuccess ||
+        device_alloc(&mp->incD, sizeof(float) * 2 * N) != cudaSuccess ||
+        (fx_all && (device_alloc(&mp->incFlo, sizeof(float) * 6 * N) != cudaSuccess ||
+                    device_alloc(&mp->incDlo, sizeof(float) * 2 * N) != cudaSuccess))) {
         cudaGetLastError();
         return cleanup(DS_ERR_OOM, "split-BF16 workspace");
     }
@@ -4049,9 +4049,9 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
                 ps_tot += (int64_t)2 * (g == 0 ? 3 * k : k) * mp->n[mu];
             }
         mp->fx_nslots = fx_all ? fx_base(2, d) + 2 + 2 * (d - 1) : 2 + 6 * (d - 1);
-        if (cudaMalloc(&mp->fxs, sizeof(FxScales)) != cudaSuccess ||
-            cudaMalloc(&mp->pscale, sizeof(float) * ps_tot) != cudaSuccess ||
-            cudaMalloc(&mp->fx_jobs, sizeof(FxMatJob) * 2 * 3 * k) != cudaSuccess) {
+        if (device_alloc(&mp->fxs, sizeof(FxScales)) != cudaSuccess ||
+            device_alloc(&mp->pscale, sizeof(float) * ps_tot) != cudaSuccess ||
+            device_alloc(&mp->fx_jobs, sizeof(FxMatJob) * 2 * 3 * k) != cudaSuccess) {
             cudaGetLastError();
             return cleanup(DS_ERR_OOM, "FX tables");
         }
@@ -4171,7 +4171,7 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
         for (int g = 0; g < 3; ++g)
             for (int mu = 0; mu < d; ++mu)
                 for (int w = 0; w < 2; ++w) need(mp->C[g][mu][w]);
-        if (ws_elems > 0 && cudaMalloc(&mp->part_ws, sizeof(float) * ws_elems) != cudaSuccess) {
+        if (ws_elems > 0 && device_alloc(&mp->part_ws, sizeof(float) * ws_elems) != cudaSuccess) {
             cudaGetLastError();
             return cleanup(DS_ERR_OOM, "split-K workspace");
         }
@@ -4186,8 +4186,8 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
                         any = any || streamk_ok(mp->C[g][mu][w]);
                     }
             if (any) {
-                if (cudaMalloc(&mp->sk_ws, sizeof(float) * streamk_ws_floats()) != cudaSuccess ||
-                    cudaMalloc(&mp->sk_cnt, sizeof(int) * units) != cudaSuccess) {
+                if (device_alloc(&mp->sk_ws, sizeof(float) * streamk_ws_floats()) != cudaSuccess ||
+                    device_alloc(&mp->sk_cnt, sizeof(int) * units) != cudaSuccess) {
                     cudaGetLastError();
                     return cleanup(DS_ERR_OOM, "stream-K workspace");
                 }
@@ -4196,7 +4196,7 @@ ds_status mixed_plan_create(const ds_grid *grid, const ds_phi_set *set, DevStatu
         }
         // scratch state for the fused epilogues while timing
         double *Us = nullptr;
-        if (cudaMalloc(&Us, sizeof(double) * 2 * N) != cudaSuccess) {
+        if (device_alloc(&Us, sizeof(double) * 2 * N) != cudaSuccess) {
             cudaGetLastError();
             return cleanup(DS_ERR_OOM, "autotuning scratch");
         }
@@ -4566,7 +4566,7 @@ ds_status mixed_group_create(const std::vector<MixedPlan *> &mps, const std::vec
     G->slots.resize(3 * d);
     auto dev_copy = [&](auto **dst, const auto &v) {
         using T = typename std::decay_t<decltype(v)>::value_type;
-        if (cudaMalloc((void **)dst, sizeof(T) * v.size()) != cudaSuccess) {
+        if (device_alloc((void **)dst, sizeof(T) * v.size()) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
@@ -4578,7 +4578,7 @@ ds_status mixed_group_create(const std::vector<MixedPlan *> &mps, const std::vec
     int64_t Ntot = 0;
     for (auto *mp : mps) Ntot += mp->N;
     double *Us = nullptr;
-    if (cudaMalloc(&Us, sizeof(double) * 2 * Ntot) != cudaSuccess) {
+    if (device_alloc(&Us, sizeof(double) * 2 * Ntot) != cudaSuccess) {
         cudaGetLastError();
         delete G;
         return fail(DS_ERR_OOM, "grouped launch scratch state");
@@ -5031,7 +5031,7 @@ static DevStatus *global_status()
     static DevStatus *s = nullptr;
     static std::once_flag once;
     std::call_once(once, [] {
-        if (cudaMalloc(&s, sizeof(DevStatus)) == cudaSuccess) cudaMemset(s, 0, sizeof(DevStatus));
+        if (device_alloc(&s, sizeof(DevStatus)) == cudaSuccess) cudaMemset(s, 0, sizeof(DevStatus));
         else s = nullptr;
     });
     return s;
