@@ -332,7 +332,9 @@ ds_status ds_integrate_ckpt(ds_plan *plan, double *U, int64_t nsteps, int64_t ck
  *   Errors: DS_ERR_INVALID_ARG, DS_ERR_UNSUPPORTED (non-FP64 plan), DS_ERR_OOM
  *   (the first call allocates a workspace of 22 N doubles and the
  *   intermediates, the first with dscale 6 N and theirs: intermediates of as
- *   many Tucker operators as fit 2 GiB, of one term where memory is short). */
+ *   many Tucker operators as fit 2 GiB, of one term where memory is short;
+ *   where there is no room for the latter dscale costs d more Tucker
+ *   operators per Tucker operator instead). */
 ds_status ds_step_backward(ds_plan *plan, const double *U, const double *lam, double *lam_n,
                            double *dparams, double *dscale, void *stream);
 

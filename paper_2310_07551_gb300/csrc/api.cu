@@ -1037,11 +1037,10 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
             zt = per_op / s->k;
             if (device_alloc(&p->tws, sizeof(double) * (6 + zt) * N) != cudaSuccess) {
                 cudaGetLastError();
-                p->tws = nullptr;
-                return fail(DS_ERR_OOM, "adjoint workspace");
+                p->tws = nullptr;   // one derivative matrix at a time, in the workspace there is
             }
         }
-        sums_create(p->tsums, s, N,
+        if (p->tws) sums_create(p->tsums, s, N,
                     {{SumKind::tangent, {0, 1, 3}}, {SumKind::tangent, {2}}, {SumKind::tangent, {4}}},
                     p->tws + 6 * N, zt, p->st);
     }
@@ -1080,20 +1079,38 @@ ds_status ds_step_backward(ds_plan *p, const double *U, const double *lam, doubl
         // each sum against the adjoint of its stage; b <- D3 = g(U3) - g(U)
         launch_dot_kterm_f64(m, N, U, F, lF, dscale, st);
         launch_gdiff_f64(m, N, U, U3, b, st);
-        double *o[3] = {p->tws, p->tws + 2 * N, p->tws + 4 * N};
-        auto dot = [&](int slot, const double *t, const double *adj) {
-            for (int c = 0; c < 2; ++c)
-                launch_dot_accum_f64(N, adj + c * N, t + c * N, kSlotW[slot] * tau, dscale + c, st);
-        };
-        const int q[3] = {0, 1, 3};
-        sums_f64(p, p->tsums, SumKind::tangent, 3, q, F, o, false, st);
-        dot(0, o[0], lU2);
-        dot(1, o[1], lU3);
-        dot(3, o[2], lam);
-        sum_f64(p, p->tsums, SumKind::tangent, 2, D2, o[0], false, st);
-        sum_f64(p, p->tsums, SumKind::tangent, 4, b, o[1], false, st);
-        dot(2, o[0], lU3);
-        dot(4, o[1], lam);
+        if (p->tws) {
+            double *o[3] = {p->tws, p->tws + 2 * N, p->tws + 4 * N};
+            auto dot = [&](int slot, const double *t, const double *adj) {
+                for (int c = 0; c < 2; ++c)
+                    launch_dot_accum_f64(N, adj + c * N, t + c * N, kSlotW[slot] * tau, dscale + c, st);
+            };
+            const int q[3] = {0, 1, 3};
+            sums_f64(p, p->tsums, SumKind::tangent, 3, q, F, o, false, st);
+            dot(0, o[0], lU2);
+            dot(1, o[1], lU3);
+            dot(3, o[2], lam);
+            sum_f64(p, p->tsums, SumKind::tangent, 2, D2, o[0], false, st);
+            sum_f64(p, p->tsums, SumKind::tangent, 4, b, o[1], false, st);
+            dot(2, o[0], lU3);
+            dot(4, o[1], lam);
+        } else {
+            // short of memory: d more Tucker operators per term, in the workspace there is
+            auto dots = [&](int slot, const double *X, const double *adj) {
+                const SplitCoeffs &co = s->co[kSlotEll[slot] - 1];
+                for (int c = 0; c < 2; ++c)
+                    for (int i = 0; i < co.k; ++i)
+                        for (int md = 0; md < s->d; ++md) {
+                            run_partial(e, c, slot, i, md, X + c * N, a, &p->prof, st);
+                            launch_dot_accum_f64(N, adj + c * N, a, kSlotW[slot] * tau * co.eta[i], dscale + c, st);
+                        }
+            };
+            dots(0, F, lU2);
+            dots(1, F, lU3);
+            dots(2, D2, lU3);
+            dots(3, F, lam);
+            dots(4, b, lam);
+        }
     }
     // K^T lam_F into F's storage
     if (tri) {

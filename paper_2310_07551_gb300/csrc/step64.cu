@@ -255,6 +255,20 @@ int run_sums(const Sums64 &e, SumKind kind, const SumOp *ops, int count, Prof *p
     return launches;
 }
 
+int run_partial(const Sums64 &e, int c, int slot, int term, int md, const double *X, double *out, Prof *prof, cudaStream_t st)
+{
+    const ds_phi_set *s = e.set;
+    int launches = 0;
+    for (int mu = 0; mu < s->d; ++mu) {
+        std::vector<Product> ps(1);
+        ps[0].A = mm::tensor_view(s->d, s->n, mu, mu ? e.z + e.N * ((mu - 1) % 2) : X);
+        ps[0].B = mm::matrix_view(s->n[mu], (mu == md ? s->dP_dev : s->P_dev) + s->P_off[c][slot][term][mu], 0);
+        ps[0].out = mu == s->d - 1 ? out : e.z + e.N * (mu % 2);
+        launches += run_phase(e, ps, prof, st);
+    }
+    return launches;
+}
+
 int run_kronsum(const Sums64 &e, const double *X, double *Y, int transpose, Prof *prof, cudaStream_t st)
 {
     int launches = 0;

@@ -47,6 +47,9 @@ void sums_create(Sums64 &e, const ds_phi_set *s, int64_t N, const std::vector<Su
 void sums_destroy(Sums64 &e);
 // Runs independent sums of one kind; returns the number of launches.
 int run_sums(const Sums64 &e, SumKind kind, const SumOp *ops, int count, Prof *prof, cudaStream_t st);
+// One term's Tucker operator with its derivative matrix in mode `md`, of component c:
+// out = T(X, P with P_md -> dP_md).  Two intermediates; returns the number of launches.
+int run_partial(const Sums64 &e, int c, int slot, int term, int md, const double *X, double *out, Prof *prof, cudaStream_t st);
 // Y_c = sum_mu X_c x_mu A_{c,mu} (transposed: A^T) for both components
 int run_kronsum(const Sums64 &e, const double *X, double *Y, int transpose, Prof *prof, cudaStream_t st);
 
