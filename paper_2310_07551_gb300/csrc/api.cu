@@ -243,6 +243,7 @@ Stencil stencil_of(const ds_phi_set *s, int c)
         t.di[mu] = base + t.n[mu];
         t.up[mu] = base + 2 * t.n[mu];
         t.sum[mu] = base + 3 * t.n[mu];
+        t.plain[mu] = mu < s->d && s->plain[c][mu];
     }
     return t;
 }
@@ -602,12 +603,17 @@ ds_status ds_phi_setup_ex(const ds_grid *grid, const double *A, int a_on_device,
                 const int64_t n = grid->n[mu];
                 const double *Am = hA.data() + s->A_off[c][mu];
                 double *lo = htri.data() + s->tri_off[c][mu], *di = lo + n, *up = lo + 2 * n, *sum = lo + 3 * n;
+                bool plain = false;
                 for (int64_t i = 0; i < n; ++i) {
                     lo[i] = i > 0 ? Am[i + n * (i - 1)] : 0.0;
                     di[i] = Am[i + n * i];
                     up[i] = i + 1 < n ? Am[i + n * (i + 1)] : 0.0;
-                    sum[i] = (lo[i] + di[i]) + up[i];
+                    // twice the diagonal: a row's error stays within three times what
+                    // its own terms' roundings are (diffusion: the bands equal it)
+                    plain = plain || !(fabs(lo[i]) + fabs(up[i]) <= 2.0 * fabs(di[i]));
                 }
+                for (int64_t i = 0; i < n; ++i) sum[i] = plain ? di[i] : (lo[i] + di[i]) + up[i];
+                s->plain[c][mu] = plain;
             }
         // phi-matrix layout [c][slot][i][mu]
         int64_t poff = 0;

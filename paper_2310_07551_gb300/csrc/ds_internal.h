@@ -114,7 +114,8 @@ struct Stencil {
     int d;
     int64_t n[kMaxD];
     const double *lo[kMaxD], *di[kMaxD], *up[kMaxD];   // device arrays of length n_mu
-    const double *sum[kMaxD];                          // row sums (lo + di) + up
+    const double *sum[kMaxD];                          // row sums (lo + di) + up; plain: di
+    bool plain[kMaxD];                                 // no differences (see stencil_point)
 };
 
 // F = K U + g(U) for both components (FP64, stencil).  Returns #launches.
@@ -241,7 +242,8 @@ struct ds_phi_set {
     double *A_dev = nullptr;                // copy of A, column-major blocks
     int64_t A_off[2][ds::kMaxD];
     bool tridiag[2];                        // every A_{c,mu} tridiagonal
-    double *tri_dev = nullptr;              // [c][mu][4][n_mu]: bands, row sums
+    bool plain[2][ds::kMaxD];               // its outer bands outweigh the diagonal somewhere
+    double *tri_dev = nullptr;              // [c][mu][4][n_mu]: bands, Stencil::sum
     int64_t tri_off[2][ds::kMaxD];
     double *P_dev = nullptr;                // FP64 phi-matrices, column-major blocks
     double *dP_dev = nullptr;               // their derivatives w.r.t. a scaling of A (same offsets)

@@ -239,7 +239,10 @@ namespace {
 // K U for one point of one component: each tridiagonal row as lo (u- - u) + up (u+ -
 // u) + (row sum) u, so that a constant state gives exactly zero where the rows sum
 // to zero, and neighbouring values lose nothing in their difference; all in one
-// chain of FMAs.  IT: 32-bit indices where the grid allows them.
+// chain of FMAs.  Where the outer bands outweigh the diagonal (advection) the
+// differences would bring in |lo| |u|, which the row itself does not have: such a
+// direction takes lo u- + up u+ + di u (plain; `sum` is its diagonal).  IT: 32-bit
+// indices where the grid allows them.
 template <typename IT>
 __device__ __forceinline__ double stencil_point(const Stencil &s, const double *U, IT p)
 {
@@ -251,8 +254,9 @@ __device__ __forceinline__ double stencil_point(const Stencil &s, const double *
         if (mu < s.d) {
             const IT nm = (IT)s.n[mu], q = rest / nm, i = rest - q * nm;
             rest = q;
-            if (i > 0) acc = fma(s.lo[mu][i], U[p - stride] - u, acc);
-            if (i + 1 < nm) acc = fma(s.up[mu][i], U[p + stride] - u, acc);
+            const double from = s.plain[mu] ? 0.0 : u;
+            if (i > 0) acc = fma(s.lo[mu][i], U[p - stride] - from, acc);
+            if (i + 1 < nm) acc = fma(s.up[mu][i], U[p + stride] - from, acc);
             const double rs = s.sum[mu][i];
             if (__double_as_longlong(rs)) acc = fma(rs, u, acc);
             stride *= nm;
