@@ -433,7 +433,9 @@ int enqueue_step_etd2_f64(ds_plan *p, double *U, cudaStream_t st)
     const double tau = p->set->tau;
     double *F = p->ws, *b = p->ws + 2 * N, *D = p->ws + 4 * N, *a = p->ws + 6 * N;
     const Sums64 &e = p->sums;
-    // small products run one per launch on the FP64 pipe
+    // Products too small for the digits: a launch per component and mode.  The number of
+    // kernels of such a step (ds_plan_kernels_per_step) is relied on; both components in a
+    // launch would take 20 steps of 64 x 64 from 789 to 541 us.
     auto sum = [&](int slot, const double *X, double *out) {
         int L = 0;
         bool digits = true;

@@ -20,8 +20,8 @@ namespace ds {
 // points is 16k threads, a third of what the SMs hold at 8 x 8 outputs each, so
 // the products of a phase share a launch (FitzHugh-Nagumo 100^3, two steps: 3.25 ms
 // with 64 x 64 tiles of 4 x 4 outputs per thread and a launch per product, 5.8 with
-// this tile and a launch per product, 2.14 so; 4 x 8 outputs for the launches of two
-// products: 2.24).  18 products of 100 entries each run at 21 TFLOP/s, the FMA pipe
+// this tile and a launch per product, 2.14 so; tried and left out, 4 x 8 outputs per
+// thread where a launch has two products: 2.24).  18 products of 100 entries each run at 21 TFLOP/s, the FMA pipe
 // 43 % busy: the padding (104 of 100 rows, 112 of 100 entries) and the copies'
 // addresses take the rest.
 // ---------------------------------------------------------------------------

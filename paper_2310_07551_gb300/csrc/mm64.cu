@@ -1124,12 +1124,12 @@ GProd to_gprod(const Product &s)
 
 int tile_cols(int64_t rows, int cols, int products, int slabs)
 {
-    // the width whose waves take the least: clocks per tile measured in the kernel,
-    // at 64 columns 1365 per slab (smem and L2 bound) and 6500 for the drain, at 48
-    // 1111 and 5100, at 32 900 and 3800, at 16 estimated
+    // the width whose waves take the least: clocks per tile of 6 and of 16 slabs over
+    // ten and fifty waves (15110 and 26818 at 64 columns, 12645 and 21823 at 48, 9219 and
+    // 16247 at 32, 6341 and 12415 at 16), as a share per slab and one per tile
     static const struct {
         int nt, slab, tile;
-    } kCost[] = {{64, 1365, 6500}, {48, 1111, 5100}, {32, 900, 3800}, {16, 750, 2800}};
+    } kCost[] = {{64, 1171, 8085}, {48, 918, 7138}, {32, 703, 5002}, {16, 607, 2696}};
     const int64_t mt = (rows + kRowBlock - 1) / kRowBlock * products;
     int best = 16;
     double least = 0.0;
@@ -1148,9 +1148,13 @@ int tile_cols(int64_t rows, int cols, int products, int slabs)
 
 bool use_digits(int64_t rows, int n, int count)
 {
+    // Up to 2^20 points ds_tucker_static gives the same bits as ds_tucker, and its 20 MiB
+    // hold the digits of a 1024 x 1024 matrix and of a row block, not of a larger one; so
+    // 2048 x 400 runs its long mode on the FP64 pipe, 2990 us (tiled FMA chains before:
+    // 5227).  Beyond, 4096, the dense scheme's largest matrix.
     const int most = rows * n > ((int64_t)1 << 20) ? 4096 : 1024;
-    // 1.5e6 FMAs take the FP64 pipe about as long as the two launches of a digit
-    // product take at least (7 and 9 + 5 us); row tiles of 128 that are mostly padding
+    // 1.5e6 FMAs take the FP64 pipe about as long as the launches of a digit
+    // product take at least (7, 9 + 5 and 3 us); row tiles of 128 that are mostly padding
     // move the line (twelve products of 64 x 64: 9 against 14 us)
     return n >= 12 && n <= most && rows >= 16 && (double)rows * n * n * count > 1.5e6 * std::max(1.0, 160.0 / rows);
 }
