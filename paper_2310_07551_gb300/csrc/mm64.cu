@@ -288,13 +288,15 @@ struct GProd {
     const double *X[kMaxCat], *L[kMaxCat];
     double sc[kMaxCat];
 };
-// Outputs of a tile that a drain leaves to k_settle: four columns (the first: c) of 32
-// rows (a lane quarter), words[j] the rows' bits in column c + j.
+// Outputs of a tile that a drain leaves to k_settle: column c of it, the rows of a lane
+// quarter that have a bit in `rows`; exps: the column's exponent and slab (Image::exps).
 struct Left {
     uint16_t prod, c;
     int entry, mi, ni;         // (ni: tile times four, plus the quarter)
-    uint32_t words[4];
+    uint32_t rows;
+    int exps;
 };
+static_assert(sizeof(Left) == 24, "as left_bytes has it");
 struct GArgs {
     int count;
     int first[kMaxProd + 1];   // prefix of tiles
@@ -525,23 +527,20 @@ __device__ __forceinline__ float leading_terms(const GProd &p, const uint8_t *A,
     return sum;
 }
 
-// Outputs that are small against the largest entries of their fibres (Left): four
-// columns of 32 rows, by W warps.  The digit sum stands where the leading digits, in the
-// slab with the column's largest entry, show terms that add up to 2^-kWeak of the
-// fibres' 2^exponents (a zero crossing of a smooth state has them, but none that is big
-// in both fibres).  The others become FMA chains.  (accumulate: all of them; their
-// digit sums were not added.)
+// Outputs that are small against the largest entries of their fibres (Left), by W warps.
+// The digit sum stands where the leading digits, in the slab with the column's largest
+// entry, show terms that add up to 2^-kWeak of the fibres' 2^exponents (a zero crossing
+// of a smooth state has them, but none that is big in both fibres).  The others become
+// FMA chains.  (accumulate: all of them; their digit sums were not added.)
 //   Few of them: sixteen lanes for an output, each with eight entries on their way.
-// Many (graded operands): a lane per row, the columns' chains over every fourth slab (in
-// each of four warps), first those whose bounds are within 2^-24 of the largest, then
-// those that are not beyond 2^-56 of the sums so far.  The FP64 pipe bounds that: a
-// DFMA of a warp takes its quarter of the SM 64 clocks.  W does not change a sum's
-// order.
-constexpr int kFew = 32, kSettleThreads = 128;
+// Many (graded operands): a lane per row, its chain over every fourth slab (in each of
+// four warps), first those whose bounds are within 2^-24 of the largest, then those that
+// are not beyond 2^-56 of the sums so far.  The FP64 pipe bounds that: a DFMA of a
+// warp takes its quarter of the SM 64 clocks.  W does not change a sum's order.
+constexpr int kFew = 8, kSettleThreads = 128, kSettleBlocks = 4;   // (blocks per SM)
 struct SettleShared {
-    uint32_t keep[4];
     int most[4][32];
-    double part[4][4][32];   // warp, column, row
+    double part[4][32];   // warp, row
 };
 template <int W>
 __device__ __forceinline__ void settle(const GProd &p, const Left &g, SettleShared &sh)
@@ -550,61 +549,42 @@ __device__ __forceinline__ void settle(const GProd &p, const Left &g, SettleShar
     const int tid = threadIdx.x % (32 * W), warp = tid / 32, lane = tid % 32;
     const int S = p.slabs, ncat = p.ncat, spc = S / ncat, n = p.n, nt = p.nt;
     const int mi = g.mi, ni = g.ni / 4, m0 = g.ni % 4 * 32, c = g.c;
-    const int64_t I = p.I, IB = p.IB, entry = g.entry;
-    auto place = [&](int row, int64_t &x, int64_t &y) {   // a row's first entry, its output in the first column
+    const int64_t I = p.I, IB = p.IB, entry = g.entry, ta = entry * p.mtiles + mi, tb = entry * p.ntiles + ni;
+    uint32_t rows = g.rows;
+    if (!p.accumulate) {
+        const int s = (g.exps >> 16) % spc, ec = (int16_t)g.exps;
+        bool look = true;
+        if constexpr (W == 1) {
+            // (graded operands: the slab's bound says no as soon)
+            const int er = (int16_t)__ldg(p.eA + ta * kRowBlock + m0 + lane);
+            int b = 0;
+            for (int t = 0; t < ncat; ++t)
+                b = max(b, (int)__ldg(p.cA + (ta * S + t * spc + s) * kRowBlock + m0 + lane) + (int)__ldg(p.cB + (tb * S + t * spc + s) * nt + c));
+            // 16 ncat <= 96 products below 2^(b - 2046)
+            look = __any_sync(all, (rows >> lane & 1) && b - 2046 + 7 > er + ec - kWeak);
+        }
+        if (look)
+            rows &= __ballot_sync(all, leading_terms(p, p.A + ta * S * kStageA, p.B + tb * S * (nt * 32 * kDigits), spc, s, m0 + lane, c) <
+                                           1.001f * (float)(1 << (28 - kWeak)));
+        if (rows == 0) return;
+    }
+    auto place = [&](int row, int64_t &x, int64_t &y) {   // a row's first entry, its output
         const int64_t rg = p.r0 + (int64_t)mi * kRowBlock + m0 + row;
         const int64_t ro = (rg | I) >> 32 ? rg / I : (int64_t)((uint32_t)rg / (uint32_t)I);
         x = entry * p.sA + ro * (I * n) + (rg - ro * I);
         y = entry * p.sOut + ro * (I * p.cols) + (rg - ro * I) + I * (ni * nt + c);
     };
-    auto column = [&](int j) {   // first entry of a column of L
-        const uint32_t col = (uint32_t)min(ni * nt + c + j, p.cols - 1), o = col / (uint32_t)IB;
-        return entry * p.sB + o * (IB * n) + (col - o * (uint32_t)IB);
-    };
-    auto put = [&](int64_t y, int j, double t) {
-        double *o = p.out + y + I * j;
-        *o = p.accumulate ? __dadd_rn(*o, t) : t;
-    };
-    uint32_t words[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        words[j] = g.words[j];
-        if (words[j] && !p.accumulate && (W == 1 || j == warp)) {
-            const uint8_t *const A = p.A + (entry * p.mtiles + mi) * S * kStageA, *const B = p.B + (entry * p.ntiles + ni) * S * (nt * 32 * kDigits);
-            const int w = __ldg(p.eB + (entry * p.ntiles + ni) * nt + c + j), s = (w >> 16) % spc;
-            if constexpr (W == 1) {
-                // (graded operands: the slab's bound says no as soon)
-                const int er = (int16_t)__ldg(p.eA + (entry * p.mtiles + mi) * kRowBlock + m0 + lane);
-                int b = 0;
-                for (int t = 0; t < ncat; ++t)
-                    b = max(b, (int)__ldg(p.cA + ((entry * p.mtiles + mi) * S + t * spc + s) * kRowBlock + m0 + lane) +
-                                   (int)__ldg(p.cB + ((entry * p.ntiles + ni) * S + t * spc + s) * nt + c + j));
-                // 16 ncat <= 96 products below 2^(b - 2046)
-                if (!__any_sync(all, (words[j] >> lane & 1) && b - 2046 + 7 > er + (int16_t)w - kWeak)) continue;
-            }
-            words[j] &= __ballot_sync(all, leading_terms(p, A, B, spc, s, m0 + lane, c + j) < 1.001f * (float)(1 << (28 - kWeak)));
-        }
-    }
-    if constexpr (W > 1) {
-        __syncthreads();   // (the outputs before are done with the shared memory)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (tid == 32 * j) sh.keep[j] = words[j];
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < 4; ++j) words[j] = sh.keep[j];
-    }
-    const int count = __popc(words[0]) + __popc(words[1]) + __popc(words[2]) + __popc(words[3]);
-    if (count == 0) return;
+    auto put = [&](int64_t y, double t) { p.out[y] = p.accumulate ? __dadd_rn(p.out[y], t) : t; };
+    const uint32_t col = (uint32_t)(ni * nt + c), co = col / (uint32_t)IB;
+    const int64_t ls = entry * p.sB + co * (IB * n) + (col - co * (uint32_t)IB);   // the column's first entry
+    int64_t xs, ys;
+    const int count = __popc(rows);
     if (count <= kFew) {
         constexpr int step = 16, share = 32 * W / step;
         const int sub = tid % step;
         for (int first = 0; first < count; first += share) {
-            int mine = min(first + tid / step, count - 1), j = 0;   // (the last one again where they run out)
-            while (mine >= __popc(words[j])) mine -= __popc(words[j++]);
-            int64_t xs, ys;
-            place((int)__fns(words[j], 0, mine + 1), xs, ys);
-            const int64_t ls = column(j);
+            const int mine = first + tid / step;
+            place((int)__fns(rows, 0, min(mine, count - 1) + 1), xs, ys);   // (the last one again where they run out)
             double total = 0.0;
             for (int t = 0; t < ncat; ++t) {
                 const double *x = p.X[t] + xs, *l = p.L[t] + ls;
@@ -625,109 +605,86 @@ __device__ __forceinline__ void settle(const GProd &p, const Left &g, SettleShar
             }
 #pragma unroll
             for (int w = step / 2; w; w /= 2) total += __shfl_xor_sync(all, total, w);
-            if (sub == 0 && first + tid / step < count) put(ys, j, total);
+            if (sub == 0 && mine < count) put(ys, total);
         }
         return;
     }
-    uint32_t weak = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) weak |= (words[j] >> lane & 1) << j;
-    const uint16_t *ca = p.cA + (entry * p.mtiles + mi) * S * kRowBlock + m0 + lane, *cb = p.cB + (entry * p.ntiles + ni) * S * nt + c;
-    // products of slab s in these columns are below 2^(bound - 2046); 0: all zero
+    const bool weak = rows >> lane & 1;
+    const uint16_t *ca = p.cA + ta * S * kRowBlock + m0 + lane, *cb = p.cB + tb * S * nt + c;
+    // products of slab s are below 2^(bound - 2046); 0: all zero
     auto bound = [&](int s) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(cb + s * nt));
-        const uint32_t r = __ldg(ca + s * kRowBlock);
-        const uint32_t b = max(max(words[0] ? v.x & 0xFFFFu : 0u, words[1] ? v.x >> 16 : 0u),
-                               max(words[2] ? v.y & 0xFFFFu : 0u, words[3] ? v.y >> 16 : 0u));
-        return weak && r && b ? (int)(r + b) : 0;
+        const int b = __ldg(cb + s * nt), r = __ldg(ca + s * kRowBlock);
+        return weak && r && b ? r + b : 0;
     };
     int most = 0;
-#pragma unroll 4
+#pragma unroll 8
     for (int s = warp; s < S; s += W) most = max(most, bound(s));
     if constexpr (W > 1) {
+        __syncthreads();   // (the outputs before are done with the shared memory)
         sh.most[warp][lane] = most;
         __syncthreads();
         most = max(max(sh.most[0][lane], sh.most[1][lane]), max(sh.most[2][lane], sh.most[3][lane]));
     }
-    int64_t xs, ys;
     place(lane, xs, ys);
-    // lane: two entries of a slab of column lane / 8
-    const int64_t ls = column(lane / 8);
-    const int ki = lane % 8 * 2, from = max(most - 24, 1);
+    const int from = max(most - 24, 1);
     int floor = from;   // slabs of a smaller bound do not matter (yet)
-    double total[4] = {};
+    double total = 0.0;
     for (int pass = 0; pass < 2; ++pass) {
-        double half[4] = {}, quarter[4] = {};   // (W = 1) parts 0 (+ 1), part 2
+        double half = 0.0, quarter = 0.0;   // (W = 1) parts 0 (+ 1), part 2
 #pragma unroll 1
         for (int first = W == 1 ? 0 : warp; first < (W == 1 ? 4 : warp + 1); ++first) {
-            double mine[4] = {}, sum[4] = {};
+            double mine = 0.0, sum = 0.0;
             int t = 0;
             for (int s = first; s < S; s += 4) {
                 const int b = bound(s), u = s / spc;
                 if (!__any_sync(all, b && b >= floor) || (pass && __any_sync(all, b >= from))) continue;
                 if (u != t) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        mine[j] = fma(p.sc[t], sum[j], mine[j]);
-                        sum[j] = 0.0;
-                    }
+                    mine = fma(p.sc[t], sum, mine);
+                    sum = 0.0;
                     t = u;
                 }
-                const int k0 = (s - u * spc) * kSlab;
-                const double *x = p.X[u] + xs, *l = p.L[u] + ls;
+                const int k0 = (s - u * spc) * kSlab, ki = lane % kSlab;
+                const double *x = p.X[u] + xs;
                 double xv[kSlab];
 #pragma unroll
                 for (int i = 0; i < kSlab; ++i) xv[i] = weak && k0 + i < n ? x[I * (k0 + i)] : 0.0;
-                const double l0 = k0 + ki < n ? l[IB * (k0 + ki)] : 0.0, l1 = k0 + ki + 1 < n ? l[IB * (k0 + ki + 1)] : 0.0;
+                const double lk = k0 + ki < n ? p.L[u][ls + IB * (k0 + ki)] : 0.0;
 #pragma unroll
-                for (int i = 0; i < kSlab; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (words[j]) sum[j] = fma(xv[i], __shfl_sync(all, i & 1 ? l1 : l0, j * 8 + i / 2), sum[j]);
+                for (int i = 0; i < kSlab; ++i) sum = fma(xv[i], __shfl_sync(all, lk, i), sum);
             }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                mine[j] = fma(p.sc[t], sum[j], mine[j]);
-                if constexpr (W > 1) {
-                    sh.part[warp][j][lane] = mine[j];
-                } else if (words[j]) {
-                    if (first == 0) half[j] = mine[j];
-                    else if (first == 1) half[j] += mine[j];
-                    else if (first == 2) quarter[j] = mine[j];
-                    else total[j] += half[j] + (quarter[j] + mine[j]);
-                }
+            mine = fma(p.sc[t], sum, mine);
+            if constexpr (W > 1) {
+                sh.part[warp][lane] = mine;
+            } else {
+                if (first == 0) half = mine;
+                else if (first == 1) half += mine;
+                else if (first == 2) quarter = mine;
+                else total += half + (quarter + mine);
             }
         }
         if constexpr (W > 1) {
             __syncthreads();
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (words[j]) total[j] += (sh.part[0][j][lane] + sh.part[1][j][lane]) + (sh.part[2][j][lane] + sh.part[3][j][lane]);
+            total += (sh.part[0][lane] + sh.part[1][lane]) + (sh.part[2][lane] + sh.part[3][lane]);
             __syncthreads();
         }
         // S slabs of 16 products below 2^(b - 2046) are below 2^-56 of |total|
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (pass == 0 && (weak >> j & 1)) {
-                const int e = total[j] == 0.0 ? -100000 : ilogb(total[j]);
-                floor = min(floor, e - 56 + 2046 - 4 - (32 - __clz(S)));
-            }
+        if (pass == 0 && weak) floor = min(floor, (total == 0.0 ? -100000 : ilogb(total)) - 56 + 2046 - 4 - (32 - __clz(S)));
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-        if ((W == 1 || j == warp) && (weak >> j & 1)) put(ys, j, total[j]);
+    if (warp == 0 && weak) put(ys, total);
 }
 
 // A kernel of its own because what is left to it clusters: settled by the CTA of their
 // tile, ten groups of outputs took 240k clocks where the other CTAs took 40k.  A block
-// takes a group where they are few (latency), each of its warps one where they are many.
-__global__ void __launch_bounds__(kSettleThreads, 4) k_settle(const __grid_constant__ GArgs a)
+// takes a column's where they are few (latency), each of its warps one where they are
+// many.  (301 x 150 four steps, late: 818 us, with four columns to a block 890; complex
+// 150 x 150 469, 496; the phi setup of 256 x 200, where they are many, 26.2 ms, 24.8.)
+__global__ void __launch_bounds__(kSettleThreads, kSettleBlocks) k_settle(const __grid_constant__ GArgs a)
 {
     __shared__ SettleShared sh;
     pdl_trigger();
     pdl_wait();
     const int items = *a.nleft;
-    if (items <= 2 * (int)gridDim.x) {
+    if (items <= 4 * (int)gridDim.x) {
         for (int i = blockIdx.x; i < items; i += gridDim.x) settle<4>(a.p[a.left[i].prod], a.left[i], sh);
     } else {
         for (int i = blockIdx.x * 4 + threadIdx.x / 32; i < items; i += gridDim.x * 4) settle<1>(a.p[a.left[i].prod], a.left[i], sh);
@@ -976,21 +933,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_digit_products(const __grid_con
                 }
                 const uint32_t some = __ballot_sync(0xffffffffu, hold);
                 if (some) {
-                    // (groups of four columns, a lane each)
-                    const uint32_t groups = (some | some >> 1 | some >> 2 | some >> 3) & 0x1111u;
-                    int at = lane == 0 ? atomicAdd(a.nleft, __popc(groups)) : 0;
-                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(groups & ((1u << (lane & ~3)) - 1));
-                    if (lane < 16 && (groups >> (lane & ~3) & 1)) {
-                        Left &g = a.left[at];
-                        g.words[lane % 4] = hold;
-                        if (lane % 4 == 0) {
-                            g.prod = (uint16_t)q;
-                            g.c = (uint16_t)(cw + lane);
-                            g.entry = be;
-                            g.mi = mi;
-                            g.ni = ni * 4 + quarter;
-                        }
-                    }
+                    int at = lane == 0 ? atomicAdd(a.nleft, __popc(some)) : 0;
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(some & ((1u << lane) - 1));
+                    if (hold) a.left[at] = {(uint16_t)q, (uint16_t)(cw + lane), be, mi, ni * 4 + quarter, hold, wc};
                     __syncwarp();
                 }
             }
@@ -1214,7 +1159,7 @@ int launch_products(const Product *s, int count, uint8_t *left, long long wait_l
     a.nleft = (int *)left;
     a.left = (Left *)(left + kAlign);
     pdl_launch(k_digit_products, dim3(std::min(tiles, kSms)), dim3(kThreads), kSmem, st, a);
-    pdl_launch(k_settle, dim3((int)std::min<int64_t>(kSms * 4, (int64_t)tiles * 64)), dim3(kSettleThreads), 0, st, a);
+    pdl_launch(k_settle, dim3((int)std::min<int64_t>(kSms * kSettleBlocks, (int64_t)tiles * 64)), dim3(kSettleThreads), 0, st, a);
     return 2;
 }
 

@@ -77,11 +77,11 @@ inline void Image::place(uint8_t *at, int batch)
 }
 
 // room for what the digit products of `rows` x `cols` outputs may leave to the FMA
-// chains: 32 bytes for each four columns of 32 rows of a tile (and, once for a launch,
-// kAlign for their count)
+// chains: 24 bytes for each column of 32 rows of a tile (and, once for a launch, kAlign
+// for their count)
 inline size_t left_bytes(int64_t rows, int cols, int batch)
 {
-    return (size_t)pad_rows(rows, kRowBlock) * ((cols + 63) / 4 + 1) * batch;
+    return (size_t)pad_rows(rows, kRowBlock) / 32 * 24 * (cols + 64) * batch;
 }
 
 // cycles a pipeline wait may take (the test hook DS_WAIT_LIMIT_CYCLES, else ~2 s)
