@@ -1,8 +1,8 @@
 // FP64 plans: a step's Tucker sums as phases of grouped mode products.  All
 // sums that share an input (every slot, term and component of the group on F)
-// advance one mode per phase, so a phase is two launches whatever their
-// number: the tensors' digit images, then the products.  The k terms of a sum
-// are one contraction in its last mode (concatenated over the terms, the
+// advance one mode per phase, so a phase is three launches whatever their
+// number: the tensors' digit images, the products, what those leave to FMA chains.
+// The k terms of a sum are one contraction in its last mode (concatenated over the terms, the
 // split weights eta folded into the matrices).
 #include <algorithm>
 
