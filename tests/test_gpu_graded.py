@@ -5,8 +5,8 @@ makes it, entry by entry, where its digits alone would lose it.
 Bound per output y = sum_k x_k l_k, S = sum_k |x_k| |l_k|.  An FMA chain of n entries is
 within n 2^-53 S, one rounding more for a term's weight.  The digit sum is one rounding
 (2^-53 |y|) and, per entry and in units of the fibres' 2^(ex + el), 2^-59.2 for the
-dropped digit products (7 pairs of at most 2^14 at 2^-76), 2^-58.6 for the rounding of
-the last classes and 2^-62 for the operands' own: below n 2^-57.7; it is kept only where
+dropped digit products (7 pairs of at most 2^14 at 2^-76), at most 2^-58.6 for what the
+last classes lose and 2^-62 for the operands' own: below n 2^-57.7; it is kept only where
 S is at least 2^-8 of that unit, so within n 2^-49.7 S."""
 import numpy as np
 import pytest
